@@ -51,7 +51,7 @@ SM_MAX_MHZ = 2070.0
 # (add + FMA + min = 3) includes is 1/(s-2) of an op per candidate here.
 OPS_PER_CANDIDATE = 2
 BK = BJ = 64              # the kernel's tile: 64 k by 64 columns
-# DRAM bytes of k_wavefront_res per interval-cost tile it copies in (64 x 64 pairs,
+# DRAM bytes of the min-plus kernel per interval-cost tile it copies in (64 x 64 pairs,
 # 34 816 B of C and Phi, plus the dp32 rows and minima that miss L2), from the committed
 # ncu capture of every launch of one solve at d = 16384; the benchmark launch is scaled
 # by the tiles it fetched (tile skipping leaves most tiles in HBM unread).
@@ -119,7 +119,7 @@ def executed_candidates(st, p, s, multipliers):
 def cost_mode_flags(E, d, s, free_bytes, share=0.6):
     """Interval-cost mode of the fast DP: the whole table resident when it fits in `share` of
     the free device memory, else band by band through a bounded buffer when that fits, else
-    the fused kernel (costs rebuilt by producer warps in every pass)."""
+    the kernel that rebuilds the costs panel by panel in every pass."""
     for flag in (E.RESIDENT_COSTS, E.STREAMED_COSTS):
         need = E.ecasq_workspace_size_flags(d, s, 1, flag)
         if 0 < need <= share * free_bytes:
@@ -425,7 +425,7 @@ def run_rows_mode(args):
 
 def run_pass_mode(args, cfg, x_np):
     """One DP pass of the configuration's vector at the --lambdas multipliers (resident
-    interval costs when they fit in 60 % of the free memory, else the fused kernel)."""
+    interval costs when they fit in 60 % of the free memory, else costs rebuilt in every pass)."""
     import torch
     import paper_2608_18147_gb300 as E
     s = cfg["s"]
@@ -635,7 +635,7 @@ def main():
                 "traffic_note": "DRAM bytes per launch: bytes per fetched cost tile from an ncu capture at "
                                 "d = 16384, times the tiles this launch fetched",
                 "tiles_fetched_per_launch": fetched_per_launch,
-                "kernel": "k_wavefront" if cost_mode_name(E, flags) == "fused" else "k_wavefront_res",
+                "kernel": "k_wavefront",
                 "peak_basis": "%d SMs (device attribute) x 128 FP32-pipe lanes (adds and mins share the issue "
                               "slots) x 2070 MHz max clock; of the 2-op count below" % n_sm,
                 "avg_launch_ms": dp_ms / max(dp_launches, 1), "launches": dp_launches,

@@ -62,21 +62,19 @@ typedef struct CUstream_st *ecasq_stream_t; /* same type as cudaStream_t */
                                      of tiles, 2.3 MB x ceil(d / 64); ecasq_workspace_size_flags with this flag) and
                                      the wavefront runs band by band; rebuilt in every pass.  RESIDENT_COSTS wins
                                      when both are given.  Results are the same as with either other mode. */
-#define ECASQ_ONE_PART_PUBLISH 128u /* fast DP with resident or streamed costs and 10 <= s <= 16: publish each column block
-                                     of the wavefront once, after all its layers, instead of in two parts (rows 2..8
-                                     after layer 8, then the rest); same results, for comparison */
-#define ECASQ_UNSEEDED_SEARCH 256u /* fast DP with resident or streamed costs and tile skipping (10 <= s <= 18, 27 <= s <= 34): in the
-                                     multiplier search, start every pass's tile skipping from scratch instead of from
-                                     the fp32 minima of the bracket's evaluated upper end (an upper bound of every
-                                     later pass's minima, Sec. 5's candidates being non-decreasing in lambda); same
-                                     results, for comparison */
+#define ECASQ_ONE_PART_PUBLISH 128u /* accepted, without effect: a column block's layers are shared one by one */
+#define ECASQ_UNSEEDED_SEARCH 256u /* fast DP with tile skipping: in the multiplier search, skip tiles by the fp32 minima a
+                                     pass finds itself, from bounds at every 32nd tile only, instead of also by the
+                                     fp32 minima of the bracket's evaluated upper end (an upper bound of every
+                                     later pass's minima, Sec. 5's candidates being non-decreasing in lambda) and
+                                     bounds at every fourth tile; same results, for comparison */
 #define ECASQ_TEST_SELF_SEED (1u << 29) /* test hook for the seeded tile skipping: with a fixed multiplier and resident
                                      or streamed costs, the pass runs twice, the second time seeded with the first
                                      one's fp32 minima (the seed then equals every output's minimum, the tightest
                                      start the seeding allows); results must equal those without the flag.
                                      ecasq_result_t.passes counts both.  Not for production use. */
 #define ECASQ_TEST_STALL (1u << 30) /* test hook for the bounded device waits: column block 0 of the fast DP's
-                                     wavefront is never published and the flag waits give up after 2^14 spins, so
+                                     wavefront is never published and the waits on it give up after 2^14 spins, so
                                      the call must return ECASQ_ETIMEOUT (nothing else) and leave the workspace
                                      usable by the next call.  Not for production use. */
 

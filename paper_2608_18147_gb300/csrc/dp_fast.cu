@@ -2,21 +2,17 @@
 //
 // Three stages per DP pass, for up to 8 multipliers at once:
 //
-// 1. k_wavefront / k_wavefront_res: an fp32 filter over the whole (k, j)
-//    triangle with every layer i = 3..s fused.  A persistent CTA owns a block of
-//    64 columns j and sweeps 64-wide tiles of k in increasing order; the tile
-//    k-block K may be used as soon as column block K has published all its
-//    layers (a flag with release/acquire order, bounded waits).  The interval
-//    costs C[k,j] and Phi[k,j] of a tile (App. E quantities rebuilt with
+// 1. k_wavefront: an fp32 filter over the whole (k, j) triangle with every layer
+//    i = 3..s in one cooperative launch, one persistent CTA per SM, in panels of 15
+//    column blocks of 64 (the phases are described at `panels` below).  The interval
+//    costs C[k,j] and Phi[k,j] of a 64 x 64 tile (App. E quantities rebuilt with
 //    compensated fp32 recurrences that add one point at a time, all terms
-//    non-negative, from a double-double anchor per tile and column) are either
-//    computed by two producer warps next to the consumers (k_wavefront), or
-//    computed once per call into a resident table (k_build_costs) and streamed
-//    in with bulk copies (k_wavefront_res, ECASQ_RESIDENT_COSTS); the values are
-//    bit-identical.  The consumer threads evaluate dp(i-1,k) + C + lambda' Phi
-//    for their (layer, column, multiplier) outputs with packed f32x2 adds and
-//    integer mins.  Per output the kernel keeps the fp32 minimum and up to two
-//    runs of tiles whose minimum came within the certified error band of it.
+//    non-negative, from a double-double anchor per tile and column) come from a
+//    table built once per call (ECASQ_RESIDENT_COSTS), from a bounded buffer that
+//    holds a band of column blocks (ECASQ_STREAMED_COSTS), or are built by the kernel
+//    itself a panel at a time; the values are bit-identical.  Per output the kernel
+//    keeps the fp32 minimum and up to two runs of tiles whose minimum came within the
+//    certified error band of it.
 // 2. k_need_layer (layers s down to 3): the outputs whose exact value the
 //    answer depends on.  eq. apx_final needs dp(i, p-1) for every i; an output
 //    resolved exactly needs the exact values of its band members in the layer
@@ -58,56 +54,27 @@ void timer_end(cudaStream_t st);
 
 constexpr int BJ = 64;         // columns per block
 constexpr int BK = 64;         // k per tile
-constexpr int LPT = 7;         // layers per consumer thread
-constexpr int JPT = 4;         // columns per consumer thread (stride 16)
-constexpr int NJQ = BJ / JPT;  // 16 column groups
-constexpr int NPROD = 64;      // producer threads: one per column of the block
+constexpr int NPROD = 64;      // threads that build a cost tile: one per column of the block
+constexpr int kTaskWords = 4;  // far tasks of a multiplier split: at most 32 of these words
 constexpr int PSTR = BK + 4;   // padded row stride (floats) of the interval-cost buffers
-constexpr int MAXCONS = 256;
+constexpr int MAXCONS = 512;   // threads of a wavefront CTA: every phase is latency-bound at 256
 constexpr int NMEM = 8;        // members kept inline per output
 constexpr int64_t kMaxFastP = (int64_t)1 << 20;
 constexpr uint32_t kSpinLimit = 1u << 26;
 constexpr uint32_t kTestSpinLimit = 1u << 14;  // the ECASQ_TEST_STALL hook: about 10-20 ms of spinning
 constexpr uint32_t kCopySpinLimit = 1u << 22;  // waits on bulk copies (microseconds when healthy)
-constexpr int kMdpMax = 36;  // block-minimum row stride bound (s + 1 rounded up to 4): tile skipping for s <= 35
 // Resident interval costs: per tile, C[64][PSTR] then Phi[64][PSTR] (the shared-memory layout).
 constexpr int kCostHalfFloats = BJ * PSTR;
 constexpr uint32_t kCostHalfBytes = (uint32_t)(kCostHalfFloats * sizeof(float));  // 17408, a multiple of 16
 constexpr size_t kCostTileFloats = 2 * (size_t)kCostHalfFloats;
 
-// Band of an output: up to two runs of tile indices K (< 2^14), tiles arriving in
-// increasing K (the diagonal block, K = J, last).  Low word: run 1 as
-// first << 16 | last; high word: run 2 the same way, 0 when absent (a second run
-// starts at a tile >= 2).  A tile within the band extends run 1 when it follows
-// run 1 directly and there is no run 2, else opens run 2, else extends run 2 to
-// itself (the gap is then scanned too: a superset, never a miss).  A tile below
-// the band restarts it: run 1 = [K, K], no run 2.
-__device__ __forceinline__ void band_update(uint32_t &w1, uint32_t &w2, bool rst, bool app, uint32_t K,
-                                            uint32_t KK) {
-    const bool has2 = w2 != 0u;
-    const bool ext1 = app && !has2 && ((w1 & 0xFFFFu) + 1u == K);
-    const uint32_t n1 = ext1 ? ((w1 & 0xFFFF0000u) | K) : w1;
-    const uint32_t n2 = (app && !ext1) ? (has2 ? ((w2 & 0xFFFF0000u) | K) : KK) : w2;
-    w1 = rst ? KK : n1;
-    w2 = rst ? 0u : n2;
-}
+// Band of an output: up to two runs of tile indices K (< 2^14), tiles appended in
+// increasing K (fold_panel).  Low word: run 1 as first << 16 | last; high word: run 2 the same way,
+// 0 when absent (a second run starts at a tile >= 2).  A tile within the band opens run 1,
+// or extends it when it follows run 1 directly and there is no run 2, else opens run 2, else
+// extends run 2 to itself (the gap is then scanned too: a superset, never a miss).  A tile
+// below the band restarts it: run 1 = [K, K], no run 2.
 __device__ __forceinline__ uint64_t band_pack(uint32_t w1, uint32_t w2) { return ((uint64_t)w2 << 32) | w1; }
-
-// Fold the minimum c of tile K (>= +0, or +inf) into an output's running minimum
-// bb and band: below bb - bb tau restarts the band, up to bb + bb tau joins it.
-// Non-negative floats order like their bit patterns, so the tests are unsigned
-// integer compares; bb = +inf makes bb - T a NaN, whose bits lie above every
-// value, so the first tile restarts the band (an all-+inf tile too, harmlessly:
-// outputs whose minimum stays +inf are never resolved).
-__device__ __forceinline__ void band_fold(float c, float &bb, float tau, uint32_t &w1, uint32_t &w2, uint32_t K,
-                                          uint32_t KK) {
-    const float T = __fmul_rn(bb, tau);
-    const uint32_t ci = __float_as_uint(c);
-    const bool rst = ci < __float_as_uint(__fsub_rn(bb, T));
-    const bool app = !rst && ci <= __float_as_uint(__fadd_rn(bb, T));
-    band_update(w1, w2, rst, app, K, KK);
-    bb = fminf(bb, c);
-}
 
 // Per-pass constants, copied once to device memory (kernels index them at run time).
 struct FastParams {
@@ -125,7 +92,8 @@ struct FastArgs {
     int64_t p, d;
     int64_t ps;            // table row stride (multiple of 64)
     float invd;            // correctly rounded 1/d
-    int G, s, lgc, Gc, nsplit, nJ, ncons;
+    int G, s, nJ;
+    int Gc, nsplit;        // far phase: multipliers per split (Gc (s-2) <= 128 tasks), splits
     const FastParams *prm;
     float *dp32;           // tile-major fp32 copy of dp: see d32()
     uint64_t *band;        // [G][s+1][ps] tile runs per output
@@ -134,26 +102,39 @@ struct FastArgs {
     uint8_t *need;         // [G][s+1][ps] output resolved exactly
     float *corner;         // [nJ(nJ-1)/2][8]: state of pair (64K+63, 64J), K < J (N, E, Ec, A, Ac, C, Cc)
     const float *costs;    // resident interval costs (tile (K, J) at J(J+1)/2 + K - tile_base), or null
-    float2 *tsum;          // with costs: per tile, {min_k C, min_k Phi} of its 64 columns (the rows' padding)
+    float2 *tsum;          // per tile, the summaries {min_k C, min_k Phi} of its 64 columns (the rows' padding);
+                           // a value is negated where it is not the one at the tile's last k
     size_t tile_base;      // index of the first tile the costs hold: 0, or J0(J0+1)/2 for a band of blocks
     int J0, J1;            // the wavefront's column blocks [J0, J1): all of them, or one band (streamed costs)
+    int build;             // the costs hold one panel's tiles, built by the wavefront itself
+    int T;                 // column blocks per panel
+    int workers;           // CTAs that share the far tiles
+    int tcap;              // tasks per far list entry, at most (16 .. 64)
+    float *part;           // [workers + T nsplit] segments: minima [Gc][s-2][64], then runs (seg_min, seg_runs)
+    uint4 *fbits;          // far tasks: 128 bits a tile, [T nsplit][ceil(nJ/32)][32] (mask_phase)
+    uint32_t *funion;      // ... and per word of 32 tiles those with any
+    int *fweight;          // ... and their work
+    unsigned long long *work;  // tasks evaluated in the pass
+    int *tmin;             // near minima by tile group [near_groups(T)][G][s-2][64], tagged with the panel's parity
+    float *tmin1;          // near minima by tile [T(T+1)/2][G][s-2][64]
     int32_t *lists;        // [s+1][2][G ps]: needed outputs of layer i (g << 24 | j); 0: <= NMEM members, 1: more
     int *list_cnt;         // [s+1][2]
     int32_t *wide;         // [G ps]: needed outputs of the layer being closed whose bands span more than
                            // kThreadTiles tiles (g << 24 | j), walked by a warp each (k_need_wide)
     int *wide_cnt;         // [s+1]
-    float *mdp;            // [nJ][G][mdp_stride]: min over the block's 64 columns of dp32(g, i, .)
+    float *mdp;            // [nJ][G][mdp_stride]: at i - 2, the min over the block's 64 columns of dp32(g, i, .)
     int mdp_stride;        // s + 1 rounded up to a multiple of 4 (16-byte rows)
-    int prune;             // skip tiles by the lower bound (resident or streamed costs)
-    int stage_tiles;       // with prune: tiles per staged batch (32, or 16 off the parked diagonal)
+    int prune;             // skip far tiles by the lower bound
+    int bound;             // the far phase starts from upper bounds of the minima (bound_phase)
+    int bound_step;        // ... from every bound_step-th tile (4; 32 in unseeded searches)
+    float *dlast;          // [nJ][G][mdp_stride]: at i - 2, dp32(g, i, .) at the block's last column
+    int *ub;               // [T][G][s-2][64]: the bounds' float bits
     const float *seed;     // with prune: fp32 dp rows [nJ][s+1][64] of an earlier pass at a multiplier >= every
                            // multiplier of this one (upper bounds of this pass's fp32 minima), or null
-    uint32_t spin_limit;   // flag waits give up after this many spins (kSpinLimit; lower in the test hook)
-    int hold0;             // test hook: column block 0 is never published (its waiters time out)
-    int split_pub;         // resident costs, two layer groups: blocks are published in two parts (below)
-    int *done;             // [nsplit][nJ]: every row of the block is stored
-    int *half;             // [nsplit][nJ]: rows 2..8 of the block are stored (split_pub)
-    int *ticket;
+    uint32_t spin_limit;   // waits on other CTAs give up after this many polls (kSpinLimit; lower in the test hook)
+    int hold0;             // test hook: column block 0's minima are never written and CTA 0 stays out of the
+                           // panel's barrier (their waiters time out)
+    int *gbar;             // grid barrier arrivals
     int *abort_flag;
     DevStatus *st;
 };
@@ -170,8 +151,10 @@ __device__ __forceinline__ size_t oidx(const FastArgs &a, int g, int i, int64_t 
 
 // ------------------------------------------------------------ named barriers
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-enum { BAR_FULL = 1, BAR_EMPTY = 3, BAR_CONS = 5, BAR_PROD = 6 };
+// BAR_BUILD .. + 5: the six 64-thread groups that build tiles; BAR_NEAR, + 1: a multiplier's eight near
+// warps
+enum { BAR_BUILD = 1, BAR_NEAR = 7 };
+constexpr int kBuildGroups = 6;  // what shared memory stages
 
 // ------------------------------------------------------------ fp32 numerics
 
@@ -299,7 +282,7 @@ __global__ void k_corners(FastArgs a) {
     }
 }
 
-// Compensated (Sum2) exclusive scan over the 64 producer threads of (x, c) pairs.
+// Compensated (Sum2) exclusive scan over the 64 threads jl = 0..63 of (x, c) pairs.
 __device__ __forceinline__ void pair_add(float &x, float &c, float y, float yc) {
     float s = __fadd_rn(x, y);
     float bb = __fsub_rn(s, x);
@@ -308,8 +291,8 @@ __device__ __forceinline__ void pair_add(float &x, float &c, float y, float yc) 
     c = __fadd_rn(__fadd_rn(c, yc), e);
 }
 
-__device__ void scan64_excl(float v, float &x_out, float &c_out, float (*wsum)[2]) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;  // producer threads 0..63
+__device__ void scan64_excl(float v, float &x_out, float &c_out, float (*wsum)[2], int jl, int bar) {
+    const int lane = jl & 31, wid = jl >> 5;
     float x = v, c = 0.f;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -317,7 +300,7 @@ __device__ void scan64_excl(float v, float &x_out, float &c_out, float (*wsum)[2
         if (lane >= o) pair_add(x, c, y, yc);
     }
     if (lane == 31) { wsum[wid][0] = x; wsum[wid][1] = c; }
-    bar_sync(BAR_PROD, NPROD);
+    bar_sync(bar, NPROD);
     if (wid == 1) pair_add(x, c, wsum[0][0], wsum[0][1]);
     // exclusive: shift by one
     float xe = __shfl_up_sync(0xffffffffu, x, 1), ce = __shfl_up_sync(0xffffffffu, c, 1);
@@ -327,7 +310,7 @@ __device__ void scan64_excl(float v, float &x_out, float &c_out, float (*wsum)[2
     }
     x_out = xe;
     c_out = ce;
-    bar_sync(BAR_PROD, NPROD);
+    bar_sync(bar, NPROD);
 }
 
 __device__ __forceinline__ Rec rec_empty() { return {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}; }
@@ -336,9 +319,6 @@ __device__ __forceinline__ int ld_acquire(const int *p) {
     int v;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-__device__ __forceinline__ void st_release(int *p, int v) {
-    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // packed fp32 pair arithmetic (sm_100+)
@@ -356,12 +336,6 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
         : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return d;
 }
-__device__ __forceinline__ float min3(float a, float b, float c) {
-    float d;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
 // ------------------------------------------- bulk copies (TMA engine) and mbarriers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned long long *bar, uint32_t count) {
@@ -380,6 +354,9 @@ __device__ __forceinline__ bool mbar_test(unsigned long long *bar, uint32_t pari
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     return ok != 0;
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // Bounded wait for phase `parity` of `bar`: on expiry record a timeout, raise the abort flag and return.
 __device__ __forceinline__ void mbar_wait_bounded(unsigned long long *bar, uint32_t parity, DevStatus *st, int *abort_flag) {
@@ -432,40 +409,41 @@ __host__ __device__ __forceinline__ size_t cost_tile_idx(int64_t K, int64_t J) {
 }
 
 // ------------------------------------------------------------ shared memory
-struct TileMeta {
-    int J, K, split, kind;  // kind: 0 off-diagonal, 1 diagonal, 2 stop
+// One panel: column blocks P0 .. P0 + nb - 1; its cost tiles are stored from linear index tbase.
+// The far lists have nb * nsplit rows (js = split * nb + Jl) of nB words, one bit per tile.
+struct Panel {
+    int P0, nb, nB, tag;
+    size_t tbase;
 };
+
+constexpr int NT = 32;  // tiles per word of the far lists, and per staged batch
 
 struct __align__(16) Smem {
-    float C[2][BJ][PSTR];
-    float Phi[2][BJ][PSTR];
-    float diag[2][kMaxG][BJ];             // dp32 of the previous / current layer inside the column
-    float kv[BK], kw[BK], kd[BK];         // v_k (k0..k0+63), w_{k+1}, v_{k+1} - v_k
-    TileMeta meta[2];
-    float wsum[2][2];                     // producer scan: per-warp totals
-    int ticket;
-    int sfront[2];                        // resident costs: frontier of the minima in stage buffer sb
-    int pad;
-    uint32_t needw[2][MAXCONS / 32];      // resident costs: per warp, the tiles of the batch it needs
-    unsigned long long mbar[2];           // resident costs: bulk-copy completion of buffer b
-    unsigned long long smbar[2];          // resident costs: completion of stage buffer sb
     float tau[kMaxS + 1];                 // FastParams::tau and lam32, read on every tile
     float lam32[kMaxG];
-    // staged dp32 block minima of a tile's column block (tile skipping): the split's
-    // multipliers' rows of a.mdp_stride floats each, flat (up to kMaxG x 20 floats)
-    __align__(16) float mdp[2][kMaxG][20];
-    // followed by dp32 slices [2][Gc * (s-2)][BK] (dynamic)
+    uint32_t tw[8 * 16];                  // mask phase: a word of each multiplier and layer (kBoundL)
+    int jstart[16 * kMaxG + 1];           // far phase: the work before each row of the list (far_plan)
+    int share, first, fpos, total;        // ... the CTAs' share; this CTA's first word, its position; all work
+    float gmin[NT / 8][kMaxG][16];        // mask phase: block minima of groups of eight tiles
+    // far phase: the CTA's next entries (far_list) and the state of the list
+    __align__(16) uint4 lbits[320];
+    uint32_t lkey[320], lwhere[320];      // ... js << 14 | K; J | first multiplier << 16
+    uint16_t tdiv[32 * kTaskWords];       // ... li | gl << 8 of task t
+    int2 lwords[MAXCONS / 32];
+    int lnext, lpos, lcount, lmore;
+    uint32_t tinfo[4][64];                // ... entry i's tasks at i % 4: t | li << 8 | gl << 16 in row order
+    uint16_t okey[256];                   // ... K of a segment's tiles by ordinal (runs_add)
+    int ok;                               // grid_sync's answer
+    unsigned long long full[3];           // ... copies of tile buffer b
+    unsigned long long smbar[2];          // copies of stage buffer sb
+    unsigned long long nbar;              // copies of the near tiles
+    // followed (dynamic, at kSmemHead) by one area that the phases use in turn: the far phase's tile
+    // buffers (costs, then a dp32 row a task), band state and partial minima, the bound and mask phases' two stage
+    // buffers and limits, the near phase's tiles and rows, or the build groups' staging
 };
+constexpr size_t kSmemHead = (sizeof(Smem) + 127) & ~(size_t)127;
 
 // ------------------------------------------------------- one tile of interval costs
-// Per-k constants of the tile starting at k0 (k = k0 + jl): v_k, w_{k+1}, v_{k+1} - v_k.
-__device__ __forceinline__ void tile_consts(const FastArgs &a, int64_t k0, int jl, float *kv, float *kw, float *kd) {
-    int64_t k = k0 + jl;
-    kv[jl] = k < a.p ? a.v[k] : 0.f;
-    kw[jl] = (k + 1 < a.p) ? a.wf[k + 1] : 0.f;
-    kd[jl] = (k + 1 < a.p) ? __fsub_rn(a.v[k + 1], a.v[k]) : 0.f;
-}
-
 // Global inputs of column jl of tile (K, J), loaded by one of the 64 threads: the tile
 // constants of k = 64K + jl (v_k, w_{k+1}, v_{k+1} - v_k), the column's increment
 // (w_{jt+1}, v_{jt+1}, v_jt, jt = 64J + jl) and v_j, and off the diagonal the corner
@@ -499,20 +477,21 @@ __device__ __forceinline__ void tile_load(const FastArgs &a, int64_t K, int64_t 
 
 // Anchor of column jl at k = 64K + 63 (off the diagonal): the corner state of (K, J)
 // advanced along j with compensated exclusive scans of non-negative increments.
-// Threads 0..63 of the block all call it (the scans synchronise them on BAR_PROD);
+// 64 threads (jl = 0..63) call it together (the scans synchronise them on barrier bar);
 // vk = v at k = 64K + 63.
-__device__ Rec tile_anchor(const TileIn &q, int64_t J, int jl, float vk, const FastArgs &a, float (*wsum)[2]) {
+__device__ Rec tile_anchor(const TileIn &q, int64_t J, int jl, float vk, const FastArgs &a, float (*wsum)[2],
+                           int bar) {
     const bool okc = J * BJ + jl + 1 < a.p;
     const float wn = q.wn, vn = q.vn;
     const float dj = okc ? __fsub_rn(vn, q.vt) : 0.f;
     const float *cp = q.c;
     float nx, nc, ax, ac, ex, ec, cx, cc;
-    scan64_excl(wn, nx, nc, wsum);                               // N (exact)
-    scan64_excl(okc ? __fmul_rn(wn, __fsub_rn(vn, vk)) : 0.f, ax, ac, wsum);  // A
+    scan64_excl(wn, nx, nc, wsum, jl, bar);                               // N (exact)
+    scan64_excl(okc ? __fmul_rn(wn, __fsub_rn(vn, vk)) : 0.f, ax, ac, wsum, jl, bar);  // A
     float Nj = __fadd_rn(cp[0], __fadd_rn(nx, nc));
     float Aj = __fadd_rn(__fadd_rn(cp[3], ax), __fadd_rn(cp[4], ac));
-    scan64_excl(__fmul_rn(dj, Nj), ex, ec, wsum);              // E
-    scan64_excl(__fmul_rn(dj, Aj), cx, cc, wsum);              // C
+    scan64_excl(__fmul_rn(dj, Nj), ex, ec, wsum, jl, bar);              // E
+    scan64_excl(__fmul_rn(dj, Aj), cx, cc, wsum, jl, bar);              // C
     Rec anchor_r;
     anchor_r.N = Nj;
     anchor_r.E = cp[1]; anchor_r.Ec = cp[2];
@@ -568,26 +547,17 @@ __device__ void tile_rows(const FastArgs &a, int64_t K, int64_t J, int jl, const
             for (int kl = 0; kl < BK; kl++) { Cr[jl][kl] = CUDART_INF_F; Pr[jl][kl] = 0.f; }
             mp = 0.f;
         }
-        Cr[jl][BK] = mc;
-        Pr[jl][BK] = mp;
+        // The column's summary: min C and min Phi, negated where the minimum is not the value at
+        // the tile's last k (then dp(., k) + C + lambda' Phi at that k is not the summary's own).
+        Cr[jl][BK] = mc == Cr[jl][BK - 1] ? mc : __int_as_float(__float_as_int(mc) | (int)0x80000000);
+        Pr[jl][BK] = mp == Pr[jl][BK - 1] ? mp : __int_as_float(__float_as_int(mp) | (int)0x80000000);
 }
 
-// tile_anchor and tile_rows for one tile (threads 0..63 of the block; kv, kw, kd hold
-// the tile constants of tile K, visible to all 64).
-__device__ void tile_columns(const FastArgs &a, int64_t K, int64_t J, int jl, const float *kv, const float *kw,
-                             const float *kd, float (*wsum)[2], float (*Cr)[PSTR], float (*Pr)[PSTR]) {
-    TileIn q;
-    tile_load(a, K, J, jl, q);
-    const Rec anchor_r = K == J ? rec_empty() : tile_anchor(q, J, jl, kv[BK - 1], a, wsum);
-    tile_rows(a, K, J, jl, anchor_r, q.vj, kv, kw, kd, Cr, Pr);
-}
-
-// Resident interval costs: every tile (K <= J) computed once, exactly as the
-// wavefront's own producer computes it (tile_anchor, tile_rows), staged in shared
-// memory and written out by a bulk copy.  64 threads per block; blocks stride over
-// the tiles.  A tile's global inputs are loaded while the previous tile's rows are
-// computed, and the wait for the previous bulk store to have read the staging rows
-// comes only just before they are overwritten.
+// Interval-cost tiles t0, t0 + stride, ... below t1 (linear index J(J+1)/2 + K), each computed
+// once (tile_anchor, tile_rows), staged in shared memory and written out by a bulk copy to
+// costs / tsum at t - tbase.  Called by 64 threads (jl = 0..63, named barrier bar).  A tile's
+// global inputs are loaded while the previous tile's rows are computed, and the wait for the
+// previous bulk store to have read the staging rows comes only just before they are overwritten.
 struct __align__(16) BuildSmem {
     float C[BJ][PSTR];
     float Phi[BJ][PSTR];
@@ -595,13 +565,10 @@ struct __align__(16) BuildSmem {
     float wsum[2][2];
 };
 
-__global__ void __launch_bounds__(NPROD) k_build_costs(FastArgs a, float *costs) {
-    __shared__ BuildSmem S;
-    const int jl = threadIdx.x;
-    // the tiles of column blocks [J0, J1): indices J0(J0+1)/2 .. J1(J1+1)/2 - 1, stored from tile_base
-    const int64_t ntiles = (int64_t)a.J1 * (a.J1 + 1) / 2;
-    int64_t t = (int64_t)a.tile_base + blockIdx.x;
-    if (t >= ntiles) return;
+__device__ __forceinline__ void build_tiles(const FastArgs &a, BuildSmem &S, int jl, int bar, int64_t t0,
+                                            int64_t stride, int64_t t1, int64_t tbase) {
+    int64_t t = t0;
+    if (t >= t1) return;
     // invert t = J(J+1)/2 + K, K <= J
     int64_t J = (int64_t)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
     while (J * (J + 1) / 2 > t) J--;
@@ -612,1067 +579,1064 @@ __global__ void __launch_bounds__(NPROD) k_build_costs(FastArgs a, float *costs)
     tile_load(a, K, J, jl, cur);
     for (;;) {
         S.kv[jl] = cur.kv; S.kw[jl] = cur.kw; S.kd[jl] = cur.kd;
-        bar_sync(BAR_PROD, NPROD);
-        const Rec anchor_r = K == J ? rec_empty() : tile_anchor(cur, J, jl, S.kv[BK - 1], a, S.wsum);
-        // the next tile of this block: t + gridDim.x, walking (J, K) along the rows
-        const int64_t tn = t + gridDim.x;
-        int64_t Jn = J, Kn = K + gridDim.x;
+        bar_sync(bar, NPROD);
+        const Rec anchor_r = K == J ? rec_empty() : tile_anchor(cur, J, jl, S.kv[BK - 1], a, S.wsum, bar);
+        // the next tile: t + stride, walking (J, K) along the rows
+        const int64_t tn = t + stride;
+        int64_t Jn = J, Kn = K + stride;
         while (Kn > Jn) { Kn -= Jn + 1; Jn++; }
         TileIn nxt;
-        if (tn < ntiles) {
+        if (tn < t1) {
             tile_load_consts(a, Kn, jl, nxt);
             tile_load(a, Kn, Jn, jl, nxt);
         }
         if (jl == 0) bulk_wait_read_all();  // the previous tile's bulk store has read the rows
-        bar_sync(BAR_PROD, NPROD);
+        bar_sync(bar, NPROD);
         tile_rows(a, K, J, jl, anchor_r, cur.vj, S.kv, S.kw, S.kd, S.C, S.Phi);
-        a.tsum[((size_t)t - a.tile_base) * BJ + jl] = make_float2(S.C[jl][BK], S.Phi[jl][BK]);  // this thread's own row
+        a.tsum[(size_t)(t - tbase) * BJ + jl] = make_float2(S.C[jl][BK], S.Phi[jl][BK]);  // this thread's own row
         fence_proxy_async_smem();
-        bar_sync(BAR_PROD, NPROD);
+        bar_sync(bar, NPROD);
         if (jl == 0) {
-            float *dst = costs + ((size_t)t - a.tile_base) * kCostTileFloats;
+            float *dst = const_cast<float *>(a.costs) + (size_t)(t - tbase) * kCostTileFloats;
             bulk_s2g(dst, &S.C[0][0], kCostHalfBytes);
             bulk_s2g(dst + kCostHalfFloats, &S.Phi[0][0], kCostHalfBytes);
             bulk_commit();
         }
-        if (tn >= ntiles) break;
+        if (tn >= t1) break;
         t = tn; J = Jn; K = Kn;
         cur = nxt;
     }
     if (jl == 0) bulk_wait_all();
 }
 
-// ------------------------------------------------------------ consumer side
-// A consumer thread owns the outputs (g = split * Gc + gl, layers 3 + lg * LPT + l,
-// columns jq + 16 q of the block) and keeps their band state in registers.
-struct ConsId {
-    int ct, jq, lg, gl;
-    bool active;
-};
-__device__ __forceinline__ ConsId cons_id(const FastArgs &a, int ct) {
-    ConsId id;
-    id.ct = ct;
-    id.jq = ct % NJQ;
-    const int rest = ct / NJQ;
-    id.lg = rest % a.lgc;
-    id.gl = rest / a.lgc;
-    id.active = ct < a.Gc * a.lgc * NJQ;
-    return id;
+static __device__ __noinline__ void build_panel(const FastArgs &a, BuildSmem &S, int jl, int bar, int64_t t0,
+                                                int64_t stride, int64_t t1, int64_t tbase) {
+    build_tiles(a, S, jl, bar, t0, stride, t1, tbase);  // the wavefront's: registers of its own
 }
 
-// The outputs a consumer thread owns: LP layers x JPT columns (LP = LPT, or 8 for the
-// generic path of the resident kernel at larger s: see launch_dp_fast).
-template <int LP>
-struct ConsStateT {
-    float best[LP][JPT];
-    uint32_t w1[LP][JPT], w2[LP][JPT];  // band runs (band_update)
-};
-using ConsState = ConsStateT<LPT>;
-template <int LP>
-__device__ __forceinline__ void cons_reset(ConsStateT<LP> &cs) {
-#pragma unroll
-    for (int l = 0; l < LP; l++)
-#pragma unroll
-        for (int q = 0; q < JPT; q++) { cs.best[l][q] = CUDART_INF_F; cs.w1[l][q] = 0u; cs.w2[l][q] = 0u; }
+// The tiles of column blocks [J0, J1): indices J0(J0+1)/2 .. J1(J1+1)/2 - 1, stored from tile_base.
+__global__ void __launch_bounds__(NPROD) k_build_costs(const __grid_constant__ FastArgs a) {
+    __shared__ BuildSmem S;
+    build_tiles(a, S, threadIdx.x, BAR_BUILD, (int64_t)a.tile_base + blockIdx.x, gridDim.x,
+                (int64_t)a.J1 * (a.J1 + 1) / 2, (int64_t)a.tile_base);
 }
 
-// Seeded running minima of block J.  Every fp32 candidate is monotone in lambda' (C and
-// Phi are >= 0 and the roundings are monotone), so by induction over the layers an
-// earlier pass's fp32 minimum at a multiplier >= this one's bounds this pass's minimum
-// m from above.  Starting the running minimum at that bound changes no result: the
-// tile holding m is never skipped (its lower bound is <= m <= the limit), so the final
-// minimum is m itself; a tile the tighter limit skips has every candidate above
-// m (1 + tau), outside the band; and band_fold keeps the band a superset of the tiles
-// with a candidate within m (1 + tau) from any starting bb >= m (a reset drops only
-// tiles whose candidates all lie above the band).  The band words keep their reset
-// state, run 1 = tile 0: a seeded output whose walk never resets its band keeps tile 0
-// in it (a superset again; a run opened at tile 0 could not be told from no run).
-// Only the skip tests see the seed: more tiles are skipped, the tables are unchanged.
-template <int LP>
-__device__ __forceinline__ void cons_seed(const FastArgs &a, ConsStateT<LP> &cs, int J, const ConsId &id) {
-    const float *sr = a.seed + (size_t)J * (size_t)(a.s + 1) * BJ;
-#pragma unroll
-    for (int l = 0; l < LP; l++) {
-        // rows past the last layer repeat the last one (cons_offdiag): so does their seed
-        const int i = 3 + min(id.lg * LP + l, a.s - 3);
-#pragma unroll
-        for (int q = 0; q < JPT; q++) {
-            const int jl = id.jq + NJQ * q;
-            const float v = ((int64_t)J * BJ + jl < a.p) ? sr[(size_t)i * BJ + jl] : CUDART_INF_F;
-            if (v < CUDART_INF_F) cs.best[l][q] = v;
-        }
-    }
-}
+// ------------------------------------------------------------ panels
+// The column blocks go in panels of a.T (15 on this GPU) consecutive blocks [P0, P0 + nb), one
+// after the other.  Within a panel, grid barriers between the steps:
+//  1. bound_phase: upper bounds of the minima over the far tiles (K < P0, whose dp rows are all
+//     final) from one candidate per tile;
+//  2. mask_phase: the far tasks -- (tile, multiplier, layer) -- that may matter, by the skip test
+//     against the bounds;
+//  3. far_phase: the tiles with tasks in one list, an equal share of the work for each CTA; a CTA's
+//     results for a column block -- a segment -- go to the outputs' minima and, with their band
+//     runs, to a slot;
+//  4. near_phase: the panel's own triangle of tiles, layer by layer.  A CTA takes up to four tiles
+//     (K, J) of one J and two multipliers, two warps one of each, with the tile's costs
+//     C + lambda' Phi in registers (a lane: one column) for all layers.  For layer i a warp gathers
+//     row i-1 of its block K -- the far minimum and the (at most four) groups' minima above it --
+//     and the CTA writes its group's minima of layer i.  A written minimum carries the panel's
+//     parity in its sign bit (values are >= +0), so the value is its own flag: a reader polls
+//     the values themselves (bounded), and no fence or counter stands between two layers;
+//  5. fold_panel: every output's band from the segments' runs and the near minima.
+// What bounds it: a wavefront of whole column blocks made the chain of blocks (one block's last
+// tile and diagonal, every layer, 22 000 cycles at s = 16) the critical path and left the SMs
+// unevenly loaded; here 15 blocks cost a few barriers and s - 2 gather/compute steps, and the
+// far tiles are shared evenly.  A pass of 8 multipliers (mean over a budgeted search, resident
+// costs): 25.6 ms instead of 46.3 at d = 2^17, s = 16; 1.69 instead of 2.93 at d = 16384, s = 16;
+// 15.1 instead of 47.7 at d = 50001, s = 32; building its own costs, 2.6 instead of 8.4 at
+// d = 12289, s = 16.  Of the 25.6 ms about 13.5 are far tiles, 3 uneven shares, 5 masks, 2.5
+// bounds and 3 the near phases; far tiles are bound by issue (one add and one min a candidate
+// on the two FP32 pipes reach about 53 candidates per cycle and SM) and by the copies and
+// barriers of a tile, which cost as much as about 8 of its tasks (kTileCost).
 
-// Off-diagonal tile K: the fp32 minimum over the tile's 64 k of every output the
-// thread owns (g must be a real multiplier), folded into its band state.
-// Candidate values are >= +0, so their bit patterns order like the floats: the
-// running minimum is kept as int bits and updated with integer min (ALU pipe)
-// next to the packed adds (FMA pipe).
-// Returns false when the warp skipped the tile (see below).
-template <int LP>
-__device__ __forceinline__ bool cons_offdiag(const FastArgs &a, const Smem &S, const float *sDPb, int b, uint32_t K,
-                                             int g, const ConsId &id, ConsStateT<LP> &cs) {
-    const int L = a.s - 2;
-    int cm[LP][JPT];
-#pragma unroll
-    for (int l = 0; l < LP; l++)
-#pragma unroll
-        for (int q = 0; q < JPT; q++) cm[l][q] = 0x7f800000;  // +inf
-    const float *dpb = sDPb + (size_t)id.gl * L * BK;
-    const float lam = S.lam32[g];
-    const float2 lam2 = make_float2(lam, lam);
-    int rowl[LP];
-#pragma unroll
-    for (int l = 0; l < LP; l++) rowl[l] = min(id.lg * LP + l, L - 1);
-    if (a.prune) {
-        // Exact tile skipping.  Every candidate of the tile for output (l, q) is
-        // >= lb = fl(min dp(i-1, .) + fl(fma(lam, min Phi, min C))) (rounding is monotone);
-        // when lb exceeds the output's band limit bb + bb tau, the tile changes neither
-        // its minimum nor its band.  The warp skips when that holds for all its outputs.
-        const float *md = &S.mdp[b][0][0] + (size_t)id.gl * a.mdp_stride + 2;
-        float lbq[JPT];
-#pragma unroll
-        for (int q = 0; q < JPT; q++) {
-            const int jl = id.jq + NJQ * q;
-            lbq[q] = __fmaf_rn(lam, S.Phi[b][jl][BK], S.C[b][jl][BK]);
-        }
-        bool need = false;
-#pragma unroll
-        for (int l = 0; l < LP; l++) {
-            const float m = md[rowl[l]], tau = S.tau[3 + rowl[l]];
-#pragma unroll
-            for (int q = 0; q < JPT; q++) {
-                const float bb = cs.best[l][q];
-                need |= __fadd_rn(m, lbq[q]) <= __fadd_rn(bb, __fmul_rn(bb, tau));
-            }
-        }
-        if (!__any_sync(__activemask(), need)) return false;
-    }
-#pragma unroll 1
-    for (int kk = 0; kk < BK; kk += 4) {
-        float2 W[JPT][2];
-#pragma unroll
-        for (int q = 0; q < JPT; q++) {
-            float4 c4 = *reinterpret_cast<const float4 *>(&S.C[b][id.jq + NJQ * q][kk]);
-            float4 f4 = *reinterpret_cast<const float4 *>(&S.Phi[b][id.jq + NJQ * q][kk]);
-            W[q][0] = fma2(lam2, make_float2(f4.x, f4.y), make_float2(c4.x, c4.y));
-            W[q][1] = fma2(lam2, make_float2(f4.z, f4.w), make_float2(c4.z, c4.w));
-        }
-#pragma unroll
-        for (int l = 0; l < LP; l++) {
-            // layer i = 3 + li uses dp row 2 + li; rows past the last layer are
-            // clamped (their results are never used)
-            const float4 d4 = *reinterpret_cast<const float4 *>(dpb + (size_t)rowl[l] * BK + kk);
-            float2 da = make_float2(d4.x, d4.y), db = make_float2(d4.z, d4.w);
-#pragma unroll
-            for (int q = 0; q < JPT; q++) {
-                float2 t0 = add2(da, W[q][0]);
-                float2 t1 = add2(db, W[q][1]);
-                int c = min(min(cm[l][q], __float_as_int(t0.x)), __float_as_int(t0.y));
-                cm[l][q] = min(min(c, __float_as_int(t1.x)), __float_as_int(t1.y));
-            }
-        }
-    }
-    // band bookkeeping (branch-free; layers past the last one carry state that is never read)
-    const uint32_t KK = (K << 16) | K;
-#pragma unroll
-    for (int l = 0; l < LP; l++) {
-        const float tau = S.tau[3 + rowl[l]];
-#pragma unroll
-        for (int q = 0; q < JPT; q++) band_fold(__int_as_float(cm[l][q]), cs.best[l][q], tau, cs.w1[l][q], cs.w2[l][q], K, KK);
-    }
-    return true;
-}
-
-// Diagonal block J (its tile in buffer b): layers in order, each needing the
-// previous layer's values inside the block; dp32 and the band words of the block
-// go to global memory.  The owner of an output computes its minimum over the
-// block's 64 k; when a.lgc == 2 the partner lane (lane ^ 16: same multiplier and
-// columns, the other layer group) takes half of the k range and the halves meet
-// by a shuffle.  All `a.ncons` consumer threads take part (BAR_CONS).
-// staged: S.diag[0] already holds layer 2 of the block (bulk copy), else it is
-// loaded here.
-template <int LP>
-__device__ __forceinline__ void cons_diag(const FastArgs &a, Smem &S, int b, int J, int split, const ConsId &id,
-                                          ConsStateT<LP> &cs, bool staged) {
-    const int L = a.s - 2;
-    const int ct = id.ct;
-    const int g = split * a.Gc + id.gl;
-    const bool own = id.active && g < a.G;
-    const int64_t j0 = (int64_t)J * BJ;
-    if (!staged) {
-        for (int q = ct; q < a.Gc * BJ; q += a.ncons) {
-            int gg = q / BJ, jj = q % BJ;
-            int g2 = split * a.Gc + gg;
-            int64_t jx = j0 + jj;
-            S.diag[0][gg][jj] = (g2 < a.G && jx < a.p) ? a.dp32[d32(a, g2, 2, jx)] : CUDART_INF_F;
-        }
-        bar_sync(BAR_CONS, a.ncons);
-    }
-    const bool pair = a.lgc == 2;  // warp-uniform
-    const float lam = own ? S.lam32[g] : 0.f;
-    const float2 lam2 = make_float2(lam, lam);
-    const uint32_t K = (uint32_t)J, KK = (K << 16) | K;
-    int cur = 0;
-    for (int li = 0; li < L; li++) {
-        if (LP != LPT && a.prune) {
-            // block minimum of the layer below (row 2 + li) for later blocks' skip tests, by the
-            // warp of that index (values >= +0: integer min on the bits); with LPT layers per
-            // thread, skipping runs on the paired diagonal only, which writes its own minima
-            const int w = ct >> 5, wl = ct & 31;
-            const int gw = split * a.Gc + w;
-            if (w < a.Gc && gw < a.G) {
-                const int v = min(__float_as_int(S.diag[cur][w][wl]), __float_as_int(S.diag[cur][w][wl + 32]));
-                const int mn = __reduce_min_sync(0xffffffffu, v);
-                if (wl == 0) a.mdp[((size_t)J * a.G + gw) * a.mdp_stride + 2 + li] = __int_as_float(mn);
-            }
-        }
-        const int i = 3 + li;
-        const int olg = li / LP, l = li - olg * LP;
-        const bool owner = own && id.lg == olg;
-        const int kbeg = (pair && !owner) ? BJ / 2 : 0;
-        const int kend = (pair && owner) ? BJ / 2 : BJ;
-        int m0[JPT], m1[JPT];
-#pragma unroll
-        for (int q = 0; q < JPT; q++) { m0[q] = 0x7f800000; m1[q] = 0x7f800000; }
-        if (own && (owner || pair)) {
-            const float *prow = &S.diag[cur][id.gl][0];
-#pragma unroll 2
-            for (int kk = kbeg; kk < kend; kk += 4) {
-                const float4 d4 = *reinterpret_cast<const float4 *>(prow + kk);
-#pragma unroll
-                for (int q = 0; q < JPT; q++) {
-                    const int jl = id.jq + NJQ * q;
-                    float4 c4 = *reinterpret_cast<const float4 *>(&S.C[b][jl][kk]);
-                    float4 f4 = *reinterpret_cast<const float4 *>(&S.Phi[b][jl][kk]);
-                    float2 v0 = fma2(lam2, make_float2(f4.x, f4.y), make_float2(c4.x, c4.y));
-                    float2 v1 = fma2(lam2, make_float2(f4.z, f4.w), make_float2(c4.z, c4.w));
-                    float2 t0 = add2(make_float2(d4.x, d4.y), v0);
-                    float2 t1 = add2(make_float2(d4.z, d4.w), v1);
-                    m0[q] = min(min(m0[q], __float_as_int(t0.x)), __float_as_int(t0.y));
-                    m1[q] = min(min(m1[q], __float_as_int(t1.x)), __float_as_int(t1.y));
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < JPT; q++) {
-            m0[q] = min(m0[q], m1[q]);
-            if (pair) m0[q] = min(m0[q], __shfl_xor_sync(0xffffffffu, m0[q], 16));
-        }
-        if (owner) {
-#pragma unroll
-            for (int lx = 0; lx < LP; lx++) {
-                if (lx != l) continue;
-#pragma unroll
-                for (int q = 0; q < JPT; q++) {
-                    const int jl = id.jq + NJQ * q;
-                    const int64_t j = j0 + jl;
-                    band_fold(__int_as_float(m0[q]), cs.best[lx][q], S.tau[i], cs.w1[lx][q], cs.w2[lx][q], K, KK);
-                    const float bb = cs.best[lx][q];
-                    S.diag[cur ^ 1][id.gl][jl] = bb;
-                    if (j < a.p) {
-                        a.dp32[d32(a, g, i, j)] = bb;
-                        a.band[oidx(a, g, i, j)] = band_pack(cs.w1[lx][q], cs.w2[lx][q]);
-                    }
-                }
-            }
-        }
-        bar_sync(BAR_CONS, a.ncons);
-        cur ^= 1;
-    }
-}
-
-// Diagonal block when a.lgc == 2 (the usual s <= 16).  Only pairs k < j of the tile
-// count, so each lane takes two whole columns of its column group jq, balanced on the
-// triangle: lanes 0-15 column jq + 48 (k < 64) and column jq (k < 16), lanes 16-31
-// column jq + 32 (k < 48) and column jq + 16 (k < 32): 80 pairs each, in 20 groups of
-// four consecutive k (kdiag_group).  The costs W = C + lambda' Phi of those pairs stay
-// in registers for all layers, so each layer reads only the previous layer's 64 values
-// from shared memory, and every column's minimum is complete within one lane (pairs
-// k >= j carry C = +inf in the tile and never win).  The band state is parked in `park`
-// ([3][LPT][JPT][ncons] words: best, run 1, run 2) and folded there; the block
-// ends with its diagonal, so the registers are not restored.  A warp holds one
-// multiplier, and the rows of S.diag and the parked slots it reads and writes are
-// that multiplier's alone, so the layers need only a warp barrier each.
-// Group g4 of a diagonal lane (half 0: lanes 0-15, half 1: lanes 16-31): its column
-// (q = 0: the long one, 1: the short one) and first k.  Groups 0-11 are k 0..47 of the
-// long column for both halves; groups 12-15 are k 48..63 of the long column (half 0)
-// or k 0..15 of the short one (half 1); groups 16-19 are k 0..15 (half 0) or 16..31
-// (half 1) of the short column.
-constexpr int kDiagGroups = 20;
-__device__ __forceinline__ void kdiag_group(int g4, int half, int &q, int &k) {
-    if (g4 < 12) { q = 0; k = 4 * g4; }
-    else if (g4 < 16) { q = half; k = half ? 4 * (g4 - 12) : 4 * g4; }
-    else { q = 1; k = half ? 4 * (g4 - 12) : 4 * (g4 - 16); }
-}
-
-// cons_diag_pair in three steps, so that the block can be published in two parts
-// (diag_prepare; diag_layers over a range of layers; diag_store over a range of rows).
-// diag_prepare: park the band state, store the block minimum of layer 2, and build the
-// lane's costs W = C + lambda' Phi of its 80 pairs (kept in registers for all layers).
-__device__ __forceinline__ void diag_prepare(const FastArgs &a, Smem &S, uint32_t *park, int b, int J, int split,
-                                             const ConsId &id, const ConsState &cs, float2 (&W)[2 * kDiagGroups]) {
-    const int ct = id.ct, nc = a.ncons;
-    const int g = split * a.Gc + id.gl;
-    const bool own = id.active && g < a.G;  // uniform over a warp (one multiplier per warp)
-    constexpr int NS = LPT * JPT;
-#pragma unroll
-    for (int l = 0; l < LPT; l++)
-#pragma unroll
-        for (int q = 0; q < JPT; q++) {
-            const int x = (l * JPT + q) * nc + ct;
-            park[x] = __float_as_uint(cs.best[l][q]);
-            park[NS * nc + x] = cs.w1[l][q];
-            park[2 * NS * nc + x] = cs.w2[l][q];
-        }
-    asm volatile("" ::: "memory");  // the state leaves the registers before W is built
-    const int lane = ct & 31;
-    if (a.prune && own) {  // block minimum of layer 2 (values are >= +0: integer min on the bits)
-        int v = min(__float_as_int(S.diag[0][id.gl][lane]), __float_as_int(S.diag[0][id.gl][lane + 32]));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (lane == 0) a.mdp[((size_t)J * a.G + g) * a.mdp_stride + 2] = __int_as_float(v);
-    }
-    const int half = (ct >> 4) & 1;
-    const int qb = 3 - half, qs = half;  // the lane's long and short columns (q of jq + 16 q)
-    const float lam = own ? S.lam32[g] : 0.f;
-    const float2 lam2 = make_float2(lam, lam);
-#pragma unroll
-    for (int g4 = 0; g4 < kDiagGroups; g4++) {  // W[2 g4], W[2 g4 + 1]: costs of group g4's four pairs
-        int q, k;
-        kdiag_group(g4, half, q, k);
-        const int jl = id.jq + NJQ * (q ? qs : qb);
-        float4 c4 = *reinterpret_cast<const float4 *>(&S.C[b][jl][k]);
-        float4 f4 = *reinterpret_cast<const float4 *>(&S.Phi[b][jl][k]);
-        W[2 * g4] = fma2(lam2, make_float2(f4.x, f4.y), make_float2(c4.x, c4.y));
-        W[2 * g4 + 1] = fma2(lam2, make_float2(f4.z, f4.w), make_float2(c4.z, c4.w));
-    }
-}
-
-// Layers li0 <= li < li1 (i = 3 + li) of the diagonal block; cur: the S.diag row
-// holding layer i - 1 (in/out).
-__device__ __forceinline__ void diag_layers(const FastArgs &a, Smem &S, uint32_t *park, int J, int split,
-                                            const ConsId &id, const float2 (&W)[2 * kDiagGroups], int li0, int li1,
-                                            int &cur) {
-    const int ct = id.ct, nc = a.ncons;
-    const int g = split * a.Gc + id.gl;
-    const bool own = id.active && g < a.G;
-    constexpr int NS = LPT * JPT;
-    const int half = (ct >> 4) & 1;
-    const int qb = 3 - half, qs = half;
-    const uint32_t K = (uint32_t)J, KK = (K << 16) | K;
-    for (int li = li0; li < li1; li++) {
-        const int i = 3 + li;
-        const int olg = li / LPT, l = li - olg * LPT;
-        // minima (float bits; candidates are >= +0) of the long and the short column:
-        // each group of four k reduces on its own, then the groups by a tree, so the
-        // layer's dependency chain is a few mins deep
-        int lmin = 0x7f800000, smin = 0x7f800000;
-        if (own) {
-            const float *prow = &S.diag[cur][id.gl][0];
-            int m[kDiagGroups];
-#pragma unroll
-            for (int g4 = 0; g4 < kDiagGroups; g4++) {
-                int q, k;
-                kdiag_group(g4, half, q, k);
-                const float4 d4 = *reinterpret_cast<const float4 *>(prow + k);
-                const float2 t0 = add2(make_float2(d4.x, d4.y), W[2 * g4]);
-                const float2 t1 = add2(make_float2(d4.z, d4.w), W[2 * g4 + 1]);
-                m[g4] = min(min(__float_as_int(t0.x), __float_as_int(t0.y)), min(__float_as_int(t1.x), __float_as_int(t1.y)));
-            }
-            // groups 0-11: the long column; 12-15: long (half 0) or short (half 1); 16-19: short
-            const int A = min(min(min(min(m[0], m[1]), min(m[2], m[3])), min(min(m[4], m[5]), min(m[6], m[7]))),
-                              min(min(m[8], m[9]), min(m[10], m[11])));
-            const int B = min(min(m[12], m[13]), min(m[14], m[15]));
-            const int C = min(min(m[16], m[17]), min(m[18], m[19]));
-            lmin = half ? A : min(A, B);
-            smin = half ? min(B, C) : C;
-        }
-        if (own) {
-            // each lane folds its two columns into the owner's slots (layer group olg,
-            // same column group: lane jq + 16 olg of the warp)
-            const int cto = (ct & ~31) | (olg << 4) | id.jq;
-#pragma unroll
-            for (int c = 0; c < 2; c++) {
-                const int q = c ? qs : qb;
-                const int mq = c ? smin : lmin;
-                const int jl = id.jq + NJQ * q;
-                const int x = (l * JPT + q) * nc + cto;
-                float bb = __uint_as_float(park[x]);
-                uint32_t w1 = park[NS * nc + x], w2 = park[2 * NS * nc + x];
-                band_fold(__int_as_float(mq), bb, S.tau[i], w1, w2, K, KK);
-                park[x] = __float_as_uint(bb);
-                park[NS * nc + x] = w1;
-                park[2 * NS * nc + x] = w2;
-                S.diag[cur ^ 1][id.gl][jl] = bb;
-            }
-        }
-        __syncwarp();  // the layer's row and parked state belong to this warp alone
-        cur ^= 1;
-    }
-}
-
-// The block's final values of layers ilo <= i <= ihi from the parked state, and the
-// block minimum of each of those layers (over the 64 columns a half-warp holds).
-__device__ __forceinline__ void diag_store(const FastArgs &a, const uint32_t *park, int J, int split,
-                                           const ConsId &id, int ilo, int ihi) {
-    const int ct = id.ct, nc = a.ncons;
-    const int g = split * a.Gc + id.gl;
-    const bool own = id.active && g < a.G;
-    const int64_t j0 = (int64_t)J * BJ;
-    if (own) {
-#pragma unroll
-        for (int l = 0; l < LPT; l++) {
-            const int i = 3 + id.lg * LPT + l;
-            const bool real = i <= a.s && i >= ilo && i <= ihi;
-            int v = 0x7f800000;
-#pragma unroll
-            for (int q = 0; q < JPT; q++) {
-                const int64_t j = j0 + id.jq + NJQ * q;
-                const int x = (l * JPT + q) * nc + ct;
-                v = min(v, (int)park[x]);
-                if (real && j < a.p) a.dp32[d32(a, g, i, j)] = __uint_as_float(park[x]);
-            }
-            if (a.prune) {
-#pragma unroll
-                for (int o = 8; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-                if (real && id.jq == 0) a.mdp[((size_t)J * a.G + g) * a.mdp_stride + i] = __int_as_float(v);
-            }
-        }
-    }
-}
-
-// The whole diagonal block at once (the block is then published in one part).
-__device__ __forceinline__ void cons_diag_pair(const FastArgs &a, Smem &S, uint32_t *park, int b, int J, int split,
-                                               const ConsId &id, ConsState &cs) {
-    float2 W[2 * kDiagGroups];
-    diag_prepare(a, S, park, b, J, split, id, cs, W);
-    int cur = 0;
-    diag_layers(a, S, park, J, split, id, W, 0, a.s - 2, cur);
-    diag_store(a, park, J, split, id, 3, a.s);
-}
-
-// Split publish (resident costs, two layer groups).  The chain of blocks runs through the
-// last off-diagonal tile (J-1, J) and the diagonal block J.  Block J-1 is published in
-// two parts -- rows 2..8 (layer group 0's inputs) after its layer 8, every row at the
-// end -- and block J takes tile (J-1, J) in the same two parts, so its layers 3..9
-// start as soon as block J-1 has finished layer 8.
-// cons_lasttile_grp: tile (J-1, J) for layer group grp (0: layers 3..9 from rows 2..8;
-// 1: layers 10..s from rows 9..s-1) by all 32 lanes of the warp -- lane 16 h + jq takes
-// columns jq + 16 q, q in {2h, 2h+1}, over the group's seven layers -- after which the
-// owners (the lanes of layer group grp) fold the tile minima of their four columns
-// into their parked band state.  There is no skip test: this tile is on the chain.
-__device__ __forceinline__ void cons_lasttile_grp(const FastArgs &a, const Smem &S, const float *sDPb, int b,
-                                                  uint32_t *park, uint32_t K, int g, const ConsId &id, int grp) {
-    const int L = a.s - 2;
-    const int ct = id.ct, nc = a.ncons;
-    const int h = (ct >> 4) & 1;
-    constexpr int NS = LPT * JPT;
-    int cm[LPT][2];
-#pragma unroll
-    for (int l = 0; l < LPT; l++) { cm[l][0] = 0x7f800000; cm[l][1] = 0x7f800000; }
-    const float *dpb = sDPb + (size_t)id.gl * L * BK;
-    const float lam = S.lam32[g];
-    const float2 lam2 = make_float2(lam, lam);
-    int rowl[LPT];
-#pragma unroll
-    for (int l = 0; l < LPT; l++) rowl[l] = min(grp * LPT + l, L - 1);
-#pragma unroll 1
-    for (int kk = 0; kk < BK; kk += 4) {
-        float2 W[2][2];
-#pragma unroll
-        for (int c = 0; c < 2; c++) {
-            const int jl = id.jq + NJQ * (2 * h + c);
-            const float4 c4 = *reinterpret_cast<const float4 *>(&S.C[b][jl][kk]);
-            const float4 f4 = *reinterpret_cast<const float4 *>(&S.Phi[b][jl][kk]);
-            W[c][0] = fma2(lam2, make_float2(f4.x, f4.y), make_float2(c4.x, c4.y));
-            W[c][1] = fma2(lam2, make_float2(f4.z, f4.w), make_float2(c4.z, c4.w));
-        }
-#pragma unroll
-        for (int l = 0; l < LPT; l++) {
-            const float4 d4 = *reinterpret_cast<const float4 *>(dpb + (size_t)rowl[l] * BK + kk);
-            const float2 da = make_float2(d4.x, d4.y), db = make_float2(d4.z, d4.w);
-#pragma unroll
-            for (int c = 0; c < 2; c++) {
-                const float2 t0 = add2(da, W[c][0]);
-                const float2 t1 = add2(db, W[c][1]);
-                const int m = min(min(cm[l][c], __float_as_int(t0.x)), __float_as_int(t0.y));
-                cm[l][c] = min(min(m, __float_as_int(t1.x)), __float_as_int(t1.y));
-            }
-        }
-    }
-    const uint32_t KK = (K << 16) | K;
-#pragma unroll
-    for (int l = 0; l < LPT; l++) {
-        const float tau = S.tau[3 + rowl[l]];
-#pragma unroll
-        for (int c = 0; c < 2; c++) {
-            const int other = __shfl_xor_sync(0xffffffffu, cm[l][c], 16);  // the partner's column q ^ 2
-            if (h == grp) {  // the owner of layer group grp (id.lg == h when there are two groups)
-#pragma unroll
-                for (int e = 0; e < 2; e++) {
-                    const int q = e ? 2 * (1 - h) + c : 2 * h + c;
-                    const int x = (l * JPT + q) * nc + ct;
-                    float bb = __uint_as_float(park[x]);
-                    uint32_t w1 = park[NS * nc + x], w2 = park[2 * NS * nc + x];
-                    band_fold(__int_as_float(e ? other : cm[l][c]), bb, tau, w1, w2, K, KK);
-                    park[x] = __float_as_uint(bb);
-                    park[NS * nc + x] = w1;
-                    park[2 * NS * nc + x] = w2;
-                }
-            }
-        }
-    }
-}
-
-// Band words of the diagonal block from the parked state (after cons_diag_pair).
-__device__ __forceinline__ void diag_pair_bands(const FastArgs &a, const uint32_t *park, int J, int split,
-                                                const ConsId &id) {
-    const int ct = id.ct, nc = a.ncons;
-    const int g = split * a.Gc + id.gl;
-    if (!(id.active && g < a.G)) return;
-    constexpr int NS = LPT * JPT;
-    const int64_t j0 = (int64_t)J * BJ;
-#pragma unroll
-    for (int l = 0; l < LPT; l++) {
-        const int i = 3 + id.lg * LPT + l;
-#pragma unroll
-        for (int q = 0; q < JPT; q++) {
-            const int64_t j = j0 + id.jq + NJQ * q;
-            const int x = (l * JPT + q) * nc + ct;
-            const uint32_t w1 = park[NS * nc + x], w2 = park[2 * NS * nc + x];
-            if (i <= a.s && j < a.p) a.band[oidx(a, g, i, j)] = band_pack(w1, w2);
-        }
-    }
-}
-
-// Bounded wait (one thread) until `flag` is set; false when the wait gave up
-// (timeout or abort).
-__device__ __forceinline__ bool wait_flag(const FastArgs &a, const int *flag) {
-    uint32_t spins = 0;
-    while (ld_acquire(flag) == 0) {
-        // the abort flag and the spin limit are checked every 64 spins, so a spin costs
-        // one flag load and a short sleep
-        if ((++spins & 63u) == 0u) {
-            if (*(volatile int *)a.abort_flag) return false;
-            if (spins > a.spin_limit) {
-                a.st->timeout = 1;
-                atomicExch(a.abort_flag, 1);
-                return false;
-            }
-        }
-        __nanosleep(32);
-    }
-    return true;
-}
-// ... until column block K of `split` is published (every row), or its rows 2..8 are.
-__device__ __forceinline__ bool wait_block(const FastArgs &a, int split, int K) {
-    return wait_flag(a, a.done + (size_t)split * a.nJ + K);
-}
-__device__ __forceinline__ bool wait_lower(const FastArgs &a, int split, int K) {
-    return wait_flag(a, a.half + (size_t)split * a.nJ + K);
-}
-
-// Publish column block J of `split` (one thread, after a barrier that follows every
-// thread's stores of the block).  The release store orders everything that happens
-// before it, the other threads' stores included through the barrier, before the flag
-// (the pattern of an acq_rel fence plus a relaxed store); readers acquire the flag.
-__device__ __forceinline__ void publish_block(const FastArgs &a, int split, int J) {
-    if (a.hold0 && J == 0) return;  // test hook: the waiters on block 0 must give up
-    st_release(a.done + (size_t)split * a.nJ + J, 1);
-}
-// The first part of a split publish: rows 2..8 of block J (and their block minima).
-__device__ __forceinline__ void publish_lower(const FastArgs &a, int split, int J) {
-    if (a.hold0 && J == 0) return;
-    st_release(a.half + (size_t)split * a.nJ + J, 1);
-}
-
-// ------------------------------------------------------------------ kernels
-// Fused producer: two producer warps compute each tile's interval costs
-// (tile_columns) and stage the dp32 rows with cp.async while the consumer warps
-// evaluate the previous tile (named barriers FULL / EMPTY per buffer).
-template <int LP>
-__global__ void __launch_bounds__(NPROD + MAXCONS, 1) k_wavefront(FastArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem &S = *reinterpret_cast<Smem *>(smem_raw);
-    float *sDP = reinterpret_cast<float *>(smem_raw + sizeof(Smem));
-    const int L = a.s - 2;                // layers 3..s
-    const int rowsDP = a.Gc * L;          // staged dp32 rows per tile (layers 2..s-1)
-    const int tid = threadIdx.x;
-    const int nall = NPROD + a.ncons;
-    for (int q = tid; q <= kMaxS; q += blockDim.x) S.tau[q] = a.prm->tau[q];
-    if (tid < kMaxG) S.lam32[tid] = a.prm->lam32[tid];
+// Grid barrier `epoch` (1, 2, ...): bounded; false when it gave up or another CTA aborted.  All
+// CTAs are resident (cooperative launch).  Orders generic and bulk-copy accesses on both sides.
+__device__ __forceinline__ bool grid_sync(const FastArgs &a, Smem &S, int epoch, bool arrive = true) {
+    asm volatile("fence.proxy.async;" ::: "memory");
     __syncthreads();
-
-    if (tid < NPROD) {
-        // =========================== producer warps ===========================
-        const int jl = tid;  // column within the block
-        uint32_t n = 0;      // tile sequence number
-        for (;;) {
-            if (tid == 0) S.ticket = atomicAdd(a.ticket, 1);
-            bar_sync(BAR_PROD, NPROD);
-            int t = S.ticket;
-            bar_sync(BAR_PROD, NPROD);
-            bool stop = t >= a.nJ * a.nsplit;
-            int J = stop ? 0 : t / a.nsplit, split = stop ? 0 : t % a.nsplit;
-            int ntiles = stop ? 1 : J + 1;
-            for (int K = 0; K < ntiles; K++) {
-                int b = n & 1;
-                if (n >= 2) bar_sync(BAR_EMPTY + b, nall);
-                if (stop) {
-                    if (tid == 0) S.meta[b] = {0, 0, 0, 2};
-                    bar_arrive(BAR_FULL + b, nall);
-                    n++;
+    if (threadIdx.x == 0) {
+        const int target = epoch * (int)gridDim.x;
+        if (arrive) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(a.gbar) : "memory");
+        uint32_t spins = 0;
+        int ok = 1;
+        while (ld_acquire(a.gbar) < target) {
+            if ((++spins & 63u) == 0u) {
+                if (*(volatile int *)a.abort_flag) { ok = 0; break; }
+                if (spins > a.spin_limit) {
+                    a.st->timeout = 1;
+                    atomicExch(a.abort_flag, 1);
+                    ok = 0;
                     break;
                 }
-                bool diag = (K == J);
-                int64_t k0 = (int64_t)K * BK;
-                // wait for column block K (bounded); the diagonal needs nothing
-                if (!diag && tid == 0) wait_block(a, split, K);
-                bar_sync(BAR_PROD, NPROD);
-                tile_consts(a, k0, jl, S.kv, S.kw, S.kd);
-                // dp32 slice of rows (g, layer 2..s-1) for k in the tile (cp.async, L2 only)
-                if (!diag) {
-                    int gbase = split * a.Gc;
-                    int n16 = rowsDP * (BK / 4);
-                    float *dst = sDP + (size_t)b * rowsDP * BK;
-                    for (int q = tid; q < n16; q += NPROD) {
-                        int row = q / (BK / 4), c4 = q % (BK / 4);
-                        int gl = row / L, li = row % L;  // layer index li -> dp row i = 2 + li
-                        int g = gbase + gl;
-                        float *sp = dst + (size_t)row * BK + c4 * 4;
-                        if (g < a.G) {
-                            const float *gp = a.dp32 + d32(a, g, 2 + li, k0 + c4 * 4);
-                            unsigned sa = (unsigned)__cvta_generic_to_shared(sp);
-                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gp) : "memory");
-                        } else {
-                            *reinterpret_cast<float4 *>(sp) = make_float4(CUDART_INF_F, CUDART_INF_F, CUDART_INF_F,
-                                                                          CUDART_INF_F);
-                        }
-                    }
-                    asm volatile("cp.async.commit_group;" ::: "memory");
-                }
-                bar_sync(BAR_PROD, NPROD);
-                tile_columns(a, K, J, jl, S.kv, S.kw, S.kd, S.wsum, S.C[b], S.Phi[b]);
-                if (!diag) asm volatile("cp.async.wait_all;" ::: "memory");
-                if (tid == 0) S.meta[b] = {J, K, split, diag ? 1 : 0};
-                bar_arrive(BAR_FULL + b, nall);
-                n++;
             }
-            if (stop) break;
+            __nanosleep(20);
         }
-        // drain: wait until the consumers released the last two buffers
-        for (uint32_t q = (n >= 2 ? n - 2 : 0); q < n; q++) bar_sync(BAR_EMPTY + (q & 1), nall);
+        S.ok = ok;
+    }
+    __syncthreads();
+    asm volatile("fence.proxy.async;" ::: "memory");
+    return S.ok != 0;
+}
+
+// Bound and mask phases: warp 0 stages up to NT consecutive far tiles of block J -- their column
+// summaries and the tiles' rows of `src` (a.dlast or a.mdp, all G multipliers) -- with two bulk copies.
+__host__ __device__ __forceinline__ size_t stage_floats(int G, int mdp_stride) {
+    return (size_t)NT * BJ * 2 + (size_t)NT * G * mdp_stride;
+}
+__device__ __forceinline__ void stage_tiles(const FastArgs &a, Smem &S, float *stg, int sb, int K0, int n, int J,
+                                            size_t tbase, const float *src, uint64_t policy) {
+    const uint32_t tb = (uint32_t)((size_t)n * BJ * sizeof(float2));
+    const uint32_t mb = (uint32_t)((size_t)n * a.G * a.mdp_stride * sizeof(float));
+    mbar_expect_tx(&S.smbar[sb], tb + mb);
+    bulk_g2s(stg, a.tsum + (cost_tile_idx(K0, J) - tbase) * BJ, tb, &S.smbar[sb], policy);
+    bulk_g2s_nohint(stg + (size_t)NT * BJ * 2, src + (size_t)K0 * a.G * a.mdp_stride, mb, &S.smbar[sb]);
+}
+
+constexpr int kNoBound = 0x7F7F7F7F;  // bits above every finite fp32 cost that occurs; a byte pattern (memset)
+__device__ __forceinline__ int *ub_at(const FastArgs &a, int Jl, int g) {
+    return a.ub + ((size_t)Jl * a.G + g) * (size_t)(a.s - 2) * BJ;
+}
+
+// Upper bounds of the panel's far minima: for every output the least candidate over the last k
+// of each far tile, dp(i-1, 64K+63) + C + lambda' Phi with C and Phi from the tile's summary (where
+// the summary is that k's, which it nearly always is) -- a candidate's own fp32 value, so never
+// below the minimum, and within the change of the candidates over one tile of it.  Tiles are then
+// skipped as if the minimum were known (far_start), whatever the order of the walk.  One candidate of
+// 64 is evaluated for it; at d = 2^17, s = 16 the share of (multiplier, tile) units with any work in a
+// search falls from 0.28 (a walk that knows the tiles to its left) to 0.17, and most of the layers
+// of those drop out too (mask_phase).
+// CTAs split the panel's (column block, tile range) pairs evenly; a thread owns one column of one
+// multiplier, kBoundL layers at a time.
+constexpr int kBoundL = 16;
+static __device__ __noinline__ void bound_phase(const FastArgs &a, Smem &S, float *stage, const Panel &pn,
+                                                uint64_t policy, uint32_t &ns) {
+    const int L = a.s - 2, ct = threadIdx.x, jl = ct & (BJ - 1), gq = ct / BJ;
+    const size_t sfl = stage_floats(a.G, a.mdp_stride);
+    const int parts = max(1, (int)gridDim.x / pn.nb);
+    const int Jl = (int)blockIdx.x % pn.nb, part = (int)blockIdx.x / pn.nb;
+    if (part >= parts) return;
+    const int Ka = (int)((int64_t)pn.P0 * part / parts), Kb = (int)((int64_t)pn.P0 * (part + 1) / parts);
+    if (Ka >= Kb) return;
+    const int J = pn.P0 + Jl, g = min(gq, a.G - 1);
+    const float lam = S.lam32[g];
+    for (int l0 = 0; l0 < L; l0 += kBoundL) {
+        int m[kBoundL];
+#pragma unroll
+        for (int l = 0; l < kBoundL; l++) m[l] = 0x7f800000;
+        if (ct == 0) stage_tiles(a, S, stage + (ns & 1) * sfl, ns & 1, Ka, min(NT, Kb - Ka), J, pn.tbase, a.dlast, policy);
+        for (int K0 = Ka; K0 < Kb; K0 += NT) {
+            const int n = min(NT, Kb - K0), sb = ns & 1;
+            const float *stg = stage + sb * sfl;
+            const uint32_t ph = (ns >> 1) & 1u;
+            ns++;
+            if (K0 + NT < Kb && ct == 0)
+                stage_tiles(a, S, stage + (ns & 1) * sfl, ns & 1, K0 + NT, min(NT, Kb - K0 - NT), J, pn.tbase, a.dlast,
+                            policy);
+            mbar_wait_bounded(&S.smbar[sb], ph, a.st, a.abort_flag);
+            const float2 *ts = reinterpret_cast<const float2 *>(stg) + jl;
+            const float *d = stg + (size_t)NT * BJ * 2 + l0 + (size_t)g * a.mdp_stride;
+            const int rs = a.G * a.mdp_stride, step = a.bound_step;
+#pragma unroll 2
+            for (int r = (step - K0 % step) % step; r < n; r += step) {
+                const float2 v = ts[r * BJ];
+                const bool last = (__float_as_int(v.x) | __float_as_int(v.y)) >= 0;
+                const float w = last ? __fmaf_rn(lam, v.y, v.x) : CUDART_INF_F;
+#pragma unroll
+                for (int l = 0; l < kBoundL; l += 4)
+                    if (l0 + l < L) {  // the rows are padded to a multiple of four
+                        const float4 x = *reinterpret_cast<const float4 *>(d + r * rs + l);
+                        m[l] = min(m[l], __float_as_int(__fadd_rn(x.x, w)));
+                        m[l + 1] = min(m[l + 1], __float_as_int(__fadd_rn(x.y, w)));
+                        m[l + 2] = min(m[l + 2], __float_as_int(__fadd_rn(x.z, w)));
+                        m[l + 3] = min(m[l + 3], __float_as_int(__fadd_rn(x.w, w)));
+                    }
+            }
+            __syncthreads();  // the stage buffer is free
+        }
+#pragma unroll
+        for (int l = 0; l < kBoundL; l++)
+            if (l0 + l < L && gq < a.G && m[l] < kNoBound)
+                atomicMin(ub_at(a, Jl, gq) + (size_t)(l0 + l) * BJ + jl, m[l]);
+    }
+}
+
+// The far phase starts each output's running minimum from +inf, lowered by an earlier pass's minimum
+// (a.seed) and the panel's bound.  Every fp32 candidate is monotone in lambda' (C and Phi are >= 0 and
+// the roundings are monotone), so by induction over the layers an earlier pass's fp32 minimum at a
+// multiplier >= this one's bounds this pass's minimum m from above, as a candidate's own value does.
+// Starting at any such bound changes no result: the tile holding m is never skipped (its lower bound is
+// <= m <= the limit), so the final minimum is m itself; a tile the tighter limit skips has every
+// candidate above m (1 + tau), outside the band; and the walk keeps the band a superset of the tiles with
+// a candidate within m (1 + tau) from any starting bb >= m (a reset drops only tiles whose candidates all
+// lie above the band).  A walk that records no tile adds none to the band.  Only the skip tests
+// see the start.
+__device__ __forceinline__ float far_bound(int w) { return w < kNoBound ? __int_as_float(w) : CUDART_INF_F; }
+// ... of the four outputs o .. o + 3 of a split and column block J: o = t * 64 + column, t = gl * L + li; u: the
+// split's bounds (ub_at).
+__device__ __forceinline__ float4 far_start(const FastArgs &a, const int *u, int J, int o) {
+    float4 v = make_float4(CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, CUDART_INF_F);
+    if (a.bound) {
+        const int4 w = __ldcg(reinterpret_cast<const int4 *>(u + o));
+        v = make_float4(far_bound(w.x), far_bound(w.y), far_bound(w.z), far_bound(w.w));
+    }
+    if (a.seed) {  // (columns past the last value hold +inf)
+        const float4 x = __ldg(reinterpret_cast<const float4 *>(
+            a.seed + ((size_t)J * (size_t)(a.s + 1) + 3 + (o / BJ) % (a.s - 2)) * BJ + (o & (BJ - 1))));
+        v = make_float4(fminf(v.x, x.x), fminf(v.y, x.y), fminf(v.z, x.z), fminf(v.w, x.w));
+    }
+    return v;
+}
+
+// The far tasks: task t = gl * L + li of a multiplier split (multiplier split * Gc + gl, layer 3 + li) on a
+// tile, needed when some column may take a candidate from the tile.  The test is exact skipping: every
+// candidate of the tile for an output is >= lb = fl(min dp(i-1, .) + fl(fma(lam, min Phi, min C))) (rounding
+// is monotone); when lb exceeds the output's band limit bb + bb tau, the tile changes neither its
+// minimum nor its band.  For row js = split * nb + Jl, a.fbits has 128 task bits a tile, and for each word
+// of 32 tiles a.funion says which have any and a.fweight the word's work: the tasks, and kTileCost a tile.
+// With the bounds a needed tile has 1.6 (first pass) to 3.4 (late passes) of its 14 layers needed per
+// multiplier that needs it at d = 2^17, s = 16, so tasks, not whole tiles, are the unit of work.
+// CTAs split the (column block, word range) pairs as in bound_phase; a thread tests one column of one
+// multiplier, kBoundL layers at a time.
+constexpr int kTileCost = 8;  // a listed tile's fixed cost (its copies, its costs into registers) in tasks
+static __device__ __noinline__ void mask_phase(const FastArgs &a, Smem &S, float *stage, const Panel &pn,
+                                               uint64_t policy, uint32_t &ns) {
+    const int L = a.s - 2, ct = threadIdx.x, lane = ct & 31, wid = ct >> 5, jl = ct & (BJ - 1), gq = ct / BJ;
+    const size_t sfl = stage_floats(a.G, a.mdp_stride);
+    const int parts = max(1, (int)gridDim.x / pn.nb);
+    const int Jl = (int)blockIdx.x % pn.nb, part = (int)blockIdx.x / pn.nb, J = pn.P0 + Jl;
+    if (part >= parts) return;
+    const int ba = pn.nB * part / parts, bz = pn.nB * (part + 1) / parts;
+    if (ba >= bz) return;
+    auto stage_word = [&](int b) {
+        stage_tiles(a, S, stage + (ns & 1) * sfl, ns & 1, b * NT, min(NT, pn.P0 - b * NT), J, pn.tbase, a.mdp, policy);
+    };
+    for (int split = 0; split < a.nsplit; split++) {
+        if (ct == 0) stage_word(ba);
+        // the outputs' band limits, into shared memory: one coalesced read, whatever the layers' order
+        float *slim = stage + 2 * sfl;  // [Gc][L][64]
+        const int gs = split * a.Gc, ngv = min(a.Gc, a.G - gs);
+        const int *u = ub_at(a, Jl, gs);
+        for (int o = 4 * ct; o < ngv * L * BJ; o += 4 * MAXCONS) {
+            const float4 v = far_start(a, u, J, o);
+            const float tau = S.tau[3 + (o / BJ) % L];
+            *reinterpret_cast<float4 *>(slim + o) =
+                make_float4(__fadd_rn(v.x, __fmul_rn(v.x, tau)), __fadd_rn(v.y, __fmul_rn(v.y, tau)),
+                            __fadd_rn(v.z, __fmul_rn(v.z, tau)), __fadd_rn(v.w, __fmul_rn(v.w, tau)));
+        }
+        const bool own = gq < ngv;
+        const int g = gs + (own ? gq : 0);
+        const float lam = S.lam32[g];
+        for (int b = ba; b < bz; b++) {
+            const int n = min(NT, pn.P0 - b * NT), sb = ns & 1;
+            const float *stg = stage + sb * sfl, *md = stg + (size_t)NT * BJ * 2;
+            const uint32_t ph = (ns >> 1) & 1u;
+            const int rs = a.G * a.mdp_stride;
+            ns++;
+            if (b + 1 < bz && ct == 0) stage_word(b + 1);
+            if (ct < 32 * kTaskWords) S.tw[ct] = 0u;
+            mbar_wait_bounded(&S.smbar[sb], ph, a.st, a.abort_flag);
+            for (int l0 = 0; l0 < L; l0 += kBoundL) {
+                // block minima of groups of eight tiles
+                for (int q = ct; q < NT / 8 * kMaxG * kBoundL; q += MAXCONS) {
+                    const int grp = q / (kMaxG * kBoundL), gg = (q / kBoundL) % kMaxG, l = q % kBoundL;
+                    float m = CUDART_INF_F;
+                    if (gg < a.G && l0 + l < L)
+#pragma unroll
+                        for (int x = 0; x < 8; x++)
+                            if (8 * grp + x < n) m = fminf(m, md[(8 * grp + x) * rs + gg * a.mdp_stride + l0 + l]);
+                    S.gmin[grp][gg][l] = m;
+                }
+                __syncthreads();  // tw is clear, gmin and slim complete
+                float lim[kBoundL];
+                uint32_t mine[kBoundL];
+#pragma unroll
+                for (int l = 0; l < kBoundL; l++) {
+                    mine[l] = 0u;
+                    lim[l] = (own && l0 + l < L) ? slim[((g - gs) * L + l0 + l) * BJ + jl] : -1.f;
+                }
+                const float2 *ts = reinterpret_cast<const float2 *>(stg) + jl;
+                for (int grp = 0; 8 * grp < n; grp++) {
+                    // a group of eight tiles at a time: the group's least block minimum and summaries bound
+                    // every tile of it, and only a layer that some lane may need there is tested tile by tile
+                    float lb[8], cx = CUDART_INF_F, cy = CUDART_INF_F;
+#pragma unroll
+                    for (int x = 0; x < 8; x++) {
+                        const float2 v = ts[(8 * grp + x) * BJ];
+                        const bool in = 8 * grp + x < n;  // (rows past n hold anything; their bits are dropped)
+                        const float c = fabsf(v.x), f = fabsf(v.y);
+                        lb[x] = __fmaf_rn(lam, f, c);
+                        cx = in ? fminf(cx, c) : cx;
+                        cy = in ? fminf(cy, f) : cy;
+                    }
+                    const uint32_t valid = n - 8 * grp >= 8 ? 0xffu : (1u << (n - 8 * grp)) - 1u;
+                    const float gb = __fmaf_rn(lam, cy, cx);
+                    const float *gm = S.gmin[grp][g];
+                    const float *d = md + (size_t)(8 * grp) * rs + (size_t)g * a.mdp_stride + l0;
+#pragma unroll
+                    for (int l = 0; l < kBoundL; l++)
+                        if (__any_sync(0xffffffffu, __fadd_rn(gm[l], gb) <= lim[l])) {
+                            uint32_t m = 0u;
+#pragma unroll
+                            for (int x = 0; x < 8; x++) m |= (__fadd_rn(d[x * rs + l], lb[x]) <= lim[l] ? 1u : 0u) << x;
+                            mine[l] |= (m & valid) << (8 * grp);
+                        }
+                }
+                // the union over the 64 columns: two warps a multiplier
+#pragma unroll
+                for (int l = 0; l < kBoundL; l++) {
+                    const uint32_t m = __reduce_or_sync(0xffffffffu, mine[l]);
+                    if (lane == 0 && m) atomicOr(&S.tw[(g - gs) * L + l0 + l], m);
+                }
+                __syncthreads();  // this part of tw is complete; gmin is free
+            }
+            // a warp turns two tiles' bits round; word totals by the first warp
+            const size_t w = (size_t)(split * pn.nb + Jl) * pn.nB + b;
+            uint32_t word[kTaskWords];
+#pragma unroll
+            for (int x = 0; x < kTaskWords; x++) word[x] = S.tw[lane + 32 * x];
+#pragma unroll
+            for (int y = 0; y < NT / (MAXCONS / 32); y++) {
+                const int r = NT / (MAXCONS / 32) * wid + y;
+                uint32_t bits[kTaskWords];
+#pragma unroll
+                for (int x = 0; x < kTaskWords; x++) bits[x] = __ballot_sync(0xffffffffu, (word[x] >> r) & 1u);
+                if (lane == 0) __stcg(a.fbits + w * NT + r, make_uint4(bits[0], bits[1], bits[2], bits[3]));
+            }
+            if (wid == 0) {
+                uint32_t any = 0u;
+                int work = 0;
+#pragma unroll
+                for (int x = 0; x < kTaskWords; x++) { any |= word[x]; work += __popc(word[x]); }
+                any = __reduce_or_sync(0xffffffffu, any);
+                work = __reduce_add_sync(0xffffffffu, work);
+                if (lane == 0) {
+                    a.funion[w] = any;
+                    a.fweight[w] = work + kTileCost * __popc(any);
+                }
+            }
+            __syncthreads();  // tw is free
+        }
+    }
+}
+
+// Without the skip test (rows too long to stage): every tile and every task.
+__device__ __forceinline__ void mask_all(const FastArgs &a, const Panel &pn) {
+    const int words = pn.nb * a.nsplit * pn.nB;
+    for (int w = (int)blockIdx.x * MAXCONS + (int)threadIdx.x; w < words; w += (int)gridDim.x * MAXCONS) {
+        const int js = w / pn.nB, n = min(NT, pn.P0 - (w - js * pn.nB) * NT), split = js / pn.nb;
+        const uint32_t u = n == 32 ? 0xffffffffu : (1u << n) - 1u;
+        const int real = min(a.Gc, a.G - split * a.Gc) * (a.s - 2);
+        uint32_t bits[kTaskWords];
+#pragma unroll
+        for (int x = 0; x < kTaskWords; x++)
+            bits[x] = real >= 32 * x + 32 ? 0xffffffffu : real <= 32 * x ? 0u : (1u << (real - 32 * x)) - 1u;
+        for (int r = 0; r < n; r++) __stcg(a.fbits + (size_t)w * NT + r, make_uint4(bits[0], bits[1], bits[2], bits[3]));
+        a.funion[w] = u;
+        a.fweight[w] = n * (real + kTileCost);
+    }
+}
+
+// The position (in work) where each row of the list starts (S.jstart), the CTAs' share (S.share),
+// this CTA's first word (S.first) and the position where it starts (S.fpos).  Every CTA computes the same.
+__device__ __forceinline__ void far_plan(const FastArgs &a, Smem &S, const Panel &pn) {
+    const int ct = threadIdx.x, lane = ct & 31, wid = ct >> 5, nj = pn.nb * a.nsplit;
+    for (int js = wid; js < nj; js += MAXCONS / 32) {
+        int n = 0;
+        for (int b = lane; b < pn.nB; b += 32) n += __ldcg(a.fweight + (size_t)js * pn.nB + b);
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0) S.jstart[js + 1] = n;
+    }
+    __syncthreads();
+    if (wid == 0) {
+        int run = 0;
+        for (int j0 = 0; j0 < nj; j0 += 32) {
+            int v = j0 + lane < nj ? S.jstart[j0 + lane + 1] : 0;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += x;
+            }
+            if (j0 + lane < nj) S.jstart[j0 + lane + 1] = run + v;
+            run += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) S.jstart[0] = 0;
+        const int share = max(1, (run + a.workers - 1) / a.workers);
+        const int pos0 = (int)blockIdx.x * share;
+        __syncwarp();
+        int first = -1, fpos = 0;
+        if ((int)blockIdx.x < a.workers && pos0 < run) {
+            // the row that holds pos0, then its word
+            int js = 0;
+            for (int j0 = 0; j0 < nj; j0 += 32) {
+                const unsigned in = __ballot_sync(0xffffffffu, j0 + lane < nj && S.jstart[j0 + lane] <= pos0 &&
+                                                                   S.jstart[j0 + lane + 1] > pos0);
+                if (in) js = j0 + __ffs(in) - 1;
+            }
+            int before = S.jstart[js];
+            for (int b0 = 0; b0 < pn.nB && first < 0; b0 += 32) {
+                const int b = b0 + lane;
+                int v = b < pn.nB ? (int)__ldcg(a.fweight + (size_t)js * pn.nB + b) : 0;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xffffffffu, v, o);
+                    if (lane >= o) v += x;
+                }
+                const unsigned past = __ballot_sync(0xffffffffu, before + v > pos0);
+                if (past) {
+                    const int l = __ffs(past) - 1;
+                    first = js * pn.nB + b0 + l;
+                    fpos = before + (l ? __shfl_sync(0xffffffffu, v, l - 1) : 0);
+                }
+                before += __shfl_sync(0xffffffffu, v, 31);
+            }
+        }
+        if (lane == 0) {
+            S.share = share;
+            S.first = first;
+            S.fpos = fpos;
+            S.total = run;
+        }
+    }
+    __syncthreads();
+}
+
+// A segment's slot: worker c's results for row js.  (c, js) pairs with work form a monotone path,
+// so c + js names each once.
+__device__ __forceinline__ float *seg_min(const FastArgs &a, int c, int js) {
+    return a.part + (size_t)(c + js) * a.Gc * (a.s - 2) * BJ * 3;
+}
+__device__ __forceinline__ uint2 *seg_runs(const FastArgs &a, float *seg) {
+    return reinterpret_cast<uint2 *>(seg + (size_t)a.Gc * (a.s - 2) * BJ);
+}
+
+// The far phase of one panel: this CTA's share of the list, the tiles whose position lies in
+// [share c, share (c + 1)), in entries of at most a.tcap tasks.  Sixteen warps take 8 of the tile's 64 k and
+// 32 of its columns each, the costs in registers (a lane: one column), and go through the entry's tasks
+// eight at a time: C + lambda' Phi once a multiplier, the task's dp row (one address a warp: a single
+// shared-memory access), the least of 8 candidates into a slot of the column's eight partial minima.
+// After one barrier a pair of warps takes each of the eight tasks, and a lane folds its column's minimum
+// into the band state (shared memory) while the next eight tasks start.  So a tile's costs are read
+// once and the warps are always even.  Shared-memory traffic is what such a loop has to save: with lanes on
+// eight k groups of four columns it took 330 cycles a task, with atomics in place of the slots 280, and
+// a warp of one multiplier with 28 outputs a lane in registers took 10 000 cycles a tile whatever it
+// needed of it.
+constexpr int kFarBufs = 3;
+constexpr int kBatch = 8;      // tasks between two barriers
+constexpr int kFarList = 320;  // list entries held
+struct Pipe {
+    uint32_t n, ns, nnear;  // far entries, stage fills and near tiles so far
+    uint32_t run, fetched;  // tasks evaluated; tiles copied in
+};
+__device__ __forceinline__ float *far_buf(const FastArgs &a, float *big, int b) {
+    return big + (size_t)b * (kCostTileFloats + (size_t)a.tcap * BK);
+}
+
+// The next entries of the share, from word S.lnext (whose position is S.lpos) on: up to 16 words, a warp
+// each, as many as the list holds.  An entry: js << 14 | K, and its tasks as 128 bits.  S.lcount: entries;
+// S.lmore: the share goes on.  All threads.
+__device__ __forceinline__ void far_list(const FastArgs &a, Smem &S, const Panel &pn) {
+    constexpr int kW = MAXCONS / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwords = pn.nb * a.nsplit * pn.nB;
+    const int pos0 = (int)blockIdx.x * S.share, end = min(pos0 + S.share, S.total);
+    const int e0 = S.lnext, e = e0 + wid;
+    // the words' positions
+    const int fw = lane < kW && e0 + lane < nwords ? __ldcg(a.fweight + e0 + lane) : 0;
+    uint32_t u = e < nwords ? __ldcg(a.funion + e) : 0u;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if ((u >> lane) & 1u) v = __ldcg(a.fbits + (size_t)e * NT + lane);
+    int before = fw;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += x;
+    }
+    const int after = S.lpos + __shfl_sync(0xffffffffu, before, kW - 1);  // position after the sixteen words
+    const int wpos = S.lpos + __shfl_sync(0xffffffffu, before - fw, wid);
+    // the word's tiles: position, in the share or not, entries
+    const int n = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+    const int weight = n ? n + kTileCost : 0;
+    int pos = weight;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, pos, o);
+        if (lane >= o) pos += x;
+    }
+    pos += wpos - weight;
+    const bool mine = n && pos >= pos0 && pos < end;
+    const int parts = mine ? (n + a.tcap - 1) / a.tcap : 0;
+    int at = parts;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += x;
+    }
+    const int total = __shfl_sync(0xffffffffu, at, 31);
+    if (lane == 0) S.lwords[wid] = make_int2(total, wpos);
+    __syncthreads();
+    int off = 0, used = 0, all = 0;  // entries of the words before; words taken and their entries
+    for (int w = 0; w < kW; w++) {
+        const int c = S.lwords[w].x;
+        if (w < wid) off += c;
+        if (used == w && all + c <= kFarList) {
+            used++;
+            all += c;
+        }
+    }
+    if (wid < used && mine) {
+        const int js = e / pn.nB, K = (e - js * pn.nB) * NT + lane, split = js / pn.nb;
+        uint32_t bits[kTaskWords] = {v.x, v.y, v.z, v.w};
+        for (int p = 0, i = off + at - parts; p < parts; p++, i++) {  // at most tcap tasks each, lowest first
+            uint32_t out[kTaskWords];
+            int m = 0;
+#pragma unroll
+            for (int x = 0; x < kTaskWords; x++) {
+                uint32_t take = bits[x];
+                while (m + __popc(take) > a.tcap) take &= ~(1u << (31 - __clz(take)));
+                m += __popc(take);
+                out[x] = take;
+                bits[x] &= ~take;
+            }
+            S.lkey[i] = (uint32_t)js << 14 | (uint32_t)K;
+            S.lwhere[i] = (uint32_t)(pn.P0 + js - split * pn.nb) | (uint32_t)(split * a.Gc) << 16;
+            S.lbits[i] = make_uint4(out[0], out[1], out[2], out[3]);
+        }
+    }
+    const int2 cut = used < kW ? S.lwords[used] : make_int2(0, 0);
+    __syncthreads();  // the list is complete, every thread has read lnext and lpos
+    if (threadIdx.x == 0) {
+        S.lcount = all;
+        S.lnext = e0 + used;
+        S.lpos = used < kW ? cut.y : after;
+        S.lmore = e0 + used < nwords && (used < kW ? cut.y : after) < end ? 1 : 0;
+    }
+    __syncthreads();
+}
+
+// Copies of list entry i into buffer b, and its tasks in row order at slot `slot`: t | li << 8 | gl << 16.
+// Five warps share it (role 0: the costs; 1 + x: the rows of the tasks in word x), as a warp that issued it all
+// came 1000 cycles late to the next barrier.  The readers look at the slot after the buffer's phase, which takes
+// one arrival of each.
+__device__ __forceinline__ void far_issue(const FastArgs &a, Smem &S, float *big, const Panel &pn, int i, int slot, int b,
+                                          int role, uint64_t policy) {
+    const int lane = threadIdx.x & 31;
+    const uint4 v = S.lbits[i];
+    const uint32_t where = S.lwhere[i], bits[kTaskWords] = {v.x, v.y, v.z, v.w};
+    const int K = (int)(S.lkey[i] & 0x3FFFu), J = (int)(where & 0xFFFFu), gs = (int)(where >> 16);
+    float *buf = far_buf(a, big, b);
+    if (role == 0) {
+        if (lane == 0) {
+            const int n = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+            mbar_expect_tx(&S.full[b], 2 * kCostHalfBytes + (uint32_t)(n * BK * sizeof(float)));
+            bulk_g2s(buf, a.costs + (cost_tile_idx(K, J) - pn.tbase) * kCostTileFloats, 2 * kCostHalfBytes, &S.full[b],
+                     policy);
+        }
         return;
     }
+    int row = 0;
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int x = 0; x < kTaskWords; x++) {
+        if (x < role - 1) row += __popc(bits[x]);
+        if (x == role - 1) mine = bits[x];
+    }
+    if ((mine >> lane) & 1u) {
+        const int t = lane + 32 * (role - 1);
+        row += __popc(mine & ((1u << lane) - 1u));
+        const uint32_t d = S.tdiv[t];  // li | gl << 8
+        S.tinfo[slot][row] = (uint32_t)t | d << 8;
+        bulk_g2s_nohint(buf + kCostTileFloats + row * BK,
+                        a.dp32 + d32(a, gs + (int)(d >> 8), 2 + (int)(d & 0xFFu), (int64_t)K * BK),
+                        (uint32_t)(BK * sizeof(float)), &S.full[b]);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&S.full[b]);
+}
 
-    // ============================= consumer warps =============================
-    const ConsId id = cons_id(a, tid - NPROD);
-    ConsStateT<LP> cs;
-    uint32_t n = 0;
-    for (;;) {
-        int b = n & 1;
-        bar_sync(BAR_FULL + b, nall);
-        TileMeta m = S.meta[b];
-        if (m.kind == 2) { bar_arrive(BAR_EMPTY + b, nall); break; }
-        const int g = m.split * a.Gc + id.gl;
-        if (m.K == 0) cons_reset(cs);
-        if (m.kind == 0) {
-            if (id.active && g < a.G) cons_offdiag(a, S, sDP + (size_t)b * rowsDP * BK, b, (uint32_t)m.K, g, id, cs);
-            bar_arrive(BAR_EMPTY + b, nall);
-        } else {
-            cons_diag(a, S, b, m.J, m.split, id, cs, false);
-            if (id.ct == 0) publish_block(a, m.split, m.J);
-            bar_arrive(BAR_EMPTY + b, nall);
+// Band runs while a segment is walked, in four bytes: first and last of run 1, then of run 2, as
+// ordinals of the segment's tiles (at most 254, then the segment is stored and goes on in a next
+// part); run 2 absent: 0 (its ordinals are >= 1); no tile yet: kNoRuns.  cont: this tile's K follows the
+// K of the tile before.
+constexpr uint32_t kNoRuns = 0xFFu;
+constexpr int kLastOrd = 254;
+// Runs r appended to the band word (w1, w2), in increasing K, as runs_add appends tiles.
+__device__ __forceinline__ void band_append(uint32_t &w1, uint32_t &w2, bool &any, uint32_t f, uint32_t l) {
+    if (!any) { w1 = (f << 16) | l; any = true; }
+    else if (!w2 && (w1 & 0xFFFFu) + 1u == f) w1 = (w1 & 0xFFFF0000u) | l;
+    else if (!w2) w2 = (f << 16) | l;
+    else w2 = (w2 & 0xFFFF0000u) | l;
+}
+__device__ __forceinline__ uint32_t runs_add(uint32_t w, bool rst, uint32_t o, bool cont) {
+    if (rst || w == kNoRuns) return o | o << 8;
+    const bool has2 = (w >> 24) != 0u;
+    if (!has2 && cont && ((w >> 8) & 0xFFu) + 1u == o) return (w & 0xFFu) | o << 8;
+    return has2 ? (w & 0x00FFFFFFu) | o << 24 : (w & 0xFFFFu) | o << 16 | o << 24;
+}
+
+__device__ __forceinline__ void far_phase(const FastArgs &a, Smem &S, float *big, const Panel &pn, uint64_t policy,
+                                          Pipe &pp) {
+    const int L = a.s - 2, nt = a.Gc * L, ct = threadIdx.x, lane = ct & 31, wid = ct >> 5;
+    const int slice = wid & 7, col = lane + 32 * (wid >> 3);
+    if (S.first < 0) return;
+    float *sbest = far_buf(a, big, kFarBufs);
+    uint32_t *sruns = reinterpret_cast<uint32_t *>(sbest + (size_t)nt * BJ);
+    int *part = reinterpret_cast<int *>(sruns + (size_t)nt * BJ);  // [2][kBatch][8][64]
+    int js = -1, ord = 0, lastK = -2;
+    bool cont = false, next = false;  // next: not the segment's first part
+    // all threads: the segment's minima into the outputs, minima and runs to its slot, behind those of its parts before
+    auto flush = [&]() {
+        const int split = js / pn.nb, real = min(a.Gc, a.G - split * a.Gc) * L * BJ;
+        const int64_t j0 = (int64_t)(pn.P0 + js - split * pn.nb) * BJ;
+        float *seg = seg_min(a, (int)blockIdx.x, js);
+        for (int o = 4 * ct; o < real; o += 4 * MAXCONS) {
+            const float4 v = *reinterpret_cast<const float4 *>(sbest + o);
+            const uint4 w = *reinterpret_cast<const uint4 *>(sruns + o);
+            const float bb[4] = {v.x, v.y, v.z, v.w};
+            const uint32_t r[4] = {w.x, w.y, w.z, w.w};
+            float out[4];
+#pragma unroll
+            for (int x = 0; x < 4; x++) {
+                out[x] = r[x] == kNoRuns ? CUDART_INF_F : bb[x];
+                if (r[x] != kNoRuns) {
+                    const int t = (o + x) / BJ, gl = t / L;
+                    uint32_t w1 = (uint32_t)S.okey[r[x] & 0xFFu] << 16 | S.okey[(r[x] >> 8) & 0xFFu];
+                    uint32_t w2 = r[x] >> 24 ? (uint32_t)S.okey[(r[x] >> 16) & 0xFFu] << 16 | S.okey[r[x] >> 24] : 0u;
+                    if (next && __ldcg(seg + o + x) <= __fadd_rn(bb[x], __fmul_rn(bb[x], S.tau[3 + t - gl * L]))) {
+                        const uint2 old = __ldcg(seg_runs(a, seg) + o + x);
+                        uint32_t f1 = old.x, f2 = old.y;
+                        bool any = true;
+                        band_append(f1, f2, any, w1 >> 16, w1 & 0xFFFFu);
+                        if (w2) band_append(f1, f2, any, w2 >> 16, w2 & 0xFFFFu);
+                        w1 = f1;
+                        w2 = f2;
+                    }
+                    __stcg(seg_runs(a, seg) + o + x, make_uint2(w1, w2));
+                    atomicMin(reinterpret_cast<int *>(
+                                  a.dp32 + d32(a, split * a.Gc + gl, 3 + t - gl * L, j0 + ((o + x) & (BJ - 1)))),
+                              __float_as_int(bb[x]));
+                }
+            }
+            if (next) {  // an output without tiles in this part keeps what it has
+#pragma unroll
+                for (int x = 0; x < 4; x++)
+                    if (r[x] != kNoRuns) __stcg(seg + o + x, out[x]);
+            } else __stcg(reinterpret_cast<float4 *>(seg + o), make_float4(out[0], out[1], out[2], out[3]));
         }
-        n++;
+    };
+    auto start = [&]() {
+        const int split = js / pn.nb, Jl = js - split * pn.nb, real = min(a.Gc, a.G - split * a.Gc) * L * BJ;
+        const int *u = ub_at(a, Jl, split * a.Gc);
+        for (int o = 4 * ct; o < real; o += 4 * MAXCONS) {
+            *reinterpret_cast<float4 *>(sbest + o) = far_start(a, u, pn.P0 + Jl, o);
+            *reinterpret_cast<uint4 *>(sruns + o) = make_uint4(kNoRuns, kNoRuns, kNoRuns, kNoRuns);
+        }
+    };
+    // the row that holds the share's start may have no tile starting in it: its segment is empty
+    auto empty = [&](int j) {
+        float *seg = seg_min(a, (int)blockIdx.x, j);
+        for (int o = ct; o < nt * BJ; o += MAXCONS) __stcg(seg + o, CUDART_INF_F);
+    };
+    const int js0 = S.first / pn.nB;
+    if (ct == 0) { S.lnext = S.first; S.lpos = S.fpos; }
+    uint32_t batch = 0;
+    for (;;) {
+        __syncthreads();  // the list before is done, its folds too
+        far_list(a, S, pn);
+        const int count = S.lcount;
+        if (wid < 5 * min(count, kFarBufs)) {
+            const int i = wid / 5;
+            far_issue(a, S, big, pn, i, i, (int)((pp.n + (uint32_t)i) % kFarBufs), wid - 5 * i, policy);
+        }
+        for (int i = 0; i < count; i++) {
+            const uint32_t key = S.lkey[i];
+            const int jsn = (int)(key >> 14), K = (int)(key & 0x3FFFu), b = (int)(pp.n % kFarBufs), slot = i & 3;
+            const uint4 bits = S.lbits[i];
+            const int n = __popc(bits.x) + __popc(bits.y) + __popc(bits.z) + __popc(bits.w);
+            if (jsn != js) {
+                __syncthreads();  // the folds of the entry before are done
+                if (js >= 0) flush();
+                else if (jsn != js0) empty(js0);
+                __syncthreads();
+                js = jsn;
+                ord = -1;
+                lastK = -2;
+                next = false;
+                start();
+            }
+            if (K != lastK) {
+                cont = K == lastK + 1;
+                if (++ord > kLastOrd) {
+                    __syncthreads();  // the folds of the entry before are done
+                    flush();
+                    __syncthreads();
+                    next = true;
+                    ord = 0;
+                    for (int o = ct; o < nt * BJ; o += MAXCONS) sruns[o] = kNoRuns;
+                }
+                if (ct == 0) S.okey[ord] = (uint16_t)K;
+                lastK = K;
+            }
+            mbar_wait_bounded(&S.full[b], (pp.n / kFarBufs) & 1u, a.st, a.abort_flag);
+            pp.n++;
+            const float *buf = far_buf(a, big, b), *rows = buf + kCostTileFloats + 8 * slice;
+            float4 C[2], F[2];
+#pragma unroll
+            for (int x = 0; x < 2; x++) {
+                C[x] = *reinterpret_cast<const float4 *>(buf + col * PSTR + 8 * slice + 4 * x);
+                F[x] = *reinterpret_cast<const float4 *>(buf + kCostHalfFloats + col * PSTR + 8 * slice + 4 * x);
+            }
+            const int g0 = (js / pn.nb) * a.Gc;
+            float2 W[4];
+            int gcur = -1;
+            for (int k0 = 0; k0 < n; k0 += kBatch, batch++) {
+                int *pt = part + (int)(batch & 1u) * kBatch * 8 * BJ;
+#pragma unroll
+                for (int y = 0; y < kBatch; y++) {
+                    if (k0 + y < n) {
+                        const int gl = (int)(S.tinfo[slot][k0 + y] >> 16);
+                        const float4 p = *reinterpret_cast<const float4 *>(rows + (k0 + y) * BK);
+                        const float4 q = *reinterpret_cast<const float4 *>(rows + (k0 + y) * BK + 4);
+                        if (gl != gcur) {
+                            gcur = gl;
+                            const float lam = S.lam32[g0 + gl];
+                            const float2 lam2 = make_float2(lam, lam);
+#pragma unroll
+                            for (int x = 0; x < 2; x++) {
+                                W[2 * x] = fma2(lam2, make_float2(F[x].x, F[x].y), make_float2(C[x].x, C[x].y));
+                                W[2 * x + 1] = fma2(lam2, make_float2(F[x].z, F[x].w), make_float2(C[x].z, C[x].w));
+                            }
+                        }
+                        // candidates are >= +0, so their bits order like the values: integer mins
+                        const float2 v0 = add2(make_float2(p.x, p.y), W[0]), v1 = add2(make_float2(p.z, p.w), W[1]);
+                        const float2 v2 = add2(make_float2(q.x, q.y), W[2]), v3 = add2(make_float2(q.z, q.w), W[3]);
+                        const int x0 = min(min(__float_as_int(v0.x), __float_as_int(v0.y)), __float_as_int(v1.x));
+                        const int x1 = min(min(__float_as_int(v2.x), __float_as_int(v2.y)), __float_as_int(v3.x));
+                        pt[(y * 8 + slice) * BJ + col] = min(min(x0, x1), min(__float_as_int(v1.y), __float_as_int(v3.y)));
+                    }
+                }
+                __syncthreads();  // the batch's partial minima are complete
+                // (the last batch: the tile's buffer is free, for the entry kFarBufs further on)
+                if (k0 + kBatch >= n && i + kFarBufs < count && ((wid - 5 * i) & 15) < 5)
+                    far_issue(a, S, big, pn, i + kFarBufs, (i + kFarBufs) & 3, b, (wid - 5 * i) & 15, policy);
+                const int k = k0 + slice;
+                if (k < n) {
+                    const uint32_t f = S.tinfo[slot][k];
+                    const int *pk = pt + slice * 8 * BJ + col;
+                    int v = pk[0];
+#pragma unroll
+                    for (int x = 1; x < 8; x++) v = min(v, pk[x * BJ]);
+                    const int o = (int)(f & 0xFFu) * BJ + col;
+                    const float tau = S.tau[3 + ((f >> 8) & 0xFFu)];
+                    const float bb = sbest[o], T = __fmul_rn(bb, tau);
+                    // a tile's minimum below bb - bb tau restarts the band, up to bb + bb tau joins it
+                    // (band limits: the tests on the bits hold for bb = +inf too)
+                    if ((uint32_t)v <= __float_as_uint(__fadd_rn(bb, T))) {
+                        sruns[o] = runs_add(sruns[o], (uint32_t)v < __float_as_uint(__fsub_rn(bb, T)), (uint32_t)ord, cont);
+                        sbest[o] = fminf(bb, __int_as_float(v));
+                    }
+                }
+            }
+            if (ct == 0) pp.run += (uint32_t)n;
+            pp.fetched++;
+        }
+        if (!S.lmore) break;
+    }
+    __syncthreads();
+    if (js >= 0) flush();
+    else empty(js0);
+}
+
+// ---------------------------------------------------------------- near phase
+constexpr int kNearTiles = 4;   // tiles (K, J) of one J per CTA, consecutive K
+constexpr int kNearMults = 2;   // multipliers per CTA
+constexpr int kPanelMax = 16;   // column blocks per panel, at most (four groups of tiles per block)
+// Groups of tiles of the blocks before Jl, and in a panel of nb blocks.
+__host__ __device__ __forceinline__ int near_groups(int nb) {
+    const int f = nb / kNearTiles, r = nb % kNearTiles;
+    return kNearTiles * f * (f + 1) / 2 + r * (f + 1);
+}
+__device__ __forceinline__ int2 ld_relaxed2(const int *p) {
+    int2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed(int *p, int v) {
+    asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Minima of tile group `grp` (near_groups(Jl) + group of Jl) and of single tiles, multiplier g: rows
+// of 64 by layer index li = i - 3.
+__device__ __forceinline__ int *near_group_min(const FastArgs &a, int grp, int g) {
+    return a.tmin + ((size_t)grp * a.G + g) * (size_t)(a.s - 2) * BJ;
+}
+__device__ __forceinline__ int near_tile(int Kl, int Jl) { return Jl * (Jl + 1) / 2 + Kl; }
+__device__ __forceinline__ float *near_tile_min(const FastArgs &a, int nt, int g) {
+    return a.tmin1 + ((size_t)nt * a.G + g) * (size_t)(a.s - 2) * BJ;
+}
+
+// Row i >= 3 of block K = P0 + Kl at multiplier g, columns 2 lane and 2 lane + 1: the far
+// minimum and the minima of the tile groups of block Kl, polled until each carries the panel's tag
+// in its sign bit.  False when the wait gave up.
+__device__ __forceinline__ bool near_gather(const FastArgs &a, int P0, int Kl, int g, int i, int tag, int lane, int &m0,
+                                            int &m1) {
+    const int2 far = ld_relaxed2(reinterpret_cast<const int *>(a.dp32 + d32(a, g, i, (int64_t)(P0 + Kl) * BJ + 2 * lane)));
+    const int *src = near_group_min(a, near_groups(Kl), g) + (size_t)(i - 3) * BJ + 2 * lane;
+    const size_t stride = (size_t)a.G * (size_t)(a.s - 2) * BJ;
+    const int n = Kl / kNearTiles;  // groups 0..n
+    uint32_t spins = 0;
+    for (;;) {
+        // every source at once: a poll is one round trip to L2, and the last writer ends it
+        int bad = 0;
+        m0 = far.x;
+        m1 = far.y;
+#pragma unroll
+        for (int u = 0; u < kPanelMax / kNearTiles; u++)
+            if (u <= n) {
+                const int2 v = ld_relaxed2(src + u * stride);
+                const int x = v.x ^ tag, y = v.y ^ tag;
+                bad |= x | y;
+                m0 = min(m0, x);
+                m1 = min(m1, y);
+            }
+        if (!__any_sync(0xffffffffu, bad < 0)) return true;
+        if ((++spins & 63u) == 0u) {
+            int stop = 0;
+            if (lane == 0) {
+                stop = *(volatile int *)a.abort_flag;
+                if (!stop && spins > a.spin_limit) {
+                    a.st->timeout = 1;
+                    atomicExch(a.abort_flag, 1);
+                    stop = 1;
+                }
+            }
+            if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+        }
     }
 }
 
-// Bulk copies of tile (K, J) into buffer b of the resident-cost kernel: the interval
-// costs from the resident table and, off the diagonal, the dp32 rows (g, layers
-// 2..s-1) of the split's real multipliers (rows of other slots are never read) and
-// their block minima; on the diagonal, row 2 of the block.  res_issue_costs (one
-// thread) expects every byte of the tile on mbar[b] and copies the costs, which no
-// block publishes; res_issue_rows(w) copies multiplier w's rows (w = 0 also the
-// minima) and needs block K made visible to the issuing thread's copies first
-// (res_probe / res_wait for warp 0, the fence after the stage wait for the others).
-// A copy may land before the expectation is posted: the phase cannot complete
-// before the single arrival, which carries the whole byte count.
-__device__ __forceinline__ void res_issue_costs(const FastArgs &a, Smem &S, int b, int K, int J, int split,
-                                                uint64_t policy) {
-    const int L = a.s - 2;
-    const int gbase = split * a.Gc;
-    const bool diag = K == J;
-    const int ngv = std::min(a.G - gbase, a.Gc);  // real multipliers of the split
-    const uint32_t rows_bytes = (uint32_t)((diag ? 1 : L) * BK * sizeof(float));
-    const uint32_t mdp_bytes = (a.prune && !diag) ? (uint32_t)(ngv * a.mdp_stride * sizeof(float)) : 0u;
-    const float *src = a.costs + (cost_tile_idx(K, J) - a.tile_base) * kCostTileFloats;
-    mbar_expect_tx(&S.mbar[b], 2 * kCostHalfBytes + (uint32_t)ngv * rows_bytes + mdp_bytes);
-    bulk_g2s(&S.C[b][0][0], src, kCostHalfBytes, &S.mbar[b], policy);
-    bulk_g2s(&S.Phi[b][0][0], src + kCostHalfFloats, kCostHalfBytes, &S.mbar[b], policy);
-}
-__device__ __forceinline__ void res_issue_rows(const FastArgs &a, Smem &S, float *sDP, int b, int K, int J, int split,
-                                               int w) {
-    const int L = a.s - 2, rowsDP = a.Gc * L;
-    const int gbase = split * a.Gc;
-    const bool diag = K == J;
-    const int ngv = std::min(a.G - gbase, a.Gc);
-    const uint32_t rows_bytes = (uint32_t)((diag ? 1 : L) * BK * sizeof(float));
-    if (w == 0 && a.prune && !diag)
-        bulk_g2s_nohint(&S.mdp[b][0][0], a.mdp + ((size_t)K * a.G + gbase) * a.mdp_stride,
-                        (uint32_t)(ngv * a.mdp_stride * sizeof(float)), &S.mbar[b]);
-    float *dst = diag ? &S.diag[0][w][0] : sDP + (size_t)b * rowsDP * BK + (size_t)w * L * BK;
-    bulk_g2s_nohint(dst, a.dp32 + d32(a, gbase + w, 2, (int64_t)K * BK), rows_bytes, &S.mbar[b]);
-}
-// Warp 0 alone issues the whole tile.
-__device__ __forceinline__ void res_issue(const FastArgs &a, Smem &S, float *sDP, int b, int K, int J, int split,
-                                          uint64_t policy, int lane) {
-    if (lane == 0) res_issue_costs(a, S, b, K, J, split, policy);
-    __syncwarp();
-    if (lane < std::min(a.G - split * a.Gc, a.Gc)) res_issue_rows(a, S, sDP, b, K, J, split, lane);
-}
-
-// Warp 0 of the resident-cost kernel tracks `frontier`: every column block <= frontier
-// of the current split is published.  A block publishes only after the block before
-// it (its last off-diagonal tile waits for that one), so one flag seen set vouches for
-// every block below it, and most tiles need no flag load at all.  When the frontier
-// advances, every lane of warp 0 fences the generic-proxy stores of the newly
-// published blocks (dp32 rows, block minima) against its later bulk copies, so the
-// copies themselves carry no fence.
-// res_probe: is block K published?  If K is past the frontier, the 32 lanes load the
-// flags of blocks K, K + st, K + 2 st, ... (below J) at once and the frontier moves to
-// the highest block seen published.
-__device__ __forceinline__ bool res_probe(const FastArgs &a, int split, int K, int J, int &frontier, int lane) {
-    if (K <= frontier) return true;
-    const int stride = (J - K + 31) / 32;
-    const int m = K + lane * stride;
-    const bool set = m < J && ld_acquire(a.done + (size_t)split * a.nJ + m) != 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, set);
-    if (bal == 0u) return false;
-    frontier = K + (31 - __clz(bal)) * stride;
-    __syncwarp();
-    fence_proxy_async_global();
+// A CTA's near item: tile group `grp` of block Jl (tiles 4 grp .. of it) and multipliers g0, g0 + 1.
+struct NearItem { int Jl, grp, g0; };
+__device__ __forceinline__ bool near_item(const FastArgs &a, int cta, int nb, NearItem &it) {
+    const int pairs = (a.G + kNearMults - 1) / kNearMults;
+    const int x = cta / pairs;
+    if (x >= near_groups(nb)) return false;
+    it.g0 = (cta - x * pairs) * kNearMults;
+    int Jl = 0;
+    while (near_groups(Jl + 1) <= x) Jl++;
+    it.Jl = Jl;
+    it.grp = x - near_groups(Jl);
     return true;
 }
-// res_wait: bounded wait until block K is published (after res_probe said no).
-__device__ __forceinline__ void res_wait(const FastArgs &a, int split, int K, int &frontier, int lane) {
-    int ok = 0;
-    if (lane == 0) ok = wait_block(a, split, K) ? 1 : 0;
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    if (ok) frontier = max(frontier, K);
-    __syncwarp();
-    fence_proxy_async_global();
-}
 
-// Tile skipping in batches (resident or streamed costs).  A batch is up to a.stage_tiles
-// (at most 32) consecutive off-diagonal tiles of block J; warp 0 stages their column
-// summaries (a.tsum) and the block minima of their column blocks (a.mdp, all G
-// multipliers) into a stage buffer with two bulk copies, one batch ahead.  The stage
-// buffers follow the dp32 rows in shared memory: where the paired diagonal parks its
-// band state (free until the diagonal; 32 tiles per batch), else in space of their own
-// (16 tiles per batch, for the larger rows of more layers).
-__host__ __device__ __forceinline__ size_t stage_floats(int G, int mdp_stride, int ntiles) {
-    return (size_t)ntiles * BJ * 2 + (size_t)ntiles * G * mdp_stride;
-}
-// The batch after the one ending at K1: 1, 1, 2, 4, ... nt tiles (the band limits are
-// +inf before the first tile and tighten fast).
-__device__ __forceinline__ int batch_end(int K1, int J, int nt) { return min(J, K1 + min(nt, max(1, K1))); }
-
-// Warp 0: stage tiles K0 <= K < K1 of block J into stage buffer sb.  Minima of blocks
-// past `frontier` may be incomplete in the copy; need_mask does not read them.
-template <int NT>
-__device__ __forceinline__ void res_stage(const FastArgs &a, Smem &S, float *stg, int sb, int K0, int K1, int J,
-                                          int frontier, uint64_t policy, int lane) {
-    if (lane == 0) {
-        const uint32_t tb = (uint32_t)((size_t)(K1 - K0) * BJ * sizeof(float2));
-        const uint32_t mb = (uint32_t)((size_t)(K1 - K0) * a.G * a.mdp_stride * sizeof(float));
-        S.sfront[sb] = frontier;  // ordered before the readers' wait by the arrive (release)
-        mbar_expect_tx(&S.smbar[sb], tb + mb);
-        bulk_g2s(stg, a.tsum + (cost_tile_idx(0, J) - a.tile_base + (size_t)K0) * BJ, tb, &S.smbar[sb], policy);
-        bulk_g2s_nohint(stg + (size_t)NT * BJ * 2, a.mdp + (size_t)K0 * a.G * a.mdp_stride, mb, &S.smbar[sb]);
-    }
-}
-
-// Batch skip test of one warp over the staged tiles K0 <= K < K1: bit K - K0 of the
-// result is set when some output of the warp may take a candidate from tile K by the
-// test of cons_offdiag, here evaluated on the staged column minima and block minima
-// with the warp's band limits as they stand.  The limits only shrink as later tiles
-// fold, and rounding is monotone, so a tile this test rules out is ruled out by
-// cons_offdiag too: walking only the tiles some warp needs changes no result.  Blocks
-// past `fr` had no published minima when staged and are always needed.
-template <int NT, int LP>
-__device__ __forceinline__ uint32_t need_mask(const FastArgs &a, const Smem &S, const float *stg, int K0, int K1, int fr,
-                                              int g, const ConsId &id, const ConsStateT<LP> &cs) {
-    const int L = a.s - 2;
+// The near phase of one panel; the item's cost tiles are in `tiles`, ex and rowbuf are scratch.  The
+// diagonal tile's warp also writes the block's final dp32 rows, its block minima and last column
+// (read by later panels' far phases).
+static __device__ __noinline__ void near_phase(const FastArgs &a, Smem &S, const float *tiles, float *rowbuf, int P0,
+                                               NearItem it, int tag) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, q = wid & 3, h = (wid >> 2) & 1, half = wid >> 3;
+    const int g = it.g0 + h;
+    if (g >= a.G) return;  // all eight warps of this multiplier
+    const int Kl = it.grp * kNearTiles + q, K = P0 + Kl, J = P0 + it.Jl;
+    const bool have = Kl <= it.Jl, diag = Kl == it.Jl;
     const float lam = S.lam32[g];
-    int rowl[LP];
-    float lim[LP][JPT];
+    const float2 lam2 = make_float2(lam, lam);
+    const int col = lane + 32 * half;
+    float2 W[BK / 2];  // costs of the lane's column
+    const float *tile = tiles + (size_t)q * kCostTileFloats + col * PSTR;
 #pragma unroll
-    for (int l = 0; l < LP; l++) {
-        rowl[l] = min(id.lg * LP + l, L - 1);
-        const float tau = S.tau[3 + rowl[l]];
-#pragma unroll
-        for (int q = 0; q < JPT; q++) lim[l][q] = __fadd_rn(cs.best[l][q], __fmul_rn(cs.best[l][q], tau));
+    for (int kk = 0; kk < BK; kk += 4) {
+        float4 c4 = make_float4(CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, CUDART_INF_F);
+        float4 f4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (have) {
+            c4 = *reinterpret_cast<const float4 *>(tile + kk);
+            f4 = *reinterpret_cast<const float4 *>(tile + kCostHalfFloats + kk);
+        }
+        W[kk / 2] = fma2(lam2, make_float2(f4.x, f4.y), make_float2(c4.x, c4.y));
+        W[kk / 2 + 1] = fma2(lam2, make_float2(f4.z, f4.w), make_float2(c4.z, c4.w));
     }
-    const float2 *ts = reinterpret_cast<const float2 *>(stg) + id.jq;
-    const float *md = stg + (size_t)NT * BJ * 2 + (size_t)g * a.mdp_stride + 2;
-    const int mstride = a.G * a.mdp_stride;
-    uint32_t mask = 0;
-#pragma unroll 2
-    for (int K = K0; K < K1; K++) {
-        bool need = true;
-        if (K <= fr) {
-            const int r = K - K0;
-            float lbq[JPT];
-#pragma unroll
-            for (int q = 0; q < JPT; q++) {
-                const float2 v = ts[r * BJ + NJQ * q];
-                lbq[q] = __fmaf_rn(lam, v.y, v.x);
-            }
-            need = false;
-#pragma unroll
-            for (int l = 0; l < LP; l++) {
-                const float m = md[r * mstride + rowl[l]];
-#pragma unroll
-                for (int q = 0; q < JPT; q++) need |= __fadd_rn(m, lbq[q]) <= lim[l][q];
+    float *row = rowbuf + wid * 2 * BK;
+    int *ex = reinterpret_cast<int *>(rowbuf + (MAXCONS / 32) * 2 * BK) + h * 2 * kNearTiles * BJ;  // [parity][tile][64]
+    const int oc = (q + 4 * half) * 8 + lane;  // lanes 0..7: the column whose group minimum this lane writes
+    int *out = near_group_min(a, near_groups(it.Jl) + it.grp, g) + oc;
+    float *out1 = near_tile_min(a, have ? near_tile(Kl, it.Jl) : 0, g) + col;
+    const bool hold = a.hold0 && J == 0;  // test hook: block 0 is never published
+    float *mdp = a.mdp + ((size_t)J * a.G + g) * a.mdp_stride, *dlast = a.dlast + ((size_t)J * a.G + g) * a.mdp_stride;
+    bool dead = false;  // a wait gave up: only the barriers are kept
+    for (int i = 3; i <= a.s; i++) {
+        int m0 = 0x7f800000, m1 = 0x7f800000;  // row i - 1 of block K, columns 2 lane, 2 lane + 1
+        if (have && !dead) {
+            if (i == 3) {
+                const int2 r = ld_relaxed2(reinterpret_cast<const int *>(a.dp32 + d32(a, g, 2, (int64_t)K * BK + 2 * lane)));
+                m0 = r.x;
+                m1 = r.y;
+            } else if (!near_gather(a, P0, Kl, g, i - 1, tag, lane, m0, m1)) {
+                dead = true;
             }
         }
-        mask |= (__any_sync(0xffffffffu, need) ? 1u : 0u) << (K - K0);
+        float *rw = row + (i & 1) * BK;
+        *reinterpret_cast<float2 *>(rw + 2 * lane) = make_float2(__int_as_float(m0), __int_as_float(m1));
+        __syncwarp();
+        int a0 = 0x7f800000, a1 = 0x7f800000, b0 = 0x7f800000, b1 = 0x7f800000;
+#pragma unroll
+        for (int kk = 0; kk < BK; kk += 8) {
+            const float4 d4 = *reinterpret_cast<const float4 *>(rw + kk), e4 = *reinterpret_cast<const float4 *>(rw + kk + 4);
+            const float2 s0 = add2(make_float2(d4.x, d4.y), W[kk / 2]), s1 = add2(make_float2(d4.z, d4.w), W[kk / 2 + 1]);
+            const float2 t0 = add2(make_float2(e4.x, e4.y), W[kk / 2 + 2]), t1 = add2(make_float2(e4.z, e4.w), W[kk / 2 + 3]);
+            a0 = min(min(a0, __float_as_int(s0.x)), __float_as_int(s0.y));
+            a1 = min(min(a1, __float_as_int(s1.x)), __float_as_int(s1.y));
+            b0 = min(min(b0, __float_as_int(t0.x)), __float_as_int(t0.y));
+            b1 = min(min(b1, __float_as_int(t1.x)), __float_as_int(t1.y));
+        }
+        a0 = min(min(a0, a1), min(b0, b1));
+        int *x = ex + (i & 1) * kNearTiles * BJ;
+        x[q * BJ + col] = a0;
+        bar_sync(BAR_NEAR + h, 256);
+        if (lane < 8 && !hold && !dead)
+            st_relaxed(out + (size_t)(i - 3) * BJ,
+                       min(min(x[oc], x[BJ + oc]), min(x[2 * BJ + oc], x[3 * BJ + oc])) ^ tag);
+        if (have) out1[(size_t)(i - 3) * BJ] = __int_as_float(a0);
+        if (diag && half == 0) {
+            if (i > 3)
+                *reinterpret_cast<float2 *>(a.dp32 + d32(a, g, i - 1, (int64_t)J * BJ + 2 * lane)) =
+                    make_float2(__int_as_float(m0), __int_as_float(m1));
+            if (a.prune) {
+                const int mn = __reduce_min_sync(0xffffffffu, min(m0, m1));  // block minimum of row i - 1
+                if (lane == 0) mdp[i - 3] = __int_as_float(mn);
+                if (lane == 31) dlast[i - 3] = __int_as_float(m1);
+            }
+        }
     }
-    return mask;
+    if (diag && half == 0 && !dead) {
+        int m0, m1;
+        if (near_gather(a, P0, Kl, g, a.s, tag, lane, m0, m1))
+            *reinterpret_cast<float2 *>(a.dp32 + d32(a, g, a.s, (int64_t)J * BJ + 2 * lane)) =
+                make_float2(__int_as_float(m0), __int_as_float(m1));
+    }
 }
 
-// Resident interval costs: no producer warps.  Warp 0 claims the column blocks,
-// waits for the flags and issues the bulk copies of the next tile while the current
-// one is evaluated (two buffers, one mbarrier each); all MAXCONS threads are
-// consumers.  With tile skipping the off-diagonal tiles go in staged batches: every
-// warp runs need_mask over the batch and only the tiles some warp needs are copied
-// in and walked, so a tile every warp rules out costs neither HBM traffic nor a
-// barrier; the next batch is staged while this one is walked.
-template <int LP>
-__global__ void __launch_bounds__(MAXCONS, 1) k_wavefront_res(FastArgs a) {
+// Band words of a panel's outputs from the far segments and the near tiles in increasing K: a
+// segment (or tile) whose minimum lies above the output's band limit adds nothing; else its runs
+// are appended as a walk appends tiles (runs_add).
+static __device__ __noinline__ void fold_panel(const FastArgs &a, const Smem &S, const Panel &pn) {
+    const int L = a.s - 2, per = a.G * L * BJ;
+    for (int idx = (int)(blockIdx.x * MAXCONS + threadIdx.x); idx < pn.nb * per;
+         idx += (int)(gridDim.x * MAXCONS)) {
+        const int Jl = idx / per, o = idx - Jl * per;
+        const int g = o / (L * BJ), li = (o / BJ) % L, jl = o & (BJ - 1);
+        const int64_t j = (int64_t)(pn.P0 + Jl) * BJ + jl;
+        if (j >= a.p) continue;
+        const float m = __ldcg(a.dp32 + d32(a, g, 3 + li, j));
+        const float lim = __fadd_rn(m, __fmul_rn(m, S.tau[3 + li]));
+        uint32_t w1 = 0, w2 = 0;
+        bool any = false;
+        auto append = [&](uint32_t f, uint32_t l) { band_append(w1, w2, any, f, l); };
+        if (pn.P0 > 0) {
+            const int split = g / a.Gc, js = split * pn.nb + Jl;
+            const int p0 = S.jstart[js], p1 = S.jstart[js + 1];
+            if (p1 > p0) {
+                const int c0 = p0 / S.share, c1 = (p1 - 1) / S.share;
+                const size_t so = (size_t)(g - split * a.Gc) * L * BJ + (size_t)li * BJ + jl;
+#pragma unroll 4
+                for (int c = c0; c <= c1; c++) {
+                    float *seg = seg_min(a, c, js);
+                    if (__ldcg(seg + so) <= lim && m < CUDART_INF_F) {
+                        const uint2 r = __ldcg(seg_runs(a, seg) + so);
+                        append(r.x >> 16, r.x & 0xFFFFu);
+                        if (r.y) append(r.y >> 16, r.y & 0xFFFFu);
+                    }
+                }
+            }
+        }
+        const int *grp = near_group_min(a, near_groups(Jl), g) + (size_t)li * BJ + jl;
+        const float *tm = near_tile_min(a, near_tile(0, Jl), g) + (size_t)li * BJ + jl;
+        const size_t step = (size_t)per;
+#pragma unroll
+        for (int u = 0; u < kPanelMax / kNearTiles; u++) {
+            if (u * kNearTiles > Jl) continue;
+            if (!(__int_as_float(__ldcg(grp + u * step) & 0x7fffffff) <= lim)) continue;
+            for (int Kl = u * kNearTiles; Kl <= min(Jl, u * kNearTiles + kNearTiles - 1); Kl++)
+                if (__ldcg(tm + Kl * step) <= lim) append((uint32_t)(pn.P0 + Kl), (uint32_t)(pn.P0 + Kl));
+        }
+        a.band[oidx(a, g, 3 + li, j)] = band_pack(w1, w2);
+    }
+}
+
+// The min-plus sweep over column blocks [J0, J1), panel by panel (see above).  build: the costs
+// buffer holds one panel's tiles, computed here before the panel's far phase (no resident or
+// streamed table).  Cooperative launch, one CTA of 512 threads per SM.
+__global__ void __launch_bounds__(MAXCONS, 1) k_wavefront(const __grid_constant__ FastArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
-    float *sDP = reinterpret_cast<float *>(smem_raw + sizeof(Smem));
-    const int L = a.s - 2;
-    const int rowsDP = a.Gc * L;
+    float *big = reinterpret_cast<float *>(smem_raw + kSmemHead);
     const int ct = threadIdx.x;
-    const int lane = ct & 31;
-    for (int q = ct; q <= kMaxS; q += blockDim.x) S.tau[q] = a.prm->tau[q];
+    for (int q = ct; q <= kMaxS; q += MAXCONS) S.tau[q] = a.prm->tau[q];
     if (ct < kMaxG) S.lam32[ct] = a.prm->lam32[ct];
+    if (ct < 32 * kTaskWords) S.tdiv[ct] = (uint16_t)(ct % (a.s - 2) | ct / (a.s - 2) << 8);
     if (ct == 0) {
-        mbar_init(&S.mbar[0], 1);
-        mbar_init(&S.mbar[1], 1);
-        mbar_init(&S.smbar[0], 1);
-        mbar_init(&S.smbar[1], 1);
+        for (int b = 0; b < 2; b++) mbar_init(&S.smbar[b], 1);
+        for (int b = 0; b < kFarBufs; b++) mbar_init(&S.full[b], 1 + kTaskWords);
+        mbar_init(&S.nbar, 1);
         mbar_fence_init();
     }
     __syncthreads();
-    const ConsId id = cons_id(a, ct);
-    ConsStateT<LP> cs;
     const uint64_t policy = policy_evict_first();
-    uint32_t n = 0;   // tile sequence number: buffer n & 1
-    uint32_t mph[2] = {0u, 0u};  // completed phases of mbar[0], mbar[1] (one per fill; two for a split last tile)
-    uint32_t ns = 0;  // batch sequence number (tile skipping): stage buffer ns & 1, its fill ns >> 1
-    float *stage = sDP + (size_t)2 * rowsDP * BK;  // the park area, free off the diagonal
-    constexpr int NT = LP == LPT ? 32 : 16;  // tiles per staged batch (a.stage_tiles, set to match)
-    const size_t sfl = stage_floats(a.G, a.mdp_stride, NT);
-    unsigned long long n_run = 0, n_skip = 0;  // lane 0 of each warp: its (warp, tile) units
-    int frontier = -1, fsplit = -1;            // warp 0 (res_probe)
-    for (;;) {
-        if (ct == 0) S.ticket = atomicAdd(a.ticket, 1);
-        __syncthreads();
-        const int t = S.ticket;
-        if (t >= (a.J1 - a.J0) * a.nsplit) break;
-        const int J = a.J0 + t / a.nsplit, split = t % a.nsplit;
-        const int g = split * a.Gc + id.gl;
-        const bool own = id.active && g < a.G;
-        if (split != fsplit) { frontier = -1; fsplit = split; }
-        cons_reset(cs);
-        if (a.seed && own) cons_seed(a, cs, J, id);
-        int issued = -1;  // the tile whose copies are in flight into buffer n & 1 (J: the diagonal), or -1
-        const int ngv = min(a.G - split * a.Gc, a.Gc);  // real multipliers of the split
-        // the tiles walked here: K < Kend (with a split publish the last one, J - 1, is the chain's)
-        const int Kend = a.split_pub ? max(J - 1, 0) : J;
-        if (a.prune && Kend > 0 && ct < 32) {  // stage the first batch
-            if (frontier < 0) res_probe(a, split, 0, J, frontier, lane);
-            res_stage<NT>(a, S, stage + (ns & 1) * sfl, ns & 1, 0, batch_end(0, Kend, NT), J, frontier, policy, lane);
+    Pipe pp{0u, 0u, 0u, 0u, 0u};
+    int epoch = 0, panel = 0;
+    bool ok = true;
+    for (int P0 = a.J0; P0 < a.J1 && ok; P0 += a.T, panel++) {
+        Panel pn;
+        pn.P0 = P0;
+        pn.nb = min(a.T, a.J1 - P0);
+        pn.nB = (P0 + NT - 1) / NT;
+        pn.tag = (panel & 1) ? (int)0x80000000 : 0;
+        pn.tbase = a.build ? (size_t)P0 * (P0 + 1) / 2 : a.tile_base;
+        if (a.build) {
+            // (a tile is one long chain of 64 steps: 14 us, so six groups beside one another, the CTAs' first ones first)
+            if (ct < kBuildGroups * NPROD)
+                build_panel(a, reinterpret_cast<BuildSmem *>(big)[ct / NPROD], ct % NPROD, BAR_BUILD + ct / NPROD,
+                            (int64_t)pn.tbase + ct / NPROD * gridDim.x + blockIdx.x, (int64_t)gridDim.x * kBuildGroups,
+                            (int64_t)(P0 + pn.nb) * (P0 + pn.nb + 1) / 2, (int64_t)pn.tbase);
+            ok = grid_sync(a, S, ++epoch);
+            if (!ok) break;
         }
-        for (int K0 = 0; K0 < Kend;) {
-            const int K1 = a.prune ? batch_end(K0, Kend, NT) : min(Kend, K0 + 32);
-            uint32_t wm = 0xffffffffu;  // the warp's tiles of the batch
-            uint32_t U = 0xffffffffu;   // the tiles some warp needs
-            int frb = -1;               // tiles <= frb: every warp issues its own rows (res_issue_rows)
-            if (a.prune) {
-                const int sb = ns & 1;
-                mbar_wait_bounded(&S.smbar[sb], (ns >> 1) & 1u, a.st, a.abort_flag);
-                frb = S.sfront[sb];
-                if (lane == 0) fence_proxy_async_global();  // blocks <= frb, published, before this warp's copies
-                wm = own ? need_mask<NT>(a, S, stage + sb * sfl, K0, K1, frb, g, id, cs) : 0u;
-                if (lane == 0) S.needw[sb][ct >> 5] = wm;
-                __syncthreads();  // needw; every read of stage buffer sb is done
-                U = 0;
-                for (int w = 0; w < (int)(blockDim.x >> 5); w++) U |= S.needw[sb][w];
-                ns++;
-                if (K1 < Kend && ct < 32) {  // stage the next batch while this one is walked
-                    const int K2 = batch_end(K1, Kend, NT);
-                    if (K2 - 1 > frontier) res_probe(a, split, frontier + 1, J, frontier, lane);
-                    res_stage<NT>(a, S, stage + (ns & 1) * sfl, ns & 1, K1, K2, J, frontier, policy, lane);
-                }
+        if (P0 > 0) {
+            if (a.bound) {
+                bound_phase(a, S, big, pn, policy, pp.ns);
+                ok = grid_sync(a, S, ++epoch);
+                if (!ok) break;
             }
-            U &= (K1 - K0 == 32) ? 0xffffffffu : ((1u << (K1 - K0)) - 1u);
-            if (own) n_skip += (unsigned long long)(K1 - K0 - __popc(U));
-            if (U && issued < 0) {
-                const int Kf = K0 + __ffs(U) - 1;
-                if (Kf <= frb) {
-                    if (ct == 0) res_issue_costs(a, S, n & 1, Kf, J, split, policy);
-                    if (lane == 0 && (ct >> 5) < ngv) res_issue_rows(a, S, sDP, n & 1, Kf, J, split, ct >> 5);
-                } else if (ct < 32) {
-                    if (!res_probe(a, split, Kf, J, frontier, lane)) res_wait(a, split, Kf, frontier, lane);
-                    res_issue(a, S, sDP, n & 1, Kf, J, split, policy, lane);
-                }
-            }
-            while (U) {
-                const int K = K0 + __ffs(U) - 1;
-                U &= U - 1;
-                // the next tile to copy: the batch's next needed one, else the diagonal after
-                // the last batch (with a split publish the tail copies its own tiles), else (no
-                // skipping) the next batch's first tile
-                const int Kn = U ? K0 + __ffs(U) - 1 : (K1 == Kend ? (a.split_pub ? -1 : J) : (a.prune ? -1 : K1));
-                const int b = n & 1;
-                bool pending = false;  // warp 0: the rows of tile Kn still to be issued
-                if (Kn >= 0 && Kn < J && Kn <= frb) {
-                    if (ct == 0) res_issue_costs(a, S, b ^ 1, Kn, J, split, policy);
-                    if (lane == 0 && (ct >> 5) < ngv) res_issue_rows(a, S, sDP, b ^ 1, Kn, J, split, ct >> 5);
-                } else if (ct < 32 && Kn >= 0) {
-                    const bool ready = Kn >= J || res_probe(a, split, Kn, J, frontier, lane);
-                    if (ready)
-                        res_issue(a, S, sDP, b ^ 1, Kn, J, split, policy, lane);
-                    else if (lane == 0)
-                        res_issue_costs(a, S, b ^ 1, Kn, J, split, policy);  // the costs publish nothing
-                    pending = !ready;
-                }
-                issued = Kn;
-                mbar_wait_bounded(&S.mbar[b], mph[b] & 1u, a.st, a.abort_flag);
-                mph[b]++;
-                if (own) {
-                    const bool ran = ((wm >> (K - K0)) & 1u) &&
-                                     cons_offdiag(a, S, sDP + (size_t)b * rowsDP * BK, b, (uint32_t)K, g, id, cs);
-                    n_run += ran ? 1 : 0;
-                    n_skip += ran ? 0 : 1;
-                }
-                __syncthreads();  // buffer b free for the tile after Kn
-                if (ct < 32 && pending) {
-                    res_wait(a, split, Kn, frontier, lane);
-                    if (lane < ngv) res_issue_rows(a, S, sDP, b ^ 1, Kn, J, split, lane);
-                }
-                n++;
-            }
-            K0 = K1;
+            if (a.prune) mask_phase(a, S, big, pn, policy, pp.ns);
+            else mask_all(a, pn);
+            ok = grid_sync(a, S, ++epoch);
+            if (!ok) break;
+            far_plan(a, S, pn);
+            far_phase(a, S, big, pn, policy, pp);
+            __syncthreads();  // the tile buffers are free
         }
-        if constexpr (LP != LPT) {  // the generic diagonal (no split publish, no parked state)
-            const int b = n & 1;
-            if (issued != J && ct < 32) res_issue(a, S, sDP, b, J, J, split, policy, lane);
-            mbar_wait_bounded(&S.mbar[b], mph[b] & 1u, a.st, a.abort_flag);
-            mph[b]++;
-            cons_diag(a, S, b, J, split, id, cs, true);
-            __syncthreads();  // every thread's dp32 and layer minima of block J are stored
-            if (ct == 0) publish_block(a, split, J);
-            n++;
-        } else if (a.split_pub) {
-            // the chain's part: tile (J-1, J) in buffer bA, the diagonal in bD (the cost copies
-            // depend on nothing published; the diagonal also copies row 2 of block J)
-            uint32_t *park = reinterpret_cast<uint32_t *>(sDP + (size_t)2 * rowsDP * BK);
-            const int bA = n & 1, bD = bA ^ 1;
-            const int gbase = split * a.Gc;
-            const uint32_t lo_bytes = (uint32_t)(LPT * BK * sizeof(float));        // rows 2..8
-            const uint32_t hi_bytes = (uint32_t)((L - LPT) * BK * sizeof(float));  // rows 9..s-1
-            float *rowsA = sDP + (size_t)bA * rowsDP * BK;
-            if (ct < 32) {
-                if (lane == 0) {
-                    if (J > 0) {
-                        mbar_expect_tx(&S.mbar[bA], 2 * kCostHalfBytes + (uint32_t)ngv * lo_bytes);
-                        const float *src = a.costs + (cost_tile_idx(J - 1, J) - a.tile_base) * kCostTileFloats;
-                        bulk_g2s(&S.C[bA][0][0], src, kCostHalfBytes, &S.mbar[bA], policy);
-                        bulk_g2s(&S.Phi[bA][0][0], src + kCostHalfFloats, kCostHalfBytes, &S.mbar[bA], policy);
-                    }
-                    res_issue_costs(a, S, bD, J, J, split, policy);
-                }
-                __syncwarp();
-                if (lane < ngv) res_issue_rows(a, S, sDP, bD, J, J, split, lane);
-            }
-            mbar_wait_bounded(&S.mbar[bD], mph[bD] & 1u, a.st, a.abort_flag);
-            mph[bD]++;
-            float2 W[2 * kDiagGroups];
-            diag_prepare(a, S, park, bD, J, split, id, cs, W);
-            int cur = 0;
-            if (J > 0) {  // layer group 0 of tile (J-1, J): rows 2..8 of block J-1
-                if (ct < 32) {
-                    if (lane == 0) wait_lower(a, split, J - 1);
-                    __syncwarp();
-                    fence_proxy_async_global();
-                    if (lane < ngv)
-                        bulk_g2s_nohint(rowsA + (size_t)lane * L * BK, a.dp32 + d32(a, gbase + lane, 2, (int64_t)(J - 1) * BK),
-                                        lo_bytes, &S.mbar[bA]);
-                }
-                mbar_wait_bounded(&S.mbar[bA], mph[bA] & 1u, a.st, a.abort_flag);
-                mph[bA]++;
-                if (own) cons_lasttile_grp(a, S, rowsA, bA, park, (uint32_t)(J - 1), g, id, 0);
-                __syncwarp();
-            }
-            diag_layers(a, S, park, J, split, id, W, 0, LPT - 1, cur);  // layers 3..8
-            diag_store(a, park, J, split, id, 3, 2 + LPT - 1);
-            __syncthreads();  // rows 3..8 and their block minima are stored
-            if (ct == 0) publish_lower(a, split, J);
-            diag_layers(a, S, park, J, split, id, W, LPT - 1, LPT, cur);  // layer 9
-            if (J > 0) {  // layer group 1: rows 9..s-1 of block J-1, after its full publish
-                if (ct < 32) {
-                    if (lane == 0) {
-                        mbar_expect_tx(&S.mbar[bA], (uint32_t)ngv * hi_bytes);
-                        wait_block(a, split, J - 1);
-                    }
-                    __syncwarp();
-                    fence_proxy_async_global();
-                    if (lane < ngv)
-                        bulk_g2s_nohint(rowsA + (size_t)lane * L * BK + LPT * BK,
-                                        a.dp32 + d32(a, gbase + lane, 2 + LPT, (int64_t)(J - 1) * BK), hi_bytes,
-                                        &S.mbar[bA]);
-                }
-                mbar_wait_bounded(&S.mbar[bA], mph[bA] & 1u, a.st, a.abort_flag);
-                mph[bA]++;
-                if (own) cons_lasttile_grp(a, S, rowsA, bA, park, (uint32_t)(J - 1), g, id, 1);
-                __syncwarp();
-                if (own) n_run++;
-            }
-            diag_layers(a, S, park, J, split, id, W, LPT, L, cur);  // layers 10..s
-            diag_store(a, park, J, split, id, 2 + LPT, a.s);
-            __syncthreads();  // every row and block minimum of block J is stored
-            if (ct == 0) publish_block(a, split, J);
-            diag_pair_bands(a, park, J, split, id);
-            n += 2;
-        } else {  // the diagonal tile (issued with the last tile walked, else now)
-            const int b = n & 1;
-            if (issued != J && ct < 32) res_issue(a, S, sDP, b, J, J, split, policy, lane);
-            mbar_wait_bounded(&S.mbar[b], mph[b] & 1u, a.st, a.abort_flag);
-            mph[b]++;
-            uint32_t *park = reinterpret_cast<uint32_t *>(sDP + (size_t)2 * rowsDP * BK);
-            if (a.lgc == 2)
-                cons_diag_pair(a, S, park, b, J, split, id, cs);
-            else
-                cons_diag(a, S, b, J, split, id, cs, true);
-            __syncthreads();  // every thread's dp32 and layer minima of block J are stored
-            if (ct == 0) publish_block(a, split, J);
-            if (a.lgc == 2) diag_pair_bands(a, park, J, split, id);
-            n++;
+        // this CTA's near tiles: their costs depend on nothing, so their copies overlap the barrier
+        NearItem it{0, 0, 0};
+        const bool near = near_item(a, (int)blockIdx.x, pn.nb, it);
+        const int Kn0 = it.grp * kNearTiles, nk = near ? min(kNearTiles, it.Jl - Kn0 + 1) : 0;
+        if (near && ct == 0) {
+            asm volatile("fence.proxy.async;" ::: "memory");
+            mbar_expect_tx(&S.nbar, (uint32_t)nk * 2 * kCostHalfBytes);
+            // consecutive K of one column block: one run of the table
+            bulk_g2s(big, a.costs + (cost_tile_idx(P0 + Kn0, P0 + it.Jl) - pn.tbase) * kCostTileFloats,
+                     (uint32_t)nk * 2 * kCostHalfBytes, &S.nbar, policy);
         }
+        if (P0 > 0) ok = grid_sync(a, S, ++epoch);  // the panel's far minima are complete
+        if (a.bound && ok) {  // the bounds were last read before this barrier: cleared for the next panel
+            const int nn = a.T * a.G * (a.s - 2) * BJ;
+            for (int q = (int)blockIdx.x * MAXCONS + ct; q < nn; q += (int)gridDim.x * MAXCONS) a.ub[q] = kNoBound;
+        }
+        if (near) {
+            mbar_wait_bounded(&S.nbar, pp.nnear & 1u, a.st, a.abort_flag);
+            pp.nnear++;
+            pp.fetched += (uint32_t)nk;
+            if (ct == 0)  // the tasks of the tiles below the diagonal
+                pp.run += (uint32_t)(min(nk, it.Jl - Kn0) * min(kNearMults, a.G - it.g0) * (a.s - 2));
+            if (ok) near_phase(a, S, big, big + kNearTiles * kCostTileFloats, P0, it, pn.tag);
+        }
+        if (!ok) break;
+        ok = grid_sync(a, S, ++epoch, !(a.hold0 && blockIdx.x == 0));  // the panel's rows are final
+        if (ok) fold_panel(a, S, pn);
     }
-    if (lane == 0 && (n_run | n_skip)) {
-        atomicAdd((unsigned long long *)&a.st->tiles_run, n_run);
-        atomicAdd((unsigned long long *)&a.st->tiles_skipped, n_skip);
-    }
-    if (ct == 0 && n) atomicAdd((unsigned long long *)&a.st->tiles_fetched, (unsigned long long)n);  // one cost tile per buffer fill
+    if (ct == 0) atomicAdd(a.work, (unsigned long long)pp.run);
+    if (ct == 0 && pp.fetched) atomicAdd((unsigned long long *)&a.st->tiles_fetched, (unsigned long long)pp.fetched);  // one cost tile per buffer fill
 }
 
 // ------------------------------------------------------------ base layer
@@ -1745,7 +1709,7 @@ __device__ void visit_tile(const FastArgs &a, int g, int i, int64_t j, int64_t K
     }
 }
 
-// Tiles listed by a band word (band_update), in increasing order.
+// Tiles listed by a band word (band_pack), in increasing order.
 template <typename F>
 __device__ void visit_band(const FastArgs &a, int g, int i, int64_t j, uint64_t w, float thr, F &&f) {
     const uint32_t w1 = (uint32_t)w, w2 = (uint32_t)(w >> 32);
@@ -1831,7 +1795,13 @@ __device__ __forceinline__ void warp_visit_band(const FastArgs &a, int g, int i,
 }
 
 // Outputs eq. apx_final reads: dp(i, p-1) for i in [ilo, s] (or every output).
+// The first thread also turns the pass's task count into (multiplier, tile) units of s - 2 tasks.
 __global__ void k_need_init(FastArgs a, int ilo, int all) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const int64_t units = (int64_t)a.G * a.nJ * (a.nJ - 1) / 2, run = (int64_t)*a.work / (a.s - 2);
+        a.st->tiles_run += run;
+        a.st->tiles_skipped += max((int64_t)0, units - run);
+    }
     int64_t tot = (int64_t)a.G * (a.s + 1) * a.ps;
     int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -2188,23 +2158,30 @@ __global__ void k_weights_f32(const int64_t *w, float *wf, int64_t p) {
     if (i < p) wf[i] = (float)w[i];
 }
 
+// One word a thread (a single thread's copy took 9.7 us).
 __global__ void k_store_params(FastParams prm, FastParams *dst) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *dst = prm;
+    static_assert(sizeof(FastParams) % 4 == 0, "copied by words");
+    for (int i = threadIdx.x; i < (int)(sizeof(FastParams) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t *>(dst)[i] = reinterpret_cast<const uint32_t *>(&prm)[i];
 }
 
 static int mdp_stride(int s) { return (s + 1 + 3) & ~3; }
 
-// The band region: band words, member lists, need marks, flags, constants, corner
-// states, block minima, the exact stage's lists; then the seed rows (cons_seed).
+// The band region: band words, need marks, flags (barrier, abort), constants, corner
+// states, block minima, list counts; member counts and lists (scratch of the wavefront before the
+// need stage writes them: scratch_bytes); then the seed rows (far_start).
+static size_t flags_bytes(int64_t d) { return align256(8 * (size_t)kMaxG * (size_t)cdiv(d, BJ) + 64); }
+static size_t scratch_bytes(int64_t d, int32_t s) {
+    const size_t rows = (size_t)kMaxG * (size_t)(s + 1) * (size_t)table_stride(d);
+    return align256(4 * rows) + align256(4 * NMEM * rows) + align256(2 * 4 * rows) +
+           align256(4 * (size_t)kMaxG * (size_t)table_stride(d));
+}
 static size_t band_core_bytes(int64_t d, int32_t s) {
     size_t rows = (size_t)kMaxG * (size_t)(s + 1) * (size_t)table_stride(d);
     size_t nJ = (size_t)cdiv(d, BJ);
-    return align256(8 * rows) + align256(4 * rows) + align256(4 * NMEM * rows) + align256(rows) +
-           align256(8 * (size_t)kMaxG * nJ + 64) + align256(sizeof(FastParams)) + align256(32 * nJ * (nJ + 1) / 2) +
-           align256(4 * (size_t)kMaxG * (size_t)mdp_stride(s) * nJ) +
-           align256(2 * 4 * (size_t)kMaxG * (size_t)(s + 1) * (size_t)table_stride(d)) +
-           align256(4 * 2 * (size_t)(s + 1)) + align256(4 * (size_t)kMaxG * (size_t)table_stride(d)) +
-           align256(4 * (size_t)(s + 1));
+    return align256(8 * rows) + align256(rows) + flags_bytes(d) + align256(sizeof(FastParams)) +
+           align256(32 * nJ * (nJ + 1) / 2) + align256(4 * (size_t)kMaxG * (size_t)mdp_stride(s) * nJ) +
+           align256(4 * 2 * (size_t)(s + 1)) + align256(4 * (size_t)(s + 1)) + scratch_bytes(d, s);
 }
 static size_t seed_rows_bytes(int64_t d, int32_t s) { return align256(4 * (size_t)cdiv(d, BJ) * BJ * (size_t)(s + 1)); }
 size_t fast_dp_band_bytes(int64_t d, int32_t s) { return band_core_bytes(d, s) + seed_rows_bytes(d, s); }
@@ -2213,7 +2190,7 @@ static float *seed_rows(void *ws, const Layout &Lw) {
 }
 
 // Keep the fp32 dp rows of multiplier g of the last pass (G multipliers over p values) as
-// the seed rows of a later pass at multipliers <= this one's (cons_seed).
+// the seed rows of a later pass at multipliers <= this one's (far_start).
 int save_dp_seed(void *ws, const Layout &Lw, int64_t p, int G, int s, int g, cudaStream_t st) {
     if (g < 0 || g >= G || s != Lw.s) return ECASQ_EINVAL;
     const size_t row = (size_t)(s + 1) * BJ * sizeof(float);
@@ -2222,8 +2199,6 @@ int save_dp_seed(void *ws, const Layout &Lw, int64_t p, int G, int s, int g, cud
                                      cudaMemcpyDeviceToDevice, st));
     return ECASQ_OK;
 }
-
-static size_t smem_bytes(int Gc, int s) { return sizeof(Smem) + (size_t)2 * Gc * (s - 2) * BK * sizeof(float); }
 
 // Certified band factors (see the file header): eps_2 = 1.0001u, eps_i = max(eps_{i-1}, 24u) + 1.0001u.
 static void band_factors(int s, FastParams &fp) {
@@ -2261,14 +2236,56 @@ size_t streamed_costs_bytes(int64_t d) {
     return band * tile_bytes_with_summary();
 }
 
+// Scratch of the wavefront (member counts and lists, unused until the need stage): the blocks'
+// last columns, the near minima, the bounds, the far lists, the far segments and, without a cost
+// table, one panel's cost tiles.  Panels of T column blocks, as many as the GPU's SMs take near items
+// of and as leave the scratch enough segments to spread a panel's far tiles over the SMs.
+// Tiles of T column blocks, at most: those of the last ones.
+static size_t panel_tiles(int T, int nJ) { return (size_t)T * nJ - (size_t)T * (T - 1) / 2; }
+struct PanelPlan { int T, workers; size_t dlast, tmin, tmin1, ub, lists, part, costs; };
+static bool plan_panels(size_t scratch, int nsm, int nJ, int G, int Gc, int nsplit, int s, bool build, PanelPlan *pl) {
+    const size_t out = (size_t)G * (s - 2) * BJ;  // outputs of a column block
+    const size_t seg = (size_t)Gc * (s - 2) * BJ * 12;
+    const int pairs = (int)cdiv(G, kNearMults);
+    int T = 1;
+    while (T < kPanelMax && near_groups(T + 1) * pairs <= nsm) T++;
+    if (near_groups(T) * pairs > nsm) return false;
+    for (T = std::min(T, nJ); T >= 1; T--) {
+        size_t off = 0;
+        auto take = [&](size_t bytes) { const size_t o = off; off += align256(bytes); return o; };
+        pl->T = T;
+        pl->workers = 0;
+        pl->dlast = take(4 * (size_t)G * mdp_stride(s) * nJ);
+        pl->tmin = take(4 * out * (size_t)near_groups(T));
+        pl->tmin1 = take(4 * out * (size_t)(T * (T + 1) / 2));
+        pl->ub = pl->lists = off;
+        if (nJ > T) {
+            pl->ub = take(4 * out * (size_t)T);
+            pl->lists = take((size_t)T * nsplit * (size_t)cdiv(nJ, NT) * (16 * NT + 8));
+        }
+        pl->costs = off;
+        if (build) take(panel_tiles(T, nJ) * (kCostTileFloats * sizeof(float) + BJ * sizeof(float2)));
+        pl->part = off;
+        if (off > scratch) continue;
+        if (nJ <= T) return true;  // one panel: no far phase
+        const int64_t slots = (int64_t)((scratch - off) / seg) - (int64_t)T * nsplit;
+        pl->workers = (int)std::min<int64_t>(slots, nsm);
+        if (pl->workers >= std::min(nsm, 2 * nJ) || (T == 1 && pl->workers >= 1)) return true;
+    }
+    return false;
+}
+
 int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, const Layout &Lw, cudaStream_t st,
                    bool exact_s, bool exact_tables, float *costs, bool build_costs, bool test_stall,
-                   size_t chunk_bytes, bool split_off, bool seeded) {
+                   size_t chunk_bytes, bool seeded, bool unbounded) {
     double *dp64 = wsp<double>(ws, Lw.dp64);
     int32_t *bp = wsp<int32_t>(ws, Lw.bp);
     // small inputs, very large ones and huge counts take the reference kernel
-    if (P.p < 2 * BJ || P.p > kMaxFastP || P.d >= (1 << 24) || s < 3 || cdiv(s - 2, LPT) * NJQ > MAXCONS)
+    if (P.p < 2 * BJ || P.p > kMaxFastP || P.d >= (1 << 24) || s < 3 || s - 2 > 112)
         return launch_dp_reference(P, lamp, G, s, dp64, bp, st);
+    int dev = 0, nsm = 0;
+    ECASQ_CUDA_TRY(cudaGetDevice(&dev));
+    ECASQ_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     FastArgs a{};
     a.v = P.v;
     a.N = P.N;
@@ -2280,30 +2297,11 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     a.invd = 1.0f / (float)P.d;  // IEEE division on the host: correctly rounded
     a.G = G;
     a.s = s;
-    // Layers per consumer thread: LPT, or 8 on the generic path (the fused kernel, or the
-    // resident one without the paired diagonal) when that costs fewer layer slots times
-    // multiplier splits; at s = 32, 4 groups of 8 layers (64 threads per multiplier, 4
-    // multipliers per split) against 5 of 7 (80 threads, 3 per split): 2 splits of 8
-    // slots per pass instead of 3 of 7.  With resident or streamed costs, also when 8
-    // layers give an even number of layer groups and LPT an odd one or more than two:
-    // only then can the generic path skip tiles (s = 17, 18; s = 27..30 with several
-    // multipliers, where the slots favour LPT).  A single multiplier at s = 27..34 keeps
-    // LPT: with one warp pair per block the skipping did not pay for the eighth layer.
-    int lp = LPT;
-    if (!(costs && cdiv(s - 2, LPT) == 2 && mdp_stride(s) <= 20)) {
-        auto slots = [&](int l) {
-            const int lgc = (int)cdiv(s - 2, l), gc = std::max(1, std::min(G, MAXCONS / (lgc * NJQ)));
-            return (int64_t)cdiv(G, gc) * l;
-        };
-        const int lg8 = (int)cdiv(s - 2, 8);
-        const bool skip8 = costs && lg8 % 2 == 0 && mdp_stride(s) <= kMdpMax && (lg8 == 2 || G > 1);
-        if (cdiv(s - 2, 8) * NJQ <= MAXCONS && (skip8 || slots(8) < slots(LPT))) lp = 8;
-    }
-    a.lgc = (int)cdiv(s - 2, lp);
-    a.Gc = std::max(1, std::min(G, MAXCONS / (a.lgc * NJQ)));
+    // far tasks: all multipliers in one split while their layers' band state fits shared memory
+    a.Gc = std::min(G, std::max(1, 32 * kTaskWords / (s - 2)));
     a.nsplit = (int)cdiv(G, a.Gc);
+    a.Gc = (int)cdiv(G, a.nsplit);
     a.nJ = (int)cdiv(P.p, BJ);
-    a.ncons = (int)cdiv((int64_t)a.Gc * a.lgc * NJQ, 32) * 32;
     FastParams fp;
     band_factors(s, fp);
     for (int g = 0; g < kMaxG; g++) {
@@ -2312,94 +2310,97 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     }
     size_t rows = (size_t)kMaxG * (size_t)(s + 1) * (size_t)table_stride(Lw.d);
     char *base = wsp<char>(ws, Lw.band);
+    auto take = [&](size_t bytes) { char *q = base; base += align256(bytes); return q; };
     a.dp32 = wsp<float>(ws, Lw.dp32);
-    a.band = reinterpret_cast<uint64_t *>(base);
-    base += align256(8 * rows);
-    a.mcnt = reinterpret_cast<int32_t *>(base);
-    base += align256(4 * rows);
-    a.members = reinterpret_cast<int32_t *>(base);
-    base += align256(4 * NMEM * rows);
-    a.need = reinterpret_cast<uint8_t *>(base);
-    base += align256(rows);
-    int *flags = reinterpret_cast<int *>(base);  // done [kMaxG][nJ], half [kMaxG][nJ], ticket, abort
-    base += align256(8 * (size_t)kMaxG * (size_t)cdiv(Lw.d, BJ) + 64);
-    FastParams *dprm = reinterpret_cast<FastParams *>(base);
-    base += align256(sizeof(FastParams));
-    a.corner = reinterpret_cast<float *>(base);
+    a.band = reinterpret_cast<uint64_t *>(take(8 * rows));
+    a.need = reinterpret_cast<uint8_t *>(take(rows));
+    int *flags = reinterpret_cast<int *>(take(flags_bytes(Lw.d)));  // abort, barrier, task count (64 bits)
+    FastParams *dprm = reinterpret_cast<FastParams *>(take(sizeof(FastParams)));
     {
         size_t nJd = (size_t)cdiv(Lw.d, BJ);
-        char *q = base + align256(32 * nJd * (nJd + 1) / 2);
-        a.mdp = reinterpret_cast<float *>(q);
-        q += align256(4 * (size_t)kMaxG * (size_t)mdp_stride(s) * nJd);
-        a.lists = reinterpret_cast<int32_t *>(q);
-        q += align256(2 * 4 * (size_t)kMaxG * (size_t)(s + 1) * (size_t)table_stride(Lw.d));
-        a.list_cnt = reinterpret_cast<int *>(q);
-        q += align256(4 * 2 * (size_t)(s + 1));
-        a.wide = reinterpret_cast<int32_t *>(q);
-        q += align256(4 * (size_t)kMaxG * (size_t)table_stride(Lw.d));
-        a.wide_cnt = reinterpret_cast<int *>(q);
+        a.corner = reinterpret_cast<float *>(take(32 * nJd * (nJd + 1) / 2));
+        a.mdp = reinterpret_cast<float *>(take(4 * (size_t)kMaxG * (size_t)mdp_stride(s) * nJd));
     }
+    a.list_cnt = reinterpret_cast<int *>(take(4 * 2 * (size_t)(s + 1)));
+    a.wide_cnt = reinterpret_cast<int *>(take(4 * (size_t)(s + 1)));
+    char *scratch = base;
+    a.mcnt = reinterpret_cast<int32_t *>(take(4 * rows));
+    a.members = reinterpret_cast<int32_t *>(take(4 * NMEM * rows));
+    a.lists = reinterpret_cast<int32_t *>(take(2 * 4 * rows));
+    a.wide = reinterpret_cast<int32_t *>(take(4 * (size_t)kMaxG * (size_t)table_stride(Lw.d)));
     a.mdp_stride = mdp_stride(s);
     a.spin_limit = test_stall ? kTestSpinLimit : kSpinLimit;
-    // two-part publishing of each block (the chain's last tile in two layer groups)
-    a.split_pub = (costs && lp == LPT && a.lgc == 2 && !split_off) ? 1 : 0;
     a.hold0 = test_stall ? 1 : 0;
-    // Tile skipping needs every warp to hold whole multipliers (its batch test is a warp
-    // vote), so an even number of layer groups (16-thread groups, 32-lane warps), and a
-    // diagonal that writes the blocks' minima: the paired one (LPT layers per thread, two
-    // groups) or the generic one with 8 layers per thread.
-    a.prune = (costs && (lp == LPT ? a.lgc == 2 : a.lgc % 2 == 0) && a.mdp_stride <= kMdpMax &&
-               a.Gc * a.mdp_stride <= kMaxG * 20) ? 1 : 0;
-    const bool parked = costs && lp == LPT && a.lgc == 2;  // the paired diagonal and its parked state
-    a.stage_tiles = lp == LPT ? 32 : 16;  // k_wavefront_res<LP>'s batch size
-    a.seed = (seeded && a.prune && s == Lw.s) ? seed_rows(ws, Lw) : nullptr;
-    a.costs = costs;
+    PanelPlan pl;
+    if (!plan_panels(scratch_bytes(Lw.d, s), nsm, a.nJ, G, a.Gc, a.nsplit, s, !costs, &pl)) return ECASQ_EWORKSPACE;
+    a.T = pl.T;
+    a.workers = pl.workers;
+    a.dlast = reinterpret_cast<float *>(scratch + pl.dlast);
+    a.tmin = reinterpret_cast<int *>(scratch + pl.tmin);
+    a.tmin1 = reinterpret_cast<float *>(scratch + pl.tmin1);
+    a.ub = reinterpret_cast<int *>(scratch + pl.ub);
+    a.fbits = reinterpret_cast<uint4 *>(scratch + pl.lists);
+    a.funion = reinterpret_cast<uint32_t *>(a.fbits + (size_t)a.T * a.nsplit * (size_t)cdiv(a.nJ, NT) * NT);
+    a.fweight = reinterpret_cast<int *>(a.funion + (size_t)a.T * a.nsplit * (size_t)cdiv(a.nJ, NT));
+    a.part = reinterpret_cast<float *>(scratch + pl.part);
+    a.build = costs ? 0 : 1;
+    a.seed = (seeded && s == Lw.s) ? seed_rows(ws, Lw) : nullptr;
+    a.costs = costs ? costs : reinterpret_cast<float *>(scratch + pl.costs);
     a.tile_base = 0;
     a.J0 = 0;
     a.J1 = a.nJ;
-    // tiles the costs buffer holds at once: the whole triangle, or (streamed) one band
-    const size_t cap_tiles = chunk_bytes ? chunk_bytes / tile_bytes_with_summary()
-                                         : (size_t)cdiv(Lw.d, BJ) * (size_t)(cdiv(Lw.d, BJ) + 1) / 2;
-    if (costs) a.tsum = reinterpret_cast<float2 *>(costs + cap_tiles * kCostTileFloats);
+    // tiles the costs buffer holds at once: the whole triangle, one band (streamed) or one panel
+    const size_t cap_tiles = !costs ? panel_tiles(a.T, a.nJ)
+                             : chunk_bytes ? chunk_bytes / tile_bytes_with_summary()
+                                           : (size_t)cdiv(Lw.d, BJ) * (size_t)(cdiv(Lw.d, BJ) + 1) / 2;
+    a.tsum = reinterpret_cast<float2 *>(const_cast<float *>(a.costs) + cap_tiles * kCostTileFloats);
     if (chunk_bytes && cap_tiles < (size_t)a.nJ) return ECASQ_EWORKSPACE;  // one column of tiles must fit
     a.prm = dprm;
-    a.done = flags;
-    a.half = flags + (size_t)kMaxG * a.nJ;
-    a.ticket = a.half + (size_t)kMaxG * a.nJ;
-    a.abort_flag = a.ticket + 1;
+    a.abort_flag = flags;
+    a.gbar = flags + 1;
+    a.work = reinterpret_cast<unsigned long long *>(flags + 2);
     a.st = wsp<DevStatus>(ws, Lw.status);
     float *wf = wsp<float>(ws, Lw.keys1);  // the sort's ping-pong buffer is free now
     a.wf = wf;
     size_t n = (size_t)G * (size_t)(s + 1) * (size_t)P.ps;
     note_launch();
-    k_store_params<<<1, 32, 0, st>>>(fp, dprm);
+    k_store_params<<<1, 256, 0, st>>>(fp, dprm);
     note_launch();
     k_fast_clear<<<4096, 256, 0, st>>>(dp64, bp, a.dp32, n);
     note_launch();
     k_weights_f32<<<(unsigned)cdiv(P.p, 256), 256, 0, st>>>(P.w, wf, P.p);
     ECASQ_LAUNCH_CHECK();
-    ECASQ_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int) * (2 * (size_t)kMaxG * a.nJ + 2), st));
+    ECASQ_CUDA_TRY(cudaMemsetAsync(flags, 0, 4 * sizeof(int), st));
     note_launch();
     k_fast_base<<<(unsigned)cdiv(P.p - 1, 128), 128, 0, st>>>(P, a, dp64, bp);
     ECASQ_LAUNCH_CHECK();
-    int dev = 0, nsm = 0;
-    ECASQ_CUDA_TRY(cudaGetDevice(&dev));
-    ECASQ_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    // corner states: needed by every tile the producer computes (per pass, or once into the table)
+    // corner states: needed by every tile that is built (per pass, or once into the table)
     if (a.nJ > 1 && (!costs || build_costs)) {
         note_launch();
         k_corners<<<(unsigned)std::min<int64_t>(cdiv((int64_t)a.nJ * (a.nJ - 1) / 2, 128), 152 * 64), 128, 0, st>>>(a);
         ECASQ_LAUNCH_CHECK();
     }
-    size_t smem = smem_bytes(a.Gc, s);
-    const size_t stage_bytes = a.prune ? 2 * stage_floats(G, a.mdp_stride, a.stage_tiles) * sizeof(float) : 0;
-    if (parked)  // parked band state; off the diagonal, the two stage buffers
-        smem += std::max((size_t)3 * LPT * JPT * a.ncons * sizeof(uint32_t), stage_bytes);
-    else
-        smem += stage_bytes;
-    auto wave = costs ? (lp == 8 ? k_wavefront_res<8> : k_wavefront_res<LPT>)
-                      : (lp == 8 ? k_wavefront<8> : k_wavefront<LPT>);
-    ECASQ_CUDA_TRY(cudaFuncSetAttribute(wave, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int smem_max = 0;
+    ECASQ_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // far tile buffers with room for tcap tasks each, next to the band state and the
+    // partial minima
+    const size_t nt = (size_t)a.Gc * (s - 2), state = 4 * (2 * nt * BJ + 2 * kBatch * 8 * BJ);
+    const size_t fixed = kSmemHead + state + 4 * (size_t)kFarBufs * kCostTileFloats, per = 4 * (size_t)kFarBufs * BK;
+    if (fixed + 16 * per > (size_t)smem_max) return ECASQ_ECUDA;
+    a.tcap = (int)std::min<size_t>(64, std::max<size_t>(16, std::min(nt, ((size_t)smem_max - fixed) / per)));
+    size_t area = std::max(fixed - kSmemHead + a.tcap * per,
+                           sizeof(float) * (kNearTiles * kCostTileFloats + (MAXCONS / 32) * 2 * BK +
+                                            kNearMults * 2 * kNearTiles * BJ));
+    if (a.build) area = std::max(area, kBuildGroups * sizeof(BuildSmem));
+    // far tasks are skipped by the lower bound wherever the staged minima fit shared memory
+    const size_t stage = (2 * stage_floats(G, a.mdp_stride) + nt * BJ) * sizeof(float);
+    a.prune = kSmemHead + stage <= (size_t)smem_max ? 1 : 0;
+    if (a.prune) area = std::max(area, stage);
+    else a.seed = nullptr;
+    a.bound = (a.prune && a.nJ > a.T) ? 1 : 0;
+    a.bound_step = unbounded ? 32 : 4;
+    const size_t smem = kSmemHead + area;
+    ECASQ_CUDA_TRY(cudaFuncSetAttribute(k_wavefront, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     if (costs && build_costs)
         ECASQ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_costs, NPROD, 0));
@@ -2422,23 +2423,28 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
         if (costs && build_costs) {
             const int64_t ntiles = (int64_t)J1 * (J1 + 1) / 2 - (int64_t)a.tile_base;
             note_launch();
-            k_build_costs<<<(unsigned)std::min<int64_t>(ntiles, (int64_t)nsm * std::max(per_sm, 1)), NPROD, 0, st>>>(
-                a, costs);
+            k_build_costs<<<(unsigned)std::min<int64_t>(ntiles, (int64_t)nsm * std::max(per_sm, 1)), NPROD, 0, st>>>(a);
             ECASQ_LAUNCH_CHECK();
         }
-        if (J0 > 0) ECASQ_CUDA_TRY(cudaMemsetAsync(a.ticket, 0, sizeof(int), st));
-        int grid = std::min(nsm, (J1 - J0) * a.nsplit);
+        if (J0 > 0) ECASQ_CUDA_TRY(cudaMemsetAsync(a.gbar, 0, sizeof(int), st));
+        // no near minimum carries the first panel's tag (sign 0) yet
+        ECASQ_CUDA_TRY(cudaMemsetAsync(a.tmin, 0xFF, 4 * (size_t)near_groups(a.T) * G * (s - 2) * BJ, st));
+        if (a.bound) ECASQ_CUDA_TRY(cudaMemsetAsync(a.ub, kNoBound & 0xFF, 4 * (size_t)a.T * G * (s - 2) * BJ, st));
+        // one panel: as many CTAs as have near items, or tiles to build
+        const int items = near_groups(a.nJ) * (int)cdiv(G, kNearMults);
+        const int grid = a.nJ > a.T ? nsm : std::max(items, a.build ? std::min(nsm, a.nJ * (a.nJ + 1) / 2) : 0);
         if (!chunk_bytes) timer_begin(st);
         note_launch();
-        wave<<<grid, (costs ? 0 : NPROD) + a.ncons, smem, st>>>(a);
+        void *args[] = {&a};
+        ECASQ_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)k_wavefront, dim3(grid), dim3(MAXCONS), args, smem, st));
         if (!chunk_bytes) timer_end(st);
         ECASQ_LAUNCH_CHECK();
         J0 = J1;
     }
     if (chunk_bytes) timer_end(st);
-    // a streamed band holds only the last band's tiles: the need and exact stages re-derive
+    // a streamed band or a panel holds only its own tiles: the need and exact stages re-derive
     // the costs they read (any evaluation within the certified bound will do)
-    if (chunk_bytes) {
+    if (chunk_bytes || !costs) {
         a.costs = nullptr;
         a.tile_base = 0;
     }

@@ -1,0 +1,42 @@
+"""The min-plus kernel at the edges of its panels, tiles and task words (run on a
+GB300: pytest -m gpu).  With every output resolved exactly, its tables equal those
+of the reference kernel, which the other tests hold to the oracle."""
+import numpy as np
+import pytest
+
+from paper_2608_18147_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def E():
+    import torch
+    assert torch.cuda.is_available(), "these tests need a CUDA GPU"
+    import paper_2608_18147_gb300 as E
+    E.lib()
+    return E
+
+
+# 15 column blocks of 64 make a panel with 7 or 8 multipliers, 16 with fewer: one block, a panel less one
+# value, exactly, plus one, two panels and a remainder; s = 3 (one layer), s = 18 and 19 (128 tasks of 8
+# multipliers and one more layer: two splits), s = 50 (four splits), s = 82 (no skip test).
+@pytest.mark.parametrize("mode", ["DEFAULT", "RESIDENT_COSTS", "STREAMED_COSTS"])
+@pytest.mark.parametrize("d,s,G", [(128, 3, 1), (959, 16, 8), (960, 16, 8), (961, 16, 7), (1024, 9, 5), (1025, 18, 6),
+                                   (2000, 3, 8), (2113, 18, 8), (2113, 19, 8), (1984, 50, 8), (1100, 82, 8),
+                                   (4097, 32, 3)])
+def test_panel_edges_match_reference_kernel(E, mode, d, s, G):
+    x = workloads.student_t(d, d + s, scale=1.0)
+    lams = [0.0, 1e-4, 1e-3, 0.01, 0.05, 0.2, 1.0, 10.0][-G:]
+    flags = getattr(E, mode, 0) | E.EXACT_TABLES
+    wsr, ws = E.workspace(d, s), E.workspace(d, s, flags=flags)
+    Qr, mr, metr = E.ecasq_dp_pass(x, s, lams, flags=E.DP_REFERENCE, ws=wsr)
+    Q, m, met = E.ecasq_dp_pass(x, s, lams, flags=flags, ws=ws)
+    st = E.native.ws_status(ws)
+    assert st["timeout"] == 0 and st["bound_viol"] == 0
+    assert m == mr
+    np.testing.assert_array_equal(Q.cpu().numpy(), Qr.cpu().numpy())
+    np.testing.assert_array_equal(met, metr)
+    for g in range(G):
+        for a, b in zip(E.ecasq_dp_tables(ws, g, s, d), E.ecasq_dp_tables(wsr, g, s, d)):
+            np.testing.assert_array_equal(a.cpu().numpy(), b.cpu().numpy())
