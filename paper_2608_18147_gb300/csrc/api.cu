@@ -41,11 +41,11 @@ int launch_refine_colour(const Prefix &P, const int32_t *a, int m, int colour, d
 size_t refine_scratch_bytes(int64_t d);
 int launch_refine_commit(int32_t *a, const int32_t *a_new, const int32_t *moved, const double *ev, int m, bool guard,
                          double budget, int32_t *ctx, cudaStream_t st);
-int launch_quantize(const float *x, int64_t d, const float *Q, int m, uint64_t seed, uint8_t *idx, uint32_t *counts,
-                    DevStatus *st, int num_sms, cudaStream_t stream);
+int launch_quantize(const float *x, int64_t d, const float *Q, int m, uint64_t seed, uint8_t *idx, const QuantOut &o,
+                    int num_sms, cudaStream_t stream);
 int launch_quantize_timeshare(const float *x, int64_t d, const float *Qm, int mm, const float *Qp, int mp,
                               double beta, uint64_t seed, uint64_t seed_ts, uint8_t *idx, uint8_t *sel,
-                              uint32_t *counts, DevStatus *st, int num_sms, cudaStream_t stream);
+                              const QuantOut &o, int num_sms, cudaStream_t stream);
 size_t fast_dp_band_bytes(int64_t d, int32_t s);
 size_t grid_pairs_bytes(int64_t n);
 int launch_dp_grid(const Prefix &P, const double *lamp, int G, int s, double *dp64, int32_t *bp, float *dp32,
@@ -1001,31 +1001,48 @@ int ecasq_evaluate(const float *x, int64_t d, const float *Q, int32_t m, void *w
     return eval_device(ws, L, P, a_dev, m, st, out);
 }
 
-int ecasq_quantize(const float *x, int64_t d, const float *Q, int32_t m, uint64_t seed, uint8_t *idx,
-                   uint32_t *counts, void *ws, size_t ws_bytes, double *h_emp, ecasq_stream_t stream) {
-    if (!x || !Q || !idx || !counts || d < 1 || d >= ((int64_t)1 << 31) || m < 1 || m > kMaxS) return ECASQ_EINVAL;
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < sizeof(DevStatus)) return ECASQ_EWORKSPACE;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    DevStatus *ds = wsp<DevStatus>(ws, 0);
-    std::vector<float> qh(m);
-    ECASQ_CUDA_TRY(cudaMemcpyAsync(qh.data(), Q, 4 * m, cudaMemcpyDeviceToHost, st));
-    ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
-    ECASQ_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * (size_t)m, st));
+// The status record of an encode, its block ticket and, where they fit the caller's workspace, its n counts,
+// so that one memset prepares them and one copy brings them back.  The codebook is checked by the kernel.
+struct QuantRecord {
+    DevStatus st;
+    uint32_t ticket;
+    uint32_t counts[2 * kMaxS];
+};
+static size_t quant_record_bytes(int n) { return offsetof(QuantRecord, counts) + 4 * (size_t)n; }
+static int quant_begin(void *scratch, size_t bytes, uint32_t *counts, int n, QuantOut *o, cudaStream_t st) {
+    QuantRecord *r = reinterpret_cast<QuantRecord *>(scratch);
+    const bool fit = bytes >= quant_record_bytes(n);
+    *o = QuantOut{fit ? r->counts : counts, counts, fit ? &r->ticket : nullptr, &r->st};
+    ECASQ_CUDA_TRY(cudaMemsetAsync(scratch, 0, fit ? quant_record_bytes(n) : sizeof(DevStatus), st));
+    if (!fit) ECASQ_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * (size_t)n, st));
+    return ECASQ_OK;
+}
+// Waits for the encode; its counts to c.
+static int quant_end(const QuantOut &o, int n, QuantRecord *h, cudaStream_t st) {
+    if (o.ticket) {
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(h, o.st, quant_record_bytes(n), cudaMemcpyDeviceToHost, st));
+    } else {
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(&h->st, o.st, sizeof(DevStatus), cudaMemcpyDeviceToHost, st));
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(h->counts, o.counts, 4 * (size_t)n, cudaMemcpyDeviceToHost, st));
+    }
     ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int r = 1; r < m; r++)
-        if (!(qh[r] > qh[r - 1])) return ECASQ_EINVAL;
-    int rc = launch_quantize(x, d, Q, m, seed, idx, counts, ds, num_sms(), st);
+    if (h->st.range_err) return h->st.range_err == kUnsortedQ ? ECASQ_EINVAL : ECASQ_ERANGE;
+    return ECASQ_OK;
+}
+static int quantize_with(void *scratch, size_t bytes, const float *x, int64_t d, const float *Q, int32_t m, uint64_t seed,
+                         uint8_t *idx, uint32_t *counts, double *h_emp, cudaStream_t st) {
+    QuantOut o;
+    int rc = quant_begin(scratch, bytes, counts, m, &o, st);
     if (rc) return rc;
-    std::vector<uint32_t> ch(m);
-    DevStatus h;
-    ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(h), cudaMemcpyDeviceToHost, st));
-    if (h_emp) ECASQ_CUDA_TRY(cudaMemcpyAsync(ch.data(), counts, 4 * (size_t)m, cudaMemcpyDeviceToHost, st));
-    ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h.range_err) return ECASQ_ERANGE;
+    rc = launch_quantize(x, d, Q, m, seed, idx, o, num_sms(), st);
+    if (rc) return rc;
+    QuantRecord h;
+    rc = quant_end(o, m, &h, st);
+    if (rc) return rc;
     if (h_emp) {
         double he = 0.0, dd_ = (double)d;
         for (int r = 0; r < m; r++) {
-            double f = (double)ch[r] / dd_;
+            double f = (double)h.counts[r] / dd_;
             if (f > 0.0) he += -f * log2(f);
         }
         *h_emp = he;
@@ -1033,8 +1050,15 @@ int ecasq_quantize(const float *x, int64_t d, const float *Q, int32_t m, uint64_
     return ECASQ_OK;
 }
 
+int ecasq_quantize(const float *x, int64_t d, const float *Q, int32_t m, uint64_t seed, uint8_t *idx,
+                   uint32_t *counts, void *ws, size_t ws_bytes, double *h_emp, ecasq_stream_t stream) {
+    if (!x || !Q || !idx || !counts || d < 1 || d >= ((int64_t)1 << 31) || m < 1 || m > kMaxS) return ECASQ_EINVAL;
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < sizeof(DevStatus)) return ECASQ_EWORKSPACE;
+    return quantize_with(ws, ws_bytes, x, d, Q, m, seed, idx, counts, h_emp, reinterpret_cast<cudaStream_t>(stream));
+}
+
 // Same checks, kernel and host arithmetic as ecasq_quantize; the status record
-// lives in the fixed scratch block and host copies in fixed-size arrays.
+// lives in the fixed scratch block.
 int ecasq_quantize_noalloc(const float *x, int64_t d, const float *Q, int32_t m, uint64_t seed, uint8_t *idx,
                            uint32_t *counts, double *h_emp, ecasq_stream_t stream) {
     if (!x || !Q || !idx || !counts || d < 1 || d >= ((int64_t)1 << 31) || m < 1 || m > kMaxS) return ECASQ_EINVAL;
@@ -1042,31 +1066,7 @@ int ecasq_quantize_noalloc(const float *x, int64_t d, const float *Q, int32_t m,
     void *scratch = nullptr;
     int rc = noalloc_scratch(st, &scratch);
     if (rc) return rc;
-    DevStatus *ds = reinterpret_cast<DevStatus *>(scratch);
-    float qh[kMaxS];
-    ECASQ_CUDA_TRY(cudaMemcpyAsync(qh, Q, 4 * (size_t)m, cudaMemcpyDeviceToHost, st));
-    ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
-    ECASQ_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * (size_t)m, st));
-    ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int r = 1; r < m; r++)
-        if (!(qh[r] > qh[r - 1])) return ECASQ_EINVAL;
-    rc = launch_quantize(x, d, Q, m, seed, idx, counts, ds, num_sms(), st);
-    if (rc) return rc;
-    uint32_t ch[kMaxS];
-    DevStatus h;
-    ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(h), cudaMemcpyDeviceToHost, st));
-    if (h_emp) ECASQ_CUDA_TRY(cudaMemcpyAsync(ch, counts, 4 * (size_t)m, cudaMemcpyDeviceToHost, st));
-    ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h.range_err) return ECASQ_ERANGE;
-    if (h_emp) {
-        double he = 0.0, dd_ = (double)d;
-        for (int r = 0; r < m; r++) {
-            double f = (double)ch[r] / dd_;
-            if (f > 0.0) he += -f * log2(f);
-        }
-        *h_emp = he;
-    }
-    return ECASQ_OK;
+    return quantize_with(scratch, kNoAllocScratchBytes, x, d, Q, m, seed, idx, counts, h_emp, st);
 }
 
 // Linear-space traceback (Sec. 5, last paragraph): the preparation layout, then four DP
@@ -1216,26 +1216,15 @@ int ecasq_quantize_timeshare(const float *x, int64_t d, const float *Qm, int32_t
         return ECASQ_EINVAL;
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < sizeof(DevStatus)) return ECASQ_EWORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    DevStatus *ds = wsp<DevStatus>(ws, 0);
-    float qh[2 * kMaxS];
-    ECASQ_CUDA_TRY(cudaMemcpyAsync(qh, Qm, 4 * (size_t)mm, cudaMemcpyDeviceToHost, st));
-    if (mp > 0) ECASQ_CUDA_TRY(cudaMemcpyAsync(qh + kMaxS, Qp, 4 * (size_t)mp, cudaMemcpyDeviceToHost, st));
-    ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
-    ECASQ_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * (size_t)(mm + mp), st));
-    ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int r = 1; r < mm; r++)
-        if (!(qh[r] > qh[r - 1])) return ECASQ_EINVAL;
-    for (int r = 1; r < mp; r++)
-        if (!(qh[kMaxS + r] > qh[kMaxS + r - 1])) return ECASQ_EINVAL;
-    int rc = launch_quantize_timeshare(x, d, Qm, mm, mp > 0 ? Qp : Qm, mp, beta, seed, seed_ts, idx, sel, counts, ds,
-                                       num_sms(), st);
+    QuantOut o;
+    int rc = quant_begin(ws, ws_bytes, counts, mm + mp, &o, st);
     if (rc) return rc;
-    uint32_t ch[2 * kMaxS];
-    DevStatus h;
-    ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(h), cudaMemcpyDeviceToHost, st));
-    if (rate) ECASQ_CUDA_TRY(cudaMemcpyAsync(ch, counts, 4 * (size_t)(mm + mp), cudaMemcpyDeviceToHost, st));
-    ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h.range_err) return ECASQ_ERANGE;
+    rc = launch_quantize_timeshare(x, d, Qm, mm, mp > 0 ? Qp : Qm, mp, beta, seed, seed_ts, idx, sel, o, num_sms(), st);
+    if (rc) return rc;
+    QuantRecord h;
+    rc = quant_end(o, mm + mp, &h, st);
+    if (rc) return rc;
+    const uint32_t *ch = h.counts;
     if (rate) {
         // each part coded with its own empirical law: -(1/d) sum_parts sum_r c_r log2(c_r / n_part)
         double bits = 0.0;

@@ -54,6 +54,14 @@ struct DevStatus {
     int64_t tiles_fetched; // fast DP, resident costs: interval-cost tiles copied in from HBM
 };
 
+// Where an encode puts its counts: o.acc is added to; with a ticket (zero at the launch) the last block copies
+// o.acc to o.counts.
+struct QuantOut {
+    uint32_t *acc, *counts, *ticket;
+    DevStatus *st;
+};
+constexpr int kUnsortedQ = 2;  // DevStatus::range_err of an encode: the codebook is not strictly ascending
+
 struct Layout {
     size_t status;         // DevStatus
     size_t keys0, keys1;   // uint32 [d]
