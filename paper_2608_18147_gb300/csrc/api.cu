@@ -25,7 +25,7 @@ int launch_rows_prepare(const float *X, int64_t rows, const RowsData &R, cudaStr
 int launch_grid_prefix(const float *P, int64_t n, const float *vX, const int64_t *NX, const double *SX,
                        const double *S2X, int64_t pX, float *v, int64_t *w, int64_t *N, double *S, double *S2,
                        DevStatus *st, cudaStream_t stream);
-int launch_rows_pass(const RowsPass &A, int nact, int pmax, cudaStream_t st);
+int launch_rows_pass(const RowsPass &A, int slots, cudaStream_t st);
 int launch_rows_gather(const RowsData &R, const int32_t *a, const int32_t *m, int64_t rows, int s, float *Q,
                        cudaStream_t st);
 int launch_traceback_eval(const Prefix &P, int G, int s, int exact_s, const double *dp64, const int32_t *bp,
@@ -193,13 +193,22 @@ static int noalloc_scratch(cudaStream_t st, void **out) {
 // results, placed after the single-row layout (which the rows that cannot take the
 // batched path still use).
 struct RowsLayout {
-    size_t v, w, N, S, S2, p, norm2, nonfinite, bp, lam, act, mcount, metrics, qidx, sel, m, pairs, total;
+    size_t v, w, N, S, S2, p, norm2, nonfinite, dp, dp64, list, need, lam, act, mcount, metrics, qidx, sel, m, pairs, total;
     int64_t pstride;
+    int slots;
 };
+// Rows searched together: all of them while their pairs' costs stay small, else as many as fit 1 GB, and at
+// least one a block slot of an SM.
+static int64_t rows_chunk(int64_t d, int64_t rows) {
+    if (d <= kRowsMaxP) return rows;
+    return std::min(rows, std::max<int64_t>(152, ((int64_t)1 << 30) / (4 * d * (d - 1))));
+}
 static size_t rows_layout(int64_t d, int32_t s, int64_t rows, RowsLayout *R) {
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
     const size_t n = (size_t)rows, dc = (size_t)d;
+    R->slots = (int)std::min<int64_t>(rows, kRowsSlots);
+    const size_t layers = (size_t)R->slots * kMaxG * (size_t)(s + 1);
     R->v = take(4 * n * dc);
     R->w = take(8 * n * dc);
     R->N = take(8 * n * (dc + 1));
@@ -208,7 +217,10 @@ static size_t rows_layout(int64_t d, int32_t s, int64_t rows, RowsLayout *R) {
     R->p = take(8 * n);
     R->norm2 = take(8 * n);
     R->nonfinite = take(4 * n);
-    R->bp = take(4 * n * kMaxG * (size_t)(s + 1) * dc);
+    R->dp = take(4 * layers * dc);
+    R->dp64 = take(8 * layers * dc);
+    R->list = take(2 * layers * dc);
+    R->need = take(4 * layers * ((dc + 31) / 32));
     R->lam = take(8 * n * kMaxG);
     R->act = take(4 * n);
     R->mcount = take(4 * n * kMaxG);
@@ -216,9 +228,7 @@ static size_t rows_layout(int64_t d, int32_t s, int64_t rows, RowsLayout *R) {
     R->qidx = take(4 * n * kMaxG * (size_t)s);
     R->sel = take(4 * n * (size_t)s);
     R->m = take(4 * n);
-    const int64_t pm = std::min<int64_t>(d, kRowsMaxP);
-    // binary64 {C, Phi} by pair, Phi^first, fp32 {C, Phi} by pair; even, so rows start on 16 bytes
-    R->pstride = (3 * (pm * (pm - 1) / 2) + pm + 1) & ~(int64_t)1;
+    R->pstride = (d * (d - 1) / 2 + 2 * d + 1) & ~(int64_t)1;  // fp32 {C, Phi} by pair, C[0, .], Phi^first[0, .]; 16-byte rows
     R->pairs = take(8 * n * (size_t)R->pstride);
     R->total = off;
     return off;
@@ -226,7 +236,7 @@ static size_t rows_layout(int64_t d, int32_t s, int64_t rows, RowsLayout *R) {
 static size_t rows_region_bytes(int64_t d, int32_t s, int64_t rows) {
     if (d > kScanTile) return 0;
     RowsLayout R;
-    return rows_layout(d, s, rows, &R);
+    return rows_layout(d, s, rows_chunk(d, rows), &R);
 }
 
 // ECASQ_RESIDENT_COSTS: the interval-cost tiles follow the common layout;
@@ -1243,11 +1253,23 @@ int ecasq_quantize_timeshare(const float *x, int64_t d, const float *Qm, int32_t
 // Short rows (d <= kScanTile, no refinement): every row runs the multiplier search
 // of ecasq_solve in lockstep with the others -- one k_rows_pass launch per round
 // for all rows still searching -- with the per-row arithmetic of the reference DP,
-// so each row's result equals ecasq_solve on that row alone.  Rows with more than
-// kRowsMaxP unique values, longer rows and refinement take ecasq_solve row by row.
+// so each row's result equals ecasq_solve on that row alone.  Rows that fp32 cannot take (rows.cu), longer
+// rows and refinement take ecasq_solve row by row, and so do rows of more than kRowsMaxP unique
+// values with a flag that only ecasq_solve knows.
 static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws,
                               size_t ws_bytes, float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
     const int s = prm->s;
+    if (rows_chunk(d, rows) < rows) {  // long rows, many of them
+        const int64_t step = rows_chunk(d, rows);
+        int status = ECASQ_OK;
+        for (int64_t r = 0; r < rows; r += step) {
+            const int rc = solve_rows_batched(X + r * d, std::min(step, rows - r), d, prm, ws, ws_bytes, Q + r * s, m_out + r,
+                                              res ? res + r : nullptr, st);
+            if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
+            if (rc == ECASQ_EINFEASIBLE) status = rc;
+        }
+        return status;
+    }
     Layout L1;
     make_layout(d, s, 1, &L1);
     int rc = add_resident_costs(prm->flags, &L1);
@@ -1286,6 +1308,7 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
         double lo, hi;
         bool done = false, failed = false;
         int sel = -1, status = ECASQ_OK, passes = 0, nlam = 0;
+        bool slow = false;  // takes ecasq_solve
         int best = -1;  // the feasible evaluation the selection rule prefers so far
     };
     std::vector<Row> st_rows(rows);
@@ -1298,7 +1321,10 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
     for (int64_t r = 0; r < rows; r++) {
         st_rows[r].lo = lo0;
         st_rows[r].hi = hi0;
-        if (ph[r] > kRowsMaxP) { slow.push_back(r); st_rows[r].done = true; }
+        if (ph[r] > kRowsMaxP && (prm->flags & (ECASQ_DP_REFERENCE | ECASQ_TEST_STALL | ECASQ_TIME_KERNELS))) {
+            slow.push_back(r);
+            st_rows[r].slow = st_rows[r].done = true;
+        }
         else if (ph[r] == 1) st_rows[r].done = true;
         else st_rows[r].evals.reserve(fixed ? 1 : 8 + 7 * (size_t)Rn + 1);
     }
@@ -1324,17 +1350,22 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
         A.R = R;
         A.rows = actd;
         A.lam = lamd;
+        A.nact = nact;
+        A.pmax = pmax;
         A.G = G;
         A.s = s;
         A.exact_s = (prm->flags & ECASQ_EXACT_S) ? 1 : 0;
-        A.bp = reinterpret_cast<int32_t *>(rb + RL.bp);
+        A.dp = reinterpret_cast<float *>(rb + RL.dp);
+        A.dp64 = reinterpret_cast<double *>(rb + RL.dp64);
+        A.list = reinterpret_cast<uint16_t *>(rb + RL.list);
+        A.need = reinterpret_cast<uint32_t *>(rb + RL.need);
         A.qidx = qid;
         A.mcount = mcd;
         A.metrics = metd;
         A.pairs = reinterpret_cast<double *>(rb + RL.pairs);
         A.pstride = RL.pstride;
         A.pairs_ready = pairs_ready ? 1 : 0;
-        int r2 = launch_rows_pass(A, nact, pmax, st);
+        int r2 = launch_rows_pass(A, RL.slots, st);
         pairs_ready = true;  // every active row of a later round was active in this one
         if (r2) return r2;
         std::vector<int32_t> mh((size_t)nact * G), qh((size_t)nact * G * s);
@@ -1345,6 +1376,11 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
         ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
         for (int b = 0; b < nact; b++) {
             Row &w = st_rows[act[b]];
+            if (mh[(size_t)b * G] < 0) {
+                slow.push_back(act[b]);
+                w.slow = w.done = true;
+                continue;
+            }
             w.passes++;
             w.nlam += G;
             bool bad = false;
@@ -1383,7 +1419,7 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
         rc = pass(act, std::vector<double>(act.size(), prm->lambda), 1);
         if (rc) return rc;
         for (int32_t r : act)
-            if (!st_rows[r].failed) st_rows[r].sel = 0;
+            if (!st_rows[r].failed && !st_rows[r].slow) st_rows[r].sel = 0;
     } else {
         double t[7];
         {  // multiplier 0 and the first round together
@@ -1398,7 +1434,7 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
             if (rc) return rc;
             for (int32_t r : act) {
                 Row &w = st_rows[r];
-                if (w.failed) continue;
+                if (w.failed || w.slow) continue;
                 if (w.evals[0].feas) { w.sel = 0; w.done = true; }
             }
         }
@@ -1415,7 +1451,7 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
             }
             for (int32_t r : act) {
                 Row &w = st_rows[r];
-                if (w.failed) continue;
+                if (w.failed || w.slow) continue;
                 const Eval *pts = &w.evals[w.evals.size() - 7];
                 int f = -1;
                 for (int q = 0; q < 7; q++)
@@ -1445,7 +1481,7 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
         if (rc) return rc;
         for (int32_t r : need_hi) {
             Row &w = st_rows[r];
-            if (w.failed) continue;
+            if (w.failed || w.slow) continue;
             w.sel = (int)w.evals.size() - 1;
             if (!w.evals[w.sel].feas) w.status = ECASQ_EINFEASIBLE;
         }
@@ -1455,7 +1491,7 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
     int status = ECASQ_OK;
     for (int64_t r = 0; r < rows; r++) {
         Row &w = st_rows[r];
-        if (std::find(slow.begin(), slow.end(), r) != slow.end()) continue;
+        if (w.slow) continue;
         double zero3[3] = {0.0, 0.0, 0.0};
         if (ph[r] == 1) {
             mh[r] = 1;
@@ -1486,10 +1522,13 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
     if (rc) return rc;
     ECASQ_CUDA_TRY(cudaMemcpyAsync(m_out, md, 4 * (size_t)rows, cudaMemcpyDeviceToDevice, st));
     ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-    // rows with many unique values: the single-row path (its layout sits before the row data)
+    // rows left to the single-row path (its layout sits before the row data); the binary64 kernel where fp32 cannot take a
+    // row whatever the path
     for (int64_t r : slow) {
         ecasq_result_t one;
-        rc = ecasq_solve(X + r * d, d, prm, ws, roff, Q + r * s, &one, reinterpret_cast<ecasq_stream_t>(st));
+        ecasq_params_t p1 = *prm;
+        if (ph[r] <= kRowsMaxP) p1.flags |= ECASQ_DP_REFERENCE;
+        rc = ecasq_solve(X + r * d, d, &p1, ws, roff, Q + r * s, &one, reinterpret_cast<ecasq_stream_t>(st));
         if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
         if (rc == ECASQ_EINFEASIBLE) status = rc;
         ECASQ_CUDA_TRY(cudaMemcpyAsync(m_out + r, &one.m, sizeof(int32_t), cudaMemcpyHostToDevice, st));

@@ -162,22 +162,27 @@ struct RowsData {
     int64_t d, dcap;
 };
 
-// One search round of the batched path: block b runs row rows[b] at G multipliers.
-constexpr int kRowsMaxP = 128;  // unique values per row the batched path holds in shared memory
+// One search round of the batched path (rows.cu): block b runs rows[b], rows[b + gridDim], .. at G multipliers.
+constexpr int kRowsMaxP = 128;   // unique values up to which a row's pair costs fit shared memory
+constexpr int kRowsSlots = 456;  // blocks of a round, at most (three an SM)
 struct RowsPass {
     RowsData R;
-    const int32_t *rows;  // [nact] row of each block
+    const int32_t *rows;  // [nact]
     const double *lam;    // [nact][G] lambda' of the row
+    int nact, pmax;       // rows; most unique values of one
     int G, s, exact_s;
-    int32_t *bp;          // [nact][G][s+1][dcap]
+    float *dp;            // [slots][s+1][dcap][kMaxG] fp32 layers
+    double *dp64;         // [slots][kMaxG][s+1][dcap] exact values of ambiguous decisions
+    uint16_t *list;       // ... and which ones
+    uint32_t *need;       // [slots][kMaxG][s+1][ceil(dcap / 32)]
     int32_t *qidx;        // [nact][G][s]
-    int32_t *mcount;      // [nact][G]
-    double *metrics;      // [nact][G][4]
-    double *pairs;        // [rows][pstride]: the row's binary64 {C, Phi} by pair, Phi^first and fp32
-                          // {C scale, Phi} by pair, kept across rounds
-    int64_t pstride;      // doubles per row: 3 npair(pmax) + pmax
+    int32_t *mcount;      // [nact][G]; -1: a row (or multiplier) that fp32 cannot take
+    double *metrics;      // [nact][G][4]: MSE, H(I,B), H(Xhat) from 1 on
+    double *pairs;        // [rows][pstride]: the row's fp32 {C, Phi} by pair, C[0, .] and Phi^first[0, .]; kept
+                          // across rounds
+    int64_t pstride;      // doubles per row
     int pairs_ready;      // the rows' interval costs are already in `pairs`
-    int bp_smem;          // backpointers in shared memory (set by the launcher)
+    float tau[kMaxS + 1]; // band factors (set by the launcher)
 };
 
 // Prefix-sum view (App. E) used by every exact pair evaluation.

@@ -1,0 +1,525 @@
+// rows.cu -- one DP pass of the multiplier search for many independent rows of at most kScanTile
+// values (Sec. 5, eqs. apx_base / apx_rec / apx_final), a block per row, all layers in one launch.
+//
+// The pass needs a codebook and its metrics per multiplier, so only decisions have to be exact:
+//  1. k_rows_build, once per search: the fp32 interval costs C, Phi of every pair k < j (cost32.cuh:
+//     one column a thread, k descending from the empty interval; a row is short enough that the
+//     compensated sums need no anchors: n^2 u^2 <= 2^-28) and the binary64 base costs C[0, j],
+//     Phi^first[0, j].  The row is scaled by a power of two that brings its largest magnitude
+//     into [2^30, 2^31), so that neither the costs nor lambda' overflow and two values at least
+//     2^-100 apart keep the relative bounds; a row with a smaller gap, or a multiplier beyond 2^120
+//     in that scale, is left to the caller (mcount = -1).
+//  2. k_rows_pass: eq. apx_rec in fp32, layer by layer, eight multipliers at a time.
+//  3. The traceback, a warp per multiplier.  At an output the candidates within the certified band
+//     of the fp32 minimum hold the exact minimiser; where it is the only one, the decision is exact.
+//     Elsewhere, and between last layers, the members' closure is evaluated in binary64 with
+//     double-double interval costs (resolve; lowest k, smallest i among exact minima).
+// The results are those of the binary64 recurrence: every output's candidate set is that of the
+// fast DP (dp_fast.cu), and an exact minimum of one candidate needs no evaluation.
+//
+// What bounds it: the chip has 2 binary64 operations a cycle and SM, so an interval cost for every pair
+// (8128 a row of 128 values) took 43 of 70 ms of device time for 8192 rows at s = 8; fp32 costs
+// and binary64 only for ambiguous decisions and the metrics take 10 (0.5 for the costs, 1.6 a round);
+// 64 rows of 300 values at s = 8: 1.1 ms of device time instead of 64 single solves of 3.6 ms.  The second bound was the
+// scan of one output a thread with a marker bit per candidate (2 candidates a cycle and SM); here a
+// unit (32 columns, 16 or 32 k) loads a pair's costs once for eight multipliers.
+#include <algorithm>
+
+#include "common.cuh"
+#include "cost32.cuh"
+
+namespace ecasq {
+
+constexpr int kRowsThreads = 512;   // at most; 256 for rows whose costs fit shared memory
+constexpr float kRowsMinGap = 0x1p-100f;
+
+// Pair (k, j) of a row at pair_at(k, j, p): k-major, so the lanes of a warp (consecutive j, one k) touch
+// consecutive words.
+__device__ __forceinline__ int pair_at(int k, int j, int p) { return k * p - k * (k + 1) / 2 + j - k - 1; }
+// The row's scale exponent: the largest magnitude is v[0]'s or v[p-1]'s.
+__device__ __forceinline__ int row_exp(const float *v, int p) { return 30 - ilogbf(fmaxf(fabsf(v[0]), fabsf(v[p - 1]))); }
+
+__device__ __forceinline__ Prefix row_prefix(const RowsData &R, int64_t row, int p) {
+    Prefix P;
+    P.v = R.v + row * R.dcap;
+    P.w = R.w + row * R.dcap;
+    P.N = R.N + row * (R.dcap + 1);
+    P.S = R.S + row * 2 * (R.dcap + 1);
+    P.S2 = R.S2 + row * 2 * (R.dcap + 1);
+    P.p = p;
+    P.d = R.d;
+    P.ps = p;
+    return P;
+}
+
+// A row's kept costs: fp32 {C, Phi} by pair, then C[0, j] and Phi^first[0, j]; Phi^first[0, 0] (unused) is 1
+// for a row that fp32 cannot take.
+struct RowCosts { float2 *cf; double *c0, *phf; };
+__device__ __forceinline__ RowCosts row_costs(const RowsPass &A, int64_t row) {
+    double *g = A.pairs + row * A.pstride;
+    double *c0 = g + (A.pstride - 2 * A.R.dcap);
+    return {reinterpret_cast<float2 *>(g), c0, c0 + A.R.dcap};
+}
+
+__global__ void __launch_bounds__(kScanTile) k_rows_build(const RowsPass A) {
+    __shared__ float v[kScanTile], w[kScanTile];
+    const int64_t row = A.rows[blockIdx.x];
+    const int p = (int)A.R.p[row];
+    const Prefix P = row_prefix(A.R, row, p);
+    const RowCosts rc = row_costs(A, row);
+    const int e = row_exp(P.v, p);
+    for (int t = threadIdx.x; t < p; t += blockDim.x) {
+        v[t] = ldexpf(P.v[t], e);
+        w[t] = (float)P.w[t];
+    }
+    __syncthreads();
+    bool narrow = false;
+    for (int t = threadIdx.x; t + 1 < p; t += blockDim.x) narrow |= !(__fsub_rn(v[t + 1], v[t]) >= kRowsMinGap);
+    narrow = __syncthreads_or(narrow);
+    if (threadIdx.x == 0) rc.phf[0] = narrow ? 1.0 : 0.0;
+    if (narrow) return;
+    const float d_f = (float)P.d, invd = 1.0f / (float)P.d;
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x; j - lane < p; j += blockDim.x) {
+        const int jt = j - lane;  // the warp's first column
+        const float vj = v[min(j, p - 1)];
+        Rec r = rec_empty();
+        for (int k = min(jt + 30, p - 2); k >= 0; k--) {
+            if (k < j && j < p) {
+                rec_step(r, vj, v[k + 1], w[k + 1], __fsub_rn(v[k + 1], v[k]));
+                float2 c;
+                rec_emit(r, vj, v[k], d_f, invd, c.x, c.y);
+                rc.cf[pair_at(k, j, p)] = c;
+            }
+        }
+        if (j >= 1 && j < p) {
+            double C, U, D;
+            pair_exact(P, 0, j, C, U, D);
+            rc.c0[j] = C;
+            rc.phf[j] = phi_exact(P, U, D, true);
+        }
+    }
+}
+
+// What a warp knows of its multiplier while it traces and resolves.
+struct RowTrace {
+    Prefix P;
+    const float2 *cf;
+    const double *c0, *phf;
+    const float *dp;       // [s+1][p][8] fp32
+    double *dp64;          // [s+1][p]: exact values of the closure's outputs
+    uint16_t *list;        // [s+1][p]: the closure's outputs by layer
+    uint32_t *need;        // [s+1][nw]: ... as bits, all zero between closures
+    uint16_t *cnt;         // [s+1]: ... their number by layer
+    const float *tau;
+    double lam;
+    float lam32, slack;
+    int p, g, nw;
+};
+__device__ __forceinline__ float row_limit(const RowTrace &T, int i, float m) {
+    return __fadd_ru(__fmul_ru(m, __fadd_ru(1.0f, T.tau[i])), T.slack);
+}
+// Members of output (i, j) among k = kb .. kb + 127, 32 a word: candidates whose fp32 value (the forward pass's) is not
+// above the limit.  One warp; the loads of the four words are in flight together.
+__device__ __forceinline__ void row_members(const RowTrace &T, int i, int j, int kb, float lim, unsigned (&in)[4]) {
+    const int lane = threadIdx.x & 31;
+    float d[4];
+    float2 c[4];
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+        const int k = kb + 32 * w + lane;
+        d[w] = CUDART_INF_F;
+        c[w] = make_float2(0.f, 0.f);
+        if (k < j) {
+            d[w] = T.dp[((size_t)(i - 1) * T.p + k) * kMaxG + T.g];
+            c[w] = T.cf[pair_at(k, j, T.p)];
+        }
+    }
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+        const float v = __fadd_rn(d[w], __fmaf_rn(T.lam32, c[w].y, c[w].x));
+        in[w] = __ballot_sync(0xffffffffu, kb + 32 * w + lane < j && !(v > lim));
+    }
+}
+__device__ __forceinline__ double row_base(const RowTrace &T, int j) {
+    return __dadd_rn(T.c0[j], __dmul_rn(T.lam, T.phf[j]));
+}
+
+// Binary64 candidate cost C[k, j] + lambda' Phi[k, j].
+__device__ __forceinline__ double row_cost(const RowTrace &T, int k, int j) {
+    double C, U, D;
+    pair_exact(T.P, k, j, C, U, D);
+    return __dadd_rn(C, __dmul_rn(T.lam, phi_exact(T.P, U, D, false)));
+}
+
+// The exact value and lowest minimiser of output (i0, j0), i0 >= 3: its members, their members and so on
+// down to layer 3 are listed (each output once), then evaluated from layer 3 up.  One warp.  A binary64 interval
+// cost is a long chain whose time 32 lanes share, so up to kRowsPairs costs of the closure (nearly
+// always all) are evaluated side by side first; larger closures go output by output.
+constexpr int kRowsPairs = 64;
+static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0, double *value) {
+    const int lane = threadIdx.x & 31, p = T.p;
+    const unsigned full = 0xffffffffu;
+    uint16_t *cnt = T.cnt;
+    // the costs and their (i, j, k) take the layers below 3 of dp64
+    double *cost = T.dp64;
+    uint32_t *key = reinterpret_cast<uint32_t *>(T.dp64 + kRowsPairs);
+    const bool room = 3 * p >= kRowsPairs + kRowsPairs / 2;
+    int np = 0;
+    if (lane == 0) {
+        T.list[(size_t)i0 * p] = (uint16_t)j0;
+        cnt[i0] = 1;
+    }
+    __syncwarp();
+    for (int i = i0; i >= 3; i--) {
+        const int n = cnt[i];
+        int nn = 0;
+        for (int e = 0; e < n; e++) {
+            const int j = T.list[(size_t)i * p + e];
+            const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
+            for (int kb = 0; kb < j; kb += 128) {
+                unsigned in[4];
+                row_members(T, i, j, kb, lim, in);
+#pragma unroll
+                for (int w = 0; w < 4; w++) {
+                    if (!in[w]) continue;
+                    const int k = kb + 32 * w + lane, q = np + __popc(in[w] & ((1u << lane) - 1u));
+                    if (((in[w] >> lane) & 1u) && room && q < kRowsPairs) key[q] = (uint32_t)(i << 20 | j << 10 | k);
+                    np += __popc(in[w]);
+                    if (i > 3) {
+                        uint32_t *word = T.need + (size_t)(i - 1) * T.nw + (kb >> 5) + w;
+                        const unsigned fresh = in[w] & ~*word;
+                        __syncwarp();
+                        if (lane == 0) *word |= in[w];
+                        if ((fresh >> lane) & 1u)
+                            T.list[(size_t)(i - 1) * p + nn + __popc(fresh & ((1u << lane) - 1u))] = (uint16_t)k;
+                        nn += __popc(fresh);
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        if (lane == 0 && i > 3) cnt[i - 1] = (uint16_t)nn;
+        __syncwarp();
+    }
+    int arg = -1;
+    double best = CUDART_INF;
+    if (room && np <= kRowsPairs) {
+        for (int q = lane; q < np; q += 32) cost[q] = row_cost(T, (int)(key[q] & 1023u), (int)(key[q] >> 10 & 1023u));
+        __syncwarp();
+        if (lane == 0) {
+            // the pairs were listed from the last layer down, k ascending: backwards, the lowest k comes last
+            for (int q = np - 1; q >= 0; q--) {
+                const uint32_t f = key[q];
+                const int i = (int)(f >> 20), k = (int)(f & 1023u);
+                const double c = __dadd_rn(i == 3 ? row_base(T, k) : T.dp64[(size_t)(i - 1) * p + k], cost[q]);
+                if (c <= best) { best = c; arg = k; }
+                if (q > 0 && key[q - 1] >> 10 != f >> 10) {  // the output's last: store it
+                    T.dp64[(size_t)i * p + (f >> 10 & 1023u)] = best;
+                    best = CUDART_INF;
+                }
+            }
+        }
+        best = __shfl_sync(full, best, 0);
+        arg = __shfl_sync(full, arg, 0);
+        for (int i = 3; i < i0; i++)
+            for (int e = lane; e < cnt[i]; e += 32) T.need[(size_t)i * T.nw + (T.list[(size_t)i * p + e] >> 5)] = 0u;
+        __syncwarp();
+        *value = best;
+        return arg;
+    }
+    for (int i = 3; i <= i0; i++) {
+        const int n = cnt[i];
+        for (int e = 0; e < n; e++) {
+            const int j = T.list[(size_t)i * p + e];
+            const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
+            best = CUDART_INF;
+            arg = 0x7fffffff;
+            for (int kb = 0; kb < j; kb += 128) {
+                unsigned in[4];
+                row_members(T, i, j, kb, lim, in);
+#pragma unroll 1
+                for (int w = 0; w < 4; w++) {
+                    const unsigned x = w == 0 ? in[0] : w == 1 ? in[1] : w == 2 ? in[2] : in[3];
+                    const int k = kb + 32 * w + lane;
+                    if ((x >> lane) & 1u) {
+                        const double c = __dadd_rn(i == 3 ? row_base(T, k) : T.dp64[(size_t)(i - 1) * p + k], row_cost(T, k, j));
+                        if (c < best) { best = c; arg = k; }
+                    }
+                    __syncwarp();
+                }
+            }
+            for (int o = 16; o; o >>= 1) {
+                const double b2 = __shfl_xor_sync(full, best, o);
+                const int a2 = __shfl_xor_sync(full, arg, o);
+                if (b2 < best || (b2 == best && a2 < arg)) { best = b2; arg = a2; }
+            }
+            if (lane == 0) {
+                T.dp64[(size_t)i * p + j] = best;
+                if (i < i0) T.need[(size_t)i * T.nw + (j >> 5)] = 0u;
+            }
+            __syncwarp();
+        }
+    }
+    *value = best;  // the last output evaluated is (i0, j0)
+    return arg;
+}
+
+// The codebook of multiplier T.g into a[0 .. m-1] (lane 0 writes); returns m, 0 when there is none.
+static __device__ __noinline__ int row_trace(const RowTrace &T, int s, int ilo, int32_t *a) {
+    const int lane = threadIdx.x & 31, p = T.p;
+    const unsigned full = 0xffffffffu;
+    // eq. apx_final: the layers whose fp32 value is within the band of the least
+    float m = CUDART_INF_F;
+    for (int i = ilo + lane; i <= s; i += 32) m = fminf(m, T.dp[((size_t)i * p + p - 1) * kMaxG + T.g]);
+    for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(full, m, o));
+    if (!(m < CUDART_INF_F)) return 0;
+    const float lim = row_limit(T, s, m);
+    int istar = -1, members = 0;
+    for (int i = ilo; i <= s; i++)
+        if (!(T.dp[((size_t)i * p + p - 1) * kMaxG + T.g] > lim)) { if (!members++) istar = i; }
+    if (members > 1) {
+        double best = CUDART_INF;
+        for (int i = ilo; i <= s; i++) {
+            if (T.dp[((size_t)i * p + p - 1) * kMaxG + T.g] > lim) continue;
+            double v;
+            if (i == 2) v = row_base(T, p - 1);
+            else row_resolve(T, i, p - 1, &v);
+            if (v < best) { best = v; istar = i; }
+        }
+    }
+    int j = p - 1;
+    if (lane == 0) a[istar - 1] = j;
+    for (int i = istar; i >= 3; i--) {
+        const float lj = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
+        int n = 0, k = 0;
+        for (int kb = 0; kb < j; kb += 128) {
+            unsigned in[4];
+            row_members(T, i, j, kb, lj, in);
+#pragma unroll
+            for (int w = 0; w < 4; w++) {
+                if (in[w] && !n) k = kb + 32 * w + __ffs(in[w]) - 1;
+                n += __popc(in[w]);
+            }
+        }
+        if (n > 1) {
+            double v;
+            k = row_resolve(T, i, j, &v);
+        }
+        j = k;
+        if (lane == 0) a[i - 2] = j;
+    }
+    if (lane == 0) a[0] = 0;
+    __syncwarp();
+    return istar;
+}
+
+// eval_codebook_lanes for the multipliers g0 .. of one warp, `width` lanes (a power of two >= s) each: the same
+// values in the same order; a binary64 sequence costs a warp the same for one lane as for 32.
+__device__ __forceinline__ void row_evaluate(const Prefix &P, const int32_t *a, int m, int width, double *out3) {
+    const unsigned full = 0xffffffffu;
+    const int l = threadIdx.x & (width - 1);
+    double C = 0.0, F = 0.0, U = 0.0, D = 0.0;
+    if (l + 1 < m) {
+        pair_exact(P, a[l], a[l + 1], C, U, D);
+        F = l == 0 ? phi_first_at(P, a[0], U, D) : phi_exact(P, U, D, false);
+    }
+    const double Uprev = __shfl_up_sync(full, U, 1, width);
+    const double Ulast = __shfl_sync(full, U, m >= 2 ? m - 2 : 0, width);
+    double ht = 0.0;
+    if (m >= 2 && l < m) {
+        const double f = l == m - 1 ? Ulast : (l == 0 ? __dadd_rn((double)P.w[a[0]], D) : __dadd_rn(Uprev, D));
+        ht = hfun(__ddiv_rn(f, (double)P.d));
+    }
+    double mse = 0.0, hs = 0.0, hx = 0.0;
+    for (int r = 0; r < width; r++) {
+        const double c = __shfl_sync(full, C, r, width), f = __shfl_sync(full, F, r, width), h = __shfl_sync(full, ht, r, width);
+        if (r + 1 < m) { mse = __dadd_rn(mse, c); hs = __dadd_rn(hs, f); }
+        if (r < m && m >= 2) hx = __dadd_rn(hx, h);
+    }
+    if (l == 0 && m > 0) { out3[0] = mse; out3[1] = hs; out3[2] = hx; }
+}
+
+// Shared memory: two layers [p][8] as float bits, the pairs' costs (p <= kRowsMaxP), the evaluation's scratch
+// (s > 32), the codebooks and the closures' counts.
+__host__ __device__ __forceinline__ size_t rows_smem_costs(int p) { return sizeof(int) * 2 * kMaxG * (size_t)p; }
+__host__ __device__ __forceinline__ size_t rows_smem_tail(int p) {
+    const size_t pc = (size_t)(p < kRowsMaxP ? p : kRowsMaxP);
+    return rows_smem_costs(p) + sizeof(float2) * (pc * (pc - 1) / 2);
+}
+static size_t rows_pass_smem(int p, int s) {
+    return rows_smem_tail(p) + (s > 32 ? sizeof(double) * 4 * kMaxS : 0) + kMaxG * (sizeof(int32_t) * s + sizeof(uint16_t) * (s + 1));
+}
+
+// WIDE: some row has more than kRowsMaxP values; its pairs' costs stay in global memory.
+template <bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_rows_pass(const __grid_constant__ RowsPass A) {
+    extern __shared__ __align__(16) unsigned char rsm[];
+    __shared__ int m_sm[kMaxG];
+    __shared__ double lam[kMaxG];
+    __shared__ float lam32[kMaxG];
+    __shared__ int refuse;
+    const RowsData &R = A.R;
+    const int G = A.G, s = A.s, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
+    const size_t dc = (size_t)R.dcap, rows_per = (size_t)(s + 1) * dc, nwc = (dc + 31) / 32;
+    double *scratch = reinterpret_cast<double *>(rsm + rows_smem_tail(A.pmax));
+    int32_t *a_sm = reinterpret_cast<int32_t *>(scratch + (s > 32 ? 4 * kMaxS : 0));
+    uint16_t *cnt_sm = reinterpret_cast<uint16_t *>(a_sm + kMaxG * s);
+    float *dp = A.dp + blockIdx.x * rows_per * kMaxG;
+    double *dp64 = A.dp64 + blockIdx.x * rows_per * kMaxG;
+    uint16_t *list = A.list + blockIdx.x * rows_per * kMaxG;
+    uint32_t *need = A.need + blockIdx.x * (size_t)(s + 1) * nwc * kMaxG;
+    for (size_t q = tid; q < (size_t)(s + 1) * nwc * kMaxG; q += blockDim.x) need[q] = 0u;
+    for (int b = blockIdx.x; b < A.nact; b += gridDim.x) {
+        const int64_t row = A.rows[b];
+        const int p = (int)R.p[row];
+        const Prefix P = row_prefix(R, row, p);
+        const RowCosts rc = row_costs(A, row);
+        const int e2 = 2 * row_exp(P.v, p);
+        __syncthreads();  // the row before is done
+        if (tid == 0) refuse = rc.phf[0] != 0.0;
+        if (tid < kMaxG) {
+            lam[tid] = tid < G ? A.lam[(size_t)b * G + tid] : 0.0;
+            lam32[tid] = __double2float_rn(ldexp(lam[tid], e2));
+        }
+        __syncthreads();
+        if (tid < G && !(lam32[tid] < 0x1p120f)) refuse = 1;
+        __syncthreads();
+        if (refuse) {
+            if (tid < G) A.mcount[(size_t)b * G + tid] = -1;
+            continue;
+        }
+        int *prev = reinterpret_cast<int *>(rsm), *out = prev + kMaxG * p;
+        float2 *csm = reinterpret_cast<float2 *>(rsm + rows_smem_costs(A.pmax));
+        const bool in_sm = !WIDE || p <= kRowsMaxP;
+        if (in_sm)
+        {
+            const int np = p * (p - 1) / 2;
+            const float4 *src = reinterpret_cast<const float4 *>(rc.cf);
+            float4 *dst = reinterpret_cast<float4 *>(csm);
+#pragma unroll 4
+            for (int t = tid; t < np / 2; t += blockDim.x) dst[t] = src[t];
+            if (tid == 0 && (np & 1)) csm[np - 1] = rc.cf[np - 1];
+        }
+        const float2 *cf = in_sm ? csm : rc.cf;
+        // eq. apx_base: dp(2, j) = C[0, j] + lambda' Phi^first[0, j]
+        for (int q = tid; q < kMaxG * p; q += blockDim.x) {
+            const int j = q / kMaxG, g = q % kMaxG;
+            float v = CUDART_INF_F;
+            if (j >= 1) v = fmaxf(__double2float_rn(ldexp(__dadd_rn(rc.c0[j], __dmul_rn(lam[g], rc.phf[j])), e2)), 0.f) + 0.f;
+            prev[q] = __float_as_int(v);
+            out[q] = 0x7f800000;
+            dp[(size_t)2 * p * kMaxG + q] = v;
+        }
+        __syncthreads();
+        // eq. apx_rec: a warp's unit is 32 columns (a lane one) and ks of their k; the values are >= +0, so
+        // their bits order like them.  Rows of at most 128 values have 20 units of 16 k for 8 warps.
+        const int ks = in_sm ? 16 : 32, ctop = (p - 1) >> 5;
+        for (int i = 3; i <= s; i++) {
+            int c = ctop, q = wid;
+            for (;;) {
+                int cnt = 0;
+                while (c >= 0 && q >= (cnt = (min(32 * c + 31, p - 1) + ks - 1) / ks)) { q -= cnt; c--; }
+                if (c < 0) break;
+                const int j = 32 * c + lane, k0 = q * ks, k1 = min(k0 + ks, min(32 * c + 31, p - 1));
+                int acc[kMaxG];
+#pragma unroll
+                for (int g = 0; g < kMaxG; g++) acc[g] = 0x7f800000;
+                float lg[kMaxG];
+#pragma unroll
+                for (int g = 0; g < kMaxG; g++) lg[g] = lam32[g];
+                const float2 *cp = cf + pair_at(k0, j, p);
+                const int jhi = j < p ? j : 0;
+#pragma unroll 4
+                for (int k = k0; k < k1; k++) {
+                    const float2 f = k < jhi ? *cp : make_float2(CUDART_INF_F, 0.f);
+                    cp += p - k - 2;  // the next k's row starts one pair later
+                    const float4 x = *reinterpret_cast<const float4 *>(prev + k * kMaxG);
+                    const float4 y = *reinterpret_cast<const float4 *>(prev + k * kMaxG + 4);
+                    const float pv[kMaxG] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+                    for (int g = 0; g < kMaxG; g++)
+                        acc[g] = min(acc[g], __float_as_int(__fadd_rn(pv[g], __fmaf_rn(lg[g], f.y, f.x))));
+                }
+                if (j < p) {
+#pragma unroll
+                    for (int g = 0; g < kMaxG; g++) atomicMin(&out[j * kMaxG + g], acc[g]);
+                }
+                q += nwarp;
+            }
+            __syncthreads();
+            for (int t = tid; t < kMaxG * p; t += blockDim.x) {
+                dp[(size_t)i * p * kMaxG + t] = __int_as_float(out[t]);
+                prev[t] = 0x7f800000;
+            }
+            int *x = prev;
+            prev = out;
+            out = x;
+            __syncthreads();
+        }
+        for (int g = wid; g < G; g += nwarp) {
+            const size_t o = (size_t)g * rows_per;
+            // underflow: C and the gaps' products 2^-149 a term, Phi where y < 1e-37 2^-118 a layer
+            const float slack = __fmul_ru(3.0f * (float)s, __fmaf_ru(lam32[g], 0x1p-114f, 8.0f * (float)P.d * 0x1p-149f));
+            const RowTrace T{P, cf, rc.c0, rc.phf, dp, dp64 + o, list + o, need + (size_t)g * (s + 1) * nwc,
+                             cnt_sm + g * (s + 1), A.tau, lam[g],
+                             lam32[g], slack, p, g, (int)nwc};
+            const int m = row_trace(T, s, A.exact_s ? s : 2, a_sm + g * s);
+            if (lane == 0) { m_sm[g] = m; A.mcount[(size_t)b * G + g] = m; }
+            for (int r = lane; r < m; r += 32) A.qidx[((size_t)b * G + g) * s + r] = a_sm[g * s + r];
+        }
+        __syncthreads();
+        if (s <= 32) {
+            const int width = s <= 4 ? 4 : s <= 8 ? 8 : s <= 16 ? 16 : 32, per = 32 / width;
+            for (int g0 = wid * per; g0 < G; g0 += nwarp * per) {
+                const int g = min(g0 + lane / width, G - 1);  // (spare lanes repeat the last one's values)
+                row_evaluate(P, a_sm + g * s, m_sm[g], width, &A.metrics[((size_t)b * G + g) * 4 + 1]);
+            }
+        } else if (wid == 0) {  // one warp, multiplier by multiplier
+            for (int g = 0; g < G; g++) {
+                if (m_sm[g] > 0) eval_codebook_warp(P, a_sm + g * s, m_sm[g], &A.metrics[((size_t)b * G + g) * 4 + 1], scratch);
+                __syncwarp();
+            }
+        }
+    }
+}
+
+int launch_rows_pass(const RowsPass &A, int slots, cudaStream_t st) {
+    if (A.nact == 0) return ECASQ_OK;
+    if (A.pmax > kScanTile) return ECASQ_EINVAL;
+    RowsPass B = A;
+    float eps[kMaxS + 1];
+    band_factors(A.s, B.tau, eps);
+    if (!A.pairs_ready) {
+        note_launch();
+        k_rows_build<<<(unsigned)A.nact, (unsigned)std::max(128, (A.pmax + 31) & ~31), 0, st>>>(B);
+        ECASQ_LAUNCH_CHECK();
+    }
+    const size_t smem = rows_pass_smem(A.pmax, A.s);
+    const bool wide = A.pmax > kRowsMaxP;
+    const void *f = wide ? (const void *)k_rows_pass<true> : (const void *)k_rows_pass<false>;
+    ECASQ_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const unsigned blocks = (unsigned)std::min(A.nact, slots);
+    note_launch();
+    if (wide) k_rows_pass<true><<<blocks, kRowsThreads, smem, st>>>(B);
+    else k_rows_pass<false><<<blocks, 256, smem, st>>>(B);
+    ECASQ_LAUNCH_CHECK();
+    return ECASQ_OK;
+}
+
+// Q[row][r] = v_row[a[row][r]] for the selected codebooks.
+__global__ void k_rows_gather(RowsData R, const int32_t *a, const int32_t *m, int s, float *Q) {
+    const int64_t row = blockIdx.x;
+    const float *v = R.v + row * R.dcap;
+    for (int r = threadIdx.x; r < m[row]; r += blockDim.x) Q[row * s + r] = v[a[row * s + r]];
+}
+
+int launch_rows_gather(const RowsData &R, const int32_t *a, const int32_t *m, int64_t rows, int s, float *Q,
+                       cudaStream_t st) {
+    note_launch();
+    k_rows_gather<<<(unsigned)rows, 32, 0, st>>>(R, a, m, s, Q);
+    ECASQ_LAUNCH_CHECK();
+    return ECASQ_OK;
+}
+
+}  // namespace ecasq

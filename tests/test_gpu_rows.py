@@ -1,0 +1,61 @@
+"""The batched rows' pass where it can go wrong (run on a GB300: pytest -m gpu): rows around the
+size whose costs fit shared memory and around units of 32 columns, up to the longest; codebook
+sizes around a warp; ties; magnitudes and gaps at the ends of the fp32 range.  Every row equals the
+single solve with the binary64 kernel."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def E():
+    import torch
+    assert torch.cuda.is_available(), "these tests need a CUDA GPU"
+    import paper_2608_18147_gb300 as E
+    E.lib()
+    return E
+
+
+def _same(E, X, s, **kw):
+    flags = kw.pop("flags", 0)
+    Q, m, res = E.ecasq_solve_batched(X, s, flags=flags, **kw)
+    Q, m = Q.cpu().numpy(), m.cpu().numpy()
+    for r in range(X.shape[0]):
+        Q1, r1 = E.ecasq_solve(X[r], s, flags=flags | E.DP_REFERENCE, **kw)
+        assert m[r] == r1["m"], r
+        np.testing.assert_array_equal(Q[r, :m[r]], Q1.cpu().numpy(), err_msg=f"row {r}")
+        for key in ("status", "lambda", "mse", "h_surrogate", "h_exact", "p", "passes", "lambdas_evaluated"):
+            assert res[r][key] == r1[key], (r, key)
+
+
+@pytest.mark.parametrize("d,s", [(2, 2), (31, 3), (33, 8), (127, 8), (128, 16), (129, 8), (160, 2), (161, 33), (300, 8),
+                                 (513, 5), (1023, 16), (1024, 8)])
+def test_rows_equal_the_binary64_solve(E, d, s):
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((5, d)).astype(np.float32)
+    X[1] = rng.standard_t(2, d).astype(np.float32)
+    X[2] = np.round(X[2] * 40) / 40                          # repeated values, evenly spaced: ties
+    X[3] = np.arange(d, dtype=np.float32) - d // 3           # every interval of one length ties
+    X[4] = np.exp(3 * X[4])
+    _same(E, X, s, budget_bits=1.5)
+    if d in (33, 129, 300):
+        _same(E, X, s, budget_bits=2.0, flags=E.EXACT_S)
+        _same(E, X, s, lambda_=0.0)
+        _same(E, X, s, lambda_=0.3)
+
+
+@pytest.mark.parametrize("d", [60, 128])
+def test_rows_at_the_ends_of_the_fp32_range(E, d):
+    """Magnitudes of 1e18 and 1e-18, values 1e-30 of the largest, gaps too small for fp32 costs
+    (left to the binary64 kernel) and a multiplier beyond fp32."""
+    rng = np.random.default_rng(9)
+    X = rng.standard_normal((6, d)).astype(np.float32)
+    X[0] *= np.float32(1e18)
+    X[1] *= np.float32(1e-18)
+    X[2, : d // 2] *= np.float32(1e-30)
+    X[3, : d // 2] = (np.arange(d // 2) * 1.4e-45).astype(np.float32)
+    X[4, 0], X[4, 1] = np.float32(3e38), np.float32(-3e38)
+    X[5] = np.linspace(0, 1e-40, d).astype(np.float32)
+    _same(E, X, 6, budget_bits=1.5)
+    _same(E, X[:3], 6, lambda_=1e37)
