@@ -17,7 +17,7 @@ int launch_dp_reference(const Prefix &P, const double *lamp, int G, int s, doubl
                         cudaStream_t st);
 int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, const Layout &L, cudaStream_t st,
                    bool exact_s, bool exact_tables, float *costs, bool build_costs, bool test_stall,
-                   size_t chunk_bytes, bool seeded, bool unbounded);
+                   size_t chunk_bytes, bool seeded, bool unbounded, bool tables);
 int save_dp_seed(void *ws, const Layout &Lw, int64_t p, int G, int s, int g, cudaStream_t st);
 size_t resident_costs_bytes(int64_t d);
 size_t streamed_costs_bytes(int64_t d);
@@ -296,8 +296,10 @@ struct PassOut {
 // seeded: the workspace's seed rows hold an earlier pass's fp32 minima at a multiplier
 // >= every multiplier of this pass (save_dp_seed); the fast kernel's tile skipping
 // starts from them.
+// tables: the caller may read the pass's tables (ecasq_dp_tables).
 static int dp_pass_prepared(void *ws, const Layout &L, const Prefix &P, int s, const double *lamp, int G,
-                            uint32_t flags, cudaStream_t st, PassOut &out, bool *costs_built, bool seeded = false) {
+                            uint32_t flags, cudaStream_t st, PassOut &out, bool *costs_built, bool seeded = false,
+                            bool tables = false) {
     double *dp64 = wsp<double>(ws, L.dp64);
     int32_t *bp = wsp<int32_t>(ws, L.bp);
     int rc;
@@ -313,7 +315,7 @@ static int dp_pass_prepared(void *ws, const Layout &L, const Prefix &P, int s, c
         rc = launch_dp_fast(P, lamp, G, s, ws, L, st, (flags & ECASQ_EXACT_S) != 0, (flags & ECASQ_EXACT_TABLES) != 0,
                             costs, costs && (L.costs_streamed || !*costs_built), (flags & ECASQ_TEST_STALL) != 0,
                             L.costs_streamed ? L.costs_bytes : 0,
-                            seeded && !(flags & ECASQ_UNSEEDED_SEARCH), (flags & ECASQ_UNSEEDED_SEARCH) != 0);
+                            seeded && !(flags & ECASQ_UNSEEDED_SEARCH), (flags & ECASQ_UNSEEDED_SEARCH) != 0, tables);
         if (costs && rc == ECASQ_OK) *costs_built = true;
     }
     if (rc != ECASQ_OK) return rc;
@@ -536,7 +538,7 @@ int ecasq_dp_pass(const float *x, int64_t d, int32_t s, const double *lambdas, i
     for (int g = 0; g < G; g++) lamp[g] = lambdas[g] * n2;
     PassOut po;
     bool costs_built = false;
-    rc = dp_pass_prepared(ws, L, P, s, lamp, G, flags, st, po, &costs_built);
+    rc = dp_pass_prepared(ws, L, P, s, lamp, G, flags, st, po, &costs_built, false, true);
     if (rc) return rc;
     rc = launch_gather_q(P.v, wsp<int32_t>(ws, L.qidx), wsp<int32_t>(ws, L.mcount), G, s, Q_out, st);
     if (rc) return rc;
