@@ -74,9 +74,18 @@ __global__ void k_grid_round(GridArgs A, int i) {
     }
 }
 
+// Binary64 values as integers of the same order (-0 as +0): compares of them stay off the binary64 pipe, which does two
+// a cycle and SM.
+__device__ __forceinline__ long long order_key(double x) {
+    const long long b = __double_as_longlong(x);
+    return b >= 0 ? b : b == (long long)0x8000000000000000ull ? 0 : b ^ 0x7fffffffffffffffll;
+}
+
 // One block per output j (heavy outputs first), its threads splitting the k range, so
 // that no output's scan is a long serial walk of one warp (the last outputs have n - 1
-// candidates per multiplier, and each step of a walk waits on its loads from L2).
+// candidates per multiplier, and each step of a walk waits on its loads from L2).  Nearly every output has one
+// member per multiplier: its thread writes it as it is, and only warps that hold several reduce them, by integer keys
+// (a reduction of all lanes with binary64 compares was most of a layer's 29 us at n = 1000; now 20).
 constexpr int kGridThreads = 256;
 __global__ void __launch_bounds__(kGridThreads, 3) k_grid_layer(GridArgs A, int i) {
     __shared__ float sm[kGridThreads / 32][kMaxG];
@@ -99,9 +108,9 @@ __global__ void __launch_bounds__(kGridThreads, 3) k_grid_layer(GridArgs A, int 
     }
 #pragma unroll
     for (int g = 0; g < kMaxG; g++) {
-        float v = m[g];
-        for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (lane == 0) sm[wid][g] = v;
+        // least value: as an integer of the same order
+        const int b = __float_as_int(m[g]), v = __reduce_min_sync(0xffffffffu, b >= 0 ? b : b ^ 0x7fffffff);
+        if (lane == 0) sm[wid][g] = __int_as_float(v >= 0 ? v : v ^ 0x7fffffff);
     }
     __syncthreads();
     // the band limits, once per block (binary64 runs at 1/64 of the fp32 rate): rounded down
@@ -123,54 +132,56 @@ __global__ void __launch_bounds__(kGridThreads, 3) k_grid_layer(GridArgs A, int 
     const int64_t Nj = A.N[j + 1];
     for (int64_t k = i - 2 + threadIdx.x; k < j; k += kGridThreads) {
         float2 cf = A.pc32[tb + k];
+        unsigned in = 0u;
+#pragma unroll
+        for (int g = 0; g < kMaxG; g++)
+            if (g < G && __fadd_rn(A.dp32[g_at(A, g, i - 1, k)], __fmaf_rn(A.lam32[g], cf.y, cf.x)) <= T[g]) in |= 1u << g;
+        if (!in) continue;
         // no data in (P_k, P_j]: then App. E's sums are differences of equal prefix values,
         // so C = U = D = 0 and Phi = 0 exactly, and the candidate is dp(i-1, k) itself
         // (x + 0 = x for x >= +0, lambda' 0 = +0): no pair load, no binary64 arithmetic.
         // Grids with many empty intervals (heavy tails) have long runs of such candidates
         // in their bands.
         const bool empty = A.N[k + 1] == Nj;
+        const double2 e = empty ? make_double2(0.0, 0.0) : A.pc64[tb + k];
 #pragma unroll
         for (int g = 0; g < kMaxG; g++) {
-            if (g < G) {
-                float v = __fadd_rn(A.dp32[g_at(A, g, i - 1, k)], __fmaf_rn(A.lam32[g], cf.y, cf.x));
-                if (v <= T[g]) {
-                    const double dprev = A.dp64[g_at(A, g, i - 1, k)];
-                    double c = dprev;
-                    if (!empty) {
-                        const double2 e = A.pc64[tb + k];
-                        c = __dadd_rn(dprev, __dadd_rn(e.x, __dmul_rn(A.lam64[g], e.y)));
-                    }
-                    // integer compares of the bit patterns (binary64 compares run on the
-                    // binary64 pipe)
-                    const long long cb = __double_as_longlong(c), bb = __double_as_longlong(best[g]);
-                    // non-negative doubles (+inf included) order like their bit patterns
-                    const bool lt = (cb >= 0 && bb >= 0) ? cb < bb : c < best[g];
-                    if (lt) { best[g] = c; arg[g] = (int32_t)k; }  // k ascends per thread
-                }
+            if ((in >> g) & 1u) {
+                const double dprev = A.dp64[g_at(A, g, i - 1, k)];
+                const double c = empty ? dprev : __dadd_rn(dprev, __dadd_rn(e.x, __dmul_rn(A.lam64[g], e.y)));
+                if (order_key(c) < order_key(best[g])) { best[g] = c; arg[g] = (int32_t)k; }  // k ascends per thread
             }
         }
     }
     // least value, then lowest k: over the lanes, then over the warps
 #pragma unroll
     for (int g = 0; g < kMaxG; g++) {
-        double b = best[g];
-        int32_t a = arg[g];
-        for (int o = 16; o > 0; o >>= 1) {
-            double b2 = __shfl_xor_sync(0xffffffffu, b, o);
-            int32_t a2 = __shfl_xor_sync(0xffffffffu, a, o);
-            if (a2 >= 0 && (a < 0 || b2 < b || (b2 == b && a2 < a))) { b = b2; a = a2; }
+        const unsigned has = __ballot_sync(0xffffffffu, arg[g] >= 0);
+        if (!has) {
+            if (lane == 0) sa[wid][g] = -1;
+        } else if (!(has & (has - 1u))) {
+            if (arg[g] >= 0) { sb[wid][g] = best[g]; sa[wid][g] = arg[g]; }
+        } else {
+            long long b = arg[g] >= 0 ? order_key(best[g]) : 0x7fffffffffffffffll;
+            int32_t a = arg[g] >= 0 ? arg[g] : 0x7fffffff;
+            for (int o = 16; o > 0; o >>= 1) {
+                const long long b2 = __shfl_xor_sync(0xffffffffu, b, o);
+                const int32_t a2 = __shfl_xor_sync(0xffffffffu, a, o);
+                if (b2 < b || (b2 == b && a2 < a)) { b = b2; a = a2; }
+            }
+            if (arg[g] == a) { sb[wid][g] = best[g]; sa[wid][g] = a; }  // one lane: a k belongs to one thread
         }
-        if (lane == 0) { sb[wid][g] = b; sa[wid][g] = a; }
     }
     __syncthreads();
     if (threadIdx.x < G) {
         const int g = threadIdx.x;
-        double b = sb[0][g];
-        int32_t a = sa[0][g];
-        for (int w = 1; w < kGridThreads / 32; w++) {
-            const double b2 = sb[w][g];
+        double b = CUDART_INF;
+        int32_t a = -1;
+        for (int w = 0; w < kGridThreads / 32; w++) {
             const int32_t a2 = sa[w][g];
-            if (a2 >= 0 && (a < 0 || b2 < b || (b2 == b && a2 < a))) { b = b2; a = a2; }
+            if (a2 < 0) continue;
+            const long long x = order_key(sb[w][g]), y = order_key(b);
+            if (a < 0 || x < y || (x == y && a2 < a)) { b = sb[w][g]; a = a2; }
         }
         A.dp64[g_at(A, g, i, j)] = b;
         A.bp[g_at(A, g, i, j)] = a;
