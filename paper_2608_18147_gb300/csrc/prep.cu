@@ -21,16 +21,42 @@ __device__ __forceinline__ float key2f(uint32_t k) {
     return __uint_as_float(u);
 }
 
-__global__ void k_make_keys(const float *__restrict__ x, int64_t d, uint32_t *__restrict__ keys,
-                            DevStatus *st) {
+// The range of the values' last-place exponents u (a value is an integer below 2^24 times 2^u), kept behind
+// the status record so that zero means none yet: hi = max u + 200, lo = 200 - min u, over non-zero values.
+struct UlpRange { uint32_t hi, lo; };
+constexpr size_t kUlpRangeAt = 128;
+static_assert(sizeof(DevStatus) <= kUlpRangeAt, "the range lies behind the status record");
+__device__ __forceinline__ UlpRange *ulp_range(DevStatus *st) {
+    return reinterpret_cast<UlpRange *>(reinterpret_cast<char *>(st) + kUlpRangeAt);
+}
+__device__ __forceinline__ int ulp_exp(uint32_t bits) { return max((int)((bits >> 23) & 255u), 1) - 150; }
+__device__ __forceinline__ void ulp_note(float f, uint32_t &hi, uint32_t &lo) {
+    const uint32_t b = __float_as_uint(f);
+    if (!(b << 1)) return;
+    hi = max(hi, (uint32_t)(ulp_exp(b) + 200));
+    lo = max(lo, (uint32_t)(200 - ulp_exp(b)));
+}
+
+__global__ void __launch_bounds__(256) k_make_keys(const float *__restrict__ x, int64_t d, uint32_t *__restrict__ keys,
+                                                   DevStatus *st) {
+    __shared__ uint32_t bhi, blo;
+    if (threadIdx.x == 0) bhi = blo = 0u;
+    __syncthreads();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    uint32_t hi = 0u, lo = 0u;
     for (; i < d; i += stride) {
         float f = x[i];
         if (!isfinite(f)) st->nonfinite = 1;
         if (f == 0.0f) f = 0.0f;
         keys[i] = f2key(f);
+        ulp_note(f, hi, lo);
     }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    if ((threadIdx.x & 31) == 0) { atomicMax(&bhi, hi); atomicMax(&blo, lo); }
+    __syncthreads();
+    if (threadIdx.x == 0) { atomicMax(&ulp_range(st)->hi, bhi); atomicMax(&ulp_range(st)->lo, blo); }
 }
 
 // counts[digit * nb + block] = number of keys of the block with that digit.
@@ -172,58 +198,220 @@ __global__ void __launch_bounds__(256) k_radix_scatter(const uint32_t *__restric
     }
 }
 
-// Pass A of the histogram scan: per tile of kScanTile sorted keys, the number
-// of unique-value heads and the double-double sums of x and x^2.
-struct DDPart { double s_hi, s_lo, q_hi, q_lo; int64_t heads; int64_t pad; };
-
-
+// ---------------------------------------------------- prefix sums of x and x^2
+// The sums are needed as double-double prefixes.  Where the data's range allows it (exact_window; all but data
+// with values 10^-24 of the largest) they are exact integers in units of the smallest last place, 128 bits
+// for x and 256 for x^2, rounded once to a double-double: the chip has 2 binary64 operations a cycle and SM, and
+// a double-double sum per key in two passes and their block scans took 863 of a preparation's 1240 us at
+// d = 4 million (220 now).  A sum that 106 bits hold has the same bits either way.  Else they are
+// double-double sums in one fixed order.
 template <typename T>
 __device__ __forceinline__ T shfl_up(T v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
 
-struct ScanVal { dd s, q; int64_t h; };
+// Exact sums of x 2^-B and x^2 2^-2B (two's complement; unsigned), and the number of heads.
+struct IntSums {
+    uint64_t s[2], q[4];
+    int64_t h;
+};
+// Double-double sums and the number of heads.
+struct DDSums { dd s, q; int64_t h; };
 
-__device__ __forceinline__ ScanVal sv_add(const ScanVal &a, const ScanVal &b) {
-    return {dd_add(a.s, b.s), dd_add(a.q, b.q), a.h + b.h};
+__device__ __forceinline__ void add_words(uint64_t (&a)[2], uint64_t b0, uint64_t b1) {
+    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(a[0]), "+l"(a[1]) : "l"(b0), "l"(b1));
+}
+__device__ __forceinline__ void add_words(uint64_t (&a)[4], uint64_t b0, uint64_t b1, uint64_t b2, uint64_t b3) {
+    asm("add.cc.u64 %0, %0, %4;\n\taddc.cc.u64 %1, %1, %5;\n\taddc.cc.u64 %2, %2, %6;\n\taddc.u64 %3, %3, %7;"
+        : "+l"(a[0]), "+l"(a[1]), "+l"(a[2]), "+l"(a[3]) : "l"(b0), "l"(b1), "l"(b2), "l"(b3));
+}
+__device__ __forceinline__ void neg_words(uint64_t (&a)[2]) {
+    a[0] = ~a[0];
+    a[1] = ~a[1];
+    add_words(a, 1, 0);
 }
 
-// Block-wide inclusive scan of one ScanVal per thread (256 threads).
-__device__ ScanVal block_scan_incl(ScanVal v, ScanVal *wtot, ScanVal &total) {
+// The top-aligned words of a non-zero integer, and by how many bits it was shifted up.
+template <int NW>
+__device__ __forceinline__ int align_words(uint64_t (&w)[NW]) {
+    int sh = 0;
+#pragma unroll
+    for (int r = 0; r < NW - 1; r++)
+        if (w[NW - 1] == 0) {
+#pragma unroll
+            for (int i = NW - 1; i > 0; i--) w[i] = w[i - 1];
+            w[0] = 0;
+            sh += 64;
+        }
+    const int c = __clzll((long long)w[NW - 1]);
+    if (c) {
+#pragma unroll
+        for (int i = NW - 1; i > 0; i--) w[i] = w[i] << c | w[i - 1] >> (64 - c);
+        w[0] <<= c;
+    }
+    return sh + c;
+}
+// The double nearest to w 2^e, ties to even (w non-zero; in the normal range); w becomes the distance to it,
+// rounded_up its direction.
+template <int NW>
+__device__ __forceinline__ double take_double(uint64_t (&w)[NW], int e, bool neg, bool &rounded_up, int &e_out) {
+    e -= align_words(w);
+    uint64_t m = w[NW - 1] >> 11, rest = w[NW - 1] & 0x7FFu, low = 0;
+#pragma unroll
+    for (int i = 0; i < NW - 1; i++) low |= w[i];
+    rounded_up = rest > 0x400u || (rest == 0x400u && (low != 0 || (m & 1u)));
+    w[NW - 1] = rest;
+    if (rounded_up) {  // the distance is 2^(64 NW - 53) - rest
+        m++;
+        uint64_t carry = 1;
+#pragma unroll
+        for (int i = 0; i < NW; i++) {
+            w[i] = ~w[i] + carry;
+            carry = carry && w[i] == 0;
+        }
+        w[NW - 1] &= 0x7FFu;
+    }
+    e_out = e;
+    int x = e + 64 * NW - 53 + 52 + 1023;
+    if (m >> 53) { m >>= 1; x++; }
+    return __longlong_as_double((long long)((neg ? 1ull << 63 : 0ull) | (uint64_t)x << 52 | (m & ((1ull << 52) - 1))));
+}
+// w 2^e (negated if neg) as the double-double nearest to it.
+template <int NW>
+__device__ __forceinline__ dd words_to_dd(uint64_t (&w)[NW], int e, bool neg) {
+    uint64_t any = 0;
+#pragma unroll
+    for (int i = 0; i < NW; i++) any |= w[i];
+    if (!any) return {0.0, 0.0};
+    bool up, up2;
+    int e1, e2;
+    const double hi = take_double(w, e, neg, up, e1);
+    any = 0;
+#pragma unroll
+    for (int i = 0; i < NW; i++) any |= w[i];
+    if (!any) return {hi, 0.0};
+    return {hi, take_double(w, e1, neg != up, up2, e2)};
+}
+
+// How a data set is summed: B < kNoWindow, exact integers in units of 2^B.
+constexpr int kNoWindow = 1 << 20;
+__device__ __forceinline__ int exact_window(UlpRange r, int64_t d) {
+    if (!r.hi) return 0;  // zeros only
+    const int umin = 200 - (int)r.lo, umax = (int)r.hi - 200, bits = 64 - __clzll(d);
+    return 24 + umax - umin + bits <= 126 ? umin : kNoWindow;  // x^2: 48 + 2 (umax - umin) + bits <= 252
+}
+
+struct SumInt {
+    using Val = IntSums;
+    int B;
+    __device__ Val zero() const { return {{0, 0}, {0, 0, 0, 0}, 0}; }
+    __device__ void add_key(Val &a, uint32_t key) const {
+        const uint32_t b = __float_as_uint(key2f(key));
+        const uint32_t m = (b & 0x7FFFFFu) | (b & 0x7F800000u ? 0x800000u : 0u);
+        const int sh = m ? ulp_exp(b) - B : 0;
+        const uint64_t v = m;
+        uint64_t x[2] = {sh < 64 ? v << sh : 0ull, sh < 64 ? (sh ? v >> (64 - sh) : 0ull) : v << (sh - 64)};
+        if (b >> 31) neg_words(x);
+        add_words(a.s, x[0], x[1]);
+        const uint64_t q = v * v;
+        const int w = 2 * sh >> 6, c = 2 * sh & 63;
+        const uint64_t l = q << c, h = c ? q >> (64 - c) : 0ull;
+        add_words(a.q, w == 0 ? l : 0ull, w == 1 ? l : w == 0 ? h : 0ull, w == 2 ? l : w == 1 ? h : 0ull,
+                  w == 3 ? l : w == 2 ? h : 0ull);
+    }
+    __device__ Val add(const Val &a, const Val &b) const {
+        Val r = a;
+        add_words(r.s, b.s[0], b.s[1]);
+        add_words(r.q, b.q[0], b.q[1], b.q[2], b.q[3]);
+        r.h += b.h;
+        return r;
+    }
+    // a - b (b summed into a before)
+    __device__ Val sub(const Val &a, const Val &b) const {
+        Val r = a;
+        asm("sub.cc.u64 %0, %0, %2;\n\tsubc.u64 %1, %1, %3;" : "+l"(r.s[0]), "+l"(r.s[1]) : "l"(b.s[0]), "l"(b.s[1]));
+        asm("sub.cc.u64 %0, %0, %4;\n\tsubc.cc.u64 %1, %1, %5;\n\tsubc.cc.u64 %2, %2, %6;\n\tsubc.u64 %3, %3, %7;"
+            : "+l"(r.q[0]), "+l"(r.q[1]), "+l"(r.q[2]), "+l"(r.q[3]) : "l"(b.q[0]), "l"(b.q[1]), "l"(b.q[2]), "l"(b.q[3]));
+        r.h -= b.h;
+        return r;
+    }
+    __device__ Val shfl_up(const Val &v, int o) const {
+        Val t;
+#pragma unroll
+        for (int i = 0; i < 2; i++) t.s[i] = ecasq::shfl_up(v.s[i], o);
+#pragma unroll
+        for (int i = 0; i < 4; i++) t.q[i] = ecasq::shfl_up(v.q[i], o);
+        t.h = ecasq::shfl_up(v.h, o);
+        return t;
+    }
+    __device__ dd s_of(const Val &v) const {
+        uint64_t w[2] = {v.s[0], v.s[1]};
+        const bool neg = w[1] >> 63;
+        if (neg) neg_words(w);
+        return words_to_dd(w, B, neg);
+    }
+    __device__ dd q_of(const Val &v) const {
+        uint64_t w[4] = {v.q[0], v.q[1], v.q[2], v.q[3]};
+        return words_to_dd(w, 2 * B, false);
+    }
+};
+
+// x^2 of a binary32 value is exact in binary64.
+struct SumDD {
+    using Val = DDSums;
+    __device__ Val zero() const { return {{0.0, 0.0}, {0.0, 0.0}, 0}; }
+    __device__ void add_key(Val &a, uint32_t key) const {
+        const double x = (double)key2f(key);
+        a.s = dd_add_d(a.s, x);
+        a.q = dd_add_d(a.q, __dmul_rn(x, x));
+    }
+    __device__ Val add(const Val &a, const Val &b) const { return {dd_add(a.s, b.s), dd_add(a.q, b.q), a.h + b.h}; }
+    __device__ Val sub(const Val &a, const Val &b) const { return {dd_sub(a.s, b.s), dd_sub(a.q, b.q), a.h - b.h}; }
+    __device__ Val shfl_up(const Val &v, int o) const {
+        return {{ecasq::shfl_up(v.s.hi, o), ecasq::shfl_up(v.s.lo, o)}, {ecasq::shfl_up(v.q.hi, o), ecasq::shfl_up(v.q.lo, o)},
+                ecasq::shfl_up(v.h, o)};
+    }
+    __device__ dd s_of(const Val &v) const { return v.s; }
+    __device__ dd q_of(const Val &v) const { return v.q; }
+};
+// One tile's partial of either kind.
+union HistPart { IntSums i; DDSums d; };
+static_assert(sizeof(HistPart) <= 192, "a tile of kHistTile keys has four scan tiles' room");
+__device__ __forceinline__ IntSums &part_of(HistPart &p, const SumInt &) { return p.i; }
+__device__ __forceinline__ DDSums &part_of(HistPart &p, const SumDD &) { return p.d; }
+
+// Block-wide inclusive scan of one value per thread (256 threads).
+template <typename Sum>
+__device__ typename Sum::Val block_scan_incl(const Sum &sum, typename Sum::Val v, HistPart *wtot, typename Sum::Val &total) {
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int o = 1; o < 32; o <<= 1) {
-        ScanVal t;
-        t.s.hi = shfl_up(v.s.hi, o); t.s.lo = shfl_up(v.s.lo, o);
-        t.q.hi = shfl_up(v.q.hi, o); t.q.lo = shfl_up(v.q.lo, o);
-        t.h = shfl_up(v.h, o);
-        if (lane >= o) v = sv_add(t, v);
+        const typename Sum::Val t = sum.shfl_up(v, o);
+        if (lane >= o) v = sum.add(t, v);
     }
-    if (lane == 31) wtot[wid] = v;
+    if (lane == 31) part_of(wtot[wid], sum) = v;
     __syncthreads();
     if (threadIdx.x == 0) {
-        ScanVal acc = wtot[0];
-        for (int w = 1; w < 8; w++) { acc = sv_add(acc, wtot[w]); wtot[w] = acc; }
+        typename Sum::Val acc = part_of(wtot[0], sum);
+        for (int w = 1; w < 8; w++) { acc = sum.add(acc, part_of(wtot[w], sum)); part_of(wtot[w], sum) = acc; }
     }
     __syncthreads();
-    if (wid > 0) v = sv_add(wtot[wid - 1], v);
-    total = wtot[7];
+    if (wid > 0) v = sum.add(part_of(wtot[wid - 1], sum), v);
+    total = part_of(wtot[7], sum);
     __syncthreads();
     return v;
 }
 
-// The thread's kHistPer consecutive sorted keys starting at base (positions >= d are
-// left out): x as binary64, the sums of x and x^2 in double-double (x^2 of a binary32
-// value is exact in binary64) and the number of heads.  One fixed order per thread, so
-// the single-row and the batched paths, which both call it, give the same bits.
-__device__ __forceinline__ ScanVal hist_thread_sums(const uint32_t *keys, int64_t d, int64_t base) {
-    ScanVal v{{0.0, 0.0}, {0.0, 0.0}, 0};
+// The thread's kHistPer consecutive sorted keys starting at base (positions >= d are left out): the sums of x and
+// x^2 and the number of heads.  One fixed order per thread, so the single-row and the batched
+// paths, which both call it, give the same bits.
+template <typename Sum>
+__device__ __forceinline__ typename Sum::Val hist_thread_sums(const Sum &sum, const uint32_t *keys, int64_t d, int64_t base) {
+    typename Sum::Val v = sum.zero();
     uint32_t prev = base > 0 && base - 1 < d ? keys[base - 1] : 0u;
 #pragma unroll 4
     for (int e = 0; e < kHistPer; e++) {
         const int64_t i = base + e;
         if (i < d) {
             const uint32_t k = keys[i];
-            const double x = (double)key2f(k);
-            v.s = dd_add_d(v.s, x);
-            v.q = dd_add_d(v.q, __dmul_rn(x, x));
+            sum.add_key(v, k);
             v.h += (i == 0 || k != prev) ? 1 : 0;
             prev = k;
         }
@@ -235,89 +423,100 @@ __device__ __forceinline__ ScanVal hist_thread_sums(const uint32_t *keys, int64_
 // i writes its unique index u = run.h, v[u], N[u] = i, S[u] and S2[u] (hi at [u], lo at
 // [lo_off + u]); the last position d - 1 also writes the totals at index p and returns
 // p and ||X||^2 through p_out and norm2_out.
-__device__ __forceinline__ void hist_thread_fill(const uint32_t *keys, int64_t d, int64_t base, ScanVal run,
-                                                 float *v, int64_t *N, double *S, double *S2, int64_t lo_off,
-                                                 int64_t *p_out, double *norm2_out) {
+template <typename Sum>
+__device__ __forceinline__ void hist_thread_fill(const Sum &sum, const uint32_t *keys, int64_t d, int64_t base,
+                                                 typename Sum::Val run, float *v, int64_t *N, double *S, double *S2,
+                                                 int64_t lo_off, int64_t *p_out, double *norm2_out) {
     uint32_t prev = base > 0 && base - 1 < d ? keys[base - 1] : 0u;
-#pragma unroll 4
+#pragma unroll 1
     for (int e = 0; e < kHistPer; e++) {
         const int64_t i = base + e;
         if (i >= d) break;
         const uint32_t k = keys[i];
-        const double x = (double)key2f(k);
         const bool head = i == 0 || k != prev;
         prev = k;
         if (head) {
             const int64_t u = run.h;
-            v[u] = (float)x;
+            const dd ss = sum.s_of(run), qq = sum.q_of(run);
+            v[u] = key2f(k);
             N[u] = i;
-            S[u] = run.s.hi; S[lo_off + u] = run.s.lo;
-            S2[u] = run.q.hi; S2[lo_off + u] = run.q.lo;
+            S[u] = ss.hi; S[lo_off + u] = ss.lo;
+            S2[u] = qq.hi; S2[lo_off + u] = qq.lo;
         }
-        run.s = dd_add_d(run.s, x);
-        run.q = dd_add_d(run.q, __dmul_rn(x, x));
+        sum.add_key(run, k);
         run.h += head ? 1 : 0;
         if (i == d - 1) {
             const int64_t p = run.h;
+            const dd ss = sum.s_of(run), qq = sum.q_of(run);
             N[p] = d;
-            S[p] = run.s.hi; S[lo_off + p] = run.s.lo;
-            S2[p] = run.q.hi; S2[lo_off + p] = run.q.lo;
+            S[p] = ss.hi; S[lo_off + p] = ss.lo;
+            S2[p] = qq.hi; S2[lo_off + p] = qq.lo;
             *p_out = p;
-            *norm2_out = run.q.hi;
+            *norm2_out = qq.hi;
         }
     }
 }
 
-__global__ void __launch_bounds__(256) k_hist_partials(const uint32_t *__restrict__ keys, int64_t d, DDPart *part) {
-    __shared__ ScanVal wtot[8];
-    const ScanVal v = hist_thread_sums(keys, d, (int64_t)blockIdx.x * kHistTile + (int64_t)threadIdx.x * kHistPer);
-    ScanVal tot;
-    block_scan_incl(v, wtot, tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = {tot.s.hi, tot.s.lo, tot.q.hi, tot.q.lo, tot.h, 0};
+// f(sum) with the data set's way of summing.
+template <typename F>
+__device__ __forceinline__ void with_sums(UlpRange r, int64_t d, F &&f) {
+    const int B = exact_window(r, d);
+    if (B < kNoWindow) f(SumInt{B});
+    else f(SumDD{});
 }
 
-// Exclusive scan of the tile partials (one thread, in order; nb is small).
+// Pass A of the histogram scan: per tile of kHistTile sorted keys, the number of unique-value heads and the sums
+// of x and x^2.
+__global__ void __launch_bounds__(256) k_hist_partials(const uint32_t *__restrict__ keys, int64_t d, HistPart *part,
+                                                       DevStatus *st) {
+    __shared__ HistPart wtot[8];
+    with_sums(*ulp_range(st), d, [&](auto sum) {
+        const auto v = hist_thread_sums(sum, keys, d, (int64_t)blockIdx.x * kHistTile + (int64_t)threadIdx.x * kHistPer);
+        auto tot = v;
+        block_scan_incl(sum, v, wtot, tot);
+        if (threadIdx.x == 0) part_of(part[blockIdx.x], sum) = tot;
+    });
+}
+
 // Exclusive scan of the tiles' partials by one block of 256 threads: each thread sums a
 // contiguous run of tiles in order, the runs' totals are scanned across the block
 // (block_scan_incl), and each thread then writes its run's exclusive prefixes.
-__global__ void __launch_bounds__(256) k_hist_scan_partials(DDPart *part, int64_t nb) {
-    __shared__ ScanVal wtot[8];
-    __shared__ ScanVal incl_all[256];
+__global__ void __launch_bounds__(256) k_hist_scan_partials(HistPart *part, int64_t nb, int64_t d, DevStatus *st) {
+    __shared__ HistPart wtot[8];
+    __shared__ HistPart incl_all[256];
     const int64_t per = cdiv(nb, (int64_t)blockDim.x);
     const int64_t lo = min((int64_t)threadIdx.x * per, nb), hi = min(lo + per, nb);
-    ScanVal s{{0.0, 0.0}, {0.0, 0.0}, 0};
-    for (int64_t b = lo; b < hi; b++) {
-        ScanVal t{{part[b].s_hi, part[b].s_lo}, {part[b].q_hi, part[b].q_lo}, part[b].heads};
-        s = sv_add(s, t);
-    }
-    ScanVal total;
-    incl_all[threadIdx.x] = block_scan_incl(s, wtot, total);
-    __syncthreads();
-    ScanVal acc = threadIdx.x > 0 ? incl_all[threadIdx.x - 1] : ScanVal{{0.0, 0.0}, {0.0, 0.0}, 0};
-    for (int64_t b = lo; b < hi; b++) {
-        ScanVal t{{part[b].s_hi, part[b].s_lo}, {part[b].q_hi, part[b].q_lo}, part[b].heads};
-        part[b] = {acc.s.hi, acc.s.lo, acc.q.hi, acc.q.lo, acc.h, 0};
-        acc = sv_add(acc, t);
-    }
+    with_sums(*ulp_range(st), d, [&](auto sum) {
+        auto s = sum.zero();
+        for (int64_t b = lo; b < hi; b++) s = sum.add(s, part_of(part[b], sum));
+        auto total = s;
+        part_of(incl_all[threadIdx.x], sum) = block_scan_incl(sum, s, wtot, total);
+        __syncthreads();
+        auto acc = threadIdx.x > 0 ? part_of(incl_all[threadIdx.x - 1], sum) : sum.zero();
+        for (int64_t b = lo; b < hi; b++) {
+            const auto t = part_of(part[b], sum);
+            part_of(part[b], sum) = acc;
+            acc = sum.add(acc, t);
+        }
+    });
 }
 
 // Pass C: per sorted position i that starts a run of equal keys (a head), the
 // unique index u and v[u], N[u] = i, S[u], S2[u] (exclusive prefix sums).
 // The last position also writes N[p] = d, S[p], S2[p], p and ||X||^2.
-__global__ void __launch_bounds__(256) k_hist_fill(const uint32_t *__restrict__ keys, int64_t d, const DDPart *part,
+__global__ void __launch_bounds__(256) k_hist_fill(const uint32_t *__restrict__ keys, int64_t d, HistPart *part,
                                                    float *v, int64_t *N, double *S, double *S2, DevStatus *st,
                                                    int64_t pcap) {
-    __shared__ ScanVal wtot[8];
+    __shared__ HistPart wtot[8];
     const int64_t base = (int64_t)blockIdx.x * kHistTile + (int64_t)threadIdx.x * kHistPer;
-    const ScanVal loc = hist_thread_sums(keys, d, base);
-    ScanVal tot;
-    const ScanVal incl = block_scan_incl(loc, wtot, tot);
-    const DDPart &pb = part[blockIdx.x];
-    const ScanVal off{{pb.s_hi, pb.s_lo}, {pb.q_hi, pb.q_lo}, pb.heads};
-    // exclusive prefix before this thread's first element
-    ScanVal run{dd_sub(incl.s, loc.s), dd_sub(incl.q, loc.q), incl.h - loc.h};
-    run = sv_add(off, run);
-    hist_thread_fill(keys, d, base, run, v, N, S, S2, pcap + 1, &st->p, &st->norm2);
+    with_sums(*ulp_range(st), d, [&](auto sum) {
+        const auto loc = hist_thread_sums(sum, keys, d, base);
+        auto tot = loc;
+        const auto incl = block_scan_incl(sum, loc, wtot, tot);
+        // exclusive prefix before this thread's first element
+        const auto run = sum.add(part_of(part[blockIdx.x], sum), sum.sub(incl, loc));
+        hist_thread_fill(sum, keys, d, base, run, v, N, S, S2, pcap + 1, &st->p, &st->norm2);
+    });
 }
 
 // The arrays were written with lo parts at offset pcap+1 (pcap = d); repack
@@ -342,13 +541,18 @@ __global__ void k_hist_finish(int64_t *N, int64_t *w, double *S, double *S2, con
 // that row alone.
 __global__ void __launch_bounds__(256) k_rows_prepare(const float *__restrict__ X, RowsData R) {
     __shared__ uint32_t keys[kScanTile];
-    __shared__ ScanVal wtot[8];
+    __shared__ HistPart wtot[8];
     __shared__ int nonfin;
+    __shared__ UlpRange range;
     const int64_t row = blockIdx.x;
     const int d = (int)R.d;
     const float *x = X + row * R.d;
-    if (threadIdx.x == 0) nonfin = 0;
+    if (threadIdx.x == 0) {
+        nonfin = 0;
+        range = {0u, 0u};
+    }
     __syncthreads();
+    uint32_t hi = 0u, lo = 0u;
     for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
         uint32_t k = 0xFFFFFFFFu;  // above every finite key: padding sorts last
         if (i < d) {
@@ -356,9 +560,13 @@ __global__ void __launch_bounds__(256) k_rows_prepare(const float *__restrict__ 
             if (!isfinite(f)) nonfin = 1;
             if (f == 0.0f) f = 0.0f;
             k = f2key(f);
+            ulp_note(f, hi, lo);
         }
         keys[i] = k;
     }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    if ((threadIdx.x & 31) == 0) { atomicMax(&range.hi, hi); atomicMax(&range.lo, lo); }
     __syncthreads();
     int n2 = 1;
     while (n2 < d) n2 <<= 1;
@@ -381,15 +589,17 @@ __global__ void __launch_bounds__(256) k_rows_prepare(const float *__restrict__ 
     double *S = R.S + row * 2 * (dcap + 1), *S2 = R.S2 + row * 2 * (dcap + 1);
     // k_hist_fill, one tile
     const int64_t base = (int64_t)threadIdx.x * kHistPer;
-    const ScanVal loc = hist_thread_sums(keys, d, base);
-    ScanVal tot;
-    const ScanVal incl = block_scan_incl(loc, wtot, tot);
-    const int64_t p = tot.h;
-    const ScanVal off{{0.0, 0.0}, {0.0, 0.0}, 0};
-    ScanVal run{dd_sub(incl.s, loc.s), dd_sub(incl.q, loc.q), incl.h - loc.h};
-    run = sv_add(off, run);
-    hist_thread_fill(keys, d, base, run, v, N, S, S2, p + 1, R.p + row, R.norm2 + row);
+    __shared__ int64_t p_sm;
+    with_sums(range, d, [&](auto sum) {
+        const auto loc = hist_thread_sums(sum, keys, d, base);
+        auto tot = loc;
+        const auto incl = block_scan_incl(sum, loc, wtot, tot);
+        const auto run = sum.add(sum.zero(), sum.sub(incl, loc));
+        hist_thread_fill(sum, keys, d, base, run, v, N, S, S2, tot.h + 1, R.p + row, R.norm2 + row);
+        if (threadIdx.x == 0) p_sm = tot.h;
+    });
     __syncthreads();
+    const int64_t p = p_sm;
     for (int u = threadIdx.x; u < p; u += blockDim.x) w[u] = N[u + 1] - N[u];
     if (threadIdx.x == 0) R.nonfinite[row] = nonfin;
 }
@@ -465,7 +675,7 @@ int prepare_device(const float *x, int64_t d, void *ws, const Layout &L, cudaStr
     DevStatus *st = wsp<DevStatus>(ws, L.status);
     uint32_t *k0 = wsp<uint32_t>(ws, L.keys0), *k1 = wsp<uint32_t>(ws, L.keys1);
     uint32_t *cnt = wsp<uint32_t>(ws, L.rcount);
-    ECASQ_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(DevStatus), stream));
+    ECASQ_CUDA_TRY(cudaMemsetAsync(st, 0, kUlpRangeAt + sizeof(UlpRange), stream));
     int nb = (int)cdiv(d, kSortTile);
     note_launch();
     k_make_keys<<<(unsigned)std::min<int64_t>(cdiv(d, 256), 4096), 256, 0, stream>>>(x, d, k0, st);
@@ -482,14 +692,14 @@ int prepare_device(const float *x, int64_t d, void *ws, const Layout &L, cudaStr
     }
     // a == k0 holds the sorted keys
     int64_t nbs = cdiv(d, kHistTile);  // the layout holds cdiv(d, kScanTile) >= nbs partials
-    DDPart *part = wsp<DDPart>(ws, L.part);
+    HistPart *part = wsp<HistPart>(ws, L.part);
     // scratch copies of N/S/S2 with lo parts at offset d+1 live in keys1 / dp area
     double *Stmp = wsp<double>(ws, L.dp64);
     double *S2tmp = Stmp + 2 * (d + 1);
     note_launch();
-    k_hist_partials<<<(unsigned)nbs, 256, 0, stream>>>(a, d, part);
+    k_hist_partials<<<(unsigned)nbs, 256, 0, stream>>>(a, d, part, st);
     note_launch();
-    k_hist_scan_partials<<<1, 256, 0, stream>>>(part, nbs);
+    k_hist_scan_partials<<<1, 256, 0, stream>>>(part, nbs, d, st);
     note_launch();
     k_hist_fill<<<(unsigned)nbs, 256, 0, stream>>>(a, d, part, wsp<float>(ws, L.v), wsp<int64_t>(ws, L.N), Stmp,
                                                  S2tmp, st, d);
