@@ -559,12 +559,12 @@ __global__ void __launch_bounds__(NPROD) k_build_costs(const __grid_constant__ F
 // tile and diagonal, every layer, 22 000 cycles at s = 16) the critical path and left the SMs
 // unevenly loaded; here 15 blocks cost a few barriers and s - 2 gather/compute steps, and the
 // far tiles are shared evenly.  A pass of 8 multipliers (mean over a budgeted search, resident
-// costs): 25.6 ms instead of 46.3 at d = 2^17, s = 16; 1.69 instead of 2.93 at d = 16384, s = 16;
-// 15.1 instead of 47.7 at d = 50001, s = 32; building its own costs, 2.6 instead of 8.4 at
-// d = 12289, s = 16.  Of the 25.6 ms about 13.5 are far tiles, 3 uneven shares, 5 masks, 2.5
+// costs): 25.1 ms instead of 46.3 at d = 2^17, s = 16; 1.55 instead of 2.93 at d = 16384, s = 16;
+// 14.7 instead of 47.7 at d = 50001, s = 32; building its own costs, 2.5 instead of 8.4 at
+// d = 12289, s = 16.  Of the 25.1 ms about 13.5 are far tiles, 2.5 uneven shares, 5 masks, 2.5
 // bounds and 3 the near phases; far tiles are bound by issue (one add and one min a candidate
 // on the two FP32 pipes reach about 53 candidates per cycle and SM) and by the copies and
-// barriers of a tile, which cost as much as about 8 of its tasks (kTileCost).
+// barriers of a tile, which cost as much as about 6 of its tasks (kTileCost).
 
 // Grid barrier `epoch` (1, 2, ...): bounded; false when it gave up or another CTA aborted.  All
 // CTAs are resident (cooperative launch).  Orders generic and bulk-copy accesses on both sides.
@@ -714,7 +714,8 @@ __device__ __forceinline__ float4 far_start(const FastArgs &a, const int *u, int
 // multiplier that needs it at d = 2^17, s = 16, so tasks, not whole tiles, are the unit of work.
 // CTAs split the (column block, word range) pairs as in bound_phase; a thread tests one column of one
 // multiplier, kBoundL layers at a time.
-constexpr int kTileCost = 8;  // a listed tile's fixed cost (its copies, its costs into registers) in tasks
+constexpr int kTileCost = 6;  // a listed tile's fixed cost (its copies, its costs into registers) in tasks (a pass at d = 2^17, s = 16: 25.1 ms
+                               // with 6, 25.7 with 4 or 8, 26.6 with 12)
 static __device__ __noinline__ void mask_phase(const FastArgs &a, Smem &S, float *stage, const Panel &pn,
                                                uint64_t policy, uint32_t &ns) {
     const int L = a.s - 2, ct = threadIdx.x, lane = ct & 31, wid = ct >> 5, jl = ct & (BJ - 1), gq = ct / BJ;
@@ -946,6 +947,17 @@ __device__ __forceinline__ float *far_buf(const FastArgs &a, float *big, int b) 
     return big + (size_t)b * (kCostTileFloats + (size_t)a.tcap * BK);
 }
 
+// The first task of a tile of n (its position: its work before it, then kTileCost, then its tasks) behind a
+// share's border at `x` from the tile's position.  A border divides a tile's tasks, in eights, where both sides
+// keep 16 or more, as a tile of 112 tasks is a whole share of a small panel (d = 16384: 1.69 ms a pass with
+// whole tiles, 1.55 now); else they go to the later share.
+__device__ __forceinline__ int share_cut(int x, int n) {
+    x -= kTileCost;
+    if (x >= n) return n;
+    if (x < 16) return 0;
+    return n - x < 16 ? n : x & ~7;
+}
+
 // The next entries of the share, from word S.lnext (whose position is S.lpos) on: up to 16 words, a warp
 // each, as many as the list holds.  An entry: js << 14 | K, and its tasks as 128 bits.  S.lcount: entries;
 // S.lmore: the share goes on.  All threads.
@@ -975,8 +987,9 @@ __device__ __forceinline__ void far_list(const FastArgs &a, Smem &S, const Panel
         if (lane >= o) pos += x;
     }
     pos += wpos - weight;
-    const bool mine = n && pos >= pos0 && pos < end;
-    const int parts = mine ? (n + a.tcap - 1) / a.tcap : 0;
+    const int lo = share_cut(pos0 - pos, n), cnt = share_cut(end - pos, n) - lo;  // the share's tasks of the tile
+    const bool mine = cnt > 0;
+    const int parts = mine ? (cnt + a.tcap - 1) / a.tcap : 0;
     int at = parts;
     for (int o = 1; o < 32; o <<= 1) {
         const int x = __shfl_up_sync(0xffffffffu, at, o);
@@ -997,13 +1010,19 @@ __device__ __forceinline__ void far_list(const FastArgs &a, Smem &S, const Panel
     if (wid < used && mine) {
         const int js = e / pn.nB, K = (e - js * pn.nB) * NT + lane, split = js / pn.nb;
         uint32_t bits[kTaskWords] = {v.x, v.y, v.z, v.w};
+        int skip = lo, left = cnt;
+#pragma unroll
+        for (int x = 0; x < kTaskWords; x++)
+            for (; skip > 0 && bits[x]; skip--) bits[x] &= bits[x] - 1u;
         for (int p = 0, i = off + at - parts; p < parts; p++, i++) {  // at most tcap tasks each, lowest first
+            const int cap = min(a.tcap, left);
+            left -= cap;
             uint32_t out[kTaskWords];
             int m = 0;
 #pragma unroll
             for (int x = 0; x < kTaskWords; x++) {
                 uint32_t take = bits[x];
-                while (m + __popc(take) > a.tcap) take &= ~(1u << (31 - __clz(take)));
+                while (m + __popc(take) > cap) take &= ~(1u << (31 - __clz(take)));
                 m += __popc(take);
                 out[x] = take;
                 bits[x] &= ~take;
@@ -1142,7 +1161,7 @@ __device__ __forceinline__ void far_phase(const FastArgs &a, Smem &S, float *big
             *reinterpret_cast<uint4 *>(sruns + o) = make_uint4(kNoRuns, kNoRuns, kNoRuns, kNoRuns);
         }
     };
-    // the row that holds the share's start may have no tile starting in it: its segment is empty
+    // the rows that hold the share's start and end may give it no task: their segments are empty
     auto empty = [&](int j) {
         float *seg = seg_min(a, (int)blockIdx.x, j);
         for (int o = ct; o < nt * BJ; o += MAXCONS) __stcg(seg + o, CUDART_INF_F);
@@ -1255,6 +1274,10 @@ __device__ __forceinline__ void far_phase(const FastArgs &a, Smem &S, float *big
     __syncthreads();
     if (js >= 0) flush();
     else empty(js0);
+    const int last = min(((int)blockIdx.x + 1) * S.share, S.total) - 1;
+    int je = max(js, js0);
+    while (je + 1 < pn.nb * a.nsplit && S.jstart[je + 1] <= last) je++;
+    if (je > max(js, js0)) empty(je);
 }
 
 // ---------------------------------------------------------------- near phase
