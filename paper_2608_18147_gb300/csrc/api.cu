@@ -37,7 +37,7 @@ int launch_gather_q(const float *v, const int32_t *qidx, const int32_t *mcount, 
 int launch_locate_q(const float *v, int64_t p, const float *Q, int m, int32_t *a, DevStatus *ds, cudaStream_t st);
 size_t refine_ctx_bytes();
 int launch_refine_colour(const Prefix &P, const int32_t *a, int m, int colour, double lamp, int32_t *a_new,
-                         int32_t *moved, void *part_buf, int32_t *ctx, cudaStream_t st, int *nblocks_out);
+                         int32_t *moved, void *part_buf, int32_t *ctx, int num_sms, cudaStream_t st, int *nblocks_out);
 size_t refine_scratch_bytes(int64_t d);
 int launch_refine_commit(int32_t *a, const int32_t *a_new, const int32_t *moved, const double *ev, int m, bool guard,
                          double budget, int32_t *ctx, cudaStream_t st);
@@ -396,7 +396,7 @@ static int refine_device(void *ws, const Layout &L, const Prefix &P, std::vector
             ECASQ_CUDA_TRY(cudaMemcpyAsync(an, a, sizeof(int32_t) * m, cudaMemcpyDeviceToDevice, st));
             ECASQ_CUDA_TRY(cudaMemsetAsync(moved, 0, sizeof(int32_t), st));
             int nblk = 0;
-            rc = launch_refine_colour(P, a, m, col, lamp, an, moved, wsp<void>(ws, L.refine_part), ctx, st, &nblk);
+            rc = launch_refine_colour(P, a, m, col, lamp, an, moved, wsp<void>(ws, L.refine_part), ctx, num_sms(), st, &nblk);
             if (rc != ECASQ_OK) return rc;
             if (nblk == 0) continue;
             // only a step that moved a value is evaluated; the step is kept or dropped on the device

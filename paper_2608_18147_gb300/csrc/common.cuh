@@ -147,6 +147,13 @@ __device__ __forceinline__ dd dd_mul(dd a, dd b) {
 }
 __device__ __forceinline__ double dd_round(dd a) { return __dadd_rn(a.hi, a.lo); }
 
+// Binary64 values as integers of the same order (-0 as +0): compares of them stay off the binary64 pipe, which does two
+// a cycle and SM.
+__device__ __forceinline__ long long order_key(double x) {
+    const long long b = __double_as_longlong(x);
+    return b >= 0 ? b : b == (long long)0x8000000000000000ull ? 0 : b ^ 0x7fffffffffffffffll;
+}
+
 // h(y) = -y log2 y, h(0) = 0 (Sec. 4).
 __device__ __forceinline__ double hfun(double y) { return y > 0.0 ? -__dmul_rn(y, log2(y)) : 0.0; }
 

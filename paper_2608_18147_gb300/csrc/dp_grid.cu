@@ -74,13 +74,6 @@ __global__ void k_grid_round(GridArgs A, int i) {
     }
 }
 
-// Binary64 values as integers of the same order (-0 as +0): compares of them stay off the binary64 pipe, which does two
-// a cycle and SM.
-__device__ __forceinline__ long long order_key(double x) {
-    const long long b = __double_as_longlong(x);
-    return b >= 0 ? b : b == (long long)0x8000000000000000ull ? 0 : b ^ 0x7fffffffffffffffll;
-}
-
 // One block per output j (heavy outputs first), its threads splitting the k range, so
 // that no output's scan is a long serial walk of one warp (the last outputs have n - 1
 // candidates per multiplier, and each step of a walk waits on its loads from L2).  Nearly every output has one
