@@ -120,6 +120,7 @@ struct FastArgs {
     float *tmin1;          // near minima by tile [T(T+1)/2][G][s-2][64]
     int32_t *lists;        // [s+1][2][G ps]: needed outputs of layer i (g << 24 | j); 0: <= NMEM members, 1: more
     int *list_cnt;         // [s+1][2]
+    uint32_t thread_tiles; // bands of at most so many tiles are walked by a thread (k_need_layer)
     int32_t *wide;         // [G ps]: needed outputs of the layer being closed whose bands span more than
                            // kThreadTiles tiles (g << 24 | j), walked by a warp each (k_need_wide)
     int *wide_cnt;         // [s+1]
@@ -1784,7 +1785,9 @@ __device__ __forceinline__ int32_t *layer_list(const FastArgs &a, int i, int kin
 // list the needed outputs for the exact stage (inline members / big bands).  A thread
 // walks an output's band when it spans at most kThreadTiles tiles; wider bands go to
 // k_need_wide, a warp each (threads of one warp walking bands of very different widths
-// would wait on the widest).
+// would wait on the widest).  Where few outputs are needed and the costs are in a table, a warp walks every band:
+// its lanes read 32 k at once (d = 50001, s = 32: 11 us a layer with k_need_wide instead of 20).  With costs
+// to re-derive a tile is one chain for a thread or a warp; for all outputs, threads fill the chip.
 constexpr uint32_t kThreadTiles = 4;
 __global__ void k_need_layer(FastArgs a, int i) {
     if (*(volatile const int *)a.abort_flag) return;  // a wait gave up: the tables are not valid
@@ -1809,7 +1812,7 @@ __global__ void k_need_layer(FastArgs a, int i) {
                 } else {
                     const uint64_t w = a.band[o];
                     packed = (int32_t)((g << 24) | (int32_t)j);
-                    if (band_tiles(w) > kThreadTiles) {
+                    if (band_tiles(w) > a.thread_tiles) {
                         wide = true;  // a warp walks it (k_need_wide): lanes' walks would diverge
                     } else {
                         int32_t *mem = a.members + o * NMEM;
@@ -1853,7 +1856,7 @@ __global__ void __launch_bounds__(128) k_need_wide(FastArgs a, int i) {
     int32_t *lsmall = layer_list(a, i, 0), *lbig = layer_list(a, i, 1);
     int *csmall = a.list_cnt + 2 * i, *cbig = csmall + 1;
     unsigned long long nmem = 0, nbig = 0, nover = 0;  // lane 0
-    for (int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); e < n; e += warps) {
+    for (int e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < n; e += warps) {
         const int32_t v = a.wide[e];
         const int g = v >> 24;
         const int64_t j = v & 0xFFFFFF;
@@ -1952,12 +1955,16 @@ __device__ __forceinline__ void count_exact(const FastArgs &a, unsigned long lon
 
 // Layer i, outputs with at most NMEM members: one thread each, binary64 re-scoring
 // with double-double interval costs; the lowest k among exact minima wins.
+constexpr int kExactBlocks = 8;  // blocks of k_exact_small per SM
 __global__ void __launch_bounds__(128) k_exact_small(Prefix P, FastArgs a, int i, double *dp64, int32_t *bp) {
     if (*(volatile const int *)a.abort_flag) return;  // a wait gave up: the tables are not valid
-    // A warp takes 32 listed outputs at a time and evaluates their members flattened
-    // (member r of the 32 outputs' lists goes to lane r mod 32), so every lane of a
+    // A warp takes up to 32 listed outputs at a time and evaluates their members flattened
+    // (member r of the outputs' lists goes to lane r mod 32), so every lane of a
     // binary64 sequence does useful work; then each output's lane takes the least value,
     // lowest k on ties, over its own members (the per-output rule, which is order-free).
+    // A short list is dealt to one warp on every SM (a sequence is 3 us of an SM's binary64 pipe, and 32
+    // outputs a warp, four warps a block, put a few hundred outputs' on three SMs: 33 us a layer at
+    // d = 50001, s = 32, now 13).
     __shared__ double sval[4][32 * NMEM];
     __shared__ int32_t sk[4][32 * NMEM];
     const int n = a.list_cnt[2 * i];
@@ -1965,9 +1972,10 @@ __global__ void __launch_bounds__(128) k_exact_small(Prefix P, FastArgs a, int i
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned long long nres = 0;
     int nviol = 0;
-    const int wstride = gridDim.x * (blockDim.x >> 5) * 32;
-    for (int base = (blockIdx.x * (blockDim.x >> 5) + wid) * 32; base < n; base += wstride) {  // warp-uniform
-        const int e = base + lane;
+    const int nsm = gridDim.x / kExactBlocks, per = min(32, (n + nsm - 1) / nsm);
+    const int wstride = gridDim.x * (blockDim.x >> 5) * per;
+    for (int base = (wid * gridDim.x + blockIdx.x) * per; base < n; base += wstride) {  // warp-uniform
+        const int e = lane < per ? base + lane : n;
         int g = 0, cnt = 0;
         int64_t j = 0;
         long long o = 0;
@@ -2040,7 +2048,7 @@ __global__ void __launch_bounds__(128) k_exact_big(Prefix P, FastArgs a, int i, 
     const int warps = gridDim.x * (blockDim.x >> 5);
     unsigned long long nres = 0;
     int nviol = 0;
-    for (int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); e < n; e += warps) {
+    for (int e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < n; e += warps) {
         const int32_t v = list[e];
         const int g = v >> 24;
         const int64_t j = v & 0xFFFFFF;
@@ -2387,6 +2395,7 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
         a.costs = nullptr;
         a.tile_base = 0;
     }
+    a.thread_tiles = !exact_tables && !tables && a.costs ? 0 : kThreadTiles;
     const int ilo = exact_s ? s : 2;
     note_launch();
     k_need_init<<<(unsigned)std::min<int64_t>(cdiv((int64_t)G * (s + 1) * P.ps, 256), (int64_t)nsm * 32), 256, 0, st>>>(
@@ -2409,7 +2418,7 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     ECASQ_LAUNCH_CHECK();
     for (int i = 3; i <= s; i++) {
         note_launch();
-        k_exact_small<<<(unsigned)nsm * 8, 128, 0, st>>>(P, a, i, dp64, bp);
+        k_exact_small<<<(unsigned)nsm * kExactBlocks, 128, 0, st>>>(P, a, i, dp64, bp);
         ECASQ_LAUNCH_CHECK();
         note_launch();
         k_exact_big<<<(unsigned)nsm * 16, 128, 0, st>>>(P, a, i, dp64, bp);
