@@ -20,7 +20,7 @@
 //    (within the certified bound; bit-identically from the resident table), keeps the members k whose fp32 value lies within the
 //    band (up to 8 inline, the count either way) and marks (i-1, k) needed.
 //    With ECASQ_EXACT_TABLES every output is needed.
-// 3. k_exact_small / k_exact_big (layers 3 up to s, over the lists the need
+// 3. k_exact_layer (layers 3 up to s, over the lists the need
 //    stage wrote; k_fill_unneeded first): re-score the members of every needed
 //    output in binary64 with double-double interval costs (the reference
 //    formulas) and take the lowest k among exact minima: dp64, bp.  Outputs
@@ -120,7 +120,6 @@ struct FastArgs {
     float *tmin1;          // near minima by tile [T(T+1)/2][G][s-2][64]
     int32_t *lists;        // [s+1][2][G ps]: needed outputs of layer i (g << 24 | j); 0: <= NMEM members, 1: more
     int *list_cnt;         // [s+1][2]
-    uint32_t thread_tiles; // bands of at most so many tiles are walked by a thread (k_need_layer)
     int32_t *wide;         // [G ps]: needed outputs of the layer being closed whose bands span more than
                            // kThreadTiles tiles (g << 24 | j), walked by a warp each (k_need_wide)
     int *wide_cnt;         // [s+1]
@@ -1785,9 +1784,7 @@ __device__ __forceinline__ int32_t *layer_list(const FastArgs &a, int i, int kin
 // list the needed outputs for the exact stage (inline members / big bands).  A thread
 // walks an output's band when it spans at most kThreadTiles tiles; wider bands go to
 // k_need_wide, a warp each (threads of one warp walking bands of very different widths
-// would wait on the widest).  Where few outputs are needed and the costs are in a table, a warp walks every band:
-// its lanes read 32 k at once (d = 50001, s = 32: 11 us a layer with k_need_wide instead of 20).  With costs
-// to re-derive a tile is one chain for a thread or a warp; for all outputs, threads fill the chip.
+// would wait on the widest).  (Not in a pass that needs few outputs: k_need_wide<true>.)
 constexpr uint32_t kThreadTiles = 4;
 __global__ void k_need_layer(FastArgs a, int i) {
     if (*(volatile const int *)a.abort_flag) return;  // a wait gave up: the tables are not valid
@@ -1812,7 +1809,7 @@ __global__ void k_need_layer(FastArgs a, int i) {
                 } else {
                     const uint64_t w = a.band[o];
                     packed = (int32_t)((g << 24) | (int32_t)j);
-                    if (band_tiles(w) > a.thread_tiles) {
+                    if (band_tiles(w) > kThreadTiles) {
                         wide = true;  // a warp walks it (k_need_wide): lanes' walks would diverge
                     } else {
                         int32_t *mem = a.members + o * NMEM;
@@ -1826,7 +1823,7 @@ __global__ void k_need_layer(FastArgs a, int i) {
                             if (mark) below[k] = 1;
                             if (v < vmin || (v == vmin && (int32_t)k < kmin)) { vmin = v; kmin = (int32_t)k; }
                         });
-                        if (cnt > NMEM) mem[0] = kmin;  // a big output keeps its fp32 argmin (k_exact_big)
+                        if (cnt > NMEM) mem[0] = kmin;  // a big output keeps its fp32 argmin (exact_big)
                         a.mcnt[o] = cnt;
                         nmem += cnt;
                         nbig += cnt > NMEM;
@@ -1846,6 +1843,11 @@ __global__ void k_need_layer(FastArgs a, int i) {
 // The closure of layer i for the outputs k_need_layer deferred: a warp per output walks
 // its band (warp_visit_band), marks (i-1, k) needed for every member, keeps the first
 // NMEM members it meets (the exact stage's rule is order-free) and lists the output.
+// CHAIN: for all outputs of the layer, those k_need_init marked and those on the chain's list, to which the layer above
+// appended each output that it marked first; so a layer takes one launch and no pass over the marks (with
+// k_need_layer 11 us a layer at d = 50001, s = 32, and 20 where its threads walked the bands; now 6).
+__device__ __forceinline__ int32_t *chain_list(const FastArgs &a, int i) { return layer_list(a, i & 1, 0); }  // (layers 0, 1: free)
+template <bool CHAIN>
 __global__ void __launch_bounds__(128) k_need_wide(FastArgs a, int i) {
     if (*(volatile const int *)a.abort_flag) return;  // a wait gave up: the tables are not valid
     const int n = a.wide_cnt[i];
@@ -1856,25 +1858,38 @@ __global__ void __launch_bounds__(128) k_need_wide(FastArgs a, int i) {
     int32_t *lsmall = layer_list(a, i, 0), *lbig = layer_list(a, i, 1);
     int *csmall = a.list_cnt + 2 * i, *cbig = csmall + 1;
     unsigned long long nmem = 0, nbig = 0, nover = 0;  // lane 0
-    for (int e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < n; e += warps) {
-        const int32_t v = a.wide[e];
+    for (int e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < n + (CHAIN ? a.G : 0); e += warps) {
+        const int32_t v = !CHAIN ? a.wide[e] : e < n ? chain_list(a, i)[e] : (int32_t)((e - n) << 24 | (int)(a.p - 1));
         const int g = v >> 24;
         const int64_t j = v & 0xFFFFFF;
         const size_t o = oidx(a, g, i, j);
+        if (CHAIN && e >= n && !a.need[o]) continue;  // no member is ever p - 1: not on the list too
+        const float m32 = a.dp32[d32(a, g, i, j)];
+        if (CHAIN && !(m32 < CUDART_INF_F)) {
+            if (lane == 0) a.mcnt[o] = 0;
+            continue;
+        }
         const uint64_t w = a.band[o];
         int32_t *mem = a.members + o * NMEM;
         uint8_t *below = a.need + oidx(a, g, i - 1, 0);
         int cnt = 0;  // warp-uniform
         float vmin = CUDART_INF_F;  // per lane: its least member value, lowest k on ties
         int32_t kmin = INT32_MAX;
-        warp_visit_band(a, g, i, j, w, band_threshold(a, i, a.dp32[d32(a, g, i, j)]), [&](bool in, int64_t k, float v) {
+        warp_visit_band(a, g, i, j, w, band_threshold(a, i, m32), [&](bool in, int64_t k, float v) {
             const unsigned mask = __ballot_sync(0xffffffffu, in);
+            bool fresh = false;
             if (in) {
                 const int pos = cnt + __popc(mask & lt);
                 if (pos < NMEM) mem[pos] = (int32_t)k;
-                if (mark) below[k] = 1;
+                if (mark && CHAIN) {
+                    const size_t at = oidx(a, g, i - 1, k);
+                    const uint32_t bit = 1u << (8 * (at & 3));
+                    fresh = !(atomicOr(reinterpret_cast<uint32_t *>(a.need + (at & ~(size_t)3)), bit) & bit);
+                } else if (mark) below[k] = 1;
                 if (v < vmin || (v == vmin && (int32_t)k < kmin)) { vmin = v; kmin = (int32_t)k; }
             }
+            if (CHAIN && mark)
+                warp_append(0xffffffffu, fresh, (int32_t)((g << 24) | (int32_t)k), chain_list(a, i - 1), a.wide_cnt + i - 1);
             cnt += __popc(mask);
         });
 #pragma unroll
@@ -1885,7 +1900,7 @@ __global__ void __launch_bounds__(128) k_need_wide(FastArgs a, int i) {
         }
         __syncwarp();  // every lane's member stores are done before lane 0 overwrites slot 0
         if (lane == 0) {
-            if (cnt > NMEM) mem[0] = kmin;  // a big output keeps its fp32 argmin (k_exact_big)
+            if (cnt > NMEM) mem[0] = kmin;  // a big output keeps its fp32 argmin (exact_big)
             a.mcnt[o] = cnt;
             nmem += cnt;
             nbig += cnt > NMEM;
@@ -1955,9 +1970,9 @@ __device__ __forceinline__ void count_exact(const FastArgs &a, unsigned long lon
 
 // Layer i, outputs with at most NMEM members: one thread each, binary64 re-scoring
 // with double-double interval costs; the lowest k among exact minima wins.
-constexpr int kExactBlocks = 8;  // blocks of k_exact_small per SM
-__global__ void __launch_bounds__(128) k_exact_small(Prefix P, FastArgs a, int i, double *dp64, int32_t *bp) {
-    if (*(volatile const int *)a.abort_flag) return;  // a wait gave up: the tables are not valid
+constexpr int kExactBlocks = 8, kExactBigBlocks = 16;  // blocks per SM
+static __device__ __forceinline__ void exact_small(const Prefix &P, const FastArgs &a, int i, double *dp64, int32_t *bp, int block) {
+    const int blocks = gridDim.x / (kExactBlocks + kExactBigBlocks) * kExactBlocks;
     // A warp takes up to 32 listed outputs at a time and evaluates their members flattened
     // (member r of the outputs' lists goes to lane r mod 32), so every lane of a
     // binary64 sequence does useful work; then each output's lane takes the least value,
@@ -1972,9 +1987,9 @@ __global__ void __launch_bounds__(128) k_exact_small(Prefix P, FastArgs a, int i
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned long long nres = 0;
     int nviol = 0;
-    const int nsm = gridDim.x / kExactBlocks, per = min(32, (n + nsm - 1) / nsm);
-    const int wstride = gridDim.x * (blockDim.x >> 5) * per;
-    for (int base = (wid * gridDim.x + blockIdx.x) * per; base < n; base += wstride) {  // warp-uniform
+    const int nsm = blocks / kExactBlocks, per = min(32, (n + nsm - 1) / nsm);
+    const int wstride = blocks * (blockDim.x >> 5) * per;
+    for (int base = (wid * blocks + block) * per; base < n; base += wstride) {  // warp-uniform
         const int e = lane < per ? base + lane : n;
         int g = 0, cnt = 0;
         int64_t j = 0;
@@ -2037,18 +2052,18 @@ __global__ void __launch_bounds__(128) k_exact_small(Prefix P, FastArgs a, int i
 // met wait in the warp's queue, and each time it holds 32 every lane re-scores one of
 // them in binary64, so the binary64 sequence runs with all lanes busy (the result,
 // least value then lowest k, does not depend on the order).
-__global__ void __launch_bounds__(128) k_exact_big(Prefix P, FastArgs a, int i, double *dp64, int32_t *bp) {
-    if (*(volatile const int *)a.abort_flag) return;  // a wait gave up: the tables are not valid
+static __device__ __forceinline__ void exact_big(const Prefix &P, const FastArgs &a, int i, double *dp64, int32_t *bp, int block) {
+    const int blocks = gridDim.x / (kExactBlocks + kExactBigBlocks) * kExactBigBlocks;
     __shared__ int32_t queue[4][32];  // per warp: band members waiting for binary64 re-scoring
     const int n = a.list_cnt[2 * i + 1];
     const int32_t *list = layer_list(a, i, 1);
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     int32_t *qw = queue[threadIdx.x >> 5];
-    const int warps = gridDim.x * (blockDim.x >> 5);
+    const int warps = blocks * (blockDim.x >> 5);
     unsigned long long nres = 0;
     int nviol = 0;
-    for (int e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < n; e += warps) {
+    for (int e = (threadIdx.x >> 5) * blocks + block; e < n; e += warps) {
         const int32_t v = list[e];
         const int g = v >> 24;
         const int64_t j = v & 0xFFFFFF;
@@ -2108,6 +2123,14 @@ __global__ void __launch_bounds__(128) k_exact_big(Prefix P, FastArgs a, int i, 
         if (lane == 0) nviol += exact_store(a, g, i, j, best, arg, dp64, bp) ? 0 : 1;
     }
     count_exact(a, nres, nviol);
+}
+
+// Layer i: the first blocks take the outputs with more members, the others the rest (one launch a layer).
+__global__ void __launch_bounds__(128) k_exact_layer(Prefix P, FastArgs a, int i, double *dp64, int32_t *bp) {
+    if (*(volatile const int *)a.abort_flag) return;  // a wait gave up: the tables are not valid
+    const int big = gridDim.x / (kExactBlocks + kExactBigBlocks) * kExactBigBlocks;
+    if ((int)blockIdx.x < big) exact_big(P, a, i, dp64, bp, (int)blockIdx.x);
+    else exact_small(P, a, i, dp64, bp, (int)blockIdx.x - big);
 }
 
 // ------------------------------------------------------------------ host
@@ -2395,7 +2418,6 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
         a.costs = nullptr;
         a.tile_base = 0;
     }
-    a.thread_tiles = !exact_tables && !tables && a.costs ? 0 : kThreadTiles;
     const int ilo = exact_s ? s : 2;
     note_launch();
     k_need_init<<<(unsigned)std::min<int64_t>(cdiv((int64_t)G * (s + 1) * P.ps, 256), (int64_t)nsm * 32), 256, 0, st>>>(
@@ -2405,11 +2427,16 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     ECASQ_CUDA_TRY(cudaMemsetAsync(a.wide_cnt, 0, sizeof(int) * (size_t)(s + 1), st));
     const unsigned gl = (unsigned)std::min<int64_t>(cdiv((int64_t)G * P.p, 128), (int64_t)nsm * 64);
     for (int i = s; i >= 3; i--) {
-        note_launch();
-        k_need_layer<<<gl, 128, 0, st>>>(a, i);
-        ECASQ_LAUNCH_CHECK();
-        note_launch();
-        k_need_wide<<<(unsigned)nsm * 16, 128, 0, st>>>(a, i);
+        if (exact_tables || tables) {
+            note_launch();
+            k_need_layer<<<gl, 128, 0, st>>>(a, i);
+            ECASQ_LAUNCH_CHECK();
+            note_launch();
+            k_need_wide<false><<<(unsigned)nsm * 16, 128, 0, st>>>(a, i);
+        } else {
+            note_launch();
+            k_need_wide<true><<<(unsigned)nsm * 16, 128, 0, st>>>(a, i);
+        }
         ECASQ_LAUNCH_CHECK();
     }
     note_launch();
@@ -2418,10 +2445,7 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     ECASQ_LAUNCH_CHECK();
     for (int i = 3; i <= s; i++) {
         note_launch();
-        k_exact_small<<<(unsigned)nsm * kExactBlocks, 128, 0, st>>>(P, a, i, dp64, bp);
-        ECASQ_LAUNCH_CHECK();
-        note_launch();
-        k_exact_big<<<(unsigned)nsm * 16, 128, 0, st>>>(P, a, i, dp64, bp);
+        k_exact_layer<<<(unsigned)nsm * (kExactBlocks + kExactBigBlocks), 128, 0, st>>>(P, a, i, dp64, bp);
         ECASQ_LAUNCH_CHECK();
     }
     return ECASQ_OK;
