@@ -51,11 +51,10 @@ SM_MAX_MHZ = 2070.0
 # (add + FMA + min = 3) includes is 1/(s-2) of an op per candidate here.
 OPS_PER_CANDIDATE = 2
 BK = BJ = 64              # the kernel's tile: 64 k by 64 columns
-# DRAM bytes of the min-plus kernel per interval-cost tile it copies in (64 x 64 pairs,
-# 34 816 B of C and Phi, plus the dp32 rows and minima that miss L2), from the committed
-# ncu capture of every launch of one solve at d = 16384; the benchmark launch is scaled
-# by the tiles it fetched (tile skipping leaves most tiles in HBM unread).
-TRAFFIC_PER_FETCHED_TILE = (6115167744 + 34815232) / 172545  # 6 launches of one solve: read + write / tiles
+# DRAM bytes of the min-plus kernel per interval-cost tile it copies in: the tile's 34 816 B of C
+# and Phi, each fetched tile read once in a pass.  (A capture of one solve at d = 16384 reads less in
+# late passes, whose tiles stay in L2; at d = 131072 a pass fetches 26 GB.)
+TRAFFIC_PER_FETCHED_TILE = 34816
 ORACLE_SAMPLE = 16384     # entries of the CPU baseline's bounded sample
 
 
@@ -632,8 +631,7 @@ def main():
                if (flags & E.RESIDENT_COSTS) and TRAFFIC_PER_FETCHED_TILE else None)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TOP/s",
                 "frac": (achieved / peak) if achieved else None, "traffic": traffic,
-                "traffic_note": "DRAM bytes per launch: bytes per fetched cost tile from an ncu capture at "
-                                "d = 16384, times the tiles this launch fetched",
+                "traffic_note": "DRAM bytes per launch: the bytes of a cost tile times the tiles this launch fetched",
                 "tiles_fetched_per_launch": fetched_per_launch,
                 "kernel": "k_wavefront",
                 "peak_basis": "%d SMs (device attribute) x 128 FP32-pipe lanes (adds and mins share the issue "
@@ -649,8 +647,8 @@ def main():
                 "effective_note": "algorithmic rate: 2 ops for every candidate of eq. apx_rec (all layers, "
                                   "multipliers, k < j), including the ones the exact tile skip never evaluates",
                 "executed_unit_frac": run_frac,
-                "executed_note": "off-diagonal (warp, tile) units evaluated; the rest were skipped by an exact "
-                                 "lower bound that proves they cannot change any minimum or band"}
+                "executed_note": "off-diagonal (multiplier, tile) units of s-2 layer tasks evaluated; the other tasks were "
+                                 "skipped by an exact lower bound that proves they cannot change any minimum or band"}
     if achieved and clocks.get("sm_mhz"):
         roofline["frac_at_measured_clock"] = achieved / (n_sm * FP32_LANES * clocks["sm_mhz"] * 1e6 / 1e12)
 
