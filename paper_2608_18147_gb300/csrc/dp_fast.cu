@@ -347,7 +347,8 @@ struct __align__(16) Smem {
     uint16_t tdiv[32 * kTaskWords];       // ... li | gl << 8 of task t
     int2 lwords[MAXCONS / 32];
     int lnext, lpos, lcount, lmore;
-    uint32_t tinfo[4][64];                // ... entry i's tasks at i % 4: t | li << 8 | gl << 16 in row order
+    __align__(16) uint32_t tinfo[4][64];  // ... entry i's tasks at i % 4: t | li << 8 | gl << 16 in row order
+    __align__(16) float tlam[4][64];      // ... and their multipliers
     uint16_t okey[256];                   // ... K of a segment's tiles by ordinal (runs_add)
     int ok;                               // grid_sync's answer
     unsigned long long full[3];           // ... copies of tile buffer b
@@ -559,9 +560,9 @@ __global__ void __launch_bounds__(NPROD) k_build_costs(const __grid_constant__ F
 // tile and diagonal, every layer, 22 000 cycles at s = 16) the critical path and left the SMs
 // unevenly loaded; here 15 blocks cost a few barriers and s - 2 gather/compute steps, and the
 // far tiles are shared evenly.  A pass of 8 multipliers (mean over a budgeted search, resident
-// costs): 25.1 ms instead of 46.3 at d = 2^17, s = 16; 1.55 instead of 2.93 at d = 16384, s = 16;
-// 14.7 instead of 47.7 at d = 50001, s = 32; building its own costs, 2.5 instead of 8.4 at
-// d = 12289, s = 16.  Of the 25.1 ms about 13.5 are far tiles, 2.5 uneven shares, 5 masks, 2.5
+// costs): 22.5 ms instead of 46.3 at d = 2^17, s = 16; 1.47 instead of 2.93 at d = 16384, s = 16;
+// 12.9 instead of 47.7 at d = 50001, s = 32; building its own costs, 2.4 instead of 8.4 at
+// d = 12289, s = 16.  Of the 22.5 ms about 10.5 are far tiles, 2.5 uneven shares, 5 masks, 2.5
 // bounds and 3 the near phases; far tiles are bound by issue (one add and one min a candidate
 // on the two FP32 pipes reach about 53 candidates per cycle and SM) and by the copies and
 // barriers of a tile, which cost as much as about 6 of its tasks (kTileCost).
@@ -714,8 +715,8 @@ __device__ __forceinline__ float4 far_start(const FastArgs &a, const int *u, int
 // multiplier that needs it at d = 2^17, s = 16, so tasks, not whole tiles, are the unit of work.
 // CTAs split the (column block, word range) pairs as in bound_phase; a thread tests one column of one
 // multiplier, kBoundL layers at a time.
-constexpr int kTileCost = 6;  // a listed tile's fixed cost (its copies, its costs into registers) in tasks (a pass at d = 2^17, s = 16: 25.1 ms
-                               // with 6, 25.7 with 4 or 8, 26.6 with 12)
+constexpr int kTileCost = 6;  // a listed tile's fixed cost (its copies, its costs into registers) in tasks (a pass at d = 2^17, s = 16: 22.5 ms
+                               // with 6, 23.9 with 3, 23.0 with 9)
 static __device__ __noinline__ void mask_phase(const FastArgs &a, Smem &S, float *stage, const Panel &pn,
                                                uint64_t policy, uint32_t &ns) {
     const int L = a.s - 2, ct = threadIdx.x, lane = ct & 31, wid = ct >> 5, jl = ct & (BJ - 1), gq = ct / BJ;
@@ -1075,6 +1076,7 @@ __device__ __forceinline__ void far_issue(const FastArgs &a, Smem &S, float *big
         row += __popc(mine & ((1u << lane) - 1u));
         const uint32_t d = S.tdiv[t];  // li | gl << 8
         S.tinfo[slot][row] = (uint32_t)t | d << 8;
+        S.tlam[slot][row] = S.lam32[gs + (int)(d >> 8)];
         bulk_g2s_nohint(buf + kCostTileFloats + row * BK,
                         a.dp32 + d32(a, gs + (int)(d >> 8), 2 + (int)(d & 0xFFu), (int64_t)K * BK),
                         (uint32_t)(BK * sizeof(float)), &S.full[b]);
@@ -1215,48 +1217,46 @@ __device__ __forceinline__ void far_phase(const FastArgs &a, Smem &S, float *big
                 C[x] = *reinterpret_cast<const float4 *>(buf + col * PSTR + 8 * slice + 4 * x);
                 F[x] = *reinterpret_cast<const float4 *>(buf + kCostHalfFloats + col * PSTR + 8 * slice + 4 * x);
             }
-            const int g0 = (js / pn.nb) * a.Gc;
-            float2 W[4];
-            int gcur = -1;
             for (int k0 = 0; k0 < n; k0 += kBatch, batch++) {
                 int *pt = part + (int)(batch & 1u) * kBatch * 8 * BJ;
+                // The tasks' multipliers come at once, and four tasks run as one block without a branch: the time of a tile
+                // is the latency of such chains (a branch where the multiplier changes and the multiplier's loads in
+                // every task's chain: 25.1 ms a pass at d = 2^17; the loads at once 23.5; now 22.5).  Tasks past
+                // the entry's last leave slots that nothing reads.
 #pragma unroll
-                for (int y = 0; y < kBatch; y++) {
-                    if (k0 + y < n) {
-                        const int gl = (int)(S.tinfo[slot][k0 + y] >> 16);
-                        const float4 p = *reinterpret_cast<const float4 *>(rows + (k0 + y) * BK);
-                        const float4 q = *reinterpret_cast<const float4 *>(rows + (k0 + y) * BK + 4);
-                        if (gl != gcur) {
-                            gcur = gl;
-                            const float lam = S.lam32[g0 + gl];
-                            const float2 lam2 = make_float2(lam, lam);
+                for (int h = 0; h < kBatch; h += 4) {
+                    if (k0 + h >= n) break;
+                    const float4 l4 = *reinterpret_cast<const float4 *>(&S.tlam[slot][k0 + h]);
+                    const float lm[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
-                            for (int x = 0; x < 2; x++) {
-                                W[2 * x] = fma2(lam2, make_float2(F[x].x, F[x].y), make_float2(C[x].x, C[x].y));
-                                W[2 * x + 1] = fma2(lam2, make_float2(F[x].z, F[x].w), make_float2(C[x].z, C[x].w));
-                            }
-                        }
+                    for (int y = 0; y < 4; y++) {
+                        const float4 p = *reinterpret_cast<const float4 *>(rows + (k0 + h + y) * BK);
+                        const float4 q = *reinterpret_cast<const float4 *>(rows + (k0 + h + y) * BK + 4);
+                        const float2 lam2 = make_float2(lm[y], lm[y]);
                         // candidates are >= +0, so their bits order like the values: integer mins
-                        const float2 v0 = add2(make_float2(p.x, p.y), W[0]), v1 = add2(make_float2(p.z, p.w), W[1]);
-                        const float2 v2 = add2(make_float2(q.x, q.y), W[2]), v3 = add2(make_float2(q.z, q.w), W[3]);
+                        const float2 v0 = add2(make_float2(p.x, p.y), fma2(lam2, make_float2(F[0].x, F[0].y), make_float2(C[0].x, C[0].y)));
+                        const float2 v1 = add2(make_float2(p.z, p.w), fma2(lam2, make_float2(F[0].z, F[0].w), make_float2(C[0].z, C[0].w)));
+                        const float2 v2 = add2(make_float2(q.x, q.y), fma2(lam2, make_float2(F[1].x, F[1].y), make_float2(C[1].x, C[1].y)));
+                        const float2 v3 = add2(make_float2(q.z, q.w), fma2(lam2, make_float2(F[1].z, F[1].w), make_float2(C[1].z, C[1].w)));
                         const int x0 = min(min(__float_as_int(v0.x), __float_as_int(v0.y)), __float_as_int(v1.x));
                         const int x1 = min(min(__float_as_int(v2.x), __float_as_int(v2.y)), __float_as_int(v3.x));
-                        pt[(y * 8 + slice) * BJ + col] = min(min(x0, x1), min(__float_as_int(v1.y), __float_as_int(v3.y)));
+                        pt[((h + y) * 8 + slice) * BJ + col] = min(min(x0, x1), min(__float_as_int(v1.y), __float_as_int(v3.y)));
                     }
                 }
+                // (what the fold needs of its task, before the barrier)
+                const int k = k0 + slice;
+                const uint32_t f = k < n ? S.tinfo[slot][k] : 0u;
+                const float tau = S.tau[3 + ((f >> 8) & 0xFFu)];
                 __syncthreads();  // the batch's partial minima are complete
                 // (the last batch: the tile's buffer is free, for the entry kFarBufs further on)
                 if (k0 + kBatch >= n && i + kFarBufs < count && ((wid - 5 * i) & 15) < 5)
                     far_issue(a, S, big, pn, i + kFarBufs, (i + kFarBufs) & 3, b, (wid - 5 * i) & 15, policy);
-                const int k = k0 + slice;
                 if (k < n) {
-                    const uint32_t f = S.tinfo[slot][k];
                     const int *pk = pt + slice * 8 * BJ + col;
                     int v = pk[0];
 #pragma unroll
                     for (int x = 1; x < 8; x++) v = min(v, pk[x * BJ]);
                     const int o = (int)(f & 0xFFu) * BJ + col;
-                    const float tau = S.tau[3 + ((f >> 8) & 0xFFu)];
                     const float bb = sbest[o], T = __fmul_rn(bb, tau);
                     // a tile's minimum below bb - bb tau restarts the band, up to bb + bb tau joins it
                     // (band limits: the tests on the bits hold for bb = +inf too)
