@@ -126,8 +126,8 @@ size_t make_layout(int64_t d, int32_t s, int64_t rows, Layout *L) {
 }
 
 // Only what the sort, histogram and prefix sums use (ecasq_prepare): the regions of
-// make_layout up to the scan partials, then a 32 (d+1)-byte scratch in place of the
-// DP tables (the fp64 sums before their double-double split).
+// make_layout up to the scan partials, then 32 (d+1) bytes in place of the DP tables (free now: the size
+// stays what callers know).
 static size_t make_prep_layout(int64_t d, Layout *L) {
     memset(L, 0, sizeof(*L));
     size_t off = 0;

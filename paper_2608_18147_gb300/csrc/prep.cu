@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(256) k_radix_scatter(const uint32_t *__restric
 // with values 10^-24 of the largest) they are exact integers in units of the smallest last place, 128 bits
 // for x and 256 for x^2, rounded once to a double-double: the chip has 2 binary64 operations a cycle and SM, and
 // a double-double sum per key in two passes and their block scans took 863 of a preparation's 1240 us at
-// d = 4 million (220 now).  A sum that 106 bits hold has the same bits either way.  Else they are
+// d = 4 million (169 now).  A sum that 106 bits hold has the same bits either way.  Else they are
 // double-double sums in one fixed order.
 template <typename T>
 __device__ __forceinline__ T shfl_up(T v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
@@ -457,6 +457,80 @@ __device__ __forceinline__ void hist_thread_fill(const Sum &sum, const uint32_t 
     }
 }
 
+// Pass C of a whole tile of kHistTile keys by exact sums: a warp takes 512 consecutive keys, 32 at a time, a lane
+// one, so that neighbouring heads' results are neighbouring stores.  (Sixteen consecutive keys a thread wrote
+// every value to a sector of its own: 186 us at 4 million values, now 136.)  Integer sums do not depend on
+// their order, so the results are hist_thread_fill's.
+__device__ __forceinline__ void hist_tile_fill(const SumInt &sum, const uint32_t *keys, int64_t d, const IntSums &before,
+                                               HistPart *wtot, float *v, int64_t *N, double *S, double *S2, int64_t lo_off,
+                                               int64_t *p_out, double *norm2_out) {
+    constexpr int kPerWarp = kHistTile / 8;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * kHistTile + wid * kPerWarp;
+    IntSums t = sum.zero();
+#pragma unroll 4
+    for (int e = 0; e < kPerWarp; e += 32) {
+        const int64_t i = base + e + lane;
+        if (i >= d) continue;
+        const uint32_t k = keys[i];
+        sum.add_key(t, k);
+        t.h += (i == 0 || k != keys[i - 1]) ? 1 : 0;
+    }
+    for (int o = 16; o; o >>= 1) {
+        IntSums x;
+#pragma unroll
+        for (int r = 0; r < 2; r++) x.s[r] = __shfl_xor_sync(full, t.s[r], o);
+#pragma unroll
+        for (int r = 0; r < 4; r++) x.q[r] = __shfl_xor_sync(full, t.q[r], o);
+        x.h = __shfl_xor_sync(full, t.h, o);
+        t = sum.add(t, x);
+    }
+    if (lane == 0) wtot[wid].i = t;
+    __syncthreads();
+    IntSums run = before;  // the sums before the warp's next 32 keys
+    for (int w = 0; w < wid; w++) run = sum.add(run, wtot[w].i);
+#pragma unroll 1
+    for (int e = 0; e < kPerWarp; e += 32) {
+        const int64_t i = base + e + lane;
+        if (base + e >= d) break;  // warp-uniform
+        const uint32_t k = i < d ? keys[i] : 0u;
+        const bool head = i < d && (i == 0 || k != keys[i - 1]);
+        const unsigned heads = __ballot_sync(full, head);
+        IntSums x = sum.zero();
+        if (i < d) sum.add_key(x, k);
+        IntSums incl = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const IntSums y = sum.shfl_up(incl, o);
+            if (lane >= o) incl = sum.add(y, incl);
+        }
+        incl = sum.add(run, incl);
+        if (head) {
+            const IntSums at = sum.sub(incl, x);
+            const int64_t u = run.h + __popc(heads & ((1u << lane) - 1u));
+            const dd ss = sum.s_of(at), qq = sum.q_of(at);
+            v[u] = key2f(k);
+            N[u] = i;
+            S[u] = ss.hi; S[lo_off + u] = ss.lo;
+            S2[u] = qq.hi; S2[lo_off + u] = qq.lo;
+        }
+        const int64_t h = run.h + __popc(heads);
+        if (i == d - 1) {
+            const dd ss = sum.s_of(incl), qq = sum.q_of(incl);
+            N[h] = d;
+            S[h] = ss.hi; S[lo_off + h] = ss.lo;
+            S2[h] = qq.hi; S2[lo_off + h] = qq.lo;
+            *p_out = h;
+            *norm2_out = qq.hi;
+        }
+#pragma unroll
+        for (int r = 0; r < 2; r++) run.s[r] = __shfl_sync(full, incl.s[r], 31);
+#pragma unroll
+        for (int r = 0; r < 4; r++) run.q[r] = __shfl_sync(full, incl.q[r], 31);
+        run.h = h;
+    }
+}
+
 // f(sum) with the data set's way of summing.
 template <typename F>
 __device__ __forceinline__ void with_sums(UlpRange r, int64_t d, F &&f) {
@@ -491,6 +565,7 @@ __global__ void __launch_bounds__(256) k_hist_scan_partials(HistPart *part, int6
         for (int64_t b = lo; b < hi; b++) s = sum.add(s, part_of(part[b], sum));
         auto total = s;
         part_of(incl_all[threadIdx.x], sum) = block_scan_incl(sum, s, wtot, total);
+        if (threadIdx.x == 0) st->p = total.h;
         __syncthreads();
         auto acc = threadIdx.x > 0 ? part_of(incl_all[threadIdx.x - 1], sum) : sum.zero();
         for (int64_t b = lo; b < hi; b++) {
@@ -503,34 +578,32 @@ __global__ void __launch_bounds__(256) k_hist_scan_partials(HistPart *part, int6
 
 // Pass C: per sorted position i that starts a run of equal keys (a head), the
 // unique index u and v[u], N[u] = i, S[u], S2[u] (exclusive prefix sums).
-// The last position also writes N[p] = d, S[p], S2[p], p and ||X||^2.
+// The last position also writes N[p] = d, S[p], S2[p] and ||X||^2.  S and S2 hold hi[0..p], then lo[0..p].
 __global__ void __launch_bounds__(256) k_hist_fill(const uint32_t *__restrict__ keys, int64_t d, HistPart *part,
-                                                   float *v, int64_t *N, double *S, double *S2, DevStatus *st,
-                                                   int64_t pcap) {
+                                                   float *v, int64_t *N, double *S, double *S2, DevStatus *st) {
     __shared__ HistPart wtot[8];
     const int64_t base = (int64_t)blockIdx.x * kHistTile + (int64_t)threadIdx.x * kHistPer;
-    with_sums(*ulp_range(st), d, [&](auto sum) {
+    const int64_t lo_off = *(volatile int64_t *)&st->p + 1;  // the number of unique values: k_hist_scan_partials
+    int64_t p;  // (the same again)
+    const int B = exact_window(*ulp_range(st), d);
+    if (B < kNoWindow) {
+        hist_tile_fill(SumInt{B}, keys, d, part[blockIdx.x].i, wtot, v, N, S, S2, lo_off, &p, &st->norm2);
+        return;
+    }
+    {
+        const SumDD sum;
         const auto loc = hist_thread_sums(sum, keys, d, base);
         auto tot = loc;
         const auto incl = block_scan_incl(sum, loc, wtot, tot);
         // exclusive prefix before this thread's first element
         const auto run = sum.add(part_of(part[blockIdx.x], sum), sum.sub(incl, loc));
-        hist_thread_fill(sum, keys, d, base, run, v, N, S, S2, pcap + 1, &st->p, &st->norm2);
-    });
+        hist_thread_fill(sum, keys, d, base, run, v, N, S, S2, lo_off, &p, &st->norm2);
+    }
 }
 
-// The arrays were written with lo parts at offset pcap+1 (pcap = d); repack
-// them to offset p+1 so that every later kernel indexes (hi[0..p], lo[0..p]).
-__global__ void k_hist_finish(int64_t *N, int64_t *w, double *S, double *S2, const DevStatus *st, int64_t pcap,
-                              double *Sp, double *S2p) {
-    int64_t p = st->p;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; i <= p; i += stride) {
-        if (i < p) w[i] = N[i + 1] - N[i];
-        Sp[i] = S[i]; Sp[p + 1 + i] = S[pcap + 1 + i];
-        S2p[i] = S2[i]; S2p[p + 1 + i] = S2[pcap + 1 + i];
-    }
+__global__ void k_hist_weights(const int64_t *N, int64_t *w, const DevStatus *st) {
+    const int64_t p = st->p, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += stride) w[i] = N[i + 1] - N[i];
 }
 
 // ------------------------------------------------------------ short rows
@@ -693,21 +766,17 @@ int prepare_device(const float *x, int64_t d, void *ws, const Layout &L, cudaStr
     // a == k0 holds the sorted keys
     int64_t nbs = cdiv(d, kHistTile);  // the layout holds cdiv(d, kScanTile) >= nbs partials
     HistPart *part = wsp<HistPart>(ws, L.part);
-    // scratch copies of N/S/S2 with lo parts at offset d+1 live in keys1 / dp area
-    double *Stmp = wsp<double>(ws, L.dp64);
-    double *S2tmp = Stmp + 2 * (d + 1);
     note_launch();
     k_hist_partials<<<(unsigned)nbs, 256, 0, stream>>>(a, d, part, st);
     note_launch();
     k_hist_scan_partials<<<1, 256, 0, stream>>>(part, nbs, d, st);
     note_launch();
-    k_hist_fill<<<(unsigned)nbs, 256, 0, stream>>>(a, d, part, wsp<float>(ws, L.v), wsp<int64_t>(ws, L.N), Stmp,
-                                                 S2tmp, st, d);
+    k_hist_fill<<<(unsigned)nbs, 256, 0, stream>>>(a, d, part, wsp<float>(ws, L.v), wsp<int64_t>(ws, L.N),
+                                                 wsp<double>(ws, L.S), wsp<double>(ws, L.S2), st);
     ECASQ_LAUNCH_CHECK();
     note_launch();
-    k_hist_finish<<<(unsigned)std::min<int64_t>(cdiv(d + 1, 256), 4096), 256, 0, stream>>>(
-        wsp<int64_t>(ws, L.N), wsp<int64_t>(ws, L.w), Stmp, S2tmp, st, d, wsp<double>(ws, L.S),
-        wsp<double>(ws, L.S2));
+    k_hist_weights<<<(unsigned)std::min<int64_t>(cdiv(d + 1, 256), 4096), 256, 0, stream>>>(
+        wsp<int64_t>(ws, L.N), wsp<int64_t>(ws, L.w), st);
     ECASQ_LAUNCH_CHECK();
     DevStatus h;
     ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, st, sizeof(DevStatus), cudaMemcpyDeviceToHost, stream));
