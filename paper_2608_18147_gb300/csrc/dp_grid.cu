@@ -78,9 +78,10 @@ __global__ void k_grid_round(GridArgs A, int i) {
 // that no output's scan is a long serial walk of one warp (the last outputs have n - 1
 // candidates per multiplier, and each step of a walk waits on its loads from L2).  Nearly every output has one
 // member per multiplier: its thread writes it as it is, and only warps that hold several reduce them, by integer keys
-// (a reduction of all lanes with binary64 compares was most of a layer's 29 us at n = 1000; now 20).
-constexpr int kGridThreads = 256;
-__global__ void __launch_bounds__(kGridThreads, 3) k_grid_layer(GridArgs A, int i) {
+// (a reduction of all lanes with binary64 compares was most of a layer's 29 us at n = 1000, then 20).  128 threads, six blocks an SM: a layer
+// is blocks' latency in waves (256 threads 20 us at n = 1000, 64 20, 32 34; now 14; the same order up to n = 12000).
+constexpr int kGridThreads = 128;
+__global__ void __launch_bounds__(kGridThreads, 6) k_grid_layer(GridArgs A, int i) {
     __shared__ float sm[kGridThreads / 32][kMaxG];
     __shared__ double sb[kGridThreads / 32][kMaxG];
     __shared__ int32_t sa[kGridThreads / 32][kMaxG];
