@@ -55,7 +55,7 @@ __device__ __forceinline__ double local_obj(const Prefix &P, const Nbr &n, int64
     return __dadd_rn(__dadd_rn(C1, C2), __dmul_rn(lamp, ent));
 }
 
-constexpr int kRefineChunk = 256;   // candidates per block: one per thread, so a value's range spreads over many SMs
+constexpr int kRefineChunk = 256;   // candidates per block, at most, one per thread (chunk_of)
 
 struct RefPart { double v; int64_t i; };
 constexpr int kRefineValues = kMaxS / 3 + 1;  // values of one colour class, at most
@@ -149,22 +149,22 @@ __global__ void __launch_bounds__(32) k_refine_bound(Prefix P, const int32_t *a,
 //    1.45 times that, __log2f errs by 2^-22 for y in [1/2, 2] and 2 ulp below, so three of them are within 2^-18, and the
 //    products with lambda' and the sums within 2^-22 of their terms.
 // What bounded it: 87 000 candidates a step at p = 131072, m = 16 at some 800 binary64 instructions each (2 a
-// cycle and SM): 105 us; about one in a hundred is left to evaluate, and bound and scan take 60.  Without
-// the screening (SCREEN false) every candidate is evaluated and the current position's goes to curval: 37 us
-// while a block per SM takes them all, against 42 for bound and scan (p = 1024), so that is where the line is.
-template <bool SCREEN>
-__global__ void __launch_bounds__(kRefineChunk) k_refine_chunks(Prefix P, const int32_t *a, int m, int colour, double lamp,
+// cycle and SM): 105 us; about one in a hundred is left to evaluate, and bound and scan take 51.  Without
+// the screening (SCREEN false) every candidate is evaluated and the current position's goes to curval: 22 us at
+// p = 1024 with blocks of 32 (38 with 256: eight sequences on one SM), against 42 for bound and scan.
+template <int CHUNK, bool SCREEN>
+__global__ void __launch_bounds__(CHUNK) k_refine_chunks(Prefix P, const int32_t *a, int m, int colour, double lamp,
                                                                 const RefineScan *scan, double *curval, RefPart *part,
                                                                 int nchunk, const int32_t *ctx) {
-    __shared__ int list[kRefineChunk];
+    __shared__ int list[CHUNK];
     __shared__ Nbr nb;
     __shared__ int count;
-    __shared__ double rv[kRefineChunk / 32];
-    __shared__ int64_t ri[kRefineChunk / 32];
+    __shared__ double rv[CHUNK / 32];
+    __shared__ int64_t ri[CHUNK / 32];
     const int l = (colour == 0 ? 3 : colour) + 3 * blockIdx.y;
     if (l > m - 2) return;
-    const int64_t lo = (int64_t)a[l - 1] + 1 + (int64_t)blockIdx.x * kRefineChunk;
-    const int64_t hi = min((int64_t)a[l + 1], lo + kRefineChunk);
+    const int64_t lo = (int64_t)a[l - 1] + 1 + (int64_t)blockIdx.x * CHUNK;
+    const int64_t hi = min((int64_t)a[l + 1], lo + CHUNK);
     if (lo >= hi || context_unchanged(a, m, l, ctx)) return;  // uniform over the block
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const RefineScan &q = scan[blockIdx.y];
@@ -235,26 +235,35 @@ __global__ void __launch_bounds__(kRefineChunk) k_refine_chunks(Prefix P, const 
     }
 }
 
-// One warp per moved value: best over the chunks (lowest index among equal
+// One block per moved value: best over the chunks (lowest index among equal
 // values), then keep the current position unless the best is strictly lower.
-__global__ void k_refine_pick(const int32_t *a, int m, int colour, const RefPart *part, const double *curval,
-                              int nchunk, int32_t *a_new, int32_t *moved, int32_t *ctx) {
+constexpr int kPickThreads = 256;
+__global__ void __launch_bounds__(kPickThreads) k_refine_pick(const int32_t *a, int m, int colour, const RefPart *part, const double *curval,
+                              int nchunk, int chunk, int32_t *a_new, int32_t *moved, int32_t *ctx) {
     int l0 = colour == 0 ? 3 : colour;
     int l = l0 + 3 * blockIdx.x;
     if (l > m - 2) return;
     if (context_unchanged(a, m, l, ctx)) return;  // a_new[l] == a[l] already
     int64_t range = (int64_t)a[l + 1] - (int64_t)a[l - 1] - 1;
-    int nc = (int)cdiv(range, kRefineChunk);
+    int nc = (int)cdiv(range, chunk);
+    __shared__ double rv[kPickThreads / 32];
+    __shared__ int64_t ri[kPickThreads / 32];
     double bv = CUDART_INF;
-    int64_t bi = -1;
-    for (int c = threadIdx.x; c < nc; c += 32) {
-        RefPart q = part[(size_t)blockIdx.x * nchunk + c];
-        if (q.i >= 0 && (q.v < bv || (q.v == bv && q.i < bi))) { bv = q.v; bi = q.i; }
+    int64_t bi = INT64_MAX;
+    auto meet = [&](double v2, int64_t i2) {  // binary64 compares as integers (order_key)
+        const long long k2 = order_key(v2), k = order_key(bv);
+        if (i2 >= 0 && (k2 < k || (k2 == k && i2 < bi))) { bv = v2; bi = i2; }
+    };
+    for (int c = threadIdx.x; c < nc; c += kPickThreads) {
+        const RefPart q = part[(size_t)blockIdx.x * nchunk + c];
+        meet(q.v, q.i);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        double v2 = __shfl_down_sync(0xffffffffu, bv, o);
-        int64_t i2 = __shfl_down_sync(0xffffffffu, bi, o);
-        if (i2 >= 0 && (bi < 0 || v2 < bv || (v2 == bv && i2 < bi))) { bv = v2; bi = i2; }
+    for (int o = 16; o > 0; o >>= 1) meet(__shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bi, o));
+    if ((threadIdx.x & 31) == 0) { rv[threadIdx.x >> 5] = bv; ri[threadIdx.x >> 5] = bi; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kPickThreads / 32; w++) meet(rv[w], ri[w]);
+        if (bi == INT64_MAX) bi = -1;
     }
     if (threadIdx.x == 0) {
         const int64_t cur = a[l];
@@ -320,23 +329,33 @@ int launch_refine_colour(const Prefix &P, const int32_t *a, int m, int colour, d
     int nblk = (m - 2 >= l0) ? (m - 2 - l0) / 3 + 1 : 0;
     *nblocks_out = nblk;
     if (nblk == 0) return ECASQ_OK;
-    int nchunk = (int)cdiv(P.p, kRefineChunk);
+    // Screened above 512 candidates an SM, where the full scan's binary64 time passes bound and scan.  A
+    // block's warps share an SM's binary64 pipe (a candidate's sequence is 5 us of it), so the blocks are as small as the
+    // room for their results allows.
+    const bool screen = P.p > (int64_t)512 * num_sms;
+    int chunk = screen ? 64 : 32;
+    while (chunk < kRefineChunk && nblk * cdiv(P.p, chunk) > kRefineValues * cdiv(P.d, kRefineChunk)) chunk *= 2;
+    const int nchunk = (int)cdiv(P.p, chunk);
     double *curval = reinterpret_cast<double *>(part_buf);  // then the values' scans and the chunks' partial results
     RefineScan *scan = reinterpret_cast<RefineScan *>(curval + kRefineValues);
     RefPart *part = reinterpret_cast<RefPart *>(scan + kRefineValues);
-    if (nchunk > num_sms) {
+    if (screen) {
         note_launch();
         k_refine_bound<<<nblk, 32, 0, st>>>(P, a, m, colour, lamp, curval, scan, ctx);
         ECASQ_LAUNCH_CHECK();
-        note_launch();
-        k_refine_chunks<true><<<dim3(nchunk, nblk), kRefineChunk, 0, st>>>(P, a, m, colour, lamp, scan, curval, part, nchunk, ctx);
-    } else {
-        note_launch();
-        k_refine_chunks<false><<<dim3(nchunk, nblk), kRefineChunk, 0, st>>>(P, a, m, colour, lamp, scan, curval, part, nchunk, ctx);
+    }
+    const dim3 grid(nchunk, nblk);
+    note_launch();
+    auto go = [&](auto kernel) { kernel<<<grid, chunk, 0, st>>>(P, a, m, colour, lamp, scan, curval, part, nchunk, ctx); };
+    switch (chunk) {
+        case 32: go(k_refine_chunks<32, false>); break;
+        case 64: screen ? go(k_refine_chunks<64, true>) : go(k_refine_chunks<64, false>); break;
+        case 128: screen ? go(k_refine_chunks<128, true>) : go(k_refine_chunks<128, false>); break;
+        default: screen ? go(k_refine_chunks<256, true>) : go(k_refine_chunks<256, false>); break;
     }
     ECASQ_LAUNCH_CHECK();
     note_launch();
-    k_refine_pick<<<nblk, 32, 0, st>>>(a, m, colour, part, curval, nchunk, a_new, moved, ctx);
+    k_refine_pick<<<nblk, kPickThreads, 0, st>>>(a, m, colour, part, curval, nchunk, chunk, a_new, moved, ctx);
     ECASQ_LAUNCH_CHECK();
     return ECASQ_OK;
 }
