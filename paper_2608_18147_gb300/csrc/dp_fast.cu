@@ -2342,7 +2342,8 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     ECASQ_LAUNCH_CHECK();
     ECASQ_CUDA_TRY(cudaMemsetAsync(flags, 0, 4 * sizeof(int), st));
     note_launch();
-    k_fast_base<<<(unsigned)cdiv(P.p - 1, 128), 128, 0, st>>>(P, a, dp64, bp);
+    // (a warp a block: its binary64 sequence is 5 us of an SM's pipe)
+    k_fast_base<<<(unsigned)cdiv(P.p - 1, 32), 32, 0, st>>>(P, a, dp64, bp);
     ECASQ_LAUNCH_CHECK();
     // corner states: needed by every tile that is built (per pass, or once into the table)
     if (a.nJ > 1 && (!costs || build_costs)) {

@@ -95,15 +95,24 @@ __global__ void k_traceback_eval(Prefix P, int G, int s, int exact_s, const doub
     __shared__ int sm_m;
     int g = blockIdx.x;
     int64_t p = P.p;
+    // eq. apx_final over the lanes: the least value, the first (i, then j) among equal ones
+    const int ilo = exact_s ? s : 2;
+    const int64_t last = (int64_t)(s - ilo + 1) * P.nR;
+    double best = CUDART_INF;
+    int64_t first = last;
+    for (int64_t q = threadIdx.x; q < last; q += 32) {
+        const double v = dp64[dp_at(g, ilo + (int)(q / P.nR), p - P.nR + q % P.nR, s, P.ps)];
+        if (v < best) { best = v; first = q; }
+    }
+    for (int o = 16; o; o >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, best, o);
+        const int64_t q = __shfl_xor_sync(0xffffffffu, first, o);
+        const long long k = order_key(v), k0 = order_key(best);
+        if (q < last && (first == last || k < k0 || (k == k0 && q < first))) { best = v; first = q; }
+    }
     if (threadIdx.x == 0) {
-        int istar = -1;
-        int64_t jstar = -1;
-        double best = CUDART_INF;
-        for (int i = exact_s ? s : 2; i <= s; i++)
-            for (int64_t jr = p - P.nR; jr < p; jr++) {
-                double v = dp64[dp_at(g, i, jr, s, P.ps)];
-                if (v < best) { best = v; istar = i; jstar = jr; }
-            }
+        const int istar = first < last ? ilo + (int)(first / P.nR) : -1;
+        const int64_t jstar = first < last ? p - P.nR + first % P.nR : -1;
         if (istar < 0) {
             sm_m = 0;
         } else {
@@ -178,7 +187,8 @@ int launch_dp_clear_base(const Prefix &P, const double *lamp, int G, int s, doub
     ECASQ_LAUNCH_CHECK();
     if (P.p >= 2) {
         note_launch();
-        k_dp_base<<<(unsigned)cdiv(P.p - 1, 128), 128, 0, st>>>(P, lam, G, s, dp64, bp);
+        // (a warp a block: its binary64 sequence is 5 us of an SM's pipe)
+        k_dp_base<<<(unsigned)cdiv(P.p - 1, 32), 32, 0, st>>>(P, lam, G, s, dp64, bp);
         ECASQ_LAUNCH_CHECK();
     }
     return ECASQ_OK;

@@ -20,7 +20,7 @@ def E():
 
 
 @pytest.mark.parametrize("kind", ["normal", "offset", "outliers", "tiny", "huge", "repeated", "integers"])
-@pytest.mark.parametrize("d,m", [(5, 5), (40, 16), (258, 3), (259, 4), (1025, 9), (4099, 16), (3000, 40), (45001, 9)])
+@pytest.mark.parametrize("d,m", [(5, 5), (40, 16), (258, 3), (259, 4), (1025, 9), (4099, 16), (3000, 40), (90001, 9)])
 def test_refinement_equals_the_oracle(E, oracle_mod, d, m, kind):
     rng = np.random.default_rng(d + m)
     x = workloads.normal(d, d)
