@@ -39,7 +39,7 @@ size_t refine_ctx_bytes();
 int launch_refine_colour(const Prefix &P, const int32_t *a, int m, int colour, double lamp, int32_t *a_new,
                          int32_t *moved, void *part_buf, int32_t *ctx, int num_sms, cudaStream_t st, int *nblocks_out);
 size_t refine_scratch_bytes(int64_t d);
-int launch_refine_commit(int32_t *a, const int32_t *a_new, const int32_t *moved, const double *ev, int m, bool guard,
+int launch_refine_commit(int32_t *a, int32_t *a_new, int32_t *moved, const double *ev, double *kept, int m, bool guard,
                          double budget, int32_t *ctx, cudaStream_t st);
 int launch_quantize(const float *x, int64_t d, const float *Q, int m, uint64_t seed, uint8_t *idx, const QuantOut &o,
                     int num_sms, cudaStream_t stream);
@@ -390,11 +390,13 @@ static int refine_device(void *ws, const Layout &L, const Prefix &P, std::vector
     if (rc != ECASQ_OK) return rc;
     double J = ev[0] + lamp * ev[2];
     double *evd = reinterpret_cast<double *>(wsp<char>(ws, L.refine) + 4 * 2 * kMaxS + 256);  // eval_device's output
+    double *kept = evd + 4;  // ... of the current codebook (k_refine_commit)
+    ECASQ_CUDA_TRY(cudaMemcpyAsync(kept, evd, 3 * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    ECASQ_CUDA_TRY(cudaMemcpyAsync(an, a, sizeof(int32_t) * m, cudaMemcpyDeviceToDevice, st));
+    ECASQ_CUDA_TRY(cudaMemsetAsync(moved, 0, sizeof(int32_t), st));
     for (int r = 0; r < max_rounds; r++) {
         double J0 = J;
         for (int col = 0; col < 3; col++) {
-            ECASQ_CUDA_TRY(cudaMemcpyAsync(an, a, sizeof(int32_t) * m, cudaMemcpyDeviceToDevice, st));
-            ECASQ_CUDA_TRY(cudaMemsetAsync(moved, 0, sizeof(int32_t), st));
             int nblk = 0;
             rc = launch_refine_colour(P, a, m, col, lamp, an, moved, wsp<void>(ws, L.refine_part), ctx, num_sms(), st, &nblk);
             if (rc != ECASQ_OK) return rc;
@@ -402,11 +404,11 @@ static int refine_device(void *ws, const Layout &L, const Prefix &P, std::vector
             // only a step that moved a value is evaluated; the step is kept or dropped on the device
             rc = launch_eval_codebook(P, an, m, evd, st, moved);
             if (rc != ECASQ_OK) return rc;
-            rc = launch_refine_commit(a, an, moved, evd, m, guard, budget, ctx, st);
+            rc = launch_refine_commit(a, an, moved, evd, kept, m, guard, budget, ctx, st);
             if (rc != ECASQ_OK) return rc;
         }
-        rc = eval_device(ws, L, P, a, m, st, ev);
-        if (rc != ECASQ_OK) return rc;
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(ev, kept, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
+        ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
         J = ev[0] + lamp * ev[2];
         *rounds_used = r + 1;
         if (last_rel) *last_rel = J0 != 0.0 ? (J0 - J) / fabs(J0) : 0.0;

@@ -292,26 +292,33 @@ __global__ void __launch_bounds__(kPickThreads) k_refine_pick(const int32_t *a, 
 // move in this step); a scan in its new context would keep it there, so a kept step gives
 // it the record such a scan writes, and the next round does not scan it again unless a
 // neighbour moves.
-__global__ void k_refine_commit(int32_t *a, const int32_t *a_new, const int32_t *moved, const double *ev, int m,
+// kept: the evaluation of the current codebook, replaced with it, so that a round's stop test needs none of its own.
+// a_new and moved are left as the next step starts: the current codebook, nothing moved.
+__global__ void k_refine_commit(int32_t *a, int32_t *a_new, int32_t *moved, const double *ev, double *kept, int m,
                                 int guard, double budget, int32_t *ctx) {
-    if (!*moved) return;
-    if (guard && ev[2] > budget) return;
-    for (int l = threadIdx.x; l < m; l += blockDim.x) {
-        if (a_new[l] == a[l]) continue;
-        int32_t c[5];
-        context_of(a_new, m, l, c);
-        int32_t *r = ctx + kCtx * l;
-        for (int q = 0; q < 5; q++) r[q] = c[q];
-        r[5] = 1;
+    if (*moved && !(guard && ev[2] > budget)) {
+        for (int l = threadIdx.x; l < m; l += blockDim.x) {
+            if (a_new[l] == a[l]) continue;
+            int32_t c[5];
+            context_of(a_new, m, l, c);
+            int32_t *r = ctx + kCtx * l;
+            for (int q = 0; q < 5; q++) r[q] = c[q];
+            r[5] = 1;
+        }
+        __syncwarp();  // every comparison with the old codebook is done
+        for (int t = threadIdx.x; t < m; t += blockDim.x) a[t] = a_new[t];
+        if (threadIdx.x < 3) kept[threadIdx.x] = ev[threadIdx.x];
+    } else {
+        for (int t = threadIdx.x; t < m; t += blockDim.x) a_new[t] = a[t];
     }
-    __syncwarp();  // every comparison with the old codebook is done
-    for (int t = threadIdx.x; t < m; t += blockDim.x) a[t] = a_new[t];
+    __syncwarp();
+    if (threadIdx.x == 0) *moved = 0;
 }
 
-int launch_refine_commit(int32_t *a, const int32_t *a_new, const int32_t *moved, const double *ev, int m, bool guard,
+int launch_refine_commit(int32_t *a, int32_t *a_new, int32_t *moved, const double *ev, double *kept, int m, bool guard,
                          double budget, int32_t *ctx, cudaStream_t st) {
     note_launch();
-    k_refine_commit<<<1, 32, 0, st>>>(a, a_new, moved, ev, m, guard ? 1 : 0, budget, ctx);
+    k_refine_commit<<<1, 32, 0, st>>>(a, a_new, moved, ev, kept, m, guard ? 1 : 0, budget, ctx);
     ECASQ_LAUNCH_CHECK();
     return ECASQ_OK;
 }
