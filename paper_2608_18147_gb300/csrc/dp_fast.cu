@@ -2371,7 +2371,8 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     a.bound = (a.prune && a.nJ > a.T) ? 1 : 0;
     a.bound_step = unbounded ? 32 : 4;
     const size_t smem = kSmemHead + area;
-    ECASQ_CUDA_TRY(cudaFuncSetAttribute(k_wavefront, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the same limit in every call: another thread's call of another shape may lie between this and the launch
+    ECASQ_CUDA_TRY(cudaFuncSetAttribute(k_wavefront, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
     int per_sm = 0;
     if (costs && build_costs)
         ECASQ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_costs, NPROD, 0));

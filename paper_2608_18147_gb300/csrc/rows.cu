@@ -498,7 +498,9 @@ int launch_rows_pass(const RowsPass &A, int slots, cudaStream_t st) {
     const size_t smem = rows_pass_smem(A.pmax, A.s);
     const bool wide = A.pmax > kRowsMaxP;
     const void *f = wide ? (const void *)k_rows_pass<true> : (const void *)k_rows_pass<false>;
-    ECASQ_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the same limit in every call (the longest rows and largest s): another thread's call of another shape may
+    // lie between this and the launch
+    ECASQ_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_pass_smem(kScanTile, kMaxS)));
     const unsigned blocks = (unsigned)std::min(A.nact, slots);
     note_launch();
     if (wide) k_rows_pass<true><<<blocks, kRowsThreads, smem, st>>>(B);
