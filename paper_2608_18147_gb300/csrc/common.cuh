@@ -47,11 +47,11 @@ struct DevStatus {
     int64_t last_d;       // d of the last DP pass
     int64_t members;      // fast DP: band members found (all outputs)
     int64_t big_bands;    // fast DP: outputs with more members than the inline list holds
-    int64_t tiles_run;    // fast DP, resident costs: (warp, tile) units evaluated
+    int64_t tiles_run;    // fast DP: (multiplier, tile) units of s - 2 tasks evaluated
     int64_t tiles_skipped; // ... and skipped by the lower bound
     int64_t grid_nL;      // permissible set: |L| = #{p_a <= min x}, |R| = #{p_b >= max x} (Sec. 5)
     int64_t grid_nR;
-    int64_t tiles_fetched; // fast DP, resident costs: interval-cost tiles copied in from HBM
+    int64_t tiles_fetched; // fast DP: interval-cost tiles copied in
 };
 
 // Where an encode puts its counts: o.acc is added to; with a ticket (zero at the launch) the last block copies
