@@ -1080,7 +1080,9 @@ int ecasq_quantize_noalloc(const float *x, int64_t d, const float *Q, int32_t m,
     void *scratch = nullptr;
     int rc = noalloc_scratch(st, &scratch);
     if (rc) return rc;
-    return quantize_with(scratch, kNoAllocScratchBytes, x, d, Q, m, seed, idx, counts, h_emp, st);
+    // The status record alone is taken from the shared block: the counts accumulate in the caller's buffer, so that calls
+    // that overlap cannot mix them.
+    return quantize_with(scratch, sizeof(DevStatus), x, d, Q, m, seed, idx, counts, h_emp, st);
 }
 
 // Linear-space traceback (Sec. 5, last paragraph): the preparation layout, then four DP

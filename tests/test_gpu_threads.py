@@ -55,3 +55,36 @@ def test_concurrent_calls_of_different_shapes(E):
     for t in threads:
         t.join()
     assert not wrong
+
+
+def test_overlapping_noalloc_encodes_keep_their_counts(E):
+    """ecasq_quantize_noalloc from several threads at once: the calls share the library's status record, their
+    counts and entropies are their own."""
+    import torch
+    rng = np.random.default_rng(3)
+    jobs = []
+    for m in (4, 8, 16, 24, 33, 40):
+        x = torch.as_tensor(rng.uniform(-1, 1, 4000003).astype(np.float32)).cuda()
+        Q = torch.linspace(-1, 1, m, device="cuda")
+        _, counts, h = E.ecasq_quantize(x, Q, m)
+        jobs.append((x, Q, m, counts, h))
+    torch.cuda.synchronize()
+    wrong = []
+
+    def work(x, Q, m, want, h):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                idx = torch.empty(x.numel(), dtype=torch.uint8, device="cuda")
+                for _ in range(30):
+                    counts = torch.full((m,), -1, dtype=torch.int32, device="cuda")
+                    assert E.ecasq_quantize_noalloc(x, Q, m, idx, counts) == pytest.approx(h, rel=1e-12)
+                    assert torch.equal(counts, want)
+        except Exception as e:  # noqa: BLE001 -- reported below, with the codebook
+            wrong.append((m, repr(e)))
+
+    threads = [threading.Thread(target=work, args=job) for job in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
