@@ -251,10 +251,13 @@ __global__ void __launch_bounds__(kQThreads, TS ? 4 : 6) k_quantize_short(const 
     const bool unsorted_q = __syncthreads_or(wrong);
     const int64_t d = unsorted_q ? 0 : a.d;  // unsorted: nothing is encoded
     if (unsorted_q && threadIdx.x == 0) o.st->range_err = kUnsortedQ;
-    // a group within [lo, hi] is within the range of either codebook
+    // a group within [lo, hi] is within the range of either codebook; NaN, which no group is within, where a codebook of one
+    // value is NaN (a longer one is refused above)
     const float q0[2] = {sq[0], TS && a.m[1] ? sq[kFastBins] : sq[0]};
     const float qm[2] = {sq[a.m[0] - 1], TS && a.m[1] ? sq[kFastBins + a.m[1] - 1] : sq[a.m[0] - 1]};
-    const float lo = fmaxf(q0[0], q0[1]), hi = fminf(qm[0], qm[1]);
+    float lo, hi;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(lo) : "f"(q0[0]), "f"(q0[1]));
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(hi) : "f"(qm[0]), "f"(qm[1]));
     const char *cq = reinterpret_cast<const char *>(sq);
     char *pc = reinterpret_cast<char *>(ph) + 4 * threadIdx.x;
     constexpr int kTop = STEPS > 0 && !TS;  // the first threshold of the search stays in a register

@@ -78,3 +78,22 @@ def test_refusals_and_small_workspace(E, oracle_mod, m):
             with pytest.raises(E.EcasqError) as ei:
                 E.ecasq_quantize(y, Q, 3, ws=ws)
             assert ei.value.code == E.native.ERANGE
+
+
+@pytest.mark.parametrize("m", [2, 16, 17])
+@pytest.mark.parametrize("d", [7, 8, 4096, 9001])
+@pytest.mark.parametrize("part", [0, 1])
+def test_a_nan_codebook_of_one_value_is_out_of_range(E, d, m, part):
+    """No entry lies within a codebook whose one value is NaN: refused whichever kernel meets the entry,
+    and no matter for the part that no entry takes."""
+    x = np.random.default_rng(d).uniform(-1, 1, d).astype(np.float32)
+    Q, nan = np.linspace(-1, 1, m).astype(np.float32), np.array([np.nan], np.float32)
+    Qm, Qp = (nan, Q) if part == 0 else (Q, nan)
+    with pytest.raises(E.EcasqError) as ei:
+        E.ecasq_quantize_timeshare(x, Qm, Qp, 0.5, 3, 4)
+    assert ei.value.code == E.native.ERANGE
+    idx, sel, counts, _ = E.ecasq_quantize_timeshare(x, Qm, Qp, 1.0 - part, 3, 4)
+    other = E.ecasq_quantize(x, Q, 3)
+    np.testing.assert_array_equal(idx.cpu().numpy(), other[0].cpu().numpy())
+    np.testing.assert_array_equal(counts.cpu().numpy()[1:] if part == 0 else counts.cpu().numpy()[:-1],
+                                  other[1].cpu().numpy())
