@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(kQThreads, TS ? 4 : 6) k_quantize_short(const 
     float lo, hi;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(lo) : "f"(q0[0]), "f"(q0[1]));
     asm("min.NaN.f32 %0, %1, %2;" : "=f"(hi) : "f"(qm[0]), "f"(qm[1]));
+    asm("min.NaN.f32 %0, %0, %1;" : "+f"(hi) : "f"(3.4028235e38f));  // +inf is not told from the padding: one by one
     const char *cq = reinterpret_cast<const char *>(sq);
     char *pc = reinterpret_cast<char *>(ph) + 4 * threadIdx.x;
     constexpr int kTop = STEPS > 0 && !TS;  // the first threshold of the search stays in a register
@@ -279,10 +280,12 @@ __global__ void __launch_bounds__(kQThreads, TS ? 4 : 6) k_quantize_short(const 
         if (__fmul_rn(k, gap) < __fsub_rn(xv, qa)) t += 4;
         return t;
     };
-    // outside its codebook's range: index 0 and the error flag
+    // outside its codebook's range: index 0 and the error flag; +inf, where it is the codebook's last value, runs into the
+    // padding behind it and is brought back
     auto checked = [&](float xv, int t) -> int {
         const int part = TS ? t / (4 * kFastBins) : 0;
-        if (xv >= (part ? q0[1] : q0[0]) && xv <= (part ? qm[1] : qm[0])) return t;
+        if (xv >= (part ? q0[1] : q0[0]) && xv <= (part ? qm[1] : qm[0]))
+            return min(t, part * 4 * kFastBins + 4 * (a.m[part] - 1));
         bad = true;
         return part * 4 * kFastBins;
     };

@@ -97,3 +97,30 @@ def test_a_nan_codebook_of_one_value_is_out_of_range(E, d, m, part):
     np.testing.assert_array_equal(idx.cpu().numpy(), other[0].cpu().numpy())
     np.testing.assert_array_equal(counts.cpu().numpy()[1:] if part == 0 else counts.cpu().numpy()[:-1],
                                   other[1].cpu().numpy())
+
+
+@pytest.mark.parametrize("m", [1, 2, 4, 5, 9, 16])
+def test_an_infinite_last_value_keeps_to_its_codebook(E, oracle_mod, m):
+    """A codebook that ends in +inf and entries equal to it: the last index, and nothing written behind the counts."""
+    import torch
+    Q = np.concatenate([np.linspace(-1, 1, max(m - 1, 1)), [np.inf]])[-m:].astype(np.float32)
+    rng = np.random.default_rng(m)
+    for d in (6, 9001):
+        x = (rng.uniform(-1, 1, d) if m > 2 else np.full(d, np.inf)).astype(np.float32)
+        x[1::5] = np.inf
+        oi, oc, _ = oracle_mod.quantize(x, Q, 3)
+        for nbytes in (128, 4096):  # the counts in the caller's buffer, or behind the status record
+            ws = torch.full((nbytes + 256,), 0x5A, dtype=torch.uint8, device="cuda")
+            out = torch.full((64,), -7, dtype=torch.int32, device="cuda")
+            idx, _, _ = E.ecasq_quantize(x, Q, 3, ws=ws[:nbytes], counts=out[:m])
+            np.testing.assert_array_equal(idx.cpu().numpy(), oi)
+            np.testing.assert_array_equal(out[:m].cpu().numpy(), oc.astype(np.int32))
+            assert bool((out[m:] == -7).all()) and bool((ws[nbytes:] == 0x5A).all())
+        for Qm, Qp in ((Q, Q), (Q, np.array([-1, 0.5, np.inf], np.float32))):
+            if Qp[0] > x.min():
+                continue
+            idx, sel, counts, _ = E.ecasq_quantize_timeshare(x, Qm, Qp, 0.4, 3, 4)
+            oi2, os2, oc2, _ = oracle_mod.quantize_timeshare(x, Qm, Qp, 0.4, 3, 4)
+            np.testing.assert_array_equal(idx.cpu().numpy(), oi2)
+            np.testing.assert_array_equal(sel.cpu().numpy(), os2)
+            np.testing.assert_array_equal(counts.cpu().numpy().astype(np.uint32), oc2)
