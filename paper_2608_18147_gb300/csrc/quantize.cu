@@ -406,13 +406,17 @@ __global__ void __launch_bounds__(256) k_quantize_timeshare(const float *__restr
                                                             uint8_t *__restrict__ sel, QuantOut o) {
     __shared__ float q[2][kMaxS];
     __shared__ uint32_t hcount[2 * kMaxS];
+    // (The order is checked here: with loops of its own for it the encode below compiles to a fifth more time, 535 against
+    // 437 us at 67 million entries and 17 or 32 values.)
+    bool wrong = false;
     for (int r = threadIdx.x; r < kMaxS; r += blockDim.x) {
         q[0][r] = r < mm ? Qm[r] : CUDART_INF_F;
         q[1][r] = r < mp ? Qp[r] : CUDART_INF_F;
+        wrong |= r > 0 && ((r < mm && !(Qm[r] > Qm[r - 1])) || (r < mp && !(Qp[r] > Qp[r - 1])));
         hcount[r] = 0;
         hcount[kMaxS + r] = 0;
     }
-    if (__syncthreads_or(unsorted(Qm, mm) || unsorted(Qp, mp))) {  // nothing is encoded
+    if (__syncthreads_or(wrong)) {  // nothing is encoded
         if (threadIdx.x == 0) o.st->range_err = kUnsortedQ;
         d = 0;
     }
