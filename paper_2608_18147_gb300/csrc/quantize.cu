@@ -43,8 +43,9 @@ __device__ __forceinline__ void finish_counts(const QuantOut &o, int n) {
     for (int r = threadIdx.x; r < n; r += blockDim.x) o.counts[r] = __ldcg(o.acc + r);
 }
 
-// half: the largest power of two <= m - 1 (0 when m = 1); q[m .. 2 half - 1] hold +inf, so
-// the search needs no bound test.  zc = seed + (i + 1) * gamma (mod 2^64) for entry i.
+// half: the largest power of two <= m - 1 (0 when m = 1); q[m .. 2 half - 1] hold NaN, which no
+// entry passes (+inf would let +inf pass), so the search needs no bound test.  zc = seed +
+// (i + 1) * gamma (mod 2^64) for entry i.
 __device__ __forceinline__ int search_half(int m) { return m > 1 ? 1 << (31 - __clz(m - 1)) : 0; }
 
 __device__ __forceinline__ int quant_one(float xv, uint64_t zc, const float *q, int m, int half, bool &bad) {
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(kQThreads) k_quantize(const float *__restrict_
     __shared__ uint32_t hcount[kMaxS];
     __shared__ uint32_t ph[PRIV ? (kPrivBins / 2) * kQThreads : 1];
     for (int r = threadIdx.x; r < kMaxS; r += blockDim.x) {
-        q[r] = r < m ? Q[r] : CUDART_INF_F;
+        q[r] = r < m ? Q[r] : CUDART_NAN_F;
         hcount[r] = 0;
     }
     const int half = search_half(m);
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(kQThreads, TS ? 4 : 6) k_quantize_short(const 
     for (int r = threadIdx.x; r < 2 * kFastBins; r += kQThreads) {
         const int part = r / kFastBins, t = r % kFastBins, m = part ? (TS ? a.m[1] : 0) : a.m[0];
         const float *Q = part ? a.Q[1] : a.Q[0];
-        sq[r] = t < m ? Q[t] : CUDART_INF_F;
+        sq[r] = t < m ? Q[t] : CUDART_NAN_F;  // (no entry passes it, +inf neither)
         sq[2 * kFastBins + r] = t + 1 < m ? __fsub_rn(Q[t + 1], Q[t]) : CUDART_INF_F;
         wrong |= t + 1 < m && !(Q[t + 1] > Q[t]);
     }
@@ -255,10 +256,9 @@ __global__ void __launch_bounds__(kQThreads, TS ? 4 : 6) k_quantize_short(const 
     // value is NaN (a longer one is refused above)
     const float q0[2] = {sq[0], TS && a.m[1] ? sq[kFastBins] : sq[0]};
     const float qm[2] = {sq[a.m[0] - 1], TS && a.m[1] ? sq[kFastBins + a.m[1] - 1] : sq[a.m[0] - 1]};
-    float lo, hi;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(lo) : "f"(q0[0]), "f"(q0[1]));
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(hi) : "f"(qm[0]), "f"(qm[1]));
-    asm("min.NaN.f32 %0, %0, %1;" : "+f"(hi) : "f"(3.4028235e38f));  // +inf is not told from the padding: one by one
+    float lo = q0[0];
+    if (TS) asm("max.NaN.f32 %0, %0, %1;" : "+f"(lo) : "f"(q0[1]));
+    const float hi = TS ? fminf(qm[0], qm[1]) : qm[0];
     const char *cq = reinterpret_cast<const char *>(sq);
     char *pc = reinterpret_cast<char *>(ph) + 4 * threadIdx.x;
     constexpr int kTop = STEPS > 0 && !TS;  // the first threshold of the search stays in a register
@@ -280,12 +280,10 @@ __global__ void __launch_bounds__(kQThreads, TS ? 4 : 6) k_quantize_short(const 
         if (__fmul_rn(k, gap) < __fsub_rn(xv, qa)) t += 4;
         return t;
     };
-    // outside its codebook's range: index 0 and the error flag; +inf, where it is the codebook's last value, runs into the
-    // padding behind it and is brought back
+    // outside its codebook's range: index 0 and the error flag
     auto checked = [&](float xv, int t) -> int {
         const int part = TS ? t / (4 * kFastBins) : 0;
-        if (xv >= (part ? q0[1] : q0[0]) && xv <= (part ? qm[1] : qm[0]))
-            return min(t, part * 4 * kFastBins + 4 * (a.m[part] - 1));
+        if (xv >= (part ? q0[1] : q0[0]) && xv <= (part ? qm[1] : qm[0])) return t;
         bad = true;
         return part * 4 * kFastBins;
     };
@@ -410,8 +408,8 @@ __global__ void __launch_bounds__(256) k_quantize_timeshare(const float *__restr
     // 437 us at 67 million entries and 17 or 32 values.)
     bool wrong = false;
     for (int r = threadIdx.x; r < kMaxS; r += blockDim.x) {
-        q[0][r] = r < mm ? Qm[r] : CUDART_INF_F;
-        q[1][r] = r < mp ? Qp[r] : CUDART_INF_F;
+        q[0][r] = r < mm ? Qm[r] : CUDART_NAN_F;
+        q[1][r] = r < mp ? Qp[r] : CUDART_NAN_F;
         wrong |= r > 0 && ((r < mm && !(Qm[r] > Qm[r - 1])) || (r < mp && !(Qp[r] > Qp[r - 1])));
         hcount[r] = 0;
         hcount[kMaxS + r] = 0;

@@ -99,7 +99,7 @@ def test_a_nan_codebook_of_one_value_is_out_of_range(E, d, m, part):
                                   other[1].cpu().numpy())
 
 
-@pytest.mark.parametrize("m", [1, 2, 4, 5, 9, 16])
+@pytest.mark.parametrize("m", [1, 2, 4, 5, 9, 16, 17, 40])
 def test_an_infinite_last_value_keeps_to_its_codebook(E, oracle_mod, m):
     """A codebook that ends in +inf and entries equal to it: the last index, and nothing written behind the counts."""
     import torch
