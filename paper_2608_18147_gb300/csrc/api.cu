@@ -22,6 +22,7 @@ int save_dp_seed(void *ws, const Layout &Lw, int64_t p, int G, int s, int g, cud
 size_t resident_costs_bytes(int64_t d);
 size_t streamed_costs_bytes(int64_t d);
 int launch_rows_prepare(const float *X, int64_t rows, const RowsData &R, cudaStream_t st);
+int launch_rows_finite(const float *x, int64_t n, DevStatus *ds, cudaStream_t st);
 int launch_grid_prefix(const float *P, int64_t n, const float *vX, const int64_t *NX, const double *SX,
                        const double *S2X, int64_t pX, float *v, int64_t *w, int64_t *N, double *S, double *S2,
                        DevStatus *st, cudaStream_t stream);
@@ -1265,25 +1266,33 @@ int ecasq_quantize_timeshare(const float *x, int64_t d, const float *Qm, int32_t
 static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws,
                               size_t ws_bytes, float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
     const int s = prm->s;
-    if (rows_chunk(d, rows) < rows) {  // long rows, many of them
-        const int64_t step = rows_chunk(d, rows);
-        int status = ECASQ_OK;
-        for (int64_t r = 0; r < rows; r += step) {
-            const int rc = solve_rows_batched(X + r * d, std::min(step, rows - r), d, prm, ws, ws_bytes, Q + r * s, m_out + r,
-                                              res ? res + r : nullptr, st);
-            if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
-            if (rc == ECASQ_EINFEASIBLE) status = rc;
-        }
-        return status;
-    }
+    const int64_t step = rows_chunk(d, rows);
     Layout L1;
     make_layout(d, s, 1, &L1);
     int rc = add_resident_costs(prm->flags, &L1);
     if (rc) return rc;
     RowsLayout RL;
-    rows_layout(d, s, rows, &RL);
+    rows_layout(d, s, step, &RL);
     const size_t roff = align256(L1.total);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < roff + RL.total) return ECASQ_EWORKSPACE;
+    if (step < rows) {  // long rows, many of them
+        // a value that is not finite refuses the call before any group's results are written
+        DevStatus *ds = wsp<DevStatus>(ws, 0), h;
+        ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
+        rc = launch_rows_finite(X, rows * d, ds, st);
+        if (rc) return rc;
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(h), cudaMemcpyDeviceToHost, st));
+        ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
+        if (h.nonfinite) return ECASQ_ENONFINITE;
+        int status = ECASQ_OK;
+        for (int64_t r = 0; r < rows; r += step) {
+            rc = solve_rows_batched(X + r * d, std::min(step, rows - r), d, prm, ws, ws_bytes, Q + r * s, m_out + r,
+                                    res ? res + r : nullptr, st);
+            if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
+            if (rc == ECASQ_EINFEASIBLE) status = rc;
+        }
+        return status;
+    }
     char *rb = static_cast<char *>(ws) + roff;
     RowsData R;
     R.v = reinterpret_cast<float *>(rb + RL.v);

@@ -713,6 +713,21 @@ __global__ void __launch_bounds__(256) k_rows_prepare(const float *__restrict__ 
     if (threadIdx.x == 0) R.nonfinite[row] = nonfin;
 }
 
+__global__ void k_rows_finite(const float *__restrict__ x, int64_t n, DevStatus *st) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    bool bad = false;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) bad |= !isfinite(x[i]);
+    if (bad) st->nonfinite = 1;
+}
+
+// Raises st->nonfinite when one of the n values is not finite.
+int launch_rows_finite(const float *x, int64_t n, DevStatus *ds, cudaStream_t st) {
+    note_launch();
+    k_rows_finite<<<(unsigned)std::min<int64_t>(cdiv(n, 256), 4096), 256, 0, st>>>(x, n, ds);
+    ECASQ_LAUNCH_CHECK();
+    return ECASQ_OK;
+}
+
 int launch_rows_prepare(const float *X, int64_t rows, const RowsData &R, cudaStream_t st) {
     if (R.d < 1 || R.d > kScanTile) return ECASQ_EINVAL;
     note_launch();

@@ -2,6 +2,8 @@
 size whose costs fit shared memory and around units of 32 columns, up to the longest; codebook
 sizes around a warp; ties; magnitudes and gaps at the ends of the fp32 range.  Every row equals the
 single solve with the binary64 kernel."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -59,3 +61,25 @@ def test_rows_at_the_ends_of_the_fp32_range(E, d):
     X[5] = np.linspace(0, 1e-40, d).astype(np.float32)
     _same(E, X, 6, budget_bits=1.5)
     _same(E, X[:3], 6, lambda_=1e37)
+
+
+def test_a_value_that_is_not_finite_refuses_every_group(E):
+    """More rows than are searched together: a NaN in the last one leaves every row's results unwritten."""
+    import torch
+    rows, d, s = 300, 1024, 4
+    X = torch.as_tensor(np.random.default_rng(5).standard_normal((rows, d)).astype(np.float32)).cuda()
+    X[299, 17] = float("nan")
+    ws = E.workspace(d, s, rows)
+    Q = torch.full((rows, s), 7.0, device="cuda")
+    m = torch.full((rows,), 7, dtype=torch.int32, device="cuda")
+    prm, ptr = E.native.make_params(s, 1.5), E.native._ptr
+    rc = E.lib().ecasq_solve_batched(ptr(X), rows, d, C.byref(prm), ptr(ws), ws.numel(), ptr(Q), ptr(m), None,
+                                     E.native._stream())
+    torch.cuda.synchronize()
+    assert rc == E.native.ENONFINITE
+    assert bool((Q == 7).all()) and bool((m == 7).all())
+    X[299, 17] = 0.25
+    Qg, mg, res = E.ecasq_solve_batched(X, s, budget_bits=1.5, ws=ws)
+    Q1, r1 = E.ecasq_solve(X[299], s, budget_bits=1.5)
+    assert mg[299] == r1["m"] and res[299]["mse"] == r1["mse"]
+    np.testing.assert_array_equal(Qg[299, : r1["m"]].cpu().numpy(), Q1.cpu().numpy())
