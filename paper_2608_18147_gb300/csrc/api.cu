@@ -1263,36 +1263,12 @@ int ecasq_quantize_timeshare(const float *x, int64_t d, const float *Qm, int32_t
 // so each row's result equals ecasq_solve on that row alone.  Rows that fp32 cannot take (rows.cu), longer
 // rows and refinement take ecasq_solve row by row, and so do rows of more than kRowsMaxP unique
 // values with a flag that only ecasq_solve knows.
-static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws,
-                              size_t ws_bytes, float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
+static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws, size_t roff,
+                            float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
     const int s = prm->s;
-    const int64_t step = rows_chunk(d, rows);
-    Layout L1;
-    make_layout(d, s, 1, &L1);
-    int rc = add_resident_costs(prm->flags, &L1);
-    if (rc) return rc;
     RowsLayout RL;
-    rows_layout(d, s, step, &RL);
-    const size_t roff = align256(L1.total);
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < roff + RL.total) return ECASQ_EWORKSPACE;
-    if (step < rows) {  // long rows, many of them
-        // a value that is not finite refuses the call before any group's results are written
-        DevStatus *ds = wsp<DevStatus>(ws, 0), h;
-        ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
-        rc = launch_rows_finite(X, rows * d, ds, st);
-        if (rc) return rc;
-        ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(h), cudaMemcpyDeviceToHost, st));
-        ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
-        if (h.nonfinite) return ECASQ_ENONFINITE;
-        int status = ECASQ_OK;
-        for (int64_t r = 0; r < rows; r += step) {
-            rc = solve_rows_batched(X + r * d, std::min(step, rows - r), d, prm, ws, ws_bytes, Q + r * s, m_out + r,
-                                    res ? res + r : nullptr, st);
-            if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
-            if (rc == ECASQ_EINFEASIBLE) status = rc;
-        }
-        return status;
-    }
+    rows_layout(d, s, rows, &RL);
+    int rc;
     char *rb = static_cast<char *>(ws) + roff;
     RowsData R;
     R.v = reinterpret_cast<float *>(rb + RL.v);
@@ -1380,6 +1356,7 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
         A.pairs = reinterpret_cast<double *>(rb + RL.pairs);
         A.pstride = RL.pstride;
         A.pairs_ready = pairs_ready ? 1 : 0;
+        A.st = wsp<DevStatus>(ws, 0);
         int r2 = launch_rows_pass(A, RL.slots, st);
         pairs_ready = true;  // every active row of a later round was active in this one
         if (r2) return r2;
@@ -1539,6 +1516,10 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
     ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
     // rows left to the single-row path (its layout sits before the row data); the binary64 kernel where fp32 cannot take a
     // row whatever the path
+    if (slow.empty()) return status;
+    DevStatus sum, h;  // each single solve starts the record anew
+    ECASQ_CUDA_TRY(cudaMemcpyAsync(&sum, ws, sizeof(sum), cudaMemcpyDeviceToHost, st));
+    ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
     for (int64_t r : slow) {
         ecasq_result_t one;
         ecasq_params_t p1 = *prm;
@@ -1547,9 +1528,49 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
         if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
         if (rc == ECASQ_EINFEASIBLE) status = rc;
         ECASQ_CUDA_TRY(cudaMemcpyAsync(m_out + r, &one.m, sizeof(int32_t), cudaMemcpyHostToDevice, st));
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ws, sizeof(h), cudaMemcpyDeviceToHost, st));
+        ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
+        sum.bound_viol += h.bound_viol;
+        sum.rescored += h.rescored;
         if (res) res[r] = one;
     }
+    h.bound_viol = sum.bound_viol;
+    h.rescored = sum.rescored;
+    ECASQ_CUDA_TRY(cudaMemcpyAsync(ws, &h, sizeof(h), cudaMemcpyHostToDevice, st));
     ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
+    return status;
+}
+
+// All rows, in groups where they are long and many.  The status record's bound_viol and rescored count all of them.
+static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws,
+                              size_t ws_bytes, float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
+    const int s = prm->s;
+    const int64_t step = rows_chunk(d, rows);
+    Layout L1;
+    make_layout(d, s, 1, &L1);
+    int rc = add_resident_costs(prm->flags, &L1);
+    if (rc) return rc;
+    RowsLayout RL;
+    rows_layout(d, s, step, &RL);
+    const size_t roff = align256(L1.total);
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < roff + RL.total) return ECASQ_EWORKSPACE;
+    DevStatus *ds = wsp<DevStatus>(ws, 0);
+    ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
+    if (step < rows) {
+        // a value that is not finite refuses the call before any group's results are written
+        DevStatus h;
+        rc = launch_rows_finite(X, rows * d, ds, st);
+        if (rc) return rc;
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(h), cudaMemcpyDeviceToHost, st));
+        ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
+        if (h.nonfinite) return ECASQ_ENONFINITE;
+    }
+    int status = ECASQ_OK;
+    for (int64_t r = 0; r < rows; r += step) {
+        rc = solve_rows_group(X + r * d, std::min(step, rows - r), d, prm, ws, roff, Q + r * s, m_out + r, res ? res + r : nullptr, st);
+        if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
+        if (rc == ECASQ_EINFEASIBLE) status = rc;
+    }
     return status;
 }
 

@@ -38,9 +38,9 @@ struct DevStatus {
     int32_t nonfinite;    // x held NaN/Inf
     int32_t range_err;    // quantize: entry outside [Q0, Qm-1]; refine: Q not in X
     int32_t timeout;      // a bounded wait ran out
-    int32_t bound_viol;   // fast DP: fp32 minima outside their certified error bound
+    int32_t bound_viol;   // fast DP, batched rows: fp32 minima outside their certified error bound
     double norm2;         // ||X||^2 (hi part of the double-double sum)
-    int64_t rescored;     // fast DP: candidates re-scored in fp64
+    int64_t rescored;     // fast DP, batched rows: candidates re-scored in fp64
     int64_t overflow;     // fast DP: needed outputs whose band spans more than 32 tiles
     int32_t last_s;       // s and G of the last DP pass (for ecasq_dp_tables)
     int32_t last_G;
@@ -189,7 +189,8 @@ struct RowsPass {
                           // across rounds
     int64_t pstride;      // doubles per row
     int pairs_ready;      // the rows' interval costs are already in `pairs`
-    float tau[kMaxS + 1]; // band factors (set by the launcher)
+    DevStatus *st;        // bound_viol and rescored are added to
+    float tau[kMaxS + 1], eps[kMaxS + 1]; // band factors and certified errors (set by the launcher)
 };
 
 // Prefix-sum view (App. E) used by every exact pair evaluation.

@@ -15,7 +15,10 @@
 //     Elsewhere, and between last layers, the members' closure is evaluated in binary64 with
 //     double-double interval costs (resolve; lowest k, smallest i among exact minima).
 // The results are those of the binary64 recurrence: every output's candidate set is that of the
-// fast DP (dp_fast.cu), and an exact minimum of one candidate needs no evaluation.
+// fast DP (dp_fast.cu), and an exact minimum of one candidate needs no evaluation.  The bound that this rests on is
+// checked at run time, as there: an output evaluated exactly, and every codebook's objective from its
+// binary64 metrics, has to lie within the certified error of its fp32 value (row_within; counted in
+// DevStatus::bound_viol).
 //
 // What bounds it: the chip has 2 binary64 operations a cycle and SM, so an interval cost for every pair
 // (8128 a row of 128 values) took 43 of 70 ms of device time for 8192 rows at s = 8; fp32 costs
@@ -111,13 +114,22 @@ struct RowTrace {
     uint16_t *list;        // [s+1][p]: the closure's outputs by layer
     uint32_t *need;        // [s+1][nw]: ... as bits, all zero between closures
     uint16_t *cnt;         // [s+1]: ... their number by layer
-    const float *tau;
-    double lam;
-    float lam32, slack;
+    const float *tau, *eps;
+    double lam, scale;
+    float lam32, slack, noise;
     int p, g, nw;
+    int *tally;            // outputs outside their certified error, candidates evaluated (shared memory)
 };
 __device__ __forceinline__ float row_limit(const RowTrace &T, int i, float m) {
     return __fadd_ru(__fmul_ru(m, __fadd_ru(1.0f, T.tau[i])), T.slack);
+}
+// Whether the fp32 value m32 of an output of layer i is within its certified error of the exact one, best * scale: eps_i
+// (and 2^-24 for the rounding of `best`, as the comparison is fp32), the underflow that row_limit allows for, and
+// what double-double interval costs and their sums leave, `noise` a layer: 2^-100 of N V^2 <= 2^10 ||X||^2 (V the
+// largest magnitude).
+__device__ __forceinline__ bool row_within(float m32, double best, float eps, float slack, double scale, int i, float noise) {
+    const float x = __double2float_rn(__dmul_rn(best, scale));
+    return fabsf(m32 - x) <= (eps * 1.0001f + 0x1p-24f) * x + (slack + (float)i * noise);
 }
 // Members of output (i, j) among k = kb .. kb + 127, 32 a word: candidates whose fp32 value (the forward pass's) is not
 // above the limit.  One warp; the loads of the four words are in flight together.
@@ -150,6 +162,10 @@ __device__ __forceinline__ double row_cost(const RowTrace &T, int k, int j) {
     double C, U, D;
     pair_exact(T.P, k, j, C, U, D);
     return __dadd_rn(C, __dmul_rn(T.lam, phi_exact(T.P, U, D, false)));
+}
+
+__device__ __forceinline__ int row_outside(const RowTrace &T, int i, int j, double best) {
+    return row_within(T.dp[((size_t)i * T.p + j) * kMaxG + T.g], best, T.eps[i], T.slack, T.scale, i, T.noise) ? 0 : 1;
 }
 
 // The exact value and lowest minimiser of output (i0, j0), i0 >= 3: its members, their members and so on
@@ -202,8 +218,9 @@ static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0
         if (lane == 0 && i > 3) cnt[i - 1] = (uint16_t)nn;
         __syncwarp();
     }
-    int arg = -1;
+    int arg = -1, bad = 0;
     double best = CUDART_INF;
+    if (lane == 0) atomicAdd(T.tally + 1, np);
     if (room && np <= kRowsPairs) {
         for (int q = lane; q < np; q += 32) cost[q] = row_cost(T, (int)(key[q] & 1023u), (int)(key[q] >> 10 & 1023u));
         __syncwarp();
@@ -214,14 +231,21 @@ static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0
                 const int i = (int)(f >> 20), k = (int)(f & 1023u);
                 const double c = __dadd_rn(i == 3 ? row_base(T, k) : T.dp64[(size_t)(i - 1) * p + k], cost[q]);
                 if (c <= best) { best = c; arg = k; }
-                if (q > 0 && key[q - 1] >> 10 != f >> 10) {  // the output's last: store it
+                if (q == 0 || key[q - 1] >> 10 != f >> 10) {  // the output's last: store it
                     T.dp64[(size_t)i * p + (f >> 10 & 1023u)] = best;
-                    best = CUDART_INF;
+                    if (q > 0) best = CUDART_INF;
                 }
             }
         }
-        best = __shfl_sync(full, best, 0);
+        best = __shfl_sync(full, best, 0);  // (dp64 is complete)
         arg = __shfl_sync(full, arg, 0);
+        __syncwarp();
+        for (int q = lane; q < np; q += 32)
+            if (q == 0 || key[q - 1] >> 10 != key[q] >> 10) {
+                const int i = (int)(key[q] >> 20), j = (int)(key[q] >> 10 & 1023u);
+                bad += row_outside(T, i, j, T.dp64[(size_t)i * p + j]);
+            }
+        if (bad) atomicAdd(T.tally, bad);
         for (int i = 3; i < i0; i++)
             for (int e = lane; e < cnt[i]; e += 32) T.need[(size_t)i * T.nw + (T.list[(size_t)i * p + e] >> 5)] = 0u;
         __syncwarp();
@@ -255,12 +279,14 @@ static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0
                 if (b2 < best || (b2 == best && a2 < arg)) { best = b2; arg = a2; }
             }
             if (lane == 0) {
+                bad += row_outside(T, i, j, best);
                 T.dp64[(size_t)i * p + j] = best;
                 if (i < i0) T.need[(size_t)i * T.nw + (j >> 5)] = 0u;
             }
             __syncwarp();
         }
     }
+    if (bad) atomicAdd(T.tally, bad);
     *value = best;  // the last output evaluated is (i0, j0)
     return arg;
 }
@@ -315,8 +341,8 @@ static __device__ __noinline__ int row_trace(const RowTrace &T, int s, int ilo, 
 }
 
 // eval_codebook_lanes for the multipliers g0 .. of one warp, `width` lanes (a power of two >= s) each: the same
-// values in the same order; a binary64 sequence costs a warp the same for one lane as for 32.
-__device__ __forceinline__ void row_evaluate(const Prefix &P, const int32_t *a, int m, int width, double *out3) {
+// values in the same order; a binary64 sequence costs a warp the same for one lane as for 32.  Returns MSE + lam H(I,B).
+__device__ __forceinline__ double row_evaluate(const Prefix &P, const int32_t *a, int m, int width, double lam, double *out3) {
     const unsigned full = 0xffffffffu;
     const int l = threadIdx.x & (width - 1);
     double C = 0.0, F = 0.0, U = 0.0, D = 0.0;
@@ -338,6 +364,7 @@ __device__ __forceinline__ void row_evaluate(const Prefix &P, const int32_t *a, 
         if (r < m && m >= 2) hx = __dadd_rn(hx, h);
     }
     if (l == 0 && m > 0) { out3[0] = mse; out3[1] = hs; out3[2] = hx; }
+    return __dadd_rn(mse, __dmul_rn(lam, hs));
 }
 
 // Shared memory: two layers [p][8] as float bits, the pairs' costs (p <= kRowsMaxP), the evaluation's scratch
@@ -359,6 +386,9 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
     __shared__ double lam[kMaxG];
     __shared__ float lam32[kMaxG];
     __shared__ int refuse;
+    __shared__ int tally[2];
+    __shared__ double scale;
+    __shared__ float noise;
     const RowsData &R = A.R;
     const int G = A.G, s = A.s, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
     const size_t dc = (size_t)R.dcap, rows_per = (size_t)(s + 1) * dc, nwc = (dc + 31) / 32;
@@ -370,6 +400,7 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
     uint16_t *list = A.list + blockIdx.x * rows_per * kMaxG;
     uint32_t *need = A.need + blockIdx.x * (size_t)(s + 1) * nwc * kMaxG;
     for (size_t q = tid; q < (size_t)(s + 1) * nwc * kMaxG; q += blockDim.x) need[q] = 0u;
+    if (tid < 2) tally[tid] = 0;
     for (int b = blockIdx.x; b < A.nact; b += gridDim.x) {
         const int64_t row = A.rows[b];
         const int p = (int)R.p[row];
@@ -378,6 +409,10 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
         const int e2 = 2 * row_exp(P.v, p);
         __syncthreads();  // the row before is done
         if (tid == 0) refuse = rc.phf[0] != 0.0;
+        if (tid == 32) {
+            scale = ldexp(1.0, e2);
+            noise = __double2float_ru(ldexp(R.norm2[row], e2 - 90));
+        }
         if (tid < kMaxG) {
             lam[tid] = tid < G ? A.lam[(size_t)b * G + tid] : 0.0;
             lam32[tid] = __double2float_rn(ldexp(lam[tid], e2));
@@ -457,30 +492,44 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
             out = x;
             __syncthreads();
         }
+        // underflow: C and the gaps' products 2^-149 a term, Phi where y < 1e-37 2^-118 a layer
+        auto slack = [&](int g) { return __fmul_ru(3.0f * (float)s, __fmaf_ru(lam32[g], 0x1p-114f, 8.0f * (float)P.d * 0x1p-149f)); };
         for (int g = wid; g < G; g += nwarp) {
             const size_t o = (size_t)g * rows_per;
-            // underflow: C and the gaps' products 2^-149 a term, Phi where y < 1e-37 2^-118 a layer
-            const float slack = __fmul_ru(3.0f * (float)s, __fmaf_ru(lam32[g], 0x1p-114f, 8.0f * (float)P.d * 0x1p-149f));
             const RowTrace T{P, cf, rc.c0, rc.phf, dp, dp64 + o, list + o, need + (size_t)g * (s + 1) * nwc,
-                             cnt_sm + g * (s + 1), A.tau, lam[g],
-                             lam32[g], slack, p, g, (int)nwc};
+                             cnt_sm + g * (s + 1), A.tau, A.eps, lam[g], scale,
+                             lam32[g], slack(g), noise, p, g, (int)nwc, tally};
             const int m = row_trace(T, s, A.exact_s ? s : 2, a_sm + g * s);
             if (lane == 0) { m_sm[g] = m; A.mcount[(size_t)b * G + g] = m; }
             for (int r = lane; r < m; r += 32) A.qidx[((size_t)b * G + g) * s + r] = a_sm[g * s + r];
         }
         __syncthreads();
+        // the codebook's objective against the fp32 value of its last output
+        auto certify = [&](int g, double objective) {
+            const int m = m_sm[g];
+            if (m > 0 && !row_within(dp[((size_t)m * p + p - 1) * kMaxG + g], objective, A.eps[m], slack(g), scale, m, noise))
+                atomicAdd(tally, 1);
+        };
         if (s <= 32) {
             const int width = s <= 4 ? 4 : s <= 8 ? 8 : s <= 16 ? 16 : 32, per = 32 / width;
             for (int g0 = wid * per; g0 < G; g0 += nwarp * per) {
                 const int g = min(g0 + lane / width, G - 1);  // (spare lanes repeat the last one's values)
-                row_evaluate(P, a_sm + g * s, m_sm[g], width, &A.metrics[((size_t)b * G + g) * 4 + 1]);
+                const double J = row_evaluate(P, a_sm + g * s, m_sm[g], width, lam[g], &A.metrics[((size_t)b * G + g) * 4 + 1]);
+                if (lane % width == 0 && g0 + lane / width < G) certify(g, J);
             }
         } else if (wid == 0) {  // one warp, multiplier by multiplier
             for (int g = 0; g < G; g++) {
-                if (m_sm[g] > 0) eval_codebook_warp(P, a_sm + g * s, m_sm[g], &A.metrics[((size_t)b * G + g) * 4 + 1], scratch);
+                double *q = &A.metrics[((size_t)b * G + g) * 4 + 1];
+                if (m_sm[g] > 0) eval_codebook_warp(P, a_sm + g * s, m_sm[g], q, scratch);
+                if (lane == 0) certify(g, __dadd_rn(q[0], __dmul_rn(lam[g], q[1])));  // (lane 0 wrote them)
                 __syncwarp();
             }
         }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        if (tally[0]) atomicAdd(&A.st->bound_viol, tally[0]);
+        if (tally[1]) atomicAdd((unsigned long long *)&A.st->rescored, (unsigned long long)tally[1]);
     }
 }
 
@@ -488,8 +537,7 @@ int launch_rows_pass(const RowsPass &A, int slots, cudaStream_t st) {
     if (A.nact == 0) return ECASQ_OK;
     if (A.pmax > kScanTile) return ECASQ_EINVAL;
     RowsPass B = A;
-    float eps[kMaxS + 1];
-    band_factors(A.s, B.tau, eps);
+    band_factors(A.s, B.tau, B.eps);
     if (!A.pairs_ready) {
         note_launch();
         k_rows_build<<<(unsigned)A.nact, (unsigned)std::max(128, (A.pmax + 31) & ~31), 0, st>>>(B);

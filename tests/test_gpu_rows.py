@@ -83,3 +83,22 @@ def test_a_value_that_is_not_finite_refuses_every_group(E):
     Q1, r1 = E.ecasq_solve(X[299], s, budget_bits=1.5)
     assert mg[299] == r1["m"] and res[299]["mse"] == r1["mse"]
     np.testing.assert_array_equal(Qg[299, : r1["m"]].cpu().numpy(), Q1.cpu().numpy())
+
+
+@pytest.mark.parametrize("rows,d,flags", [(5, 100, 0), (5, 300, 0), (260, 1024, 0), (5, 300, "TIME_KERNELS")])
+def test_rows_check_their_certificate(E, rows, d, flags):
+    """The status record tells how many candidates the call evaluated in binary64 (over all rows, in groups or one by
+    one) and that no fp32 value left its certified error."""
+    flags = getattr(E, flags) if flags else 0
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((rows, d)).astype(np.float32)
+    X[3] = np.arange(d)                                      # ties: many members an output
+    X[4] = 1 + rng.integers(0, 40, d) * 2.0 ** -23           # neighbours far from zero
+    ws = E.workspace(d, 8, rows, flags=flags)
+    ws.fill_(0xFF)
+    _, _, res = E.ecasq_solve_batched(X, 8, budget_bits=2.0, flags=flags, ws=ws)
+    st = E.native.ws_status(ws)
+    assert st["bound_viol"] == 0 and st["timeout"] == 0
+    assert st["rescored"] > rows
+    if flags:
+        assert st["rescored"] >= sum(r["rescored"] for r in res)
