@@ -2152,8 +2152,12 @@ static int mdp_stride(int s) { return (s + 1 + 3) & ~3; }
 // states, block minima, list counts; member counts and lists (scratch of the wavefront before the
 // need stage writes them: scratch_bytes); then the seed rows (far_start).
 static size_t flags_bytes(int64_t d) { return align256(8 * (size_t)kMaxG * (size_t)cdiv(d, BJ) + 64); }
+// For 3 <= s < 6 as much as for s = 6: without a cost table a panel's tiles go there, 552 d bytes a column block, and the lists of
+// three to five layers left room for two or three blocks a panel; the panels' barriers and tile chains then made a
+// budgeted search slower than whole column blocks had (d = 12000, s = 3: 36 ms against 26; with four blocks 18).
+constexpr int kScratchS = 6;
 static size_t scratch_bytes(int64_t d, int32_t s) {
-    const size_t rows = (size_t)kMaxG * (size_t)(s + 1) * (size_t)table_stride(d);
+    const size_t rows = (size_t)kMaxG * (size_t)((s < 3 ? s : std::max(s, kScratchS)) + 1) * (size_t)table_stride(d);
     return align256(4 * rows) + align256(4 * NMEM * rows) + align256(2 * 4 * rows) +
            align256(4 * (size_t)kMaxG * (size_t)table_stride(d));
 }
