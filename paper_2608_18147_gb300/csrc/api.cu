@@ -1261,8 +1261,8 @@ int ecasq_quantize_timeshare(const float *x, int64_t d, const float *Qm, int32_t
 // of ecasq_solve in lockstep with the others -- one k_rows_pass launch per round
 // for all rows still searching -- with the per-row arithmetic of the reference DP,
 // so each row's result equals ecasq_solve on that row alone.  Rows that fp32 cannot take (rows.cu), longer
-// rows and refinement take ecasq_solve row by row, and so do rows of more than kRowsMaxP unique
-// values with a flag that only ecasq_solve knows.
+// rows and refinement take ecasq_solve row by row, and so do one long row alone and rows of more than
+// kRowsMaxP unique values with a flag that only ecasq_solve knows.
 static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws, size_t roff,
                             float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
     const int s = prm->s;
@@ -1309,10 +1309,15 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
     const int Rn = prm->search_rounds > 0 ? prm->search_rounds : 6;
     if (!fixed && !(hi0 > lo0)) return ECASQ_EINVAL;
     std::vector<int64_t> slow;  // rows that take ecasq_solve
+    // A pass keeps a row to one block, p^2 s candidates a multiplier; the single solve, as before, spreads it over the chip.
+    // For one long row alone the single solve is faster from about 6e6 on (batched / single, ms): p = 1024 5.3 / 4.5 at s = 8,
+    // 10.8 / 5.2 at 16, 44 / 11 at 64; p = 640 5.0 / 3.9 at 16; p = 400 9.6 / 9.2 at 64.  Below: p = 1024 2.4 / 4.0 at s = 4,
+    // p = 640 3.8 / 3.9 at 12, p = 400 4.7 / 5.5 at 32, p = 300 9.6 / 9.7 at 64.
+    const bool alone = rows == 1 && ph[0] * ph[0] * s >= 6000000;
     for (int64_t r = 0; r < rows; r++) {
         st_rows[r].lo = lo0;
         st_rows[r].hi = hi0;
-        if (ph[r] > kRowsMaxP && (prm->flags & (ECASQ_DP_REFERENCE | ECASQ_TEST_STALL | ECASQ_TIME_KERNELS))) {
+        if (alone || (ph[r] > kRowsMaxP && (prm->flags & (ECASQ_DP_REFERENCE | ECASQ_TEST_STALL | ECASQ_TIME_KERNELS)))) {
             slow.push_back(r);
             st_rows[r].slow = st_rows[r].done = true;
         }

@@ -102,3 +102,14 @@ def test_rows_check_their_certificate(E, rows, d, flags):
     assert st["rescored"] > rows
     if flags:
         assert st["rescored"] >= sum(r["rescored"] for r in res)
+
+
+@pytest.mark.parametrize("d,s", [(1024, 5), (1024, 6), (612, 16), (614, 16), (400, 38), (1024, 33)])
+def test_one_long_row_alone(E, d, s):
+    """Around the line from which the single solve takes one row."""
+    X = np.random.default_rng(s).standard_normal((1, d)).astype(np.float32)
+    X[0, :3] = 0.5  # (two values fewer)
+    _same(E, X, s, budget_bits=1.5)
+    _same(E, X, s, lambda_=0.3)
+    X[0, 1:3] = [0.25, 0.75]
+    _same(E, X, s, budget_bits=1.5)
