@@ -125,12 +125,12 @@ struct FastArgs {
     int *wide_cnt;         // [s+1]
     float *mdp;            // [nJ][G][mdp_stride]: at i - 2, the min over the block's 64 columns of dp32(g, i, .)
     int mdp_stride;        // s + 1 rounded up to a multiple of 4 (16-byte rows)
-    int prune;             // skip far tiles by the lower bound
+    int nstage;            // stage buffers of the bound and mask phases: 2, or 1 where two do not fit shared memory
     int bound;             // the far phase starts from upper bounds of the minima (bound_phase)
     int bound_step;        // ... from every bound_step-th tile (4; 32 in unseeded searches)
     float *dlast;          // [nJ][G][mdp_stride]: at i - 2, dp32(g, i, .) at the block's last column
     int *ub;               // [T][G][s-2][64]: the bounds' float bits
-    const float *seed;     // with prune: fp32 dp rows [nJ][s+1][64] of an earlier pass at a multiplier >= every
+    const float *seed;     // fp32 dp rows [nJ][s+1][64] of an earlier pass at a multiplier >= every
                            // multiplier of this one (upper bounds of this pass's fp32 minima), or null
     uint32_t spin_limit;   // waits on other CTAs give up after this many polls (kSpinLimit; lower in the test hook)
     int hold0;             // test hook: column block 0's minima are never written and CTA 0 stays out of the
@@ -601,6 +601,9 @@ __device__ __forceinline__ bool grid_sync(const FastArgs &a, Smem &S, int epoch,
 __host__ __device__ __forceinline__ size_t stage_floats(int G, int mdp_stride) {
     return (size_t)NT * BJ * 2 + (size_t)NT * G * mdp_stride;
 }
+// Stage number ns: its buffer, and the parity of its barrier's phase.
+__device__ __forceinline__ int stage_buf(const FastArgs &a, uint32_t ns) { return a.nstage == 2 ? (int)(ns & 1u) : 0; }
+__device__ __forceinline__ uint32_t stage_parity(const FastArgs &a, uint32_t ns) { return (a.nstage == 2 ? ns >> 1 : ns) & 1u; }
 __device__ __forceinline__ void stage_tiles(const FastArgs &a, Smem &S, float *stg, int sb, int K0, int n, int J,
                                             size_t tbase, const float *src, uint64_t policy) {
     const uint32_t tb = (uint32_t)((size_t)n * BJ * sizeof(float2));
@@ -641,15 +644,18 @@ static __device__ __noinline__ void bound_phase(const FastArgs &a, Smem &S, floa
         int m[kBoundL];
 #pragma unroll
         for (int l = 0; l < kBoundL; l++) m[l] = 0x7f800000;
-        if (ct == 0) stage_tiles(a, S, stage + (ns & 1) * sfl, ns & 1, Ka, min(NT, Kb - Ka), J, pn.tbase, a.dlast, policy);
+        auto stage_from = [&](int K) {
+            const int sb = stage_buf(a, ns);
+            stage_tiles(a, S, stage + sb * sfl, sb, K, min(NT, Kb - K), J, pn.tbase, a.dlast, policy);
+        };
+        if (ct == 0) stage_from(Ka);
         for (int K0 = Ka; K0 < Kb; K0 += NT) {
-            const int n = min(NT, Kb - K0), sb = ns & 1;
+            const int n = min(NT, Kb - K0), sb = stage_buf(a, ns);
             const float *stg = stage + sb * sfl;
-            const uint32_t ph = (ns >> 1) & 1u;
+            const uint32_t ph = stage_parity(a, ns);
             ns++;
-            if (K0 + NT < Kb && ct == 0)
-                stage_tiles(a, S, stage + (ns & 1) * sfl, ns & 1, K0 + NT, min(NT, Kb - K0 - NT), J, pn.tbase, a.dlast,
-                            policy);
+            const bool more = K0 + NT < Kb && ct == 0;
+            if (more && a.nstage == 2) stage_from(K0 + NT);
             mbar_wait_bounded(&S.smbar[sb], ph, a.st, a.abort_flag);
             const float2 *ts = reinterpret_cast<const float2 *>(stg) + jl;
             const float *d = stg + (size_t)NT * BJ * 2 + l0 + (size_t)g * a.mdp_stride;
@@ -670,6 +676,7 @@ static __device__ __noinline__ void bound_phase(const FastArgs &a, Smem &S, floa
                     }
             }
             __syncthreads();  // the stage buffer is free
+            if (more && a.nstage != 2) stage_from(K0 + NT);
         }
 #pragma unroll
         for (int l = 0; l < kBoundL; l++)
@@ -727,12 +734,13 @@ static __device__ __noinline__ void mask_phase(const FastArgs &a, Smem &S, float
     const int ba = pn.nB * part / parts, bz = pn.nB * (part + 1) / parts;
     if (ba >= bz) return;
     auto stage_word = [&](int b) {
-        stage_tiles(a, S, stage + (ns & 1) * sfl, ns & 1, b * NT, min(NT, pn.P0 - b * NT), J, pn.tbase, a.mdp, policy);
+        const int sb = stage_buf(a, ns);
+        stage_tiles(a, S, stage + sb * sfl, sb, b * NT, min(NT, pn.P0 - b * NT), J, pn.tbase, a.mdp, policy);
     };
     for (int split = 0; split < a.nsplit; split++) {
         if (ct == 0) stage_word(ba);
         // the outputs' band limits, into shared memory: one coalesced read, whatever the layers' order
-        float *slim = stage + 2 * sfl;  // [Gc][L][64]
+        float *slim = stage + a.nstage * sfl;  // [Gc][L][64]
         const int gs = split * a.Gc, ngv = min(a.Gc, a.G - gs);
         const int *u = ub_at(a, Jl, gs);
         for (int o = 4 * ct; o < ngv * L * BJ; o += 4 * MAXCONS) {
@@ -746,12 +754,13 @@ static __device__ __noinline__ void mask_phase(const FastArgs &a, Smem &S, float
         const int g = gs + (own ? gq : 0);
         const float lam = S.lam32[g];
         for (int b = ba; b < bz; b++) {
-            const int n = min(NT, pn.P0 - b * NT), sb = ns & 1;
+            const int n = min(NT, pn.P0 - b * NT), sb = stage_buf(a, ns);
             const float *stg = stage + sb * sfl, *md = stg + (size_t)NT * BJ * 2;
-            const uint32_t ph = (ns >> 1) & 1u;
+            const uint32_t ph = stage_parity(a, ns);
             const int rs = a.G * a.mdp_stride;
             ns++;
-            if (b + 1 < bz && ct == 0) stage_word(b + 1);
+            const bool more = b + 1 < bz && ct == 0;
+            if (more && a.nstage == 2) stage_word(b + 1);
             if (ct < 32 * kTaskWords) S.tw[ct] = 0u;
             mbar_wait_bounded(&S.smbar[sb], ph, a.st, a.abort_flag);
             for (int l0 = 0; l0 < L; l0 += kBoundL) {
@@ -833,25 +842,9 @@ static __device__ __noinline__ void mask_phase(const FastArgs &a, Smem &S, float
                     a.fweight[w] = work + kTileCost * __popc(any);
                 }
             }
-            __syncthreads();  // tw is free
+            __syncthreads();  // tw and, of one, the stage buffer are free
+            if (more && a.nstage != 2) stage_word(b + 1);
         }
-    }
-}
-
-// Without the skip test (rows too long to stage): every tile and every task.
-__device__ __forceinline__ void mask_all(const FastArgs &a, const Panel &pn) {
-    const int words = pn.nb * a.nsplit * pn.nB;
-    for (int w = (int)blockIdx.x * MAXCONS + (int)threadIdx.x; w < words; w += (int)gridDim.x * MAXCONS) {
-        const int js = w / pn.nB, n = min(NT, pn.P0 - (w - js * pn.nB) * NT), split = js / pn.nb;
-        const uint32_t u = n == 32 ? 0xffffffffu : (1u << n) - 1u;
-        const int real = min(a.Gc, a.G - split * a.Gc) * (a.s - 2);
-        uint32_t bits[kTaskWords];
-#pragma unroll
-        for (int x = 0; x < kTaskWords; x++)
-            bits[x] = real >= 32 * x + 32 ? 0xffffffffu : real <= 32 * x ? 0u : (1u << (real - 32 * x)) - 1u;
-        for (int r = 0; r < n; r++) __stcg(a.fbits + (size_t)w * NT + r, make_uint4(bits[0], bits[1], bits[2], bits[3]));
-        a.funion[w] = u;
-        a.fweight[w] = n * (real + kTileCost);
     }
 }
 
@@ -1432,11 +1425,9 @@ static __device__ __noinline__ void near_phase(const FastArgs &a, Smem &S, const
             if (i > 3)
                 *reinterpret_cast<float2 *>(a.dp32 + d32(a, g, i - 1, (int64_t)J * BJ + 2 * lane)) =
                     make_float2(__int_as_float(m0), __int_as_float(m1));
-            if (a.prune) {
-                const int mn = __reduce_min_sync(0xffffffffu, min(m0, m1));  // block minimum of row i - 1
-                if (lane == 0) mdp[i - 3] = __int_as_float(mn);
-                if (lane == 31) dlast[i - 3] = __int_as_float(m1);
-            }
+            const int mn = __reduce_min_sync(0xffffffffu, min(m0, m1));  // block minimum of row i - 1
+            if (lane == 0) mdp[i - 3] = __int_as_float(mn);
+            if (lane == 31) dlast[i - 3] = __int_as_float(m1);
         }
     }
     if (diag && half == 0 && !dead) {
@@ -1538,8 +1529,7 @@ __global__ void __launch_bounds__(MAXCONS, 1) k_wavefront(const __grid_constant_
                 ok = grid_sync(a, S, ++epoch);
                 if (!ok) break;
             }
-            if (a.prune) mask_phase(a, S, big, pn, policy, pp.ns);
-            else mask_all(a, pn);
+            mask_phase(a, S, big, pn, policy, pp.ns);
             ok = grid_sync(a, S, ++epoch);
             if (!ok) break;
             far_plan(a, S, pn);
@@ -2367,12 +2357,12 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
                            sizeof(float) * (kNearTiles * kCostTileFloats + (MAXCONS / 32) * 2 * BK +
                                             kNearMults * 2 * kNearTiles * BJ));
     if (a.build) area = std::max(area, kBuildGroups * sizeof(BuildSmem));
-    // far tasks are skipped by the lower bound wherever the staged minima fit shared memory
-    const size_t stage = (2 * stage_floats(G, a.mdp_stride) + nt * BJ) * sizeof(float);
-    a.prune = kSmemHead + stage <= (size_t)smem_max ? 1 : 0;
-    if (a.prune) area = std::max(area, stage);
-    else a.seed = nullptr;
-    a.bound = (a.prune && a.nJ > a.T) ? 1 : 0;
+    // one stage buffer where two do not fit (8 multipliers: s >= 80).  Such codebooks once went without the skip test: a search
+    // at d = 30000, s = 114 with a table took 503 ms (441 with whole column blocks), and takes 206.
+    auto stage = [&](int n) { return (n * stage_floats(G, a.mdp_stride) + nt * BJ) * sizeof(float); };
+    a.nstage = kSmemHead + stage(2) <= (size_t)smem_max ? 2 : 1;
+    area = std::max(area, stage(a.nstage));
+    a.bound = a.nJ > a.T ? 1 : 0;
     a.bound_step = unbounded ? 32 : 4;
     const size_t smem = kSmemHead + area;
     // the same limit in every call: another thread's call of another shape may lie between this and the launch

@@ -20,11 +20,12 @@ def E():
 
 # 15 column blocks of 64 make a panel with 7 or 8 multipliers, 16 with fewer: one block, a panel less one
 # value, exactly, plus one, two panels and a remainder; s = 3 (one layer), s = 18 and 19 (128 tasks of 8
-# multipliers and one more layer: two splits), s = 50 (four splits), s = 82 (no skip test).
+# multipliers and one more layer: two splits), s = 50 (four splits), s = 79 to 114 (one stage
+# buffer of the skip test with 8 multipliers above s = 79).
 @pytest.mark.parametrize("mode", ["DEFAULT", "RESIDENT_COSTS", "STREAMED_COSTS"])
 @pytest.mark.parametrize("d,s,G", [(128, 3, 1), (959, 16, 8), (960, 16, 8), (961, 16, 7), (1024, 9, 5), (1025, 18, 6),
                                    (2000, 3, 8), (2113, 18, 8), (2113, 19, 8), (1984, 50, 8), (1100, 82, 8),
-                                   (4097, 32, 3)])
+                                   (4097, 32, 3), (2113, 79, 8), (1500, 80, 8), (2113, 114, 8), (2113, 114, 7)])
 def test_panel_edges_match_reference_kernel(E, mode, d, s, G):
     x = workloads.student_t(d, d + s, scale=1.0)
     lams = [0.0, 1e-4, 1e-3, 0.01, 0.05, 0.2, 1.0, 10.0][-G:]
