@@ -68,6 +68,10 @@ typedef struct CUstream_st *ecasq_stream_t; /* same type as cudaStream_t */
                                      fp32 minima of the bracket's evaluated upper end (an upper bound of every
                                      later pass's minima, Sec. 5's candidates being non-decreasing in lambda) and
                                      bounds at every fourth tile; same results, for comparison */
+#define ECASQ_TEST_SHORT_PARTS (1u << 28) /* test hook for the far segments of the fast DP: four CTAs share a panel's far tiles and
+                                     store a column block's results after every three tiles instead of 255, so that
+                                     small inputs have segments of several parts; results must equal those
+                                     without the flag.  Not for production use. */
 #define ECASQ_TEST_SELF_SEED (1u << 29) /* test hook for the seeded tile skipping: with a fixed multiplier and resident
                                      or streamed costs, the pass runs twice, the second time seeded with the first
                                      one's fp32 minima (the seed then equals every output's minimum, the tightest

@@ -16,7 +16,7 @@ namespace ecasq {
 int launch_dp_reference(const Prefix &P, const double *lamp, int G, int s, double *dp64, int32_t *bp,
                         cudaStream_t st);
 int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, const Layout &L, cudaStream_t st,
-                   bool exact_s, bool exact_tables, float *costs, bool build_costs, bool test_stall,
+                   bool exact_s, bool exact_tables, float *costs, bool build_costs, bool test_stall, bool short_parts,
                    size_t chunk_bytes, bool seeded, bool unbounded, bool tables);
 int save_dp_seed(void *ws, const Layout &Lw, int64_t p, int G, int s, int g, cudaStream_t st);
 size_t resident_costs_bytes(int64_t d);
@@ -315,6 +315,7 @@ static int dp_pass_prepared(void *ws, const Layout &L, const Prefix &P, int s, c
         // streamed costs are rebuilt band by band in every pass
         rc = launch_dp_fast(P, lamp, G, s, ws, L, st, (flags & ECASQ_EXACT_S) != 0, (flags & ECASQ_EXACT_TABLES) != 0,
                             costs, costs && (L.costs_streamed || !*costs_built), (flags & ECASQ_TEST_STALL) != 0,
+                            (flags & ECASQ_TEST_SHORT_PARTS) != 0,
                             L.costs_streamed ? L.costs_bytes : 0,
                             seeded && !(flags & ECASQ_UNSEEDED_SEARCH), (flags & ECASQ_UNSEEDED_SEARCH) != 0, tables);
         if (costs && rc == ECASQ_OK) *costs_built = true;

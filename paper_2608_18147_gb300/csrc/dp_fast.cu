@@ -111,6 +111,7 @@ struct FastArgs {
     int T;                 // column blocks per panel
     int workers;           // CTAs that share the far tiles
     int tcap;              // tasks per far list entry, at most (16 .. 64)
+    int last_ord;          // a far segment's part: tiles 0 .. last_ord (kLastOrd; lower in the test hook)
     float *part;           // [workers + T nsplit] segments: minima [Gc][s-2][64], then runs (seg_min, seg_runs)
     uint4 *fbits;          // far tasks: 128 bits a tile, [T nsplit][ceil(nJ/32)][32] (mask_phase)
     uint32_t *funion;      // ... and per word of 32 tiles those with any
@@ -1190,7 +1191,7 @@ __device__ __forceinline__ void far_phase(const FastArgs &a, Smem &S, float *big
             }
             if (K != lastK) {
                 cont = K == lastK + 1;
-                if (++ord > kLastOrd) {
+                if (++ord > a.last_ord) {
                     __syncthreads();  // the folds of the entry before are done
                     flush();
                     __syncthreads();
@@ -2240,7 +2241,7 @@ static bool plan_panels(size_t scratch, int nsm, int nJ, int G, int Gc, int nspl
 }
 
 int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, const Layout &Lw, cudaStream_t st,
-                   bool exact_s, bool exact_tables, float *costs, bool build_costs, bool test_stall,
+                   bool exact_s, bool exact_tables, float *costs, bool build_costs, bool test_stall, bool short_parts,
                    size_t chunk_bytes, bool seeded, bool unbounded, bool tables) {
     double *dp64 = wsp<double>(ws, Lw.dp64);
     int32_t *bp = wsp<int32_t>(ws, Lw.bp);
@@ -2298,7 +2299,8 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     PanelPlan pl;
     if (!plan_panels(scratch_bytes(Lw.d, s), nsm, a.nJ, G, a.Gc, a.nsplit, s, !costs, &pl)) return ECASQ_EWORKSPACE;
     a.T = pl.T;
-    a.workers = pl.workers;
+    a.workers = short_parts ? std::min(pl.workers, 4) : pl.workers;
+    a.last_ord = short_parts ? 2 : kLastOrd;
     a.dlast = reinterpret_cast<float *>(scratch + pl.dlast);
     a.tmin = reinterpret_cast<int *>(scratch + pl.tmin);
     a.tmin1 = reinterpret_cast<float *>(scratch + pl.tmin1);

@@ -132,7 +132,7 @@ def test_binding_constants_match_the_header():
         defs[name] = eval(expr, {"__builtins__": {}})
     codes = {"OK", "EINVAL", "ENONFINITE", "EINFEASIBLE", "EWORKSPACE", "ECUDA", "ETIMEOUT", "ERANGE"}
     flags = {"EXACT_S", "NO_REFINE_GUARD", "DP_REFERENCE", "TIME_KERNELS", "EXACT_TABLES", "RESIDENT_COSTS",
-             "STREAMED_COSTS", "ONE_PART_PUBLISH", "UNSEEDED_SEARCH", "TEST_STALL", "TEST_SELF_SEED"}
+             "STREAMED_COSTS", "ONE_PART_PUBLISH", "UNSEEDED_SEARCH", "TEST_STALL", "TEST_SELF_SEED", "TEST_SHORT_PARTS"}
     for name in codes | flags:
         assert name in defs, name
         assert getattr(native, name) == defs[name], (name, getattr(native, name), defs[name])
