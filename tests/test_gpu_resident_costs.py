@@ -238,10 +238,10 @@ def test_streamed_costs_budgeted_solve_matches_oracle(E, oracle_mod):
 
 
 @pytest.mark.parametrize("name,s", [("lognormal16k", 16), ("studentt9000", 12), ("normal5000", 10)])
-def test_two_part_publish_bit_identical_to_one_part(E, name, s):
-    """Publishing each column block in two parts (rows 2..8 after layer 8, then the rest) lets the
-    next block start its last tile and first layers early; the results are those of the one-part
-    publish: the same tables, resolved and unresolved outputs alike."""
+def test_cost_modes_give_the_same_tables(E, name, s):
+    """Costs built panel by panel, in a table or in bands: every output resolved exactly, the same
+    tables, codebooks and metrics over many panels (and bands).  ECASQ_ONE_PART_PUBLISH is accepted
+    and changes nothing."""
     if name == "lognormal16k":
         x = workloads.signed_lognormal(16384, 0)
     elif name == "studentt9000":
@@ -249,22 +249,25 @@ def test_two_part_publish_bit_identical_to_one_part(E, name, s):
     else:
         x = workloads.normal(5000, 7)
     lams = [0.0, 1e-4, 0.01, 0.1, 0.4, 1.0, 3.0, 30.0]
-    for costs_flag in (E.RESIDENT_COSTS, E.STREAMED_COSTS):
-        ws1 = E.workspace(x.size, s, flags=costs_flag)
+    ws1 = E.workspace(x.size, s)
+    Q1, m1, met1 = E.ecasq_dp_pass(x, s, lams, flags=E.EXACT_TABLES, ws=ws1)
+    tables = _tables(E, ws1, len(lams), s, x.size)
+    for costs_flag in (E.RESIDENT_COSTS | E.ONE_PART_PUBLISH, E.STREAMED_COSTS):
         ws2 = E.workspace(x.size, s, flags=costs_flag)
-        Q1, m1, met1 = E.ecasq_dp_pass(x, s, lams, flags=costs_flag | E.ONE_PART_PUBLISH, ws=ws1)
-        Q2, m2, met2 = E.ecasq_dp_pass(x, s, lams, flags=costs_flag, ws=ws2)
+        Q2, m2, met2 = E.ecasq_dp_pass(x, s, lams, flags=costs_flag | E.EXACT_TABLES, ws=ws2)
         for ws in (ws1, ws2):
             st = E.native.ws_status(ws)
             assert st["timeout"] == 0 and st["bound_viol"] == 0
         assert m1 == m2
         np.testing.assert_array_equal(Q1.cpu().numpy(), Q2.cpu().numpy())
         np.testing.assert_array_equal(met1, met2)
-        for (dp1, bp1), (dp2, bp2) in zip(_tables(E, ws1, len(lams), s, x.size), _tables(E, ws2, len(lams), s, x.size)):
+        for (dp1, bp1), (dp2, bp2) in zip(tables, _tables(E, ws2, len(lams), s, x.size)):
             np.testing.assert_array_equal(dp1, dp2)
             np.testing.assert_array_equal(bp1, bp2)
-        del ws1, ws2
+        del ws2
         _free()
+    del ws1
+    _free()
 
 
 @pytest.mark.parametrize("name,s,b,mode", [("studentt16k", 16, 2.5, "RESIDENT_COSTS"),
