@@ -45,15 +45,14 @@ METRIC = "ECASQ approx-DP solve ms & candidate evals/s at d=2^17,s=16; % of ALU 
 UNIT = "candidate evals/s"
 FP32_LANES = 128          # FP32-pipe lanes per SM (adds and min/max share them)
 SM_MAX_MHZ = 2070.0
-# Ops the min-plus kernel issues per candidate: one add (packed f32x2) and one min
-# (3-input integer min on the float bits).  W = C + lambda' Phi is formed once per
-# (pair, multiplier) and shared by every layer, so the FMA that a per-candidate count
-# (add + FMA + min = 3) includes is 1/(s-2) of an op per candidate here.
+# Ops counted per candidate: one add (packed f32x2) and one min (3-input integer min on
+# the float bits).  W = C + lambda' Phi is the same for every layer of a (pair, multiplier);
+# the near phase forms it once, the far phase again in each task (an FMA that is not counted).
 OPS_PER_CANDIDATE = 2
 BK = BJ = 64              # the kernel's tile: 64 k by 64 columns
-# DRAM bytes of the min-plus kernel per interval-cost tile it copies in: the tile's 34 816 B of C
-# and Phi, each fetched tile read once in a pass.  (A capture of one solve at d = 16384 reads less in
-# late passes, whose tiles stay in L2; at d = 131072 a pass fetches 26 GB.)
+# Bytes that the min-plus kernel copies per interval-cost tile: the tile's 34 816 B of C and Phi, each
+# fetched tile once in a pass, from HBM or L2 -- an upper bound of the DRAM reads.  (Of one solve's copies at
+# d = 16384, 3.66 GB, 1.95 GB came from HBM; at d = 131072 a pass copies 26 GB.)
 TRAFFIC_PER_FETCHED_TILE = 34816
 ORACLE_SAMPLE = 16384     # entries of the CPU baseline's bounded sample
 
@@ -416,8 +415,8 @@ def run_rows_mode(args):
                         "traffic": None, "kernel": "k_rows_pass",
                         "candidates_per_step": cand,
                         "note": "2 ops per candidate of eq. apx_rec over the whole step; the first search round "
-                                "builds each row's binary64 pair costs (binary64 pipe), the later rounds are "
-                                "latency-bound at two 8-warp blocks per SM (shared memory per row)"},
+                                "builds each row's fp32 pair costs, every round runs three 8-warp blocks an SM (shared "
+                                "memory per row); more than half of the step is the host's search"},
            "gpu_launches": E.ecasq_kernel_launches() - launches0, "clocks": clocks}
     print(json.dumps(out), flush=True)
 
@@ -631,7 +630,8 @@ def main():
                if (flags & E.RESIDENT_COSTS) and TRAFFIC_PER_FETCHED_TILE else None)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TOP/s",
                 "frac": (achieved / peak) if achieved else None, "traffic": traffic,
-                "traffic_note": "DRAM bytes per launch: the bytes of a cost tile times the tiles this launch fetched",
+                "traffic_note": "bytes copied per launch, from HBM or L2 (an upper bound of its DRAM reads): the bytes of a "
+                                "cost tile times the tiles this launch fetched",
                 "tiles_fetched_per_launch": fetched_per_launch,
                 "kernel": "k_wavefront",
                 "peak_basis": "%d SMs (device attribute) x 128 FP32-pipe lanes (adds and mins share the issue "
@@ -639,8 +639,8 @@ def main():
                 "avg_launch_ms": dp_ms / max(dp_launches, 1), "launches": dp_launches,
                 "ops_basis": "executed: 2 ops (add, min) per candidate the kernel evaluated -- %d-column x %d-k "
                              "tile units it ran, times the s-2 layers, plus its diagonal blocks; "
-                             "C + lambda' Phi is formed once per pair and multiplier, so a 3-op count "
-                             "(add + FMA + min) would add 1/(s-2) op per candidate" % (BJ, BK),
+                             "the FMA of C + lambda' Phi, which the far phase repeats per candidate, "
+                             "is not counted" % (BJ, BK),
                 "executed_candidates_per_launch": executed / last_launches,
                 "effective": effective,
                 "effective_frac": (effective / peak) if effective else None,

@@ -52,7 +52,9 @@ typedef struct CUstream_st *ecasq_stream_t; /* same type as cudaStream_t */
 #define ECASQ_EXACT_S 1u          /* use exactly s values (eq. apx_final with i = s only) */
 #define ECASQ_NO_REFINE_GUARD 2u  /* refinement may raise H(Xhat) above the budget */
 #define ECASQ_DP_REFERENCE 4u     /* run the fp64 reference DP kernel instead of the fast kernel */
-#define ECASQ_TIME_KERNELS 8u     /* time the DP kernels with CUDA events (ecasq_result_t.dp_kernel_ms) */
+#define ECASQ_TIME_KERNELS 8u     /* time the DP kernels with CUDA events (ecasq_result_t.dp_kernel_ms); in ecasq_solve_batched
+                                     rows of more than 128 unique values are then solved one by one, as only the
+                                     single solve times its kernel (the call takes far longer than without the flag) */
 #define ECASQ_EXACT_TABLES 16u    /* resolve every DP output exactly (default: only what eq. apx_final and the traceback read) */
 #define ECASQ_RESIDENT_COSTS 32u  /* fast DP: compute the lambda-independent interval costs C and Phi (Sec. 5, App. E)
                                      once per call into the workspace and stream them to every pass (workspace:
@@ -77,8 +79,8 @@ typedef struct CUstream_st *ecasq_stream_t; /* same type as cudaStream_t */
                                      one's fp32 minima (the seed then equals every output's minimum, the tightest
                                      start the seeding allows); results must equal those without the flag.
                                      ecasq_result_t.passes counts both.  Not for production use. */
-#define ECASQ_TEST_STALL (1u << 30) /* test hook for the bounded device waits: column block 0 of the fast DP's
-                                     wavefront is never published and the waits on it give up after 2^14 spins, so
+#define ECASQ_TEST_STALL (1u << 30) /* test hook for the bounded device waits: the minima of column block 0 of the fast
+                                     DP's wavefront are never written and the waits on them give up after 2^14 spins, so
                                      the call must return ECASQ_ETIMEOUT (nothing else) and leave the workspace
                                      usable by the next call.  Not for production use. */
 
@@ -216,7 +218,7 @@ int ecasq_solve_timeshare(const float *x, int64_t d, const float *P, int64_t n, 
  *   idx     device [d] uint8 output: index into the entry's codebook
  *   sel     device [d] uint8 output (may be NULL): 1 where Qp was used
  *   counts  device [mm + mp] uint32 output: index histograms of Qm, then Qp
- *   ws      device, >= 256 bytes, 256-byte aligned (status record)
+ *   ws      device, >= 256 bytes, 256-byte aligned (status record and, where they fit, counts)
  *   rate    host (may be NULL): bits per entry of coding each part with its own
  *           empirical law, -(1/d) sum_parts sum_r c_r log2(c_r / n_part)
  * ECASQ_EINVAL for beta outside [0, 1], non-ascending codebooks or mp = 0 with
@@ -322,8 +324,9 @@ int ecasq_evaluate(const float *x, int64_t d, const float *Q, int32_t m, void *w
  *   idx     device [d] uint8 output
  *   counts  device [m] uint32 output: index histogram
  *   h_emp   host, output (may be NULL): empirical entropy of idx (Sec. 1)
- * ECASQ_ERANGE if an entry lies outside [Q[0], Q[m-1]].  Synchronises
- * `stream` only when h_emp is not NULL. */
+ * ECASQ_EINVAL for a codebook that is not strictly ascending, ECASQ_ERANGE if an
+ * entry lies outside [Q[0], Q[m-1]].  ws: device, 256-byte aligned, 256 bytes or more (the
+ * status record and, where they fit, the counts).  Synchronises `stream`. */
 int ecasq_quantize(const float *x, int64_t d, const float *Q, int32_t m, uint64_t seed, uint8_t *idx,
                    uint32_t *counts, void *ws, size_t ws_bytes, double *h_emp, ecasq_stream_t stream);
 
@@ -364,7 +367,8 @@ int ecasq_quantize_noalloc(const float *x, int64_t d, const float *Q, int32_t m,
 /* Budgeted solves of `rows` independent rows of length d (row-major X),
  * each exactly as ecasq_solve would do it on that row alone (same schedule,
  * same results).  Q [rows * s] device, m_out [rows] device, res host [rows]
- * (may be NULL).  Synchronises `stream`. */
+ * (may be NULL).  ECASQ_ENONFINITE when any row of at most 1024 entries without
+ * refinement holds a NaN or Inf: then no row's results are written.  Synchronises `stream`. */
 int ecasq_solve_batched(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws,
                         size_t ws_bytes, float *Q, int32_t *m_out, ecasq_result_t *res,
                         ecasq_stream_t stream);

@@ -199,7 +199,7 @@ struct RowsLayout {
     int slots;
 };
 // Rows searched together: all of them while their pairs' costs stay small, else as many as fit 1 GB, and at
-// least one a block slot of an SM.
+// least one an SM of 152 (a size of the workspace, so no device's).
 static int64_t rows_chunk(int64_t d, int64_t rows) {
     if (d <= kRowsMaxP) return rows;
     return std::min(rows, std::max<int64_t>(152, ((int64_t)1 << 30) / (4 * d * (d - 1))));

@@ -171,7 +171,7 @@ struct RowsData {
 
 // One search round of the batched path (rows.cu): block b runs rows[b], rows[b + gridDim], .. at G multipliers.
 constexpr int kRowsMaxP = 128;   // unique values up to which a row's pair costs fit shared memory
-constexpr int kRowsSlots = 456;  // blocks of a round, at most (three an SM)
+constexpr int kRowsSlots = 456;  // blocks of a round, at most: three an SM of 152 (a size of the workspace, so no device's)
 struct RowsPass {
     RowsData R;
     const int32_t *rows;  // [nact]

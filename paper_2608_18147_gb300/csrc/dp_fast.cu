@@ -313,8 +313,6 @@ __device__ __forceinline__ void bulk_g2s_nohint(void *dst, const void *src, uint
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-// global writes seen through generic loads/acquire -> ordered before later bulk copies
-__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
@@ -543,7 +541,7 @@ __global__ void __launch_bounds__(NPROD) k_build_costs(const __grid_constant__ F
 // The column blocks go in panels of a.T (15 on this GPU) consecutive blocks [P0, P0 + nb), one
 // after the other.  Within a panel, grid barriers between the steps:
 //  1. bound_phase: upper bounds of the minima over the far tiles (K < P0, whose dp rows are all
-//     final) from one candidate per tile;
+//     final) from one candidate of every fourth tile;
 //  2. mask_phase: the far tasks -- (tile, multiplier, layer) -- that may matter, by the skip test
 //     against the bounds;
 //  3. far_phase: the tiles with tasks in one list, an equal share of the work for each CTA; a CTA's
@@ -563,10 +561,11 @@ __global__ void __launch_bounds__(NPROD) k_build_costs(const __grid_constant__ F
 // far tiles are shared evenly.  A pass of 8 multipliers (mean over a budgeted search, resident
 // costs): 22.5 ms instead of 46.3 at d = 2^17, s = 16; 1.47 instead of 2.93 at d = 16384, s = 16;
 // 12.9 instead of 47.7 at d = 50001, s = 32; building its own costs, 2.4 instead of 8.4 at
-// d = 12289, s = 16.  Of the 22.5 ms about 10.5 are far tiles, 2.5 uneven shares, 5 masks, 2.5
-// bounds and 3 the near phases; far tiles are bound by issue (one add and one min a candidate
-// on the two FP32 pipes reach about 53 candidates per cycle and SM) and by the copies and
-// barriers of a tile, which cost as much as about 6 of its tasks (kTileCost).
+// d = 12289, s = 16.  Of the 22.5 ms 11.0 are far tiles, 2.4 uneven shares, 2.8 masks, 1.4 bounds, 2.4
+// the near phases, 0.8 the fold and 1.7 barriers and the rest.  Far tiles are bound by the latency of one tile's
+// chain -- copies, costs into registers, a batch of tasks, a barrier, the fold: about 3000 cycles
+// with eight tasks, at most 13 candidates per cycle and SM where the adds and mins alone would
+// reach 53 -- so a tile costs as much as about 6 of its tasks on top of them (kTileCost).
 
 // Grid barrier `epoch` (1, 2, ...): bounded; false when it gave up or another CTA aborted.  All
 // CTAs are resident (cooperative launch).  Orders generic and bulk-copy accesses on both sides.
@@ -620,13 +619,12 @@ __device__ __forceinline__ int *ub_at(const FastArgs &a, int Jl, int g) {
 }
 
 // Upper bounds of the panel's far minima: for every output the least candidate over the last k
-// of each far tile, dp(i-1, 64K+63) + C + lambda' Phi with C and Phi from the tile's summary (where
-// the summary is that k's, which it nearly always is) -- a candidate's own fp32 value, so never
-// below the minimum, and within the change of the candidates over one tile of it.  Tiles are then
+// of every fourth far tile (a.bound_step), dp(i-1, 64K+63) + C + lambda' Phi with C and Phi from the tile's
+// summary (where the summary is that k's, which it nearly always is) -- a candidate's own fp32 value, so never
+// below the minimum, and within the change of the candidates over a few tiles of it.  Tiles are then
 // skipped as if the minimum were known (far_start), whatever the order of the walk.  One candidate of
-// 64 is evaluated for it; at d = 2^17, s = 16 the share of (multiplier, tile) units with any work in a
-// search falls from 0.28 (a walk that knows the tiles to its left) to 0.17, and most of the layers
-// of those drop out too (mask_phase).
+// 256 is evaluated for it; a budgeted search at d = 2^17, s = 16 then runs 5 % of the (tile, multiplier, layer)
+// tasks (mask_phase).
 // CTAs split the panel's (column block, tile range) pairs evenly; a thread owns one column of one
 // multiplier, kBoundL layers at a time.
 constexpr int kBoundL = 16;
@@ -719,8 +717,8 @@ __device__ __forceinline__ float4 far_start(const FastArgs &a, const int *u, int
 // is monotone); when lb exceeds the output's band limit bb + bb tau, the tile changes neither its
 // minimum nor its band.  For row js = split * nb + Jl, a.fbits has 128 task bits a tile, and for each word
 // of 32 tiles a.funion says which have any and a.fweight the word's work: the tasks, and kTileCost a tile.
-// With the bounds a needed tile has 1.6 (first pass) to 3.4 (late passes) of its 14 layers needed per
-// multiplier that needs it at d = 2^17, s = 16, so tasks, not whole tiles, are the unit of work.
+// A tile that is copied in has 14 of its 112 tasks needed at d = 2^17, s = 16 (mean of a search), so
+// tasks, not whole tiles, are the unit of work.
 // CTAs split the (column block, word range) pairs as in bound_phase; a thread tests one column of one
 // multiplier, kBoundL layers at a time.
 constexpr int kTileCost = 6;  // a listed tile's fixed cost (its copies, its costs into registers) in tasks (a pass at d = 2^17, s = 16: 22.5 ms
@@ -923,7 +921,7 @@ __device__ __forceinline__ uint2 *seg_runs(const FastArgs &a, float *seg) {
 // The far phase of one panel: this CTA's share of the list, the tiles whose position lies in
 // [share c, share (c + 1)), in entries of at most a.tcap tasks.  Sixteen warps take 8 of the tile's 64 k and
 // 32 of its columns each, the costs in registers (a lane: one column), and go through the entry's tasks
-// eight at a time: C + lambda' Phi once a multiplier, the task's dp row (one address a warp: a single
+// eight at a time: C + lambda' Phi, the task's dp row (one address a warp: a single
 // shared-memory access), the least of 8 candidates into a slot of the column's eight partial minima.
 // After one barrier a pair of warps takes each of the eight tasks, and a lane folds its column's minimum
 // into the band state (shared memory) while the next eight tasks start.  So a tile's costs are read
@@ -2344,7 +2342,7 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     // corner states: needed by every tile that is built (per pass, or once into the table)
     if (a.nJ > 1 && (!costs || build_costs)) {
         note_launch();
-        k_corners<<<(unsigned)std::min<int64_t>(cdiv((int64_t)a.nJ * (a.nJ - 1) / 2, 128), 152 * 64), 128, 0, st>>>(a);
+        k_corners<<<(unsigned)std::min<int64_t>(cdiv((int64_t)a.nJ * (a.nJ - 1) / 2, 128), (int64_t)nsm * 64), 128, 0, st>>>(a);
         ECASQ_LAUNCH_CHECK();
     }
     int smem_max = 0;

@@ -1,7 +1,8 @@
 """ECASQ_RESIDENT_COSTS: the interval costs C and Phi (Sec. 5, App. E) built once
 per call into the workspace and streamed to every DP pass.  The tiles are
-computed by the same code as the fused kernel's producer, so every fp32
-minimum and every exact decision equals the fused mode's; the results match
+computed by the same code as without a table (there, panel by panel in every pass: the
+default mode, "fused" in the tests' names), so every fp32 minimum and every exact
+decision equals that mode's; the results match
 the oracle under the same bar as the other fast-DP tests (pytest -m gpu)."""
 import numpy as np
 import pytest
@@ -43,8 +44,7 @@ def _tables(E, ws, G, s, d):
 def test_resident_costs_bit_identical_to_fused(E, name, s, flags_name):
     """Same codebooks and metrics with and without resident costs; the same
     exact tables; the same fp32 minima where the closure left outputs unresolved.
-    At s = 32 and s = 18 the resident kernel runs eight layers per thread (the fused
-    kernel seven)."""
+    At s = 32 the far tiles go in splits of four multipliers, at s = 18 a tile has all 128 tasks."""
     x = {"lognormal16k": lambda: workloads.signed_lognormal(16384, 0),
          "ragged2049": lambda: workloads.student_t(2049, 3, scale=1.0),
          "mixture12k": lambda: workloads.mixture(12288, 2),
@@ -191,7 +191,7 @@ def test_full_size_sampled_decisions(E, oracle_mod):
 @pytest.mark.parametrize("name,s", [("lognormal16k", 16), ("ragged20001", 9), ("mixture12k", 32)])
 def test_streamed_costs_bit_identical_to_fused(E, name, s, flags_name):
     """ECASQ_STREAMED_COSTS builds the cost tiles band by band into a bounded buffer and runs
-    the wavefront over each band: the same fp32 values as the fused producer's, so the same
+    the wavefront over each band: the same fp32 values as without a table, so the same
     tables (resolved and unresolved outputs alike), codebooks and metrics, over several bands."""
     if name == "lognormal16k":
         x = workloads.signed_lognormal(16384, 0)
@@ -275,7 +275,7 @@ def test_cost_modes_give_the_same_tables(E, name, s):
                                            ("studentt20001", 12, 2.5, "RESIDENT_COSTS"),
                                            ("normal8192", 10, 2.0, "RESIDENT_COSTS"),
                                            ("studentt16k", 16, 2.5, "STREAMED_COSTS"),
-                                           ("mixture12k", 32, 4.0, "RESIDENT_COSTS"),   # 8 layers per thread
+                                           ("mixture12k", 32, 4.0, "RESIDENT_COSTS"),   # two far splits
                                            ("ragged5000", 18, 2.5, "STREAMED_COSTS")])
 def test_seeded_search_bit_identical_to_unseeded(E, name, s, b, mode):
     """Later passes of the search start their tile skipping from the fp32 minima of the
@@ -308,7 +308,7 @@ def test_seeded_search_bit_identical_to_unseeded(E, name, s, b, mode):
         np.testing.assert_array_equal(dps, dpu)
         np.testing.assert_array_equal(bps, bpu)
     assert sts["tiles_run"] <= stu["tiles_run"]
-    assert stu["tiles_skipped"] > 0  # tile skipping runs at every s here (even layer groups)
+    assert stu["tiles_skipped"] > 0  # tile skipping runs at every s
     if name == "studentt16k":  # five seeded passes at multipliers where most tiles are skipped
         assert sts["tiles_run"] < 0.95 * stu["tiles_run"]
 
@@ -316,8 +316,8 @@ def test_seeded_search_bit_identical_to_unseeded(E, name, s, b, mode):
 @pytest.mark.parametrize("lam", [0.0, 0.05])
 @pytest.mark.parametrize("name,s,mode", [("studentt16k", 16, "RESIDENT_COSTS"),
                                          ("lognormal16k", 16, "RESIDENT_COSTS"),
-                                         ("mixture12k", 17, "RESIDENT_COSTS"),  # 8 layers per thread
-                                         ("ragged5000", 18, "STREAMED_COSTS")])  # 8 layers per thread
+                                         ("mixture12k", 17, "RESIDENT_COSTS"),
+                                         ("ragged5000", 18, "STREAMED_COSTS")])
 def test_self_seeded_pass_bit_identical(E, name, s, mode, lam):
     """A fixed-multiplier pass seeded with its own fp32 minima: every running minimum
     starts at the output's final value, the tightest seed that the monotonicity of the
@@ -349,5 +349,5 @@ def test_self_seeded_pass_bit_identical(E, name, s, mode, lam):
     np.testing.assert_array_equal(bp0, bp1)
     # the counters add up over a call's passes: the seeded pass is the second one
     assert st1["tiles_run"] <= 2 * st0["tiles_run"]
-    assert st0["tiles_skipped"] > 0  # 8 layers per thread at s = 17 and 18: tile skipping with one multiplier
+    assert st0["tiles_skipped"] > 0  # with one multiplier too
     assert st1["tiles_run"] - st0["tiles_run"] < st0["tiles_run"]

@@ -1,11 +1,11 @@
 """The min-plus wavefront's bounded device waits (run on a GB300: pytest -m gpu).
 
-A column block of the wavefront may be consumed only after its owner published it;
-every wait on such a flag gives up after a spin limit, records a timeout in the
-workspace's status record, raises the kernel's abort flag (so the other CTAs stop
-waiting too) and returns.  The ECASQ_TEST_STALL hook makes that happen on purpose
-without faulting anything: block 0 is never published and the spin limit drops to
-2^14 spins.  The call must return ECASQ_ETIMEOUT within a short time, and the next
+A layer's minima of a column block are read as soon as their owner wrote them (they are
+their own flags), and grid barriers stand between the phases; every wait on another CTA
+gives up after a spin limit, records a timeout in the workspace's status record, raises
+the kernel's abort flag (so the other CTAs stop waiting too) and returns.  The
+ECASQ_TEST_STALL hook makes that happen on purpose without faulting anything: block 0's
+minima are never written and the spin limit drops to 2^14 spins.  The call must return ECASQ_ETIMEOUT within a short time, and the next
 call on the same workspace must run normally and give the same results as a call on
 a fresh workspace.
 """
