@@ -111,7 +111,7 @@ struct FastArgs {
     int T;                 // column blocks per panel
     int workers;           // CTAs that share the far tiles
     int tcap;              // tasks per far list entry, at most (16 .. 64)
-    int last_ord;          // a far segment's part: tiles 0 .. last_ord (kLastOrd; lower in the test hook)
+    int first_ord;         // ordinal of a far segment's first tile: 0 (higher in the test hook: shorter parts)
     float *part;           // [workers + T nsplit] segments: minima [Gc][s-2][64], then runs (seg_min, seg_runs)
     uint4 *fbits;          // far tasks: 128 bits a tile, [T nsplit][ceil(nJ/32)][32] (mask_phase)
     uint32_t *funion;      // ... and per word of 32 tiles those with any
@@ -1182,19 +1182,19 @@ __device__ __forceinline__ void far_phase(const FastArgs &a, Smem &S, float *big
                 else if (jsn != js0) empty(js0);
                 __syncthreads();
                 js = jsn;
-                ord = -1;
+                ord = a.first_ord - 1;
                 lastK = -2;
                 next = false;
                 start();
             }
             if (K != lastK) {
                 cont = K == lastK + 1;
-                if (++ord > a.last_ord) {
+                if (++ord > kLastOrd) {
                     __syncthreads();  // the folds of the entry before are done
                     flush();
                     __syncthreads();
                     next = true;
-                    ord = 0;
+                    ord = a.first_ord;
                     for (int o = ct; o < nt * BJ; o += MAXCONS) sruns[o] = kNoRuns;
                 }
                 if (ct == 0) S.okey[ord] = (uint16_t)K;
@@ -2298,7 +2298,7 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     if (!plan_panels(scratch_bytes(Lw.d, s), nsm, a.nJ, G, a.Gc, a.nsplit, s, !costs, &pl)) return ECASQ_EWORKSPACE;
     a.T = pl.T;
     a.workers = short_parts ? std::min(pl.workers, 4) : pl.workers;
-    a.last_ord = short_parts ? 2 : kLastOrd;
+    a.first_ord = short_parts ? kLastOrd - 2 : 0;
     a.dlast = reinterpret_cast<float *>(scratch + pl.dlast);
     a.tmin = reinterpret_cast<int *>(scratch + pl.tmin);
     a.tmin1 = reinterpret_cast<float *>(scratch + pl.tmin1);
