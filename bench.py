@@ -354,7 +354,7 @@ def run_hbm_mode(args):
                config={"workload": "normal, 2^28 entries (encode), 2^26 (prepare)", "mode": "hbm",
                        "codebook": int(Q.numel()), "l2": "vectors of 1 GiB and 256 MiB, far above the 129 MB L2"},
                roofline={"bound": "hbm", "achieved": gbs_q, "peak": peak, "unit": "GB/s", "frac": gbs_q / peak,
-                         "traffic": None, "kernel": "k_quantize", "peak_basis": "MEASURED_PEAKS.json hbm_gbs"},
+                         "traffic": None, "kernel": "k_quantize_short", "peak_basis": "MEASURED_PEAKS.json hbm_gbs"},
                rows={"encode": {"ms": ms_q, "bytes_per_entry": 5, "GBs": gbs_q, "frac": gbs_q / peak},
                      "encode_timeshare": {"ms": ms_t, "bytes_per_entry": 6, "GBs": gbs_t, "frac": gbs_t / peak},
                      "prepare": {"ms": ms_p, "bytes_per_entry": 32, "GBs": gbs_p, "frac": gbs_p / peak,
@@ -408,15 +408,15 @@ def run_rows_mode(args):
     achieved = 2.0 * cand / (ms / args.steps / 1000.0) / 1e12
     out = {"metric": "ECASQ batched solve: rows/s", "value": args.steps * rows / (ms / 1000.0), "unit": "rows/s",
            "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
-           "higher_is_better": True, "vs_baseline": None, "dtype": "f64", "data": "synthetic",
-           "config": {"workload": name, "mode": "rows", "rows": rows, "d": d, "s": s, "budget_bits": budget},
+           "higher_is_better": True, "vs_baseline": None, "dtype": "f32 (fp64 where a decision is ambiguous)",
+           "data": "synthetic", "config": {"workload": name, "mode": "rows", "rows": rows, "d": d, "s": s, "budget_bits": budget},
            "rows_ok": ok, "mean_m": float(m.float().mean().item()),
            "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TOP/s", "frac": achieved / peak,
                         "traffic": None, "kernel": "k_rows_pass",
                         "candidates_per_step": cand,
                         "note": "2 ops per candidate of eq. apx_rec over the whole step; the first search round "
                                 "builds each row's fp32 pair costs, every round runs three 8-warp blocks an SM (shared "
-                                "memory per row); more than half of the step is the host's search"},
+                                "memory per row); about half of the step is the host's search"},
            "gpu_launches": E.ecasq_kernel_launches() - launches0, "clocks": clocks}
     print(json.dumps(out), flush=True)
 

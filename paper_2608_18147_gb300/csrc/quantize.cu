@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(kQThreads) k_quantize(const float *__restrict_
 
 // ------------------------------------------------ short codebooks (m <= 16)
 // The same decisions as k_quantize, and as k_quantize_timeshare with two codebooks (TS), with fewer
-// instructions per entry.  What bounds it: instructions, 69 an entry in an earlier form and 46 now, half of
-// them on the pipe for integer logic and compares.  So
+// instructions per entry.  What bounds it: instruction issue, 69 instructions an entry in an earlier form and 50 now
+// (16 values; issue 76 %), then the pipe for integer logic and compares (63 %).  So
 //  * the search takes STEPS = ceil(log2 m) unrolled steps (a template argument); its position is a byte offset
 //    that steps by predicated float adds of denormals (bit patterns 4, 8, ..: exact), which the otherwise
 //    idle fp32 pipe takes;
