@@ -1258,6 +1258,16 @@ int ecasq_quantize_timeshare(const float *x, int64_t d, const float *Qm, int32_t
     return ECASQ_OK;
 }
 
+// The result of a row without a codebook of the required size (ecasq_solve leaves its result alone then).
+static ecasq_result_t no_codebook(int64_t d, int64_t p) {
+    ecasq_result_t one;
+    memset(&one, 0, sizeof(one));
+    one.status = ECASQ_EINFEASIBLE;
+    one.d = d;
+    one.p = p;
+    return one;
+}
+
 // Short rows (d <= kScanTile, no refinement): every row runs the multiplier search
 // of ecasq_solve in lockstep with the others -- one k_rows_pass launch per round
 // for all rows still searching -- with the per-row arithmetic of the reference DP,
@@ -1500,7 +1510,7 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
         }
         if (w.failed || w.sel < 0) {
             status = ECASQ_EINFEASIBLE;
-            if (res) { memset(&res[r], 0, sizeof(res[r])); res[r].status = ECASQ_EINFEASIBLE; res[r].d = d; res[r].p = ph[r]; }
+            if (res) res[r] = no_codebook(d, ph[r]);
             continue;
         }
         const Eval &e = w.evals[w.sel];
@@ -1527,7 +1537,7 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
     ECASQ_CUDA_TRY(cudaMemcpyAsync(&sum, ws, sizeof(sum), cudaMemcpyDeviceToHost, st));
     ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
     for (int64_t r : slow) {
-        ecasq_result_t one;
+        ecasq_result_t one = no_codebook(d, ph[r]);
         ecasq_params_t p1 = *prm;
         if (ph[r] <= kRowsMaxP) p1.flags |= ECASQ_DP_REFERENCE;
         rc = ecasq_solve(X + r * d, d, &p1, ws, roff, Q + r * s, &one, reinterpret_cast<ecasq_stream_t>(st));
@@ -1588,7 +1598,7 @@ int ecasq_solve_batched(const float *X, int64_t rows, int64_t d, const ecasq_par
         return solve_rows_batched(X, rows, d, prm, ws, ws_bytes, Q, m_out, res, st);
     int status = ECASQ_OK;
     for (int64_t r = 0; r < rows; r++) {
-        ecasq_result_t one;
+        ecasq_result_t one = no_codebook(d, 0);
         int rc = ecasq_solve(X + r * d, d, prm, ws, ws_bytes, Q + r * prm->s, &one, stream);
         if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
         if (rc == ECASQ_EINFEASIBLE) status = rc;

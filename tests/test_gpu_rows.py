@@ -113,3 +113,27 @@ def test_one_long_row_alone(E, d, s):
     _same(E, X, s, lambda_=0.3)
     X[0, 1:3] = [0.25, 0.75]
     _same(E, X, s, budget_bits=1.5)
+
+
+@pytest.mark.parametrize("kw", [dict(lambda_=0.3), dict(lambda_=1e30), dict(lambda_=0.3, refine_max_rounds=2)])
+def test_rows_without_a_codebook(E, kw):
+    """Exactly s values from fewer: status and sizes whichever path a row takes (1e30 is beyond fp32, refinement goes row
+    by row), and m = 0."""
+    import torch
+    X = np.random.default_rng(2).standard_normal((3, 9)).astype(np.float32)
+    X[1] = np.round(X[1])
+    rows, d = X.shape
+    ws = E.workspace(d, 17, rows)
+    prm, ptr = E.native.make_params(17, flags=E.EXACT_S, **kw), E.native._ptr
+    Q, m = torch.zeros((rows, 17), device="cuda"), torch.full((rows,), -7, dtype=torch.int32, device="cuda")
+    Xd, res = torch.as_tensor(X).cuda(), (E.native.Result * rows)()
+    C.memset(res, 0x5A, C.sizeof(res))
+    rc = E.lib().ecasq_solve_batched(ptr(Xd), rows, d, C.byref(prm), ptr(ws), ws.numel(), ptr(Q), ptr(m),
+                                     res, E.native._stream())
+    assert rc == E.native.EINFEASIBLE
+    assert m.cpu().numpy().tolist() == [0] * rows
+    for r in range(rows):
+        got = res[r].as_dict()
+        assert got["status"] == E.native.EINFEASIBLE and got["m"] == 0 and got["d"] == d and got["passes"] == 0
+        if not kw.get("refine_max_rounds"):
+            assert got["p"] == np.unique(X[r]).size
