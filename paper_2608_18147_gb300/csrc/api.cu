@@ -194,7 +194,7 @@ static int noalloc_scratch(cudaStream_t st, void **out) {
 // results, placed after the single-row layout (which the rows that cannot take the
 // batched path still use).
 struct RowsLayout {
-    size_t v, w, N, S, S2, p, norm2, nonfinite, dp, dp64, list, need, lam, act, mcount, metrics, qidx, sel, m, pairs, total;
+    size_t v, w, N, S, S2, p, norm2, nonfinite, dp, dp64, list, need, arg, cost, lam, act, mcount, metrics, qidx, sel, m, pairs, total;
     int64_t pstride;
     int slots;
 };
@@ -222,6 +222,8 @@ static size_t rows_layout(int64_t d, int32_t s, int64_t rows, RowsLayout *R) {
     R->dp64 = take(8 * layers * dc);
     R->list = take(2 * layers * dc);
     R->need = take(4 * layers * ((dc + 31) / 32));
+    R->arg = take(2 * layers * dc);
+    R->cost = take(8 * (size_t)R->slots * kMaxG * 96);
     R->lam = take(8 * n * kMaxG);
     R->act = take(4 * n);
     R->mcount = take(4 * n * kMaxG);
@@ -1366,6 +1368,8 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
         A.dp64 = reinterpret_cast<double *>(rb + RL.dp64);
         A.list = reinterpret_cast<uint16_t *>(rb + RL.list);
         A.need = reinterpret_cast<uint32_t *>(rb + RL.need);
+        A.arg = reinterpret_cast<uint16_t *>(rb + RL.arg);
+        A.cost = reinterpret_cast<double *>(rb + RL.cost);
         A.qidx = qid;
         A.mcount = mcd;
         A.metrics = metd;

@@ -182,6 +182,8 @@ struct RowsPass {
     double *dp64;         // [slots][kMaxG][s+1][dcap] exact values of ambiguous decisions
     uint16_t *list;       // ... and which ones
     uint32_t *need;       // [slots][kMaxG][s+1][ceil(dcap / 32)]
+    uint16_t *arg;        // [slots][kMaxG][s+1][dcap] their minimisers
+    double *cost;         // [slots][kMaxG][96] pairs that a warp evaluates side by side
     int32_t *qidx;        // [nact][G][s]
     int32_t *mcount;      // [nact][G]; -1: a row (or multiplier) that fp32 cannot take
     double *metrics;      // [nact][G][4]: MSE, H(I,B), H(Xhat) from 1 on

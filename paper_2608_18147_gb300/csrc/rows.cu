@@ -112,8 +112,11 @@ struct RowTrace {
     const float *dp;       // [s+1][p][8] fp32
     double *dp64;          // [s+1][p]: exact values of the closure's outputs
     uint16_t *list;        // [s+1][p]: the closure's outputs by layer
-    uint32_t *need;        // [s+1][nw]: ... as bits, all zero between closures
-    uint16_t *cnt;         // [s+1]: ... their number by layer
+    uint32_t *need;        // [s+1][nw]: ... as bits, all zero between traces
+    uint16_t *arg;         // [s+1][p]: ... their lowest minimisers
+    uint16_t *cnt, *from;  // [s+1]: ... their number by layer; before the present closure
+    uint32_t *key;         // [kRowsPairs]: pairs to evaluate
+    double *cost;          // [kRowsPairs]: ... and their costs
     const float *tau, *eps;
     double lam, scale;
     float lam32, slack, noise;
@@ -168,126 +171,229 @@ __device__ __forceinline__ int row_outside(const RowTrace &T, int i, int j, doub
     return row_within(T.dp[((size_t)i * T.p + j) * kMaxG + T.g], best, T.eps[i], T.slack, T.scale, i, T.noise) ? 0 : 1;
 }
 
+// Whether output (i, j) is listed, and so resolved once its closure is.
+__device__ __forceinline__ bool row_listed(const RowTrace &T, int i, int j) {
+    return (T.need[(size_t)i * T.nw + (j >> 5)] >> (j & 31)) & 1u;
+}
+// Lists the outputs kb + bits of `any` of layer i that are not listed yet, behind the n that are; their number then.
+__device__ __forceinline__ int row_list(const RowTrace &T, int i, int kb, unsigned any, int n) {
+    const int lane = threadIdx.x & 31;
+    uint32_t *word = T.need + (size_t)i * T.nw + (kb >> 5);
+    const unsigned fresh = any & ~*word;
+    __syncwarp();
+    if (lane == 0) *word |= any;
+    if ((fresh >> lane) & 1u) T.list[(size_t)i * T.p + n + __popc(fresh & ((1u << lane) - 1u))] = (uint16_t)(kb + lane);
+    return n + __popc(fresh);
+}
+// row_members for 32 outputs of layer i at once, a lane one: members among k = kb .. kb + 31 of output j.
+__device__ __forceinline__ unsigned row_members_of(const RowTrace &T, int i, int j, int kb, float lim) {
+    unsigned in = 0u;
+    const float *d = T.dp + ((size_t)(i - 1) * T.p + kb) * kMaxG + T.g;
+    const float2 *cp = T.cf + pair_at(kb, j, T.p);
+#pragma unroll 8
+    for (int t = 0; t < 32; t++) {
+        const int k = kb + t;
+        float v = CUDART_INF_F;
+        if (k < j) {
+            const float2 c = *cp;
+            v = __fadd_rn(d[t * kMaxG], __fmaf_rn(T.lam32, c.y, c.x));
+        }
+        cp += T.p - k - 2;  // the next k's row starts one pair later
+        if (k < j && !(v > lim)) in |= 1u << t;
+    }
+    return in;
+}
+constexpr int kRowsPairs = 64;  // costs that are evaluated side by side (RowsPass::cost: 64 costs, 64 keys)
+constexpr int kRowsWide = 8;    // outputs of a layer from which a lane takes one
+
+// Candidates T.key[at .. at + n - 1] (j << 10 | k) of layer i, n <= 32, a lane one: into their outputs' least value and
+// lowest minimiser.
+__device__ __forceinline__ void row_evaluate_pairs(const RowTrace &T, int i, int at, int n) {
+    const int lane = threadIdx.x & 31, p = T.p;
+    const unsigned full = 0xffffffffu;
+    const bool have = lane < n;
+    const uint32_t f = have ? T.key[at + lane] : 0u;
+    int k = (int)(f & 1023u);
+    const int j = have ? (int)(f >> 10) : -1 - lane;
+    double c = CUDART_INF;
+    if (have) c = __dadd_rn(i == 3 ? row_base(T, k) : T.dp64[(size_t)(i - 1) * p + k], row_cost(T, k, j));
+    const unsigned peers = __match_any_sync(full, j);
+    const bool leader = have && lane == __ffs(peers) - 1;
+    for (unsigned rest = __ballot_sync(full, leader && (peers & (peers - 1u))); rest; rest &= rest - 1u) {
+        const int l = __ffs(rest) - 1;
+        const bool mine = (__shfl_sync(full, peers, l) >> lane) & 1u;
+        const long long own = mine ? order_key(c) : 0x7fffffffffffffffll;
+        long long x = own;
+        int y = mine ? k : 0x7fffffff;
+        for (int o = 16; o; o >>= 1) {
+            const long long x2 = __shfl_xor_sync(full, x, o);
+            const int y2 = __shfl_xor_sync(full, y, o);
+            if (x2 < x || (x2 == x && y2 < y)) { x = x2; y = y2; }
+        }
+        const double least = __shfl_sync(full, c, __ffs(__ballot_sync(full, mine && own == x && k == y)) - 1);
+        if (lane == l) { c = least; k = y; }
+    }
+    if (leader) {
+        const size_t o = (size_t)i * p + j;
+        const long long x = order_key(c), y = order_key(T.dp64[o]);
+        if (x < y || (x == y && k < (int)T.arg[o])) { T.dp64[o] = c; T.arg[o] = (uint16_t)k; }
+    }
+    __syncwarp();
+}
+
+// The listed outputs of a large closure from layer 3 up, those behind `from` in each layer's list: members are found again and
+// queued, 32 candidates at a time evaluated side by side, whatever outputs they are of.
+static __device__ __noinline__ void row_resolve_many(const RowTrace &T, int i0) {
+    const int lane = threadIdx.x & 31, p = T.p;
+    const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
+    int bad = 0;
+    for (int i = 3; i <= i0; i++) {
+        const int n0 = T.from[i], n1 = T.cnt[i];
+        const uint16_t *list = T.list + (size_t)i * p;
+        for (int e = n0 + lane; e < n1; e += 32) {
+            T.dp64[(size_t)i * p + list[e]] = CUDART_INF;
+            T.arg[(size_t)i * p + list[e]] = 0xFFFFu;
+        }
+        __syncwarp();
+        int qn = 0;
+        auto queue = [&](bool in, int j, int k) {  // whole warp
+            const unsigned m = __ballot_sync(full, in);
+            if (in) T.key[qn + __popc(m & lt)] = (uint32_t)(j << 10 | k);
+            qn += __popc(m);
+            __syncwarp();
+            if (qn >= 32) row_evaluate_pairs(T, i, qn -= 32, 32);
+        };
+        if (n1 - n0 >= kRowsWide) {
+            for (int b = n0; b < n1; b += 32) {
+                const int j = b + lane < n1 ? (int)list[b + lane] : 0, jmax = __reduce_max_sync(full, j);
+                const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
+                for (int kb = 0; kb < jmax; kb += 32) {
+                    unsigned in = row_members_of(T, i, j, kb, lim);
+                    while (__any_sync(full, in)) {
+                        queue(in != 0u, j, kb + __ffs(in) - 1);
+                        in &= in - 1u;
+                    }
+                }
+            }
+        } else {
+            for (int e = n0; e < n1; e++) {
+                const int j = list[e];
+                const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
+                for (int kb = 0; kb < j; kb += 128) {
+                    unsigned in[4];
+                    row_members(T, i, j, kb, lim, in);
+#pragma unroll 1
+                    for (int w = 0; w < 4; w++) {
+                        const unsigned x = w == 0 ? in[0] : w == 1 ? in[1] : w == 2 ? in[2] : in[3];
+                        if (x) queue((x >> lane) & 1u, j, kb + 32 * w + lane);
+                    }
+                }
+            }
+        }
+        if (qn) row_evaluate_pairs(T, i, 0, qn);
+        for (int e = n0 + lane; e < n1; e += 32) bad += row_outside(T, i, list[e], T.dp64[(size_t)i * p + list[e]]);
+    }
+    if (bad) atomicAdd(T.tally, bad);
+    __syncwarp();
+}
+
 // The exact value and lowest minimiser of output (i0, j0), i0 >= 3: its members, their members and so on
-// down to layer 3 are listed (each output once), then evaluated from layer 3 up.  One warp.  A binary64 interval
+// down to layer 3 are listed (each output once a trace), then evaluated from layer 3 up.  One warp.  A binary64 interval
 // cost is a long chain whose time 32 lanes share, so up to kRowsPairs costs of the closure (nearly
-// always all) are evaluated side by side first; larger closures go output by output.
-constexpr int kRowsPairs = 64;
+// always all) are evaluated side by side first; larger closures -- evenly spaced values tie in thousands of
+// outputs -- layer by layer (row_resolve_many).  What was resolved stays known until the trace ends (dp64, arg), so
+// that a trace evaluates an output once, not once a step: 4 rows of 107 integers at s = 64 took 261 ms output by output
+// and closure by closure, and take 4.3 (5.0 with every pair's binary64 cost kept).
 static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0, double *value) {
     const int lane = threadIdx.x & 31, p = T.p;
     const unsigned full = 0xffffffffu;
     uint16_t *cnt = T.cnt;
-    // the costs and their (i, j, k) take the layers below 3 of dp64
-    double *cost = T.dp64;
-    uint32_t *key = reinterpret_cast<uint32_t *>(T.dp64 + kRowsPairs);
-    const bool room = 3 * p >= kRowsPairs + kRowsPairs / 2;
-    int np = 0;
+    if (row_listed(T, i0, j0)) {
+        *value = T.dp64[(size_t)i0 * p + j0];
+        return T.arg[(size_t)i0 * p + j0];
+    }
+    for (int i = 3 + lane; i <= i0; i += 32) T.from[i] = cnt[i];
+    __syncwarp();
     if (lane == 0) {
-        T.list[(size_t)i0 * p] = (uint16_t)j0;
-        cnt[i0] = 1;
+        T.need[(size_t)i0 * T.nw + (j0 >> 5)] |= 1u << (j0 & 31);
+        T.list[(size_t)i0 * p + cnt[i0]++] = (uint16_t)j0;
     }
     __syncwarp();
+    int np = 0;
+    bool wide = false;
     for (int i = i0; i >= 3; i--) {
-        const int n = cnt[i];
-        int nn = 0;
-        for (int e = 0; e < n; e++) {
-            const int j = T.list[(size_t)i * p + e];
-            const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
-            for (int kb = 0; kb < j; kb += 128) {
-                unsigned in[4];
-                row_members(T, i, j, kb, lim, in);
-#pragma unroll
-                for (int w = 0; w < 4; w++) {
-                    if (!in[w]) continue;
-                    const int k = kb + 32 * w + lane, q = np + __popc(in[w] & ((1u << lane) - 1u));
-                    if (((in[w] >> lane) & 1u) && room && q < kRowsPairs) key[q] = (uint32_t)(i << 20 | j << 10 | k);
-                    np += __popc(in[w]);
-                    if (i > 3) {
-                        uint32_t *word = T.need + (size_t)(i - 1) * T.nw + (kb >> 5) + w;
-                        const unsigned fresh = in[w] & ~*word;
-                        __syncwarp();
-                        if (lane == 0) *word |= in[w];
-                        if ((fresh >> lane) & 1u)
-                            T.list[(size_t)(i - 1) * p + nn + __popc(fresh & ((1u << lane) - 1u))] = (uint16_t)k;
-                        nn += __popc(fresh);
-                    }
+        const int n0 = T.from[i], n1 = cnt[i];
+        if (n0 == n1) continue;
+        int nn = i > 3 ? cnt[i - 1] : 0;
+        if (n1 - n0 >= kRowsWide) {
+            wide = true;
+            for (int b = n0; b < n1; b += 32) {
+                const int j = b + lane < n1 ? (int)T.list[(size_t)i * p + b + lane] : 0, jmax = __reduce_max_sync(full, j);
+                const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
+                for (int kb = 0; kb < jmax; kb += 32) {
+                    const unsigned in = row_members_of(T, i, j, kb, lim), any = __reduce_or_sync(full, in);
+                    np += __reduce_add_sync(full, __popc(in));
+                    if (any && i > 3) nn = row_list(T, i - 1, kb, any, nn);
                     __syncwarp();
+                }
+            }
+        } else {
+            for (int e = n0; e < n1; e++) {
+                const int j = T.list[(size_t)i * p + e];
+                const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
+                for (int kb = 0; kb < j; kb += 128) {
+                    unsigned in[4];
+                    row_members(T, i, j, kb, lim, in);
+#pragma unroll
+                    for (int w = 0; w < 4; w++) {
+                        if (!in[w]) continue;
+                        const int k = kb + 32 * w + lane, q = np + __popc(in[w] & ((1u << lane) - 1u));
+                        if (((in[w] >> lane) & 1u) && q < kRowsPairs) T.key[q] = (uint32_t)(i << 20 | j << 10 | k);
+                        np += __popc(in[w]);
+                        if (i > 3) nn = row_list(T, i - 1, kb + 32 * w, in[w], nn);
+                        __syncwarp();
+                    }
                 }
             }
         }
         if (lane == 0 && i > 3) cnt[i - 1] = (uint16_t)nn;
         __syncwarp();
     }
+    if (lane == 0) atomicAdd(T.tally + 1, np);
+    if (wide || np > kRowsPairs) {
+        row_resolve_many(T, i0);
+        *value = T.dp64[(size_t)i0 * p + j0];
+        return T.arg[(size_t)i0 * p + j0];
+    }
+    for (int q = lane; q < np; q += 32) T.cost[q] = row_cost(T, (int)(T.key[q] & 1023u), (int)(T.key[q] >> 10 & 1023u));
+    __syncwarp();
     int arg = -1, bad = 0;
     double best = CUDART_INF;
-    if (lane == 0) atomicAdd(T.tally + 1, np);
-    if (room && np <= kRowsPairs) {
-        for (int q = lane; q < np; q += 32) cost[q] = row_cost(T, (int)(key[q] & 1023u), (int)(key[q] >> 10 & 1023u));
-        __syncwarp();
-        if (lane == 0) {
-            // the pairs were listed from the last layer down, k ascending: backwards, the lowest k comes last
-            for (int q = np - 1; q >= 0; q--) {
-                const uint32_t f = key[q];
-                const int i = (int)(f >> 20), k = (int)(f & 1023u);
-                const double c = __dadd_rn(i == 3 ? row_base(T, k) : T.dp64[(size_t)(i - 1) * p + k], cost[q]);
-                if (c <= best) { best = c; arg = k; }
-                if (q == 0 || key[q - 1] >> 10 != f >> 10) {  // the output's last: store it
-                    T.dp64[(size_t)i * p + (f >> 10 & 1023u)] = best;
-                    if (q > 0) best = CUDART_INF;
-                }
+    if (lane == 0) {
+        // the pairs were listed from the last layer down, k ascending: backwards, the lowest k comes last
+        for (int q = np - 1; q >= 0; q--) {
+            const uint32_t f = T.key[q];
+            const int i = (int)(f >> 20), k = (int)(f & 1023u);
+            const double c = __dadd_rn(i == 3 ? row_base(T, k) : T.dp64[(size_t)(i - 1) * p + k], T.cost[q]);
+            if (c <= best) { best = c; arg = k; }
+            if (q == 0 || T.key[q - 1] >> 10 != f >> 10) {  // the output's last: store it
+                const size_t o = (size_t)i * p + (f >> 10 & 1023u);
+                T.dp64[o] = best;
+                T.arg[o] = (uint16_t)arg;
+                if (q > 0) best = CUDART_INF;
             }
         }
-        best = __shfl_sync(full, best, 0);  // (dp64 is complete)
-        arg = __shfl_sync(full, arg, 0);
-        __syncwarp();
-        for (int q = lane; q < np; q += 32)
-            if (q == 0 || key[q - 1] >> 10 != key[q] >> 10) {
-                const int i = (int)(key[q] >> 20), j = (int)(key[q] >> 10 & 1023u);
-                bad += row_outside(T, i, j, T.dp64[(size_t)i * p + j]);
-            }
-        if (bad) atomicAdd(T.tally, bad);
-        for (int i = 3; i < i0; i++)
-            for (int e = lane; e < cnt[i]; e += 32) T.need[(size_t)i * T.nw + (T.list[(size_t)i * p + e] >> 5)] = 0u;
-        __syncwarp();
-        *value = best;
-        return arg;
     }
-    for (int i = 3; i <= i0; i++) {
-        const int n = cnt[i];
-        for (int e = 0; e < n; e++) {
-            const int j = T.list[(size_t)i * p + e];
-            const float lim = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
-            best = CUDART_INF;
-            arg = 0x7fffffff;
-            for (int kb = 0; kb < j; kb += 128) {
-                unsigned in[4];
-                row_members(T, i, j, kb, lim, in);
-#pragma unroll 1
-                for (int w = 0; w < 4; w++) {
-                    const unsigned x = w == 0 ? in[0] : w == 1 ? in[1] : w == 2 ? in[2] : in[3];
-                    const int k = kb + 32 * w + lane;
-                    if ((x >> lane) & 1u) {
-                        const double c = __dadd_rn(i == 3 ? row_base(T, k) : T.dp64[(size_t)(i - 1) * p + k], row_cost(T, k, j));
-                        if (c < best) { best = c; arg = k; }
-                    }
-                    __syncwarp();
-                }
-            }
-            for (int o = 16; o; o >>= 1) {
-                const double b2 = __shfl_xor_sync(full, best, o);
-                const int a2 = __shfl_xor_sync(full, arg, o);
-                if (b2 < best || (b2 == best && a2 < arg)) { best = b2; arg = a2; }
-            }
-            if (lane == 0) {
-                bad += row_outside(T, i, j, best);
-                T.dp64[(size_t)i * p + j] = best;
-                if (i < i0) T.need[(size_t)i * T.nw + (j >> 5)] = 0u;
-            }
-            __syncwarp();
+    best = __shfl_sync(full, best, 0);  // (dp64 is complete)
+    arg = __shfl_sync(full, arg, 0);
+    __syncwarp();
+    for (int q = lane; q < np; q += 32)
+        if (q == 0 || T.key[q - 1] >> 10 != T.key[q] >> 10) {
+            const int i = (int)(T.key[q] >> 20), j = (int)(T.key[q] >> 10 & 1023u);
+            bad += row_outside(T, i, j, T.dp64[(size_t)i * p + j]);
         }
-    }
     if (bad) atomicAdd(T.tally, bad);
-    *value = best;  // the last output evaluated is (i0, j0)
+    *value = best;
     return arg;
 }
 
@@ -297,11 +403,14 @@ static __device__ __noinline__ int row_trace(const RowTrace &T, int s, int ilo, 
     const unsigned full = 0xffffffffu;
     // eq. apx_final: the layers whose fp32 value is within the band of the least
     float m = CUDART_INF_F;
+    for (int i = lane; i <= s; i += 32) T.cnt[i] = 0;
+    __syncwarp();
     for (int i = ilo + lane; i <= s; i += 32) m = fminf(m, T.dp[((size_t)i * p + p - 1) * kMaxG + T.g]);
     for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(full, m, o));
     if (!(m < CUDART_INF_F)) return 0;
     const float lim = row_limit(T, s, m);
     int istar = -1, members = 0;
+    bool known = false;  // some outputs are resolved
     for (int i = ilo; i <= s; i++)
         if (!(T.dp[((size_t)i * p + p - 1) * kMaxG + T.g] > lim)) { if (!members++) istar = i; }
     if (members > 1) {
@@ -310,13 +419,18 @@ static __device__ __noinline__ int row_trace(const RowTrace &T, int s, int ilo, 
             if (T.dp[((size_t)i * p + p - 1) * kMaxG + T.g] > lim) continue;
             double v;
             if (i == 2) v = row_base(T, p - 1);
-            else row_resolve(T, i, p - 1, &v);
+            else { row_resolve(T, i, p - 1, &v); known = true; }
             if (v < best) { best = v; istar = i; }
         }
     }
     int j = p - 1;
     if (lane == 0) a[istar - 1] = j;
     for (int i = istar; i >= 3; i--) {
+        if (known && row_listed(T, i, j)) {
+            j = T.arg[(size_t)i * p + j];
+            if (lane == 0) a[i - 2] = j;
+            continue;
+        }
         const float lj = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
         int n = 0, k = 0;
         for (int kb = 0; kb < j; kb += 128) {
@@ -331,11 +445,16 @@ static __device__ __noinline__ int row_trace(const RowTrace &T, int s, int ilo, 
         if (n > 1) {
             double v;
             k = row_resolve(T, i, j, &v);
+            known = true;
         }
         j = k;
         if (lane == 0) a[i - 2] = j;
     }
     if (lane == 0) a[0] = 0;
+    __syncwarp();
+    if (known)
+        for (int i = 3; i <= s; i++)
+            for (int e = lane; e < T.cnt[i]; e += 32) T.need[(size_t)i * T.nw + (T.list[(size_t)i * p + e] >> 5)] = 0u;
     __syncwarp();
     return istar;
 }
@@ -375,7 +494,7 @@ __host__ __device__ __forceinline__ size_t rows_smem_tail(int p) {
     return rows_smem_costs(p) + sizeof(float2) * (pc * (pc - 1) / 2);
 }
 static size_t rows_pass_smem(int p, int s) {
-    return rows_smem_tail(p) + (s > 32 ? sizeof(double) * 4 * kMaxS : 0) + kMaxG * (sizeof(int32_t) * s + sizeof(uint16_t) * (s + 1));
+    return rows_smem_tail(p) + (s > 32 ? sizeof(double) * 4 * kMaxS : 0) + kMaxG * (sizeof(int32_t) * s + 2 * sizeof(uint16_t) * (s + 1));
 }
 
 // WIDE: some row has more than kRowsMaxP values; its pairs' costs stay in global memory.
@@ -399,6 +518,8 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
     double *dp64 = A.dp64 + blockIdx.x * rows_per * kMaxG;
     uint16_t *list = A.list + blockIdx.x * rows_per * kMaxG;
     uint32_t *need = A.need + blockIdx.x * (size_t)(s + 1) * nwc * kMaxG;
+    uint16_t *arg = A.arg + blockIdx.x * rows_per * kMaxG;
+    double *cost = A.cost + (size_t)blockIdx.x * kMaxG * (kRowsPairs + kRowsPairs / 2);  // kRowsPairs costs, then as many keys
     for (size_t q = tid; q < (size_t)(s + 1) * nwc * kMaxG; q += blockDim.x) need[q] = 0u;
     if (tid < 2) tally[tid] = 0;
     for (int b = blockIdx.x; b < A.nact; b += gridDim.x) {
@@ -497,7 +618,9 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
         for (int g = wid; g < G; g += nwarp) {
             const size_t o = (size_t)g * rows_per;
             const RowTrace T{P, cf, rc.c0, rc.phf, dp, dp64 + o, list + o, need + (size_t)g * (s + 1) * nwc,
-                             cnt_sm + g * (s + 1), A.tau, A.eps, lam[g], scale,
+                             arg + o, cnt_sm + g * (s + 1), cnt_sm + (kMaxG + g) * (s + 1),
+                             reinterpret_cast<uint32_t *>(cost + (size_t)g * (kRowsPairs + kRowsPairs / 2) + kRowsPairs),
+                             cost + (size_t)g * (kRowsPairs + kRowsPairs / 2), A.tau, A.eps, lam[g], scale,
                              lam32[g], slack(g), noise, p, g, (int)nwc, tally};
             const int m = row_trace(T, s, A.exact_s ? s : 2, a_sm + g * s);
             if (lane == 0) { m_sm[g] = m; A.mcount[(size_t)b * G + g] = m; }

@@ -137,3 +137,20 @@ def test_rows_without_a_codebook(E, kw):
         assert got["status"] == E.native.EINFEASIBLE and got["m"] == 0 and got["d"] == d and got["passes"] == 0
         if not kw.get("refine_max_rounds"):
             assert got["p"] == np.unique(X[r]).size
+
+
+@pytest.mark.parametrize("d,s", [(9, 5), (31, 12), (64, 16), (107, 64), (128, 40), (129, 64), (300, 33)])
+def test_rows_that_tie(E, d, s):
+    """Evenly spaced values, repeated ones and few distinct gaps: outputs tie by the thousand, layers of a closure from one
+    output to whole rows, traces that meet outputs they resolved before."""
+    rng = np.random.default_rng(d + s)
+    X = np.tile(np.arange(d, dtype=np.float32), (5, 1))
+    X[1] = X[1] * np.float32(0.1) - np.float32(d / 3)
+    X[2] = rng.integers(-d // 3, d // 3, d)
+    X[3] = np.cumsum(rng.integers(1, 3, d))
+    X[4, : d // 2] = 2 * X[4, : d // 2]
+    _same(E, X, s, lambda_=0.0)
+    _same(E, X, s, lambda_=1e-3)
+    _same(E, X, s, budget_bits=min(2.0, 0.6 * np.log2(s)))
+    enough = [x for x in X if np.unique(x).size >= s]
+    _same(E, np.stack(enough), s, budget_bits=min(3.0, 0.8 * np.log2(s)), flags=E.EXACT_S)
