@@ -274,6 +274,15 @@ static Prefix make_prefix(void *ws, const Layout &L, int64_t p, int64_t d) {
     return P;
 }
 
+// P = X: the fast DP's fp32 costs are of the size of ||X||^2 and, times a multiplier of up to 1e3 and an entropy, above it, and
+// the squares of the smallest gaps far below.  From 2^-60 to 2^60 they are what they are (no factor); beyond, the values go by a
+// power of two that brings ||X||^2 into [1, 4).  (fp32 took ||X||^2 of 4e37 for infinite, and of 1e-57 for ties.)
+static double plain_scale32(double n2) {
+    if (!(n2 > 0.0) || (n2 >= 0x1p-60 && n2 <= 0x1p60)) return 1.0;
+    const int e = ilogb(n2);
+    return ldexp(1.0, -(e & ~1));
+}
+
 // The 7 interior points of [lo, hi] from three levels of geometric midpoints
 // sqrt(a*b): correctly rounded multiply and sqrt only.
 static void midpoints7(double lo, double hi, double *t) {
@@ -531,6 +540,7 @@ int ecasq_dp_pass(const float *x, int64_t d, int32_t s, const double *lambdas, i
     rc = prepare_device(x, d, ws, L, st, &p, &n2);
     if (rc) return rc;
     Prefix P = make_prefix(ws, L, p, d);
+    P.scale32 = plain_scale32(n2);
     if (p == 1) {
         for (int g = 0; g < G; g++) {
             ECASQ_CUDA_TRY(cudaMemcpyAsync(Q_out + (size_t)g * s, P.v, 4, cudaMemcpyDeviceToDevice, st));
@@ -780,6 +790,7 @@ static int prepare_plain(const float *x, int64_t d, const ecasq_params_t *prm, v
     rc = prepare_device(x, d, ws, *L, st, &p, n2);
     if (rc) return rc;
     *P = make_prefix(ws, *L, p, d);
+    P->scale32 = plain_scale32(*n2);
     return ECASQ_OK;
 }
 

@@ -207,7 +207,8 @@ struct Prefix {
     int64_t ps;           // DP-table row stride, table_stride(p)
     int64_t nL = 1;       // first-value set L = {0..nL-1}, last-value set R = {p-nR..p-1}
     int64_t nR = 1;       // (Sec. 5); both 1 when the candidates are the unique values of x
-    double scale32 = 1.0; // grid DP: power of two that brings ||X||^2 into [1, 2) for fp32 copies
+    double scale32 = 1.0; // for fp32 copies of costs.  Permissible sets: the power of two that brings ||X||^2 into
+                          // [1, 2); P = X: 1, or outside the range that fp32 is fit for a power of four that does about that
 };
 
 // Largest permissible set whose pair costs the grid DP caches (24 bytes per pair).

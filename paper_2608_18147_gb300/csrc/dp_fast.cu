@@ -42,6 +42,7 @@
 // computed from the complementary mass.  The exact stage re-checks
 // |m32 - dp64| <= eps_i dp64 for every resolved output and counts violations.
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "cost32.cuh"
@@ -86,7 +87,8 @@ struct FastParams {
 };
 
 struct FastArgs {
-    const float *v;
+    const float *v;        // the unique values, times sc
+    double sc, sc2, isc2;  // sc: a power of two (Prefix::scale32 = sc^2); the fp32 costs are sc2 times the binary64 ones
     const float *wf;       // multiplicities as fp32 (exact below 2^24)
     const int64_t *N;
     const double *S, *S2;  // hi [p+1] | lo [p+1]
@@ -170,6 +172,10 @@ __device__ void rec_anchor(const FastArgs &a, int64_t k, int64_t j, Rec &r) {
     double nd = (double)n;
     dd dS = dd_sub(load_dd(a.S, a.p, j + 1), load_dd(a.S, a.p, k + 1));
     dd dS2 = dd_sub(load_dd(a.S2, a.p, j + 1), load_dd(a.S2, a.p, k + 1));
+    if (a.sc2 != 1.0) {
+        dS = {dS.hi * a.sc, dS.lo * a.sc};
+        dS2 = {dS2.hi * a.sc2, dS2.lo * a.sc2};
+    }
     double vk = (double)a.v[k], vj = (double)a.v[j];
     dd A = dd_sub(dS, two_prod(vk, nd));
     dd E = dd_sub(two_prod(vj, nd), dS);
@@ -1586,7 +1592,7 @@ __global__ void k_fast_base(Prefix P, FastArgs a, double *dp64, int32_t *bp) {
         double v = __dadd_rn(C, __dmul_rn(a.prm->lam64[g], phi));
         dp64[oidx(a, g, 2, j)] = v;
         bp[oidx(a, g, 2, j)] = 0;
-        a.dp32[d32(a, g, 2, j)] = __fadd_rn(__double2float_rn(v), 0.0f);  // >= +0 (no -0)
+        a.dp32[d32(a, g, 2, j)] = __fadd_rn(__double2float_rn(v * a.sc2), 0.0f);  // >= +0 (no -0)
     }
 }
 
@@ -1917,7 +1923,7 @@ __global__ void k_fill_unneeded(FastArgs a, double *dp64, int32_t *bp) {
         const int g = (int)(o / (a.ps * (a.s + 1)));
         if (i < 3 || j >= a.p || j < i - 1 || a.need[o]) continue;
         const float m32 = a.dp32[d32(a, g, i, j)];
-        if (m32 < CUDART_INF_F) { dp64[o] = (double)m32; bp[o] = -2; }
+        if (m32 < CUDART_INF_F) { dp64[o] = (double)m32 * a.isc2; bp[o] = -2; }
     }
 }
 
@@ -1941,8 +1947,8 @@ __device__ __forceinline__ bool exact_store(const FastArgs &a, int g, int i, int
     dp64[o] = best;
     bp[o] = arg == INT32_MAX ? -1 : arg;
     const float m32 = a.dp32[d32(a, g, i, j)];
-    const double e = (double)a.prm->eps[i];
-    return fabs((double)m32 - best) <= e * best * 1.0001;
+    const double e = (double)a.prm->eps[i], x = best * a.sc2;
+    return fabs((double)m32 - x) <= e * x * 1.0001;
 }
 
 __device__ __forceinline__ void count_exact(const FastArgs &a, unsigned long long nres, int nviol) {
@@ -2078,7 +2084,7 @@ static __device__ __forceinline__ void exact_big(const Prefix &P, const FastArgs
         b0 = __shfl_sync(0xffffffffu, b0, 0);
         if (lane == 0 && kb >= 0) { best = b0; arg = kb; nres++; }
         const float thr2 = b0 < CUDART_INF
-                               ? __double2float_ru(__dmul_ru(b0, __dadd_ru(1.0 + 0x1p-30, (double)a.prm->eps[i])))
+                               ? __double2float_ru(__dmul_ru(b0 * a.sc2, __dadd_ru(1.0 + 0x1p-30, (double)a.prm->eps[i])))
                                : CUDART_INF_F;
         warp_visit_band(a, g, i, j, w, thr, [&](bool in0, int64_t k, float v) {
             const bool in = in0 && v <= thr2 && (int32_t)k != kb;
@@ -2123,6 +2129,15 @@ __global__ void __launch_bounds__(128) k_exact_layer(Prefix P, FastArgs a, int i
 }
 
 // ------------------------------------------------------------------ host
+// The values times sc (exact but below 2^-126); narrow: two of them end up too close for fp32 intervals.
+__global__ void k_scale_values(const float *v, float *out, int64_t p, double sc, int *narrow) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p) return;
+    const float x = (float)((double)v[i] * sc);
+    out[i] = x;
+    if (i > 0 && !(__fsub_rn(x, (float)((double)v[i - 1] * sc)) >= 0x1p-100f)) *narrow = 1;
+}
+
 __global__ void k_weights_f32(const int64_t *w, float *wf, int64_t p) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < p) wf[i] = (float)w[i];
@@ -2258,6 +2273,24 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     a.d = P.d;
     a.ps = P.ps;
     a.invd = 1.0f / (float)P.d;  // IEEE division on the host: correctly rounded
+    a.sc = a.sc2 = a.isc2 = 1.0;
+    if (P.scale32 != 1.0) {
+        // values of another order than fp32 costs are fit for (rare, so that the wait does not matter)
+        float *vs = wsp<float>(ws, Lw.keys0);  // the sort's buffers are free now
+        int *narrow = reinterpret_cast<int *>(wsp<char>(ws, Lw.keys1)), h = 0;
+        ECASQ_CUDA_TRY(cudaMemsetAsync(narrow, 0, sizeof(int), st));
+        note_launch();
+        k_scale_values<<<(unsigned)cdiv(P.p, 256), 256, 0, st>>>(P.v, vs, P.p, sqrt(P.scale32), narrow);
+        ECASQ_LAUNCH_CHECK();
+        ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, narrow, sizeof(int), cudaMemcpyDeviceToHost, st));
+        ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
+        if (!h) {
+            a.v = vs;
+            a.sc2 = P.scale32;
+            a.sc = sqrt(a.sc2);
+            a.isc2 = 1.0 / a.sc2;
+        }
+    }
     a.G = G;
     a.s = s;
     // far tasks: all multipliers in one split while their layers' band state fits shared memory
@@ -2269,7 +2302,7 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
     band_factors(s, fp);
     for (int g = 0; g < kMaxG; g++) {
         fp.lam64[g] = g < G ? lamp[g] : 0.0;
-        fp.lam32[g] = (float)fp.lam64[g];
+        fp.lam32[g] = (float)(fp.lam64[g] * a.sc2);
     }
     size_t rows = (size_t)kMaxG * (size_t)(s + 1) * (size_t)table_stride(Lw.d);
     char *base = wsp<char>(ws, Lw.band);

@@ -82,3 +82,33 @@ def test_segments_of_several_parts_match_reference_kernel(E, mode, d, s, G, ties
         far, segments = _far_tiles(st["tiles_fetched"], (st["p"] + 63) // 64, G,
                                    torch.cuda.get_device_properties(0).multi_processor_count)
         assert far > 3 * segments
+
+
+# ||X||^2 beyond what fp32 costs hold: 1e38 (its multiples overflow), 1e63, 1e-31, 1e-57 (its gaps' squares vanish); 2^60 and 2^-60 are
+# about the ends of the range that is taken as it is.
+@pytest.mark.parametrize("mode", ["DEFAULT", "RESIDENT_COSTS", "STREAMED_COSTS"])
+@pytest.mark.parametrize("scale", [1e17, 1e30, 1e-17, 1e-30, 2.0 ** 24, 2.0 ** 26, 2.0 ** -34, 2.0 ** -36])
+def test_magnitudes_beyond_fp32_match_reference_kernel(E, mode, scale):
+    d, s = 1500, 9
+    x = (workloads.normal(d, 4).astype(np.float64) * scale).astype(np.float32)
+    x[::7] = x[0]
+    lams = [0.0, 1e-8, 1e-3, 0.1, 1.0, 1e3]
+    flags = getattr(E, mode, 0)
+    wsr, ws = E.workspace(d, s), E.workspace(d, s, flags=flags)
+    Qr, mr, metr = E.ecasq_dp_pass(x, s, lams, flags=E.DP_REFERENCE, ws=wsr)
+    Q, m, met = E.ecasq_dp_pass(x, s, lams, flags=flags | E.EXACT_TABLES, ws=ws)
+    assert E.native.ws_status(ws)["bound_viol"] == 0
+    assert m == mr
+    np.testing.assert_array_equal(Q.cpu().numpy(), Qr.cpu().numpy())
+    np.testing.assert_array_equal(met, metr)
+    tables = [[t.cpu().numpy() for t in E.ecasq_dp_tables(wsr, g, s, d)] for g in range(len(lams))]
+    for g in range(len(lams)):
+        for a, b in zip(E.ecasq_dp_tables(ws, g, s, d), tables[g]):
+            np.testing.assert_array_equal(a.cpu().numpy(), b)
+    E.ecasq_dp_pass(x, s, lams, flags=flags, ws=ws)  # what is not resolved: the fp32 values, in x's own scale
+    for g in range(len(lams)):
+        dp, bp = (t.cpu().numpy() for t in E.ecasq_dp_tables(ws, g, s, d))
+        np.testing.assert_allclose(dp[bp == -2], tables[g][0][bp == -2], rtol=1e-5)
+    got, want = (E.ecasq_solve(x, s, budget_bits=1.7, refine_max_rounds=3, flags=f) for f in (flags, E.DP_REFERENCE))
+    np.testing.assert_array_equal(got[0].cpu().numpy(), want[0].cpu().numpy())
+    assert [got[1][k] for k in ("lambda", "mse", "h_exact")] == [want[1][k] for k in ("lambda", "mse", "h_exact")]
