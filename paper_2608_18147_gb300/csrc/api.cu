@@ -1324,6 +1324,7 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
         bool done = false, failed = false;
         int sel = -1, status = ECASQ_OK, passes = 0, nlam = 0;
         bool slow = false;  // takes ecasq_solve
+        bool refused = false;  // ... as fp32 cannot take it
         int best = -1;  // the feasible evaluation the selection rule prefers so far
     };
     std::vector<Row> st_rows(rows);
@@ -1401,7 +1402,7 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
             Row &w = st_rows[act[b]];
             if (mh[(size_t)b * G] < 0) {
                 slow.push_back(act[b]);
-                w.slow = w.done = true;
+                w.slow = w.done = w.refused = true;
                 continue;
             }
             w.passes++;
@@ -1554,7 +1555,7 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
     for (int64_t r : slow) {
         ecasq_result_t one = no_codebook(d, ph[r]);
         ecasq_params_t p1 = *prm;
-        if (ph[r] <= kRowsMaxP) p1.flags |= ECASQ_DP_REFERENCE;
+        if (st_rows[r].refused) p1.flags |= ECASQ_DP_REFERENCE;
         rc = ecasq_solve(X + r * d, d, &p1, ws, roff, Q + r * s, &one, reinterpret_cast<ecasq_stream_t>(st));
         if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
         if (rc == ECASQ_EINFEASIBLE) status = rc;

@@ -2284,6 +2284,8 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
         ECASQ_LAUNCH_CHECK();
         ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, narrow, sizeof(int), cudaMemcpyDeviceToHost, st));
         ECASQ_CUDA_TRY(cudaStreamSynchronize(st));
+        // a spread that no factor brings into fp32: the reference kernel, while its time is seconds
+        if (h && P.p <= 32768) return launch_dp_reference(P, lamp, G, s, dp64, bp, st);
         if (!h) {
             a.v = vs;
             a.sc2 = P.scale32;

@@ -6,9 +6,9 @@
 //     one column a thread, k descending from the empty interval; a row is short enough that the
 //     compensated sums need no anchors: n^2 u^2 <= 2^-28) and the binary64 base costs C[0, j],
 //     Phi^first[0, j].  The row is scaled by a power of two that brings its largest magnitude
-//     into [2^30, 2^31), so that neither the costs nor lambda' overflow and two values at least
-//     2^-100 apart keep the relative bounds; a row with a smaller gap, or a multiplier beyond 2^120
-//     in that scale, is left to the caller (mcount = -1).
+//     into [2^30, 2^31), or lower where a multiplier of the first pass is beyond 2^118 then, so that
+//     neither the costs nor lambda' overflow and two values at least 2^-100 apart keep the relative bounds;
+//     a row with a smaller gap, or a later multiplier beyond 2^120, is left to the caller (mcount = -1).
 //  2. k_rows_pass: eq. apx_rec in fp32, layer by layer, eight multipliers at a time.
 //  3. The traceback, a warp per multiplier.  At an output the candidates within the certified band
 //     of the fp32 minimum hold the exact minimiser; where it is the only one, the decision is exact.
@@ -39,8 +39,11 @@ constexpr float kRowsMinGap = 0x1p-100f;
 // Pair (k, j) of a row at pair_at(k, j, p): k-major, so the lanes of a warp (consecutive j, one k) touch
 // consecutive words.
 __device__ __forceinline__ int pair_at(int k, int j, int p) { return k * p - k * (k + 1) / 2 + j - k - 1; }
-// The row's scale exponent: the largest magnitude is v[0]'s or v[p-1]'s.
-__device__ __forceinline__ int row_exp(const float *v, int p) { return 30 - ilogbf(fmaxf(fabsf(v[0]), fabsf(v[p - 1]))); }
+// The row's scale exponent for multipliers up to lam: the largest magnitude is v[0]'s or v[p-1]'s.
+__device__ __forceinline__ int row_exp(const float *v, int p, double lam) {
+    const int e = 30 - ilogbf(fmaxf(fabsf(v[0]), fabsf(v[p - 1])));
+    return lam > 0.0 ? min(e, (117 - ilogb(lam)) >> 1) : e;
+}
 
 __device__ __forceinline__ Prefix row_prefix(const RowsData &R, int64_t row, int p) {
     Prefix P;
@@ -55,8 +58,8 @@ __device__ __forceinline__ Prefix row_prefix(const RowsData &R, int64_t row, int
     return P;
 }
 
-// A row's kept costs: fp32 {C, Phi} by pair, then C[0, j] and Phi^first[0, j]; Phi^first[0, 0] (unused) is 1
-// for a row that fp32 cannot take.
+// A row's kept costs: fp32 {C, Phi} by pair, then C[0, j] and Phi^first[0, j]; Phi^first[0, 0] (unused) is its scale
+// exponent, C[0, 0] (unused) 1 for a row that fp32 cannot take.
 struct RowCosts { float2 *cf; double *c0, *phf; };
 __device__ __forceinline__ RowCosts row_costs(const RowsPass &A, int64_t row) {
     double *g = A.pairs + row * A.pstride;
@@ -70,7 +73,9 @@ __global__ void __launch_bounds__(kScanTile) k_rows_build(const RowsPass A) {
     const int p = (int)A.R.p[row];
     const Prefix P = row_prefix(A.R, row, p);
     const RowCosts rc = row_costs(A, row);
-    const int e = row_exp(P.v, p);
+    double lmax = 0.0;
+    for (int g = 0; g < A.G; g++) lmax = fmax(lmax, A.lam[(size_t)blockIdx.x * A.G + g]);
+    const int e = row_exp(P.v, p, lmax);
     for (int t = threadIdx.x; t < p; t += blockDim.x) {
         v[t] = ldexpf(P.v[t], e);
         w[t] = (float)P.w[t];
@@ -79,7 +84,10 @@ __global__ void __launch_bounds__(kScanTile) k_rows_build(const RowsPass A) {
     bool narrow = false;
     for (int t = threadIdx.x; t + 1 < p; t += blockDim.x) narrow |= !(__fsub_rn(v[t + 1], v[t]) >= kRowsMinGap);
     narrow = __syncthreads_or(narrow);
-    if (threadIdx.x == 0) rc.phf[0] = narrow ? 1.0 : 0.0;
+    if (threadIdx.x == 0) {
+        rc.phf[0] = (double)e;
+        rc.c0[0] = narrow ? 1.0 : 0.0;
+    }
     if (narrow) return;
     const float d_f = (float)P.d, invd = 1.0f / (float)P.d;
     const int lane = threadIdx.x & 31;
@@ -527,9 +535,9 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
         const int p = (int)R.p[row];
         const Prefix P = row_prefix(R, row, p);
         const RowCosts rc = row_costs(A, row);
-        const int e2 = 2 * row_exp(P.v, p);
+        const int e2 = 2 * (int)rc.phf[0];
         __syncthreads();  // the row before is done
-        if (tid == 0) refuse = rc.phf[0] != 0.0;
+        if (tid == 0) refuse = rc.c0[0] != 0.0;
         if (tid == 32) {
             scale = ldexp(1.0, e2);
             noise = __double2float_ru(ldexp(R.norm2[row], e2 - 90));

@@ -87,11 +87,13 @@ def test_segments_of_several_parts_match_reference_kernel(E, mode, d, s, G, ties
 # ||X||^2 beyond what fp32 costs hold: 1e38 (its multiples overflow), 1e63, 1e-31, 1e-57 (its gaps' squares vanish); 2^60 and 2^-60 are
 # about the ends of the range that is taken as it is.
 @pytest.mark.parametrize("mode", ["DEFAULT", "RESIDENT_COSTS", "STREAMED_COSTS"])
-@pytest.mark.parametrize("scale", [1e17, 1e30, 1e-17, 1e-30, 2.0 ** 24, 2.0 ** 26, 2.0 ** -34, 2.0 ** -36])
+@pytest.mark.parametrize("scale", [1e17, 1e30, 1e-17, 1e-30, 2.0 ** 24, 2.0 ** 26, 2.0 ** -34, 2.0 ** -36, None])
 def test_magnitudes_beyond_fp32_match_reference_kernel(E, mode, scale):
     d, s = 1500, 9
-    x = (workloads.normal(d, 4).astype(np.float64) * scale).astype(np.float32)
+    x = (workloads.normal(d, 4).astype(np.float64) * (scale or 1.0)).astype(np.float32)
     x[::7] = x[0]
+    if scale is None:  # a spread that no factor brings into fp32
+        x[1], x[2] = 3e38, -3e38
     lams = [0.0, 1e-8, 1e-3, 0.1, 1.0, 1e3]
     flags = getattr(E, mode, 0)
     wsr, ws = E.workspace(d, s), E.workspace(d, s, flags=flags)
@@ -109,6 +111,7 @@ def test_magnitudes_beyond_fp32_match_reference_kernel(E, mode, scale):
     for g in range(len(lams)):
         dp, bp = (t.cpu().numpy() for t in E.ecasq_dp_tables(ws, g, s, d))
         np.testing.assert_allclose(dp[bp == -2], tables[g][0][bp == -2], rtol=1e-5)
+        assert (bp == -2).any() or scale is None
     got, want = (E.ecasq_solve(x, s, budget_bits=1.7, refine_max_rounds=3, flags=f) for f in (flags, E.DP_REFERENCE))
     np.testing.assert_array_equal(got[0].cpu().numpy(), want[0].cpu().numpy())
     assert [got[1][k] for k in ("lambda", "mse", "h_exact")] == [want[1][k] for k in ("lambda", "mse", "h_exact")]

@@ -47,7 +47,7 @@ def test_rows_equal_the_binary64_solve(E, d, s):
         _same(E, X, s, lambda_=0.3)
 
 
-@pytest.mark.parametrize("d", [60, 128])
+@pytest.mark.parametrize("d", [60, 128, 200])
 def test_rows_at_the_ends_of_the_fp32_range(E, d):
     """Magnitudes of 1e18 and 1e-18, values 1e-30 of the largest, gaps too small for fp32 costs
     (left to the binary64 kernel) and a multiplier beyond fp32."""
