@@ -21,7 +21,7 @@ int launch_dp_fast(const Prefix &P, const double *lamp, int G, int s, void *ws, 
 int save_dp_seed(void *ws, const Layout &Lw, int64_t p, int G, int s, int g, cudaStream_t st);
 size_t resident_costs_bytes(int64_t d);
 size_t streamed_costs_bytes(int64_t d);
-int launch_rows_prepare(const float *X, int64_t rows, const RowsData &R, cudaStream_t st);
+int launch_rows_prepare(const float *X, int64_t rows, const RowsData &R, DevStatus *ds, cudaStream_t st);
 int launch_rows_finite(const float *x, int64_t n, DevStatus *ds, cudaStream_t st);
 int launch_grid_prefix(const float *P, int64_t n, const float *vX, const int64_t *NX, const double *SX,
                        const double *S2X, int64_t pX, float *v, int64_t *w, int64_t *N, double *S, double *S2,
@@ -1288,7 +1288,7 @@ static ecasq_result_t no_codebook(int64_t d, int64_t p) {
 // rows and refinement take ecasq_solve row by row, and so do one long row alone and rows of more than
 // kRowsMaxP unique values with a flag that only ecasq_solve knows.
 static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq_params_t *prm, void *ws, size_t roff,
-                            float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
+                            bool first, float *Q, int32_t *m_out, ecasq_result_t *res, cudaStream_t st) {
     const int s = prm->s;
     RowsLayout RL;
     rows_layout(d, s, rows, &RL);
@@ -1305,7 +1305,7 @@ static int solve_rows_group(const float *X, int64_t rows, int64_t d, const ecasq
     R.nonfinite = reinterpret_cast<int32_t *>(rb + RL.nonfinite);
     R.d = d;
     R.dcap = d;
-    rc = launch_rows_prepare(X, rows, R, st);
+    rc = launch_rows_prepare(X, rows, R, first ? wsp<DevStatus>(ws, 0) : nullptr, st);
     if (rc) return rc;
     std::vector<int64_t> ph(rows);
     std::vector<double> n2h(rows);
@@ -1586,11 +1586,10 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
     rows_layout(d, s, step, &RL);
     const size_t roff = align256(L1.total);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < roff + RL.total) return ECASQ_EWORKSPACE;
-    DevStatus *ds = wsp<DevStatus>(ws, 0);
-    ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
     if (step < rows) {
         // a value that is not finite refuses the call before any group's results are written
-        DevStatus h;
+        DevStatus *ds = wsp<DevStatus>(ws, 0), h;
+        ECASQ_CUDA_TRY(cudaMemsetAsync(ds, 0, sizeof(DevStatus), st));
         rc = launch_rows_finite(X, rows * d, ds, st);
         if (rc) return rc;
         ECASQ_CUDA_TRY(cudaMemcpyAsync(&h, ds, sizeof(h), cudaMemcpyDeviceToHost, st));
@@ -1599,7 +1598,8 @@ static int solve_rows_batched(const float *X, int64_t rows, int64_t d, const eca
     }
     int status = ECASQ_OK;
     for (int64_t r = 0; r < rows; r += step) {
-        rc = solve_rows_group(X + r * d, std::min(step, rows - r), d, prm, ws, roff, Q + r * s, m_out + r, res ? res + r : nullptr, st);
+        rc = solve_rows_group(X + r * d, std::min(step, rows - r), d, prm, ws, roff, r == 0, Q + r * s, m_out + r,
+                              res ? res + r : nullptr, st);
         if (rc != ECASQ_OK && rc != ECASQ_EINFEASIBLE) return rc;
         if (rc == ECASQ_EINFEASIBLE) status = rc;
     }

@@ -192,7 +192,7 @@ struct RowsPass {
     int64_t pstride;      // doubles per row
     int pairs_ready;      // the rows' interval costs are already in `pairs`
     DevStatus *st;        // bound_viol and rescored are added to
-    float tau[kMaxS + 1], eps[kMaxS + 1]; // band factors and certified errors (set by the launcher)
+    float tau[kMaxS + 1]; // band factors (set by the launcher)
 };
 
 // Prefix-sum view (App. E) used by every exact pair evaluation.

@@ -648,7 +648,9 @@ __global__ void k_hist_weights(const int64_t *N, int64_t *w, const DevStatus *st
 // then the arithmetic of k_hist_fill for a single tile (zero tile offset), so that
 // v, w, N, S, S2, p and ||X||^2 of every row equal what prepare_device gives for
 // that row alone.
-__global__ void __launch_bounds__(256) k_rows_prepare(const float *__restrict__ X, RowsData R) {
+// st, where given: the status record, which starts at zero.
+__global__ void __launch_bounds__(256) k_rows_prepare(const float *__restrict__ X, RowsData R, DevStatus *st) {
+    if (st && blockIdx.x == 0 && threadIdx.x < sizeof(DevStatus) / 8) reinterpret_cast<int64_t *>(st)[threadIdx.x] = 0;
     __shared__ uint32_t keys[kScanTile];
     __shared__ HistPart wtot[8];
     __shared__ int nonfin;
@@ -728,10 +730,11 @@ int launch_rows_finite(const float *x, int64_t n, DevStatus *ds, cudaStream_t st
     return ECASQ_OK;
 }
 
-int launch_rows_prepare(const float *X, int64_t rows, const RowsData &R, cudaStream_t st) {
+int launch_rows_prepare(const float *X, int64_t rows, const RowsData &R, DevStatus *ds, cudaStream_t st) {
     if (R.d < 1 || R.d > kScanTile) return ECASQ_EINVAL;
     note_launch();
-    k_rows_prepare<<<(unsigned)rows, 256, 0, st>>>(X, R);
+    static_assert(sizeof(DevStatus) % 8 == 0, "cleared by 64-bit words");
+    k_rows_prepare<<<(unsigned)rows, 256, 0, st>>>(X, R, ds);
     ECASQ_LAUNCH_CHECK();
     return ECASQ_OK;
 }

@@ -16,9 +16,9 @@
 //     double-double interval costs (resolve; lowest k, smallest i among exact minima).
 // The results are those of the binary64 recurrence: every output's candidate set is that of the
 // fast DP (dp_fast.cu), and an exact minimum of one candidate needs no evaluation.  The bound that this rests on is
-// checked at run time, as there: an output evaluated exactly, and every codebook's objective from its
-// binary64 metrics, has to lie within the certified error of its fp32 value (row_within; counted in
-// DevStatus::bound_viol).
+// checked at run time, as there: an output resolved, those of its closure where that is large, and every
+// codebook's objective from its binary64 metrics have to lie within the certified error of their fp32
+// values (row_within; counted in DevStatus::bound_viol).
 //
 // What bounds it: the chip has 2 binary64 operations a cycle and SM, so an interval cost for every pair
 // (8128 a row of 128 values) took 43 of 70 ms of device time for 8192 rows at s = 8; fp32 costs
@@ -58,8 +58,8 @@ __device__ __forceinline__ Prefix row_prefix(const RowsData &R, int64_t row, int
     return P;
 }
 
-// A row's kept costs: fp32 {C, Phi} by pair, then C[0, j] and Phi^first[0, j]; Phi^first[0, 0] (unused) is its scale
-// exponent, C[0, 0] (unused) 1 for a row that fp32 cannot take.
+// A row's kept costs: fp32 {C, Phi} by pair, then C[0, j] and Phi^first[0, j].  Phi^first[0, 0] (unused) is its costs' scale, C[0, 0]
+// (unused) the noise that row_within allows a layer, or -1 for a row that fp32 cannot take.
 struct RowCosts { float2 *cf; double *c0, *phf; };
 __device__ __forceinline__ RowCosts row_costs(const RowsPass &A, int64_t row) {
     double *g = A.pairs + row * A.pstride;
@@ -74,7 +74,9 @@ __global__ void __launch_bounds__(kScanTile) k_rows_build(const RowsPass A) {
     const Prefix P = row_prefix(A.R, row, p);
     const RowCosts rc = row_costs(A, row);
     double lmax = 0.0;
-    for (int g = 0; g < A.G; g++) lmax = fmax(lmax, A.lam[(size_t)blockIdx.x * A.G + g]);
+#pragma unroll
+    for (int g = 0; g < kMaxG; g++)  // (as integers: multipliers are >= 0)
+        lmax = __longlong_as_double(max(__double_as_longlong(lmax), __double_as_longlong(g < A.G ? A.lam[(size_t)blockIdx.x * A.G + g] : 0.0)));
     const int e = row_exp(P.v, p, lmax);
     for (int t = threadIdx.x; t < p; t += blockDim.x) {
         v[t] = ldexpf(P.v[t], e);
@@ -85,8 +87,8 @@ __global__ void __launch_bounds__(kScanTile) k_rows_build(const RowsPass A) {
     for (int t = threadIdx.x; t + 1 < p; t += blockDim.x) narrow |= !(__fsub_rn(v[t + 1], v[t]) >= kRowsMinGap);
     narrow = __syncthreads_or(narrow);
     if (threadIdx.x == 0) {
-        rc.phf[0] = (double)e;
-        rc.c0[0] = narrow ? 1.0 : 0.0;
+        rc.phf[0] = ldexp(1.0, 2 * e);
+        rc.c0[0] = narrow ? -1.0 : ldexp(A.R.norm2[row], 2 * e - 90);
     }
     if (narrow) return;
     const float d_f = (float)P.d, invd = 1.0f / (float)P.d;
@@ -125,7 +127,7 @@ struct RowTrace {
     uint16_t *cnt, *from;  // [s+1]: ... their number by layer; before the present closure
     uint32_t *key;         // [kRowsPairs]: pairs to evaluate
     double *cost;          // [kRowsPairs]: ... and their costs
-    const float *tau, *eps;
+    const float *tau;
     double lam, scale;
     float lam32, slack, noise;
     int p, g, nw;
@@ -135,12 +137,12 @@ __device__ __forceinline__ float row_limit(const RowTrace &T, int i, float m) {
     return __fadd_ru(__fmul_ru(m, __fadd_ru(1.0f, T.tau[i])), T.slack);
 }
 // Whether the fp32 value m32 of an output of layer i is within its certified error of the exact one, best * scale: eps_i
-// (and 2^-24 for the rounding of `best`, as the comparison is fp32), the underflow that row_limit allows for, and
-// what double-double interval costs and their sums leave, `noise` a layer: 2^-100 of N V^2 <= 2^10 ||X||^2 (V the
-// largest magnitude).
-__device__ __forceinline__ bool row_within(float m32, double best, float eps, float slack, double scale, int i, float noise) {
+// and 2^-24 for the rounding of `best`, as the comparison is fp32 (tau_i / 2 is above both; layer 2 has no band), the
+// underflow that row_limit allows for, and what double-double interval costs and their sums leave, `noise` a layer: 2^-100 of
+// N V^2 <= 2^10 ||X||^2 (V the largest magnitude).
+__device__ __forceinline__ bool row_within(float m32, double best, float tau, float slack, double scale, int i, float noise) {
     const float x = __double2float_rn(__dmul_rn(best, scale));
-    return fabsf(m32 - x) <= (eps * 1.0001f + 0x1p-24f) * x + (slack + (float)i * noise);
+    return fabsf(m32 - x) <= (i > 2 ? 0.5f * tau : 0x1.001p-23f) * x + (slack + (float)i * noise);
 }
 // Members of output (i, j) among k = kb .. kb + 127, 32 a word: candidates whose fp32 value (the forward pass's) is not
 // above the limit.  One warp; the loads of the four words are in flight together.
@@ -176,7 +178,7 @@ __device__ __forceinline__ double row_cost(const RowTrace &T, int k, int j) {
 }
 
 __device__ __forceinline__ int row_outside(const RowTrace &T, int i, int j, double best) {
-    return row_within(T.dp[((size_t)i * T.p + j) * kMaxG + T.g], best, T.eps[i], T.slack, T.scale, i, T.noise) ? 0 : 1;
+    return row_within(T.dp[((size_t)i * T.p + j) * kMaxG + T.g], best, T.tau[i], T.slack, T.scale, i, T.noise) ? 0 : 1;
 }
 
 // Whether output (i, j) is listed, and so resolved once its closure is.
@@ -187,9 +189,9 @@ __device__ __forceinline__ bool row_listed(const RowTrace &T, int i, int j) {
 __device__ __forceinline__ int row_list(const RowTrace &T, int i, int kb, unsigned any, int n) {
     const int lane = threadIdx.x & 31;
     uint32_t *word = T.need + (size_t)i * T.nw + (kb >> 5);
-    const unsigned fresh = any & ~*word;
+    const unsigned old = *word, fresh = any & ~old;
     __syncwarp();
-    if (lane == 0) *word |= any;
+    if (lane == 0) *word = old | any;
     if ((fresh >> lane) & 1u) T.list[(size_t)i * T.p + n + __popc(fresh & ((1u << lane) - 1u))] = (uint16_t)(kb + lane);
     return n + __popc(fresh);
 }
@@ -310,20 +312,21 @@ static __device__ __noinline__ void row_resolve_many(const RowTrace &T, int i0) 
 // cost is a long chain whose time 32 lanes share, so up to kRowsPairs costs of the closure (nearly
 // always all) are evaluated side by side first; larger closures -- evenly spaced values tie in thousands of
 // outputs -- layer by layer (row_resolve_many).  What was resolved stays known until the trace ends (dp64, arg), so
-// that a trace evaluates an output once, not once a step: 4 rows of 107 integers at s = 64 took 261 ms output by output
+// that a trace evaluates an output once and follows the rest of its path (row_follow): 4 rows of 107 integers at s = 64 took 261 ms output by output
 // and closure by closure, and take 4.3 (5.0 with every pair's binary64 cost kept).
-static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0, double *value) {
+// known: the trace has resolved outputs.
+static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0, bool known, double *value) {
     const int lane = threadIdx.x & 31, p = T.p;
     const unsigned full = 0xffffffffu;
     uint16_t *cnt = T.cnt;
-    if (row_listed(T, i0, j0)) {
+    if (known && row_listed(T, i0, j0)) {
         *value = T.dp64[(size_t)i0 * p + j0];
         return T.arg[(size_t)i0 * p + j0];
     }
     for (int i = 3 + lane; i <= i0; i += 32) T.from[i] = cnt[i];
     __syncwarp();
     if (lane == 0) {
-        T.need[(size_t)i0 * T.nw + (j0 >> 5)] |= 1u << (j0 & 31);
+        atomicOr(&T.need[(size_t)i0 * T.nw + (j0 >> 5)], 1u << (j0 & 31));
         T.list[(size_t)i0 * p + cnt[i0]++] = (uint16_t)j0;
     }
     __syncwarp();
@@ -375,7 +378,7 @@ static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0
     }
     for (int q = lane; q < np; q += 32) T.cost[q] = row_cost(T, (int)(T.key[q] & 1023u), (int)(T.key[q] >> 10 & 1023u));
     __syncwarp();
-    int arg = -1, bad = 0;
+    int arg = -1;
     double best = CUDART_INF;
     if (lane == 0) {
         // the pairs were listed from the last layer down, k ascending: backwards, the lowest k comes last
@@ -391,54 +394,56 @@ static __device__ __noinline__ int row_resolve(const RowTrace &T, int i0, int j0
                 if (q > 0) best = CUDART_INF;
             }
         }
+        if (row_outside(T, i0, j0, best)) atomicAdd(T.tally, 1);
     }
-    best = __shfl_sync(full, best, 0);  // (dp64 is complete)
+    best = __shfl_sync(full, best, 0);
     arg = __shfl_sync(full, arg, 0);
-    __syncwarp();
-    for (int q = lane; q < np; q += 32)
-        if (q == 0 || T.key[q - 1] >> 10 != T.key[q] >> 10) {
-            const int i = (int)(T.key[q] >> 20), j = (int)(T.key[q] >> 10 & 1023u);
-            bad += row_outside(T, i, j, T.dp64[(size_t)i * p + j]);
-        }
-    if (bad) atomicAdd(T.tally, bad);
     *value = best;
     return arg;
 }
 
+// The path from the resolved output (i, j) down to layer 3 into a[]: a closure holds every layer below, so all of it is
+// resolved; then what the trace listed is forgotten.
+static __device__ __noinline__ void row_follow(const RowTrace &T, int i, int j, int s, int32_t *a) {
+    const int lane = threadIdx.x & 31, p = T.p;
+    for (; i >= 3; i--) {
+        j = T.arg[(size_t)i * p + j];
+        if (lane == 0) a[i - 2] = j;
+    }
+    for (int l = 3 + lane; l <= s; l += 32) {
+        for (int e = 0; e < T.cnt[l]; e++) T.need[(size_t)l * T.nw + (T.list[(size_t)l * p + e] >> 5)] = 0u;
+        T.cnt[l] = 0;
+    }
+}
+
 // The codebook of multiplier T.g into a[0 .. m-1] (lane 0 writes); returns m, 0 when there is none.
-static __device__ __noinline__ int row_trace(const RowTrace &T, int s, int ilo, int32_t *a) {
+static __device__ __forceinline__ int row_trace(const RowTrace &T, int s, int ilo, int32_t *a) {
     const int lane = threadIdx.x & 31, p = T.p;
     const unsigned full = 0xffffffffu;
     // eq. apx_final: the layers whose fp32 value is within the band of the least
     float m = CUDART_INF_F;
-    for (int i = lane; i <= s; i += 32) T.cnt[i] = 0;
-    __syncwarp();
     for (int i = ilo + lane; i <= s; i += 32) m = fminf(m, T.dp[((size_t)i * p + p - 1) * kMaxG + T.g]);
     for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(full, m, o));
     if (!(m < CUDART_INF_F)) return 0;
     const float lim = row_limit(T, s, m);
     int istar = -1, members = 0;
-    bool known = false;  // some outputs are resolved
     for (int i = ilo; i <= s; i++)
         if (!(T.dp[((size_t)i * p + p - 1) * kMaxG + T.g] > lim)) { if (!members++) istar = i; }
-    if (members > 1) {
+    bool resolved = members > 1;
+    if (resolved) {
         double best = CUDART_INF;
+        bool known = false;
         for (int i = ilo; i <= s; i++) {
             if (T.dp[((size_t)i * p + p - 1) * kMaxG + T.g] > lim) continue;
             double v;
             if (i == 2) v = row_base(T, p - 1);
-            else { row_resolve(T, i, p - 1, &v); known = true; }
+            else { row_resolve(T, i, p - 1, known, &v); known = true; }
             if (v < best) { best = v; istar = i; }
         }
     }
-    int j = p - 1;
+    int j = p - 1, i = istar;
     if (lane == 0) a[istar - 1] = j;
-    for (int i = istar; i >= 3; i--) {
-        if (known && row_listed(T, i, j)) {
-            j = T.arg[(size_t)i * p + j];
-            if (lane == 0) a[i - 2] = j;
-            continue;
-        }
+    for (; i >= 3 && !resolved; i--) {
         const float lj = row_limit(T, i, T.dp[((size_t)i * p + j) * kMaxG + T.g]);
         int n = 0, k = 0;
         for (int kb = 0; kb < j; kb += 128) {
@@ -452,19 +457,33 @@ static __device__ __noinline__ int row_trace(const RowTrace &T, int s, int ilo, 
         }
         if (n > 1) {
             double v;
-            k = row_resolve(T, i, j, &v);
-            known = true;
+            row_resolve(T, i, j, false, &v);
+            resolved = true;
+            break;
         }
         j = k;
         if (lane == 0) a[i - 2] = j;
     }
+    if (resolved) row_follow(T, i, j, s, a);
     if (lane == 0) a[0] = 0;
     __syncwarp();
-    if (known)
-        for (int i = 3; i <= s; i++)
-            for (int e = lane; e < T.cnt[i]; e += 32) T.need[(size_t)i * T.nw + (T.list[(size_t)i * p + e] >> 5)] = 0u;
-    __syncwarp();
     return istar;
+}
+
+// A block's scratch of multiplier g and row_trace on it.  Not in line, and with pointers of its own: what the forward pass does
+// not need then takes none of its 80 registers (8192 rows of 128 values: 9.8 ms of passes, 10.1 otherwise).
+static __device__ __noinline__ int row_codebook(const RowsPass &A, int64_t row, int p, int g, const float2 *cf, double lam,
+                                                float lam32, float slack, double scale, float noise, uint16_t *cnt, int *tally,
+                                                int32_t *a) {
+    const size_t dc = (size_t)A.R.dcap, rows_per = (size_t)(A.s + 1) * dc, nwc = (dc + 31) / 32;
+    const size_t at = (size_t)blockIdx.x * kMaxG + g;
+    const RowCosts rc = row_costs(A, row);
+    double *cost = A.cost + at * (kRowsPairs + kRowsPairs / 2);  // kRowsPairs costs, then as many keys
+    const RowTrace T{row_prefix(A.R, row, p), cf, rc.c0, rc.phf, A.dp + blockIdx.x * rows_per * kMaxG, A.dp64 + at * rows_per,
+                     A.list + at * rows_per, A.need + at * (size_t)(A.s + 1) * nwc, A.arg + at * rows_per, cnt + g * (A.s + 1),
+                     cnt + (kMaxG + g) * (A.s + 1), reinterpret_cast<uint32_t *>(cost + kRowsPairs), cost, A.tau, lam, scale,
+                     lam32, slack, noise, p, g, (int)nwc, tally};
+    return row_trace(T, A.s, A.exact_s ? A.s : 2, a);
 }
 
 // eval_codebook_lanes for the multipliers g0 .. of one warp, `width` lanes (a power of two >= s) each: the same
@@ -514,37 +533,35 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
     __shared__ float lam32[kMaxG];
     __shared__ int refuse;
     __shared__ int tally[2];
-    __shared__ double scale;
     __shared__ float noise;
     const RowsData &R = A.R;
     const int G = A.G, s = A.s, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
-    const size_t dc = (size_t)R.dcap, rows_per = (size_t)(s + 1) * dc, nwc = (dc + 31) / 32;
+    const size_t dc = (size_t)R.dcap, rows_per = (size_t)(s + 1) * dc;
     double *scratch = reinterpret_cast<double *>(rsm + rows_smem_tail(A.pmax));
     int32_t *a_sm = reinterpret_cast<int32_t *>(scratch + (s > 32 ? 4 * kMaxS : 0));
     uint16_t *cnt_sm = reinterpret_cast<uint16_t *>(a_sm + kMaxG * s);
     float *dp = A.dp + blockIdx.x * rows_per * kMaxG;
-    double *dp64 = A.dp64 + blockIdx.x * rows_per * kMaxG;
-    uint16_t *list = A.list + blockIdx.x * rows_per * kMaxG;
-    uint32_t *need = A.need + blockIdx.x * (size_t)(s + 1) * nwc * kMaxG;
-    uint16_t *arg = A.arg + blockIdx.x * rows_per * kMaxG;
-    double *cost = A.cost + (size_t)blockIdx.x * kMaxG * (kRowsPairs + kRowsPairs / 2);  // kRowsPairs costs, then as many keys
-    for (size_t q = tid; q < (size_t)(s + 1) * nwc * kMaxG; q += blockDim.x) need[q] = 0u;
+    {
+        const size_t n = (size_t)(s + 1) * ((dc + 31) / 32) * kMaxG;
+        for (size_t q = tid; q < n; q += blockDim.x) A.need[blockIdx.x * n + q] = 0u;
+    }
     if (tid < 2) tally[tid] = 0;
+    for (int q = tid; q < kMaxG * (s + 1); q += blockDim.x) cnt_sm[q] = 0;  // (row_follow leaves it at zero)
     for (int b = blockIdx.x; b < A.nact; b += gridDim.x) {
         const int64_t row = A.rows[b];
         const int p = (int)R.p[row];
         const Prefix P = row_prefix(R, row, p);
         const RowCosts rc = row_costs(A, row);
-        const int e2 = 2 * (int)rc.phf[0];
+        const double scale = rc.phf[0];
         __syncthreads();  // the row before is done
-        if (tid == 0) refuse = rc.c0[0] != 0.0;
-        if (tid == 32) {
-            scale = ldexp(1.0, e2);
-            noise = __double2float_ru(ldexp(R.norm2[row], e2 - 90));
+        if (tid == 0) {
+            const double x = rc.c0[0];
+            refuse = x < 0.0;
+            noise = __double2float_ru(x);
         }
         if (tid < kMaxG) {
             lam[tid] = tid < G ? A.lam[(size_t)b * G + tid] : 0.0;
-            lam32[tid] = __double2float_rn(ldexp(lam[tid], e2));
+            lam32[tid] = __double2float_rn(__dmul_rn(lam[tid], scale));
         }
         __syncthreads();
         if (tid < G && !(lam32[tid] < 0x1p120f)) refuse = 1;
@@ -570,7 +587,7 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
         for (int q = tid; q < kMaxG * p; q += blockDim.x) {
             const int j = q / kMaxG, g = q % kMaxG;
             float v = CUDART_INF_F;
-            if (j >= 1) v = fmaxf(__double2float_rn(ldexp(__dadd_rn(rc.c0[j], __dmul_rn(lam[g], rc.phf[j])), e2)), 0.f) + 0.f;
+            if (j >= 1) v = fmaxf(__double2float_rn(__dmul_rn(__dadd_rn(rc.c0[j], __dmul_rn(lam[g], rc.phf[j])), scale)), 0.f) + 0.f;
             prev[q] = __float_as_int(v);
             out[q] = 0x7f800000;
             dp[(size_t)2 * p * kMaxG + q] = v;
@@ -624,13 +641,7 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
         // underflow: C and the gaps' products 2^-149 a term, Phi where y < 1e-37 2^-118 a layer
         auto slack = [&](int g) { return __fmul_ru(3.0f * (float)s, __fmaf_ru(lam32[g], 0x1p-114f, 8.0f * (float)P.d * 0x1p-149f)); };
         for (int g = wid; g < G; g += nwarp) {
-            const size_t o = (size_t)g * rows_per;
-            const RowTrace T{P, cf, rc.c0, rc.phf, dp, dp64 + o, list + o, need + (size_t)g * (s + 1) * nwc,
-                             arg + o, cnt_sm + g * (s + 1), cnt_sm + (kMaxG + g) * (s + 1),
-                             reinterpret_cast<uint32_t *>(cost + (size_t)g * (kRowsPairs + kRowsPairs / 2) + kRowsPairs),
-                             cost + (size_t)g * (kRowsPairs + kRowsPairs / 2), A.tau, A.eps, lam[g], scale,
-                             lam32[g], slack(g), noise, p, g, (int)nwc, tally};
-            const int m = row_trace(T, s, A.exact_s ? s : 2, a_sm + g * s);
+            const int m = row_codebook(A, row, p, g, cf, lam[g], lam32[g], slack(g), scale, noise, cnt_sm, tally, a_sm + g * s);
             if (lane == 0) { m_sm[g] = m; A.mcount[(size_t)b * G + g] = m; }
             for (int r = lane; r < m; r += 32) A.qidx[((size_t)b * G + g) * s + r] = a_sm[g * s + r];
         }
@@ -638,7 +649,7 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
         // the codebook's objective against the fp32 value of its last output
         auto certify = [&](int g, double objective) {
             const int m = m_sm[g];
-            if (m > 0 && !row_within(dp[((size_t)m * p + p - 1) * kMaxG + g], objective, A.eps[m], slack(g), scale, m, noise))
+            if (m > 0 && !row_within(dp[((size_t)m * p + p - 1) * kMaxG + g], objective, A.tau[m], slack(g), scale, m, noise))
                 atomicAdd(tally, 1);
         };
         if (s <= 32) {
@@ -668,7 +679,8 @@ int launch_rows_pass(const RowsPass &A, int slots, cudaStream_t st) {
     if (A.nact == 0) return ECASQ_OK;
     if (A.pmax > kScanTile) return ECASQ_EINVAL;
     RowsPass B = A;
-    band_factors(A.s, B.tau, B.eps);
+    float eps[kMaxS + 1];
+    band_factors(A.s, B.tau, eps);
     if (!A.pairs_ready) {
         note_launch();
         k_rows_build<<<(unsigned)A.nact, (unsigned)std::max(128, (A.pmax + 31) & ~31), 0, st>>>(B);
