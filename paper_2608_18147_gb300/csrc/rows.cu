@@ -638,8 +638,11 @@ __global__ void __launch_bounds__(WIDE ? kRowsThreads : 256, WIDE ? 1 : 3) k_row
             out = x;
             __syncthreads();
         }
-        // underflow: C and the gaps' products 2^-149 a term, Phi where y < 1e-37 2^-118 a layer
-        auto slack = [&](int g) { return __fmul_ru(3.0f * (float)s, __fmaf_ru(lam32[g], 0x1p-114f, 8.0f * (float)P.d * 0x1p-149f)); };
+        // underflow: C and the gaps' products 2^-149 a term, Phi where y < 1e-37 2^-118 a layer; and what the binary64 costs of
+        // an output and of its rival are off by (row_within), which decides where fp32's are exact: the rounding of ||X||^2
+        auto slack = [&](int g) {
+            return __fmul_ru(3.0f * (float)s, __fadd_ru(noise, __fmaf_ru(lam32[g], 0x1p-114f, 8.0f * (float)P.d * 0x1p-149f)));
+        };
         for (int g = wid; g < G; g += nwarp) {
             const int m = row_codebook(A, row, p, g, cf, lam[g], lam32[g], slack(g), scale, noise, cnt_sm, tally, a_sm + g * s);
             if (lane == 0) { m_sm[g] = m; A.mcount[(size_t)b * G + g] = m; }

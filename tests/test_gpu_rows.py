@@ -154,3 +154,16 @@ def test_rows_that_tie(E, d, s):
     _same(E, X, s, budget_bits=min(2.0, 0.6 * np.log2(s)))
     enough = [x for x in X if np.unique(x).size >= s]
     _same(E, np.stack(enough), s, budget_bits=min(3.0, 0.8 * np.log2(s)), flags=E.EXACT_S)
+
+
+@pytest.mark.parametrize("d,s", [(11, 64), (13, 32), (40, 33), (130, 64)])
+@pytest.mark.parametrize("kw", [dict(lambda_=0.0)])
+def test_rows_whose_least_cost_is_rounding(E, d, s, kw):
+    # magnitudes from 1e-20 to 1e17: past the last codeword that matters, double-double costs are rounding (2^-100 of ||X||^2)
+    # and tie or differ by it, where fp32's are exactly zero or ordered
+    rng = np.random.default_rng(1000 * d + s)
+    X = rng.standard_normal((24, d))
+    X[:, : d // 3] *= 1e17
+    X[:, d // 3 : d // 3 + 3] *= 1e-20
+    X[1::2] = X[1::2, ::-1] + 0.0
+    _same(E, X.astype(np.float32), s, **kw)
