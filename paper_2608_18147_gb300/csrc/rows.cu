@@ -7,8 +7,11 @@
 //     compensated sums need no anchors: n^2 u^2 <= 2^-28) and the binary64 base costs C[0, j],
 //     Phi^first[0, j].  The row is scaled by a power of two that brings its largest magnitude
 //     into [2^30, 2^31), or lower where a multiplier of the first pass is beyond 2^118 then, so that
-//     neither the costs nor lambda' overflow and two values at least 2^-100 apart keep the relative bounds;
-//     a row with a smaller gap, or a later multiplier beyond 2^120, is left to the caller (mcount = -1).
+//     neither the costs nor lambda' overflow and two values at least 2^-100 apart keep the relative bounds.
+//     A row with a smaller gap, or one below 2^-70 of its largest magnitude (an interval of that length has its
+//     Phi only as well as double-double sums have its mean), takes its binary64 costs rounded; one whose binary64
+//     costs are not costs (a mean outside its interval, an entropy below zero), or a later multiplier beyond
+//     2^120, is left to the caller (mcount = -1).
 //  2. k_rows_pass: eq. apx_rec in fp32, layer by layer, eight multipliers at a time.
 //  3. The traceback, a warp per multiplier.  At an output the candidates within the certified band
 //     of the fp32 minimum hold the exact minimiser; where it is the only one, the decision is exact.
@@ -67,6 +70,30 @@ __device__ __forceinline__ RowCosts row_costs(const RowsPass &A, int64_t row) {
     return {reinterpret_cast<float2 *>(g), c0, c0 + A.R.dcap};
 }
 
+// The binary64 costs of a row's pairs, rounded (2 binary64 operations a cycle and SM: a search of 512 rows of 128 values takes
+// 5.3 ms instead of 2.1).  C below zero is within the run-time check's noise of it.  Returns whether this thread met what is
+// no cost.
+static __device__ __noinline__ bool rows_build_rounded(const Prefix &P, const RowCosts &rc, double scale) {
+    const int p = (int)P.p;
+    bool lost = false;
+    for (int j = threadIdx.x; j < p; j += blockDim.x)
+        for (int k = 0; k < j; k++) {
+            double C, U, D;
+            pair_exact(P, k, j, C, U, D);
+            if (k == 0) {
+                rc.c0[j] = C;
+                const double F = phi_exact(P, U, D, true);
+                rc.phf[j] = F;
+                lost |= !(F >= 0.0);
+            }
+            const double F = phi_exact(P, U, D, false);
+            rc.cf[pair_at(k, j, p)] = make_float2(fmaxf(__double2float_rn(__dmul_rn(C, scale)), 0.f) + 0.f,
+                                                  __double2float_rn(F) + 0.f);
+            lost |= !(F >= 0.0);
+        }
+    return lost;
+}
+
 __global__ void __launch_bounds__(kScanTile) k_rows_build(const RowsPass A) {
     __shared__ float v[kScanTile], w[kScanTile];
     const int64_t row = A.rows[blockIdx.x];
@@ -83,12 +110,15 @@ __global__ void __launch_bounds__(kScanTile) k_rows_build(const RowsPass A) {
         w[t] = (float)P.w[t];
     }
     __syncthreads();
+    const float gap = fmaxf(kRowsMinGap, 0x1p-70f * fmaxf(fabsf(v[0]), fabsf(v[p - 1])));
     bool narrow = false;
-    for (int t = threadIdx.x; t + 1 < p; t += blockDim.x) narrow |= !(__fsub_rn(v[t + 1], v[t]) >= kRowsMinGap);
+    for (int t = threadIdx.x; t + 1 < p; t += blockDim.x) narrow |= !(__fsub_rn(v[t + 1], v[t]) >= gap);
     narrow = __syncthreads_or(narrow);
+    bool lost = false;
+    if (narrow) lost = __syncthreads_or(rows_build_rounded(P, rc, ldexp(1.0, 2 * e)));
     if (threadIdx.x == 0) {
         rc.phf[0] = ldexp(1.0, 2 * e);
-        rc.c0[0] = narrow ? -1.0 : ldexp(A.R.norm2[row], 2 * e - 90);
+        rc.c0[0] = lost ? -1.0 : ldexp(A.R.norm2[row], 2 * e - 90);
     }
     if (narrow) return;
     const float d_f = (float)P.d, invd = 1.0f / (float)P.d;

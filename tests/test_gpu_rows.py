@@ -50,7 +50,7 @@ def test_rows_equal_the_binary64_solve(E, d, s):
 @pytest.mark.parametrize("d", [60, 128, 200])
 def test_rows_at_the_ends_of_the_fp32_range(E, d):
     """Magnitudes of 1e18 and 1e-18, values 1e-30 of the largest, gaps too small for fp32 costs
-    (left to the binary64 kernel) and a multiplier beyond fp32."""
+    (binary64 costs, rounded) and a multiplier beyond fp32."""
     rng = np.random.default_rng(9)
     X = rng.standard_normal((6, d)).astype(np.float32)
     X[0] *= np.float32(1e18)
@@ -157,7 +157,7 @@ def test_rows_that_tie(E, d, s):
 
 
 @pytest.mark.parametrize("d,s", [(11, 64), (13, 32), (40, 33), (130, 64)])
-@pytest.mark.parametrize("kw", [dict(lambda_=0.0)])
+@pytest.mark.parametrize("kw", [dict(lambda_=0.0), dict(lambda_=1e-6), dict(budget_bits=1.7)])
 def test_rows_whose_least_cost_is_rounding(E, d, s, kw):
     # magnitudes from 1e-20 to 1e17: past the last codeword that matters, double-double costs are rounding (2^-100 of ||X||^2)
     # and tie or differ by it, where fp32's are exactly zero or ordered
